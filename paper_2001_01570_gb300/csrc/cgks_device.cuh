@@ -21,6 +21,9 @@
 #include <stdint.h>
 
 #include "cgks_erfcx_table.h"
+#ifndef CGKS_OPCOUNT_HOST
+#include "cgks_split.cuh"
+#endif
 #include "../../include/cgks.h"
 
 namespace cgks {
@@ -110,7 +113,10 @@ enum ReconK {
     RK_Q0 = RK_W + 7, RK_Q13 = RK_Q0 + 2, RK_Q2 = RK_Q13 + 2, RK_Q4 = RK_Q2 + 3, RK_Q5 = RK_Q4 + 2,
     RK_Q6 = RK_Q5 + 4,    // candidate values (d_k folded where one candidate carries the weight)
     RK_S0 = RK_Q6 + 4, RK_S2 = RK_S0 + 2, RK_S5 = RK_S2 + 3, RK_S6 = RK_S5 + 4,   // candidate slopes
-    RK_N = RK_S6 + 4
+    // the linear reconstruction in differences (linear_diff_rk): value, h*slope, h^2*curvature
+    RK_HALF = RK_S6 + 4, RK_MHALF, RK_M2, RK_M6TH,
+    RK_DV, RK_DS = RK_DV + 3, RK_DC = RK_DS + 3,
+    RK_N = RK_DC + 2
 };
 
 // ------------------------------------------------------------------------
@@ -143,6 +149,48 @@ __device__ __forceinline__ void linear_recon_rk(const RegK& r, double a, double 
         h2vxx = r.kfma(RK_LC + 1, AmD, r.kfma(RK_LC + 2, BmC, diff));
     }
 }
+
+#ifndef CGKS_OPCOUNT_HOST   // the host operation count takes the plain forms
+// The same reconstruction in differences of the stencil data (the notation of
+// cgks_split.cuh; 8th order: t + u = s3 + s4 - 2((d1-A) + (D-d3)) and so on):
+//   P7       = b + d2/2 - (s3+s4)/12 + (t+u)/140 + 17(p-q)/70
+//   h P7_x   = d2 - 10w/27 - (t-u)/72 - 11(p+q)/12
+//   h^2 P7_xx = (s3+s4)/2 - (t+u)/8 - 9(p-q)/4
+// (order 6: -(s3+s4)/12 + (p-q)/5;  -11w/36 - 2(p+q)/3;  (s3+s4)/2 - 3(p-q)/2).
+// The sums of order-one values cancel exactly in the differences, so the value is
+// one rounding from exact (largest error over random smooth rows 0.11e-15 against
+// 0.36e-15 of the form above) and the operations are fewer: the differences are
+// shared with the nonlinear part.
+struct RowDiffs { double d1, d2, d3, s3, s4, w, t, u, p, q; };
+
+__device__ __forceinline__ void row_diffs_rk(const RegK& r, const double Q[4], const double S[4], RowDiffs& x)
+{
+    x.d1 = r.sub(Q[1], Q[0]); x.d2 = r.sub(Q[2], Q[1]); x.d3 = r.sub(Q[3], Q[2]);
+    x.s3 = r.sub(x.d2, x.d1); x.s4 = r.sub(x.d3, x.d2);
+    x.w = r.sub(x.s4, x.s3);
+    x.t = r.kfma(RK_M2, r.sub(x.d1, S[0]), x.s3);
+    x.u = r.kfma(RK_M2, r.sub(S[3], x.d3), x.s4);
+    x.p = r.kfma(RK_MHALF, r.add(x.d1, x.d2), S[1]);
+    x.q = r.kfma(RK_MHALF, r.add(x.d2, x.d3), S[2]);
+}
+
+template <int ORDER>
+__device__ __forceinline__ void linear_diff_rk(const RegK& r, double b, double hd2, const RowDiffs& x, double& v,
+                                               double& hvx, double& h2vxx)
+{
+    const double ss = r.add(x.s3, x.s4), pm = r.sub(x.p, x.q), pp = r.add(x.p, x.q);
+    double y = r.kfma(RK_DV + 1, pm, r.kfma(RK_DV + 0, ss, hd2));
+    hvx = r.kfma(RK_DS + 1, pp, r.kfma(RK_DS + 0, x.w, x.d2));
+    h2vxx = r.kfma(RK_HALF, ss, r.kmul(RK_DC + 0, pm));
+    if constexpr (ORDER != 6) {
+        const double tu = r.add(x.t, x.u);
+        y = r.kfma(RK_DV + 2, tu, y);
+        hvx = r.kfma(RK_DS + 2, r.sub(x.t, x.u), hvx);
+        h2vxx = r.kfma(RK_DC + 1, tu, h2vxx);
+    }
+    v = r.add(b, y);
+}
+#endif
 
 // ------------------------------------------------------------------------
 // Sec. 3.3: nonlinear compact reconstruction.  With d1 = b-a, d2 = c-b,
@@ -249,42 +297,90 @@ __device__ __forceinline__ void weno_pair_rk(const RegK& r, double a, double b, 
     sr = -s;
 }
 
+#ifndef CGKS_OPCOUNT_HOST
+// The pair of one row: the split form of cgks_split.cuh where it loses nothing
+// (split_ok), else the FP64 form above.  Same outputs as weno_pair_rk.
+template <int ORDER>
+__device__ __forceinline__ void weno_pair_row(const RegK& r, const double Q[4], const double S[4], const RowDiffs& x,
+                                              double hd2, double eps, int scale_hi, double& vl, double& sl,
+                                              double& vr, double& sr)
+{
+    if (split_ok(scale_hi, eps, x.w, x.t, x.u, x.p, x.q, x.s3)) {
+        const ff e = ff_from(eps);
+        DiffData m{ff_from(x.d2), ff_from(x.s3), ff_from(x.s4), ff_from(x.w), ff_from(x.t), ff_from(x.u),
+                   ff_from(x.p), ff_from(x.q)};
+        ff dv, ds;
+        weno_side_split<ORDER>(m, e, dv, ds);
+        vl = r.add(Q[1], r.add(r.kfma(RK_M6TH, x.s3, hd2), r.add(d_from(dv.h), d_from(dv.l))));
+        sl = r.add(x.d2, r.add(d_from(ds.h), d_from(ds.l)));
+        // the right-biased side is the left-biased one of the mirrored row
+        m = DiffData{ff_neg(m.d2), m.s4, m.s3, ff_neg(m.w), m.u, m.t, ff_neg(m.q), ff_neg(m.p)};
+        weno_side_split<ORDER>(m, e, dv, ds);
+        vr = r.add(Q[2], r.add(r.kfma(RK_M6TH, x.s4, -hd2), r.add(d_from(dv.h), d_from(dv.l))));
+        sr = r.sub(x.d2, r.add(d_from(ds.h), d_from(ds.l)));
+    } else {
+        weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], eps, vl, sl, vr, sr);
+    }
+}
+#endif
+
 // ------------------------------------------------------------------------
 // Characteristic variables (Sec. 3.2 allows them for the reconstruction):
 // eigenvectors of the normal Euler flux Jacobian in the face frame at the state
 // W (rho, m_n, m_t, E); fields 0: U-c, 1: entropy, 2: shear, 3: U+c.
 struct CharState { double U, V, c, H, q2, b1, b2, ic; };
 
-__device__ __forceinline__ void char_state(const double W[4], double gamma, CharState& s)
+// (every operation in an explicitly rounded form, so that each kernel that inlines
+// the characteristic path gets the same bits)
+__device__ __forceinline__ void char_state(const RegK& r, const double W[4], double gamma, CharState& s)
 {
-    const double ir = __drcp_rn(W[0]);
-    s.U = W[1] * ir;
-    s.V = W[2] * ir;
-    s.q2 = s.U * s.U + s.V * s.V;
-    const double p = (gamma - 1.0) * (W[3] - 0.5 * W[0] * s.q2);
-    s.c = sqrt(gamma * p * ir);
+    const double ir = __drcp_rn(W[0]), gm1 = r.sub(gamma, r.one);
+    s.U = r.mul(W[1], ir);
+    s.V = r.mul(W[2], ir);
+    s.q2 = fma(s.V, s.V, r.mul(s.U, s.U));
+    const double p = r.mul(gm1, fma(r.mul(-0.5, W[0]), s.q2, W[3]));
+    s.c = __dsqrt_rn(r.mul(r.mul(gamma, p), ir));
     s.ic = __drcp_rn(s.c);
-    s.H = (W[3] + p) * ir;
-    s.b2 = (gamma - 1.0) * s.ic * s.ic;
-    s.b1 = 0.5 * s.b2 * s.q2;
+    s.H = r.mul(r.add(W[3], p), ir);
+    s.b2 = r.mul(r.mul(gm1, s.ic), s.ic);
+    s.b1 = r.mul(r.mul(0.5, s.b2), s.q2);
 }
 
 // row m of the left eigenvector matrix
-__device__ __forceinline__ void char_left_row(const CharState& s, int m, double l[4])
+__device__ __forceinline__ void char_left_row(const RegK& r, const CharState& s, int m, double l[4])
 {
-    if (m == 0) { l[0] = 0.5 * (s.b1 + s.U * s.ic); l[1] = -0.5 * (s.b2 * s.U + s.ic); l[2] = -0.5 * s.b2 * s.V; l[3] = 0.5 * s.b2; }
-    else if (m == 1) { l[0] = 1.0 - s.b1; l[1] = s.b2 * s.U; l[2] = s.b2 * s.V; l[3] = -s.b2; }
-    else if (m == 2) { l[0] = -s.V; l[1] = 0.0; l[2] = 1.0; l[3] = 0.0; }
-    else { l[0] = 0.5 * (s.b1 - s.U * s.ic); l[1] = -0.5 * (s.b2 * s.U - s.ic); l[2] = -0.5 * s.b2 * s.V; l[3] = 0.5 * s.b2; }
+    if (m == 0 || m == 3) {
+        const double ic = m == 0 ? s.ic : -s.ic, hb = r.mul(0.5, s.b2);
+        l[0] = r.mul(0.5, fma(s.U, ic, s.b1));
+        l[1] = r.mul(-0.5, fma(s.b2, s.U, ic));
+        l[2] = r.mul(-hb, s.V);
+        l[3] = hb;
+    } else if (m == 1) {
+        l[0] = r.sub(r.one, s.b1);
+        l[1] = r.mul(s.b2, s.U);
+        l[2] = r.mul(s.b2, s.V);
+        l[3] = -s.b2;
+    } else {
+        l[0] = -s.V; l[1] = 0.0; l[2] = 1.0; l[3] = 0.0;
+    }
+}
+
+// l . (q0, q1, q2, q3) for row m of the left eigenvectors
+__device__ __forceinline__ double char_project(const RegK& r, int m, const double l[4], double q0, double q1, double q2,
+                                               double q3)
+{
+    if (m == 2) return fma(l[0], q0, q2);   // the shear field: (-V, 0, 1, 0)
+    return fma(l[3], q3, fma(l[2], q2, fma(l[1], q1, r.mul(l[0], q0))));
 }
 
 // conservative = R . characteristic
-__device__ __forceinline__ void char_to_cons(const CharState& s, const double w[4], double out[4])
+__device__ __forceinline__ void char_to_cons(const RegK& r, const CharState& s, const double w[4], double out[4])
 {
-    out[0] = w[0] + w[1] + w[3];
-    out[1] = (s.U - s.c) * w[0] + s.U * w[1] + (s.U + s.c) * w[3];
-    out[2] = s.V * (w[0] + w[1] + w[3]) + w[2];
-    out[3] = (s.H - s.U * s.c) * w[0] + 0.5 * s.q2 * w[1] + s.V * w[2] + (s.H + s.U * s.c) * w[3];
+    const double sum = r.add(w[0], w[3]), dif = r.mul(s.c, r.sub(w[3], w[0]));
+    out[0] = r.add(sum, w[1]);
+    out[1] = fma(s.U, out[0], dif);
+    out[2] = fma(s.V, out[0], w[2]);
+    out[3] = fma(s.U, dif, fma(s.H, sum, fma(r.mul(0.5, s.q2), w[1], r.mul(s.V, w[2]))));
 }
 
 }  // namespace cgks

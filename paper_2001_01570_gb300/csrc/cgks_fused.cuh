@@ -146,8 +146,10 @@ struct FusedTile {
                 double Qv[4], S[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) { Qv[c] = cell(c, pv); S[c] = rr.mul(h, cell(c, gn + pv)); }
-                if (G.order == 6) cons_record<6>(rr, Qv, S, ih, G.weno_eps, inner, k, out);
-                else cons_record<8>(rr, Qv, S, ih, G.weno_eps, inner, k, out);
+                const bool mom = inner && (k == 1 || k == 2);
+                const int sc = scale_of(k, Qv[1], Qv[2], mom ? cell(1, 0) : 0.0, mom ? cell(1, 3) : 0.0);
+                if (G.order == 6) cons_record<6>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
+                else cons_record<8>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
             } else {
                 double Qa[4][4], Sa[4][4];
 #pragma unroll
@@ -289,8 +291,10 @@ struct FusedTile {
                 double Qv[4], S[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) { Qv[c] = cell(c, pv); S[c] = rr.mul(h, cell(c, gn + pv)); }
-                if (G.order == 6) cons_record<6>(rr, Qv, S, ih, G.weno_eps, inner, k, out);
-                else cons_record<8>(rr, Qv, S, ih, G.weno_eps, inner, k, out);
+                const bool mom = inner && (k == 1 || k == 2);
+                const int sc = scale_of(k, Qv[1], Qv[2], mom ? cell(1, 0) : 0.0, mom ? cell(1, 3) : 0.0);
+                if (G.order == 6) cons_record<6>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
+                else cons_record<8>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
             } else {
                 double Qa[4][4], Sa[4][4];
 #pragma unroll

@@ -122,7 +122,10 @@ inline int tile_h(int s) { static const int v[TILE_COUNT] = {CGKS_FOR_EACH_TILE(
 #undef CGKS_TILE_W
 #undef CGKS_TILE_H
 
-// the record kernel's work queue: chunks of 256 (record, variable) items of one
+// the record kernel's CTA and chunk: one warp per FP64 unit of an SM, so that a
+// small grid's items spread over the SMs one warp per unit
+constexpr int kRecordChunk = 128;
+// the record kernel's work queue: chunks of kRecordChunk (record, variable) items of one
 // grid (one record per item in characteristic mode); TileRef.x0 is the first item
 std::vector<TileRef> record_chunks(int nx, int ny, int dim, int recon_vars, int grid);
 // the update kernel's work queue: chunks of 256 cells of one grid (TileRef.x0
@@ -146,11 +149,11 @@ inline int stage_blocks(int ntiles, int nsm)
     return ntiles < kStageCtasPerSm * nsm ? ntiles : kStageCtasPerSm * nsm;
 }
 
-// persistent grid of the record kernel: its resident CTAs (two per SM with
-// conservative variables, one with characteristic ones), at most one per chunk
+// persistent grid of the record kernel: its resident CTAs (four per SM with
+// conservative variables, two with characteristic ones), at most one per chunk
 inline int record_blocks(int nchunks, int nsm, int char_vars)
 {
-    const int cap = (char_vars ? 1 : 2) * nsm;
+    const int cap = (char_vars ? 2 : 4) * nsm;
     return nchunks < cap ? nchunks : cap;
 }
 

@@ -29,7 +29,7 @@ constexpr int kMaxSide = CGKS_NOALLOC_MAX_SIDE;
 // face-row records of the largest admissible grid: 2 nx ny + 5 (nx + ny) + 8
 // rows is largest for nx ny = kMaxCells with one side at kMaxSide
 constexpr size_t kMaxRecordRows = 2 * kMaxCells + 5 * ((size_t)kMaxSide + kMaxCells / kMaxSide) + 8;
-constexpr int kMaxChunks = (int)((4 * kMaxRecordRows + 255) / 256);
+constexpr int kMaxChunks = (int)((4 * kMaxRecordRows + cgks::kRecordChunk - 1) / cgks::kRecordChunk);
 // face results: 16 per face, (nx+1) ny + nx (ny+1) faces
 constexpr size_t kMaxFaces = 2 * kMaxCells + (size_t)kMaxSide + kMaxCells / kMaxSide;
 constexpr int kMaxCellChunks = (int)((kMaxCells + 255) / 256);
@@ -97,7 +97,7 @@ __global__ void noalloc_init_kernel(cgks::GridDev G, int tw, int th, int nchunks
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntx * nty; t += gridDim.x * blockDim.x)
         g_tiles[t] = cgks::TileRef{0, (t % ntx) * tw, (t / ntx) * th, 0};
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nchunks; c += gridDim.x * blockDim.x)
-        g_rchunks[c] = cgks::TileRef{0, 256 * c, 0, 0};
+        g_rchunks[c] = cgks::TileRef{0, cgks::kRecordChunk * c, 0, 0};
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncchunks; c += gridDim.x * blockDim.x)
         g_cchunks[c] = cgks::TileRef{0, 256 * c, 0, 0};
 }
@@ -187,7 +187,7 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     const int nt = (int)ntiles;
     const int cv = prob->recon_vars;
     const long long items = (long long)(cv ? 1 : 4) * record_rows(prob->nx, prob->ny, 2);
-    const int nrc = (int)((items + 255) / 256);
+    const int nrc = (int)((items + kRecordChunk - 1) / kRecordChunk);
     const int ncc = (int)((cells + 255) / 256);
     const int work = nt > nrc ? nt : nrc;
     noalloc_init_kernel<<<(work + 255) / 256, 256, 0, stream>>>(G, tw, th, nrc, ncc);

@@ -20,8 +20,16 @@ __constant__ ReconTab kReconTab = make_recon_tab();
 // CHAR = 0: conservative variables, one (record, variable) per thread;
 // CHAR = 1: characteristic variables, one record (all four variables) per thread.
 // The reconstruction order is per grid (a uniform branch per chunk).
+// Bound by the FP64 unit and FP32 issue together: about 55 FP64 instructions of 68
+// cycles per warp (differences, linear reconstruction, the sums that bring the
+// corrections back) beside some 1,900 FP32 and integer ones of the split WENO-Z
+// pair (cgks_split.cuh); rows that fail split_ok take 240 more FP64 instructions.
+// Measured per stage on the 2048^2 vortex: 15.73 ms with the pair in FP64, 4.08 ms;
+// 512^2: 1.010 -> 0.333 ms; 97x61 (three warps per FP64 unit): 44.5 -> 17.5 us.
+// CTAs of 128 threads, four per SM: one of 256 left a small grid's items on half
+// of the SMs (100 cells in 1D: 24.7 us; spread over twice the CTAs: 20.9).
 template <int STAGE, int CHAR>
-__global__ void __launch_bounds__(256, CHAR ? 1 : 2) records_kernel(const GridDev* __restrict__ grids,
+__global__ void __launch_bounds__(kRecordChunk, CHAR ? 2 : 4) records_kernel(const GridDev* __restrict__ grids,
                                                                     const TileRef* __restrict__ chunks, int nchunks,
                                                                     const int* __restrict__ dcount)
 {
@@ -56,7 +64,7 @@ std::vector<TileRef> record_chunks(int nx, int ny, int dim, int recon_vars, int 
 {
     const long long items = (long long)(recon_vars ? 1 : 4) * record_rows(nx, ny, dim);
     std::vector<TileRef> c;
-    for (long long s = 0; s < items; s += 256) c.push_back(TileRef{grid, (int)s, 0, 0});
+    for (long long s = 0; s < items; s += kRecordChunk) c.push_back(TileRef{grid, (int)s, 0, 0});
     return c;
 }
 
@@ -65,11 +73,11 @@ cudaError_t launch_records(int stage, int char_vars, const GridDev* grids, const
 {
     if (nchunks <= 0 || nblocks <= 0) return cudaSuccess;
     if (char_vars) {
-        if (stage == 1) records_kernel<1, 1><<<nblocks, 256, 0, st>>>(grids, chunks, nchunks, dcount);
-        else records_kernel<2, 1><<<nblocks, 256, 0, st>>>(grids, chunks, nchunks, dcount);
+        if (stage == 1) records_kernel<1, 1><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
+        else records_kernel<2, 1><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
     } else {
-        if (stage == 1) records_kernel<1, 0><<<nblocks, 256, 0, st>>>(grids, chunks, nchunks, dcount);
-        else records_kernel<2, 0><<<nblocks, 256, 0, st>>>(grids, chunks, nchunks, dcount);
+        if (stage == 1) records_kernel<1, 0><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
+        else records_kernel<2, 0><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
     }
     return cudaGetLastError();
 }

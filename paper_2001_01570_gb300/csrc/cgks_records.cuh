@@ -93,6 +93,11 @@ constexpr ReconTab make_recon_tab()
             k[RK_LS + 3] = -99.0 / 108.0;
             k[RK_LC + 0] = 1.0; k[RK_LC + 1] = -0.25; k[RK_LC + 2] = -2.25;
         }
+        k[RK_HALF] = 0.5; k[RK_MHALF] = -0.5; k[RK_M2] = -2.0; k[RK_M6TH] = -1.0 / 6.0;
+        k[RK_DV + 0] = -1.0 / 12.0; k[RK_DV + 1] = six ? 0.2 : 17.0 / 70.0; k[RK_DV + 2] = six ? 0.0 : 1.0 / 140.0;
+        k[RK_DS + 0] = six ? -11.0 / 36.0 : -10.0 / 27.0; k[RK_DS + 1] = six ? -2.0 / 3.0 : -11.0 / 12.0;
+        k[RK_DS + 2] = six ? 0.0 : -1.0 / 72.0;
+        k[RK_DC + 0] = six ? -1.5 : -2.25; k[RK_DC + 1] = six ? 0.0 : -0.125;
         const double e0[3] = {16.0 / 3.0, -38.0 / 3.0, 25.0 / 3.0};
         const double e1[6] = {801.0 / 80.0, -2443.0 / 80.0, 761.0 / 80.0, 23627.0 / 960.0, -7769.0 / 480.0,
                               3443.0 / 960.0};
@@ -133,25 +138,52 @@ constexpr ReconTab make_recon_tab()
 // The arithmetic of one record in conservative variables: variable k from its
 // four stencil cells (values Q, h times the normal gradients S), written through
 // out(field, k, value); the WENO-Z fields only where `inner` (the rows the
-// non-equilibrium states are needed on).
+// non-equilibrium states are needed on).  scale_hi: see scale_of.
 template <int ORDER, class Out>
 __device__ __forceinline__ void cons_record(const RegK& r, const double Q[4], const double S[4], double ih,
-                                            double weno_eps, bool inner, int k, Out out)
+                                            double weno_eps, bool inner, int k, int scale_hi, Out out)
 {
     double v, hvx, h2vxx;
+#ifdef CGKS_OPCOUNT_HOST
     linear_recon_rk<ORDER>(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], v, hvx, h2vxx);
+#else
+    RowDiffs x;
+    row_diffs_rk(r, Q, S, x);
+    const double hd2 = r.kmul(RK_HALF, x.d2);
+    linear_diff_rk<ORDER>(r, Q[1], hd2, x, v, hvx, h2vxx);
+#endif
     out(RV, k, v);
     out(RN, k, r.mul(hvx, ih));
     out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
     if (inner) {
         double vl, sl, vr, sr;
+#ifdef CGKS_OPCOUNT_HOST
         weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, vl, sl, vr, sr);
+#else
+        weno_pair_row<ORDER>(r, Q, S, x, hd2, weno_eps, scale_hi, vl, sl, vr, sr);
+#endif
         out(RL, k, vl);
         out(RR, k, vr);
         out(RLN, k, r.mul(sl, ih));
         out(RRN, k, r.mul(sr, ih));
     }
 }
+
+#ifdef CGKS_OPCOUNT_HOST
+inline int scale_of(int, double, double, double, double) { return 0; }
+#else
+// High word of the scale a variable's rounding is measured against: density and
+// energy against the values on the face's two sides (b, c); a momentum also
+// against sqrt(rho E) (its high word: the mean of the two), the momentum whose
+// changes the pressure fluxes' last bits amount to -- a gas at rest has no
+// momentum of its own to measure against.
+__device__ __forceinline__ int scale_of(int k, double b, double c, double rho, double E)
+{
+    int s = i_max(hi_abs(b), hi_abs(c));
+    if (k == 1 || k == 2) s = i_max(s, (int)(((unsigned)hi_abs(rho) + (unsigned)hi_abs(E)) >> 1));
+    return s;
+}
+#endif
 
 // The arithmetic of one record in characteristic variables: all four variables
 // from the stencil cells' values Qa[var][cell] and h times normal gradients
@@ -162,12 +194,18 @@ __device__ __forceinline__ void char_record(const RegK& r, double gamma, const d
 {
     double Wref[4];
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) Wref[kk] = 0.5 * (Qa[kk][1] + Qa[kk][2]);
+    for (int kk = 0; kk < 4; ++kk) Wref[kk] = r.mul(0.5, r.add(Qa[kk][1], Qa[kk][2]));
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         double v, hvx, h2vxx;
+#ifdef CGKS_OPCOUNT_HOST
         linear_recon_rk<ORDER>(r, Qa[k][0], Qa[k][1], Qa[k][2], Qa[k][3], Sa[k][0], Sa[k][1], Sa[k][2], Sa[k][3], v,
                                hvx, h2vxx);
+#else
+        RowDiffs x;
+        row_diffs_rk(r, Qa[k], Sa[k], x);
+        linear_diff_rk<ORDER>(r, Qa[k][1], r.kmul(RK_HALF, x.d2), x, v, hvx, h2vxx);
+#endif
         out(RV, k, v);
         out(RN, k, r.mul(hvx, ih));
         out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
@@ -176,32 +214,40 @@ __device__ __forceinline__ void char_record(const RegK& r, double gamma, const d
     // project on the left eigenvectors of the normal flux Jacobian at the
     // mean of the two cells sharing the face, WENO-Z per field, map back
     CharState cs;
-    char_state(Wref, gamma, cs);
+    char_state(r, Wref, gamma, cs);
     double cvl[4], csl[4], cvr[4], csr[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         double l[4], Q[4], S[4];
-        char_left_row(cs, m, l);
+        char_left_row(r, cs, m, l);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            Q[c] = l[0] * Qa[0][c] + l[1] * Qa[1][c] + l[2] * Qa[2][c] + l[3] * Qa[3][c];
-            S[c] = l[0] * Sa[0][c] + l[1] * Sa[1][c] + l[2] * Sa[2][c] + l[3] * Sa[3][c];
+            Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
+            S[c] = char_project(r, m, l, Sa[0][c], Sa[1][c], Sa[2][c], Sa[3][c]);
         }
+#ifdef CGKS_OPCOUNT_HOST
         weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, cvl[m], csl[m], cvr[m], csr[m]);
+#else
+        // every characteristic field is measured against the density, whose dimension it has
+        RowDiffs x;
+        row_diffs_rk(r, Q, S, x);
+        weno_pair_row<ORDER>(r, Q, S, x, r.kmul(RK_HALF, x.d2), weno_eps, hi_abs(Wref[0]), cvl[m], csl[m], cvr[m],
+                             csr[m]);
+#endif
         csl[m] = r.mul(csl[m], ih);
         csr[m] = r.mul(csr[m], ih);
     }
     double o4[4];
-    char_to_cons(cs, cvl, o4);
+    char_to_cons(r, cs, cvl, o4);
 #pragma unroll
     for (int k = 0; k < 4; ++k) out(RL, k, o4[k]);
-    char_to_cons(cs, cvr, o4);
+    char_to_cons(r, cs, cvr, o4);
 #pragma unroll
     for (int k = 0; k < 4; ++k) out(RR, k, o4[k]);
-    char_to_cons(cs, csl, o4);
+    char_to_cons(r, cs, csl, o4);
 #pragma unroll
     for (int k = 0; k < 4; ++k) out(RLN, k, o4[k]);
-    char_to_cons(cs, csr, o4);
+    char_to_cons(r, cs, csr, o4);
 #pragma unroll
     for (int k = 0; k < 4; ++k) out(RRN, k, o4[k]);
 }
@@ -214,7 +260,8 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
     const RowRef q = row_ref(G, row);
     if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
     const int pv = q.xo ? k : ((k == 1) ? 2 : (k == 2) ? 1 : k);   // face frame: normal momentum first
-    double Q[4], S[4];
+    double Q[4], S[4], rho = 0.0, E = 0.0;   // rho, E: cell b's, where a momentum's scale needs them
+    const bool mom = k == 1 || k == 2;
     const int i3 = q.i0 + 3 * q.di, j3 = q.j0 + 3 * q.dj;
     if (q.i0 >= 0 && q.j0 >= 0 && i3 < G.nx && j3 < G.ny) {
         // stencil inside the grid: no boundary mapping
@@ -223,6 +270,11 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
         const size_t step = q.di ? 1 : (size_t)G.nx;
 #pragma unroll
         for (int c = 0; c < 4; ++c) { Q[c] = __ldg(v + c * step); S[c] = r.mul(q.h, __ldg(d + c * step)); }
+        if (mom && q.inner) {
+            const double* b = src + (size_t)q.j0 * G.nx + q.i0 + step;
+            rho = __ldg(b);
+            E = __ldg(b + 3 * PL);
+        }
     } else {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -230,10 +282,14 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
             Q[c] = cell_value(G, src, PL, i, j, pv);
             S[c] = r.mul(q.h, cell_value(G, src, PL, i, j, q.gn + pv));
         }
+        if (mom && q.inner) {
+            rho = cell_value(G, src, PL, q.i0 + q.di, q.j0 + q.dj, 0);
+            E = cell_value(G, src, PL, q.i0 + q.di, q.j0 + q.dj, 3);
+        }
     }
     double* o = q.base + q.idx;
     const size_t st = q.stride;
-    cons_record<ORDER>(r, Q, S, q.ih, G.weno_eps, q.inner, k,
+    cons_record<ORDER>(r, Q, S, q.ih, G.weno_eps, q.inner, k, scale_of(k, Q[1], Q[2], rho, E),
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
 
