@@ -39,15 +39,6 @@ cgks_status cuda_fail(cudaError_t e, const char* where)
         if (e_ != cudaSuccess) return cuda_fail(e_, #call);  \
     } while (0)
 
-std::vector<TileRef> make_tiles(int nx, int ny, int shape, int grid)
-{
-    const int tw = tile_w(shape), th = tile_h(shape);
-    std::vector<TileRef> t;
-    for (int y0 = 0; y0 < ny; y0 += th)
-        for (int x0 = 0; x0 < nx; x0 += tw) t.push_back(TileRef{grid, x0, y0, 0});
-    return t;
-}
-
 cgks_status validate(const cgks_problem* p)
 {
     if (!p) return fail(CGKS_E_INVAL, "problem is NULL");
@@ -86,21 +77,8 @@ cgks_status read_ctrl(cgks_solver* s, Ctrl* c)
     return CGKS_OK;
 }
 
-// The flux kernel's tile shape for a grid: 64x1 in 1D; in 2D 8x16 (two face segments per thread of
-// the 128-thread CTA) or 14x8 (1.75), whichever needs less time over the passes of the persistent
-// grid (two CTAs per SM): on 2048^2, where partial passes do not matter, a pass of 14x8 tiles takes
-// 0.883 of a pass of 8x16 tiles (27.67 ms for 107.8 passes against 28.05 ms for 123.8), so 8x16
-// wins on large grids and 14x8 where it needs no more passes than 8x16 (256^2: 2 passes each).
-int pick_shape(const cgks_problem& p, int nsm)
-{
-    if (p.dim == 1) return TILE_64x1;
-    const long long cap = 2LL * (nsm > 0 ? nsm : 1);
-    auto passes = [&](int tx, int ty) {
-        const long long tiles = (long long)((p.nx + tx - 1) / tx) * ((p.ny + ty - 1) / ty);
-        return (double)((tiles + cap - 1) / cap);
-    };
-    return 0.883 * passes(14, 8) < passes(8, 16) ? TILE_14x8 : TILE_8x16;
-}
+// The flux kernel's tile shape for a grid: 64x1 in 1D, 8x16 in 2D.
+int pick_shape(const cgks_problem& p) { return p.dim == 1 ? TILE_64x1 : TILE_8x16; }
 
 }  // namespace
 
@@ -147,6 +125,17 @@ void fill_grid_desc(const cgks_problem& p, double* planes, double* records, doub
         G.inflow[side][2] = r * v;
         G.inflow[side][3] = pr / (p.gamma - 1.0) + 0.5 * r * (u * u + v * v);
     }
+}
+
+std::vector<TileRef> make_tiles(int nx, int ny, int dim, int shape, int grid, bool last_faces)
+{
+    const int tw = tile_w(shape), th = tile_h(shape);
+    std::vector<TileRef> t;
+    const int xn = nx + (last_faces ? 1 : 0), yn = ny + (last_faces && dim == 2 ? 1 : 0);
+    for (int y0 = 0; y0 < yn; y0 += th)
+        for (int x0 = 0; x0 < xn; x0 += tw)
+            if (x0 < nx || y0 < ny) t.push_back(TileRef{grid, x0, y0, 0});
+    return t;
 }
 
 size_t grid_device_bytes(const cgks_problem& p)
@@ -209,7 +198,7 @@ cgks_status cgks_create(const cgks_problem* prob, void* cuda_stream, cgks_solver
     s->stream = (cudaStream_t)cuda_stream;
     cudaError_t e = cudaGetDevice(&s->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->nsm, cudaDevAttrMultiProcessorCount, s->device);
-    s->shape = pick_shape(*prob, s->nsm);
+    s->shape = pick_shape(*prob);
     const size_t PL = (size_t)s->nx * s->ny;
     const size_t rec = record_doubles(s->nx, s->ny, prob->dim), fac = face_doubles(s->nx, s->ny, prob->dim);
     s->device_bytes = 3 * 12 * PL * sizeof(double) + (rec + fac) * sizeof(double);
@@ -219,7 +208,7 @@ cgks_status cgks_create(const cgks_problem* prob, void* cuda_stream, cgks_solver
     if (e == cudaSuccess) e = cudaMalloc(&s->d_ctrl, sizeof(Ctrl));
     if (e == cudaSuccess) e = cudaMalloc(&s->d_desc, sizeof(GridDev));
     if (e == cudaSuccess && prob->dim == 1) e = cudaMalloc(&s->d_stage1d, 6 * PL * sizeof(double));
-    std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, s->shape, 0);
+    std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, prob->dim, s->shape, 0);
     s->ntiles = (int)tiles.size();
     if (e == cudaSuccess) e = cudaMalloc(&s->d_tiles, tiles.size() * sizeof(TileRef));
     std::vector<TileRef> rchunks = record_chunks(s->nx, s->ny, prob->dim, prob->recon_vars, 0);
@@ -259,10 +248,10 @@ extern "C" void cgks_forget_solver_plans(cgks_solver* s);
 cgks_status cgks_set_tile_shape(cgks_solver* s, int shape)
 {
     if (!s) return fail(CGKS_E_INVAL, "solver is NULL");
-    if (shape < 0) shape = pick_shape(s->prob, s->nsm);
+    if (shape < 0) shape = pick_shape(s->prob);
     if (shape >= TILE_COUNT) return fail(CGKS_E_INVAL, "unknown tile shape");
     if ((s->prob.dim == 1) != (shape == TILE_64x1)) return fail(CGKS_E_INVAL, "tile shape does not fit the dimension");
-    std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, shape, 0);
+    std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, s->prob.dim, shape, 0);
     TileRef* d = nullptr;
     CK(cudaMalloc(&d, tiles.size() * sizeof(TileRef)));
     cudaError_t e = cudaMemcpyAsync(d, tiles.data(), tiles.size() * sizeof(TileRef), cudaMemcpyHostToDevice, s->stream);
@@ -354,7 +343,7 @@ cgks_status cgks_get_state(cgks_solver* s, double* planes, int on_device, double
 
 static cgks_status enqueue_steps(cgks_solver* s, int nsteps, long* launches, bool fused)
 {
-    const int nblocks = stage_blocks(s->ntiles, s->nsm);
+    const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
     const int rblocks = record_blocks(s->nrchunks, s->nsm, cv);
     const int ublocks = update_blocks(s->ncchunks, s->nsm, 4);
@@ -389,7 +378,7 @@ static cgks_status step_impl(cgks_solver* s, int nsteps, double t_end, double* t
     if (!s || nsteps < 0) return fail(CGKS_E_INVAL, "bad arguments");
     if (fused && s->prob.dim != 2) return fail(CGKS_E_INVAL, "the fused step is 2D only");
     if (fused && !s->d_ftiles) {
-        const std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, TILE_16x8, 0);
+        const std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, 2, TILE_16x8, 0, false);
         TileRef* d = nullptr;
         CK(cudaMalloc(&d, tiles.size() * sizeof(TileRef)));
         cudaError_t e = cudaMemcpyAsync(d, tiles.data(), tiles.size() * sizeof(TileRef), cudaMemcpyHostToDevice,
@@ -449,7 +438,7 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
     constexpr int NK = 8;
     std::vector<cudaEvent_t> ev((size_t)nsteps * (NK + 1));
     for (auto& e : ev) CK(cudaEventCreate(&e));
-    const int nblocks = stage_blocks(s->ntiles, s->nsm);
+    const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
     const int rblocks = record_blocks(s->nrchunks, s->nsm, cv);
     const int ublocks = update_blocks(s->ncchunks, s->nsm, 4);

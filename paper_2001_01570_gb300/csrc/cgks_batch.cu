@@ -39,7 +39,7 @@ __global__ void dummy_ctrl_kernel(Ctrl* c)
     c->steps_target = 0;
 }
 
-constexpr int kShapeCands[] = {TILE_8x16, TILE_14x8, TILE_16x8, TILE_16x16};
+constexpr int kShapeCands[] = {TILE_8x16, TILE_14x8};
 constexpr int kCptCands[] = {2, 4};
 
 }  // namespace
@@ -139,9 +139,8 @@ cudaError_t BatchEngine::set_members(const std::vector<std::pair<int, GridDev>>&
         table[slot] = G;
         cells_ += (long long)G.nx * G.ny;
         for (int s : shapes) {
-            const int tw = tile_w(s), th = tile_h(s);
-            for (int y0 = 0; y0 < G.ny; y0 += th)
-                for (int x0 = 0; x0 < G.nx; x0 += tw) q[s].push_back(TileRef{slot, x0, y0, 0});
+            const std::vector<TileRef> t = make_tiles(G.nx, G.ny, G.dim, s, slot);
+            q[s].insert(q[s].end(), t.begin(), t.end());
         }
         std::vector<TileRef> r = record_chunks(G.nx, G.ny, G.dim, G.recon_vars, slot);
         q[TILE_COUNT + G.recon_vars].insert(q[TILE_COUNT + G.recon_vars].end(), r.begin(), r.end());
@@ -210,7 +209,7 @@ cudaError_t BatchEngine::capture(int cand)
                                     record_blocks(1 << 30, nsm_, v), cap, cnt + TILE_COUNT + v);
             if (e1 == cudaSuccess)
                 e1 = launch_stage(c.shape, stage, d_grids_, d_q_[c.shape], (int)cap_[c.shape],
-                                  stage_blocks(1 << 30, nsm_), cap, cnt + c.shape);
+                                  stage_blocks(1 << 30, nsm_, c.shape), cap, cnt + c.shape);
             if (e1 == cudaSuccess)
                 e1 = launch_update(stage, d_grids_, d_q_[TILE_COUNT + 2], (int)cap_[TILE_COUNT + 2],
                                    update_blocks(1 << 30, nsm_, c.cpt), cap, cnt + TILE_COUNT + 2, c.cpt);

@@ -76,6 +76,8 @@ struct RegK {
     double kfma(int i, double x, double y) const { return fma(k(i), x, y); }
     double kmul(int i, double x) const { return k(i) * x; }
     double rcp(double x) const { return cgks_opcount_rcp(x); }
+    double rcp3(double x) const { return cgks_opcount_rcp(x); }
+    double rsq(double x) const { return rsqrt(x); }
 #else
     __device__ __forceinline__ double add(double x, double y) const { return fma(x, one, y); }
     __device__ __forceinline__ double sub(double x, double y) const { return fma(x, one, -y); }
@@ -95,8 +97,37 @@ struct RegK {
         e = fma(-x, y, one);
         return fma(y, e, y);
     }
+    // the same in one third-order step, y (1 + e + e^2): one instruction fewer, the last
+    // bit of the result not always the correctly rounded one (error below 0.51 ulp)
+    __device__ __forceinline__ double rcp3(double x) const
+    {
+        double y;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+        const double e = fma(-x, y, one);
+        return fma(y, fma(e, e, e), y);
+    }
+    // 1/sqrt(x), x normal and positive, likewise: y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2
+    __device__ __forceinline__ double rsq(double x) const
+    {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+        const double e = fma(-mul(x, y), y, one);
+        return fma(mul(y, e), fma(0.375, e, 0.5), y);
+    }
 #endif
 };
+
+// x > 0 (normal or infinite, not NaN), from the high word: a comparison instruction would
+// take a slot of the FP64 unit
+#ifdef CGKS_OPCOUNT_HOST
+inline bool positive(double x) { return x > 0.0; }
+#else
+__device__ __forceinline__ bool positive(double x)
+{
+    const int hi = __double2hiint(x);
+    return hi >= 0x00100000 && hi <= 0x7ff00000;
+}
+#endif
 
 // Layout of the reconstruction coefficient table: one block per order (8, 6),
 // each starting with 1.0 and -0.0.  Indices are offsets within a block.
@@ -309,15 +340,19 @@ __device__ __forceinline__ void weno_pair_row(const RegK& r, const double Q[4], 
         const ff e = ff_from(eps);
         DiffData m{ff_from(x.d2), ff_from(x.s3), ff_from(x.s4), ff_from(x.w), ff_from(x.t), ff_from(x.u),
                    ff_from(x.p), ff_from(x.q)};
-        ff dv, ds;
-        weno_side_split<ORDER>(m, e, dv, ds);
-        vl = r.add(Q[1], r.add(r.kfma(RK_M6TH, x.s3, hd2), r.add(d_from(dv.h), d_from(dv.l))));
-        sl = r.add(x.d2, r.add(d_from(ds.h), d_from(ds.l)));
-        // the right-biased side is the left-biased one of the mirrored row
-        m = DiffData{ff_neg(m.d2), m.s4, m.s3, ff_neg(m.w), m.u, m.t, ff_neg(m.q), ff_neg(m.p)};
-        weno_side_split<ORDER>(m, e, dv, ds);
-        vr = r.add(Q[2], r.add(r.kfma(RK_M6TH, x.s4, -hd2), r.add(d_from(dv.h), d_from(dv.l))));
-        sr = r.sub(x.d2, r.add(d_from(ds.h), d_from(ds.l)));
+        // the right-biased side is the left-biased one of the mirrored row: a rolled loop, one
+        // copy of its instructions (with two, a third of the issue slots waited for instructions)
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            ff dv, ds;
+            weno_side_split<ORDER>(m, e, dv, ds);
+            const double y = r.add(r.kfma(RK_M6TH, side ? x.s4 : x.s3, side ? -hd2 : hd2), r.add(d_from(dv.h), d_from(dv.l)));
+            const double v = r.add(side ? Q[2] : Q[1], y), c = r.add(d_from(ds.h), d_from(ds.l));
+            const double sl_ = r.add(x.d2, side ? -c : c);
+            if (side) { vr = v; sr = sl_; }
+            else { vl = v; sl = sl_; }
+            m = DiffData{ff_neg(m.d2), m.s4, m.s3, ff_neg(m.w), m.u, m.t, ff_neg(m.q), ff_neg(m.p)};
+        }
     } else {
         weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], eps, vl, sl, vr, sr);
     }

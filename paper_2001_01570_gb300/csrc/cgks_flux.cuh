@@ -18,14 +18,11 @@ namespace cgks {
 // (copied from kFluxFixed), then the values of the tile's grid and time step
 // (written by the CTA's first thread at the start of each tile).
 enum FluxK {
-    FK_ONE = 0, FK_NZERO, FK_HALF, FK_MHALF, FK_2, FK_M2, FK_3, FK_4, FK_5, FK_M3, FK_M4, FK_QUARTER, FK_EIGHTH,
-    FK_ERFC_TMAX,                          // last table piece of erfcx
+    FK_ONE = 0, FK_NZERO, FK_HALF, FK_MHALF, FK_2, FK_M2, FK_3, FK_4, FK_M4,
     FK_T13_3, FK_DLO, FK_DHI,              // tangential WENO-Z: 4 x beta weight, linear weights at the Gauss points
     FK_HG, FK_MHG,                         // +-eta/2 at the Gauss point eta = 1/(2 sqrt 3)
-    FK_A1T, FK_A2T, FK_S1T, FK_S2T, FK_M0T,         // quartic: d/deta coefficients
-    FK_S1TT, FK_S2TT, FK_M0TT,                      // quartic: d^2/deta^2 coefficients
-    FK_M0N, FK_S1N, FK_S2N, FK_A1N, FK_A2N,         // quartic: value at the Gauss points
-    FK_C0P, FK_C0M,                                  // +-1/(2 sqrt(pi))
+    FK_M12TH, FK_M9TH, FK_M4320TH, FK_M7_72,         // quartic through the five means: coefficients
+    FK_C1P, FK_C1M,                                  // +-1/sqrt(pi)
     FK_X32LN2, FK_SHIFT, FK_LN2HI, FK_LN2LO,         // exponential: argument reduction
     FK_P2, FK_P3, FK_P4, FK_P5, FK_P6,               // exponential: 1/k! of the Taylor polynomial
     FK_NFIX,
@@ -34,10 +31,14 @@ enum FluxK {
     // per grid and tile
     FK_DT = FK_NFIX2, FK_IDT, FK_4IDT2, FK_HDT, FK_MHDT, FK_EPSDT, FK_CTAUDT, FK_C8, FK_C6,
     FK_W1A, FK_W1B, FK_W2A, FK_W2B, FK_W3,          // Gauss-average weights of the face results
-    FK_GAMMA, FK_GM1, FK_K, FK_K2, FK_KK2, FK_INVK2, FK_K2INV2, FK_KHEAT, FK_MU,
+    FK_GAMMA, FK_GM1, FK_K1, FK_K3, FK_K2INV2, FK_KHEAT, FK_MU,
     FK_IDX, FK_IDY, FK_WEPS, FK_WEPS4,
     FK_N
 };
+
+// the linear weights of the outer candidates along a face over the centre one's, 11/18
+constexpr double kTangLo = (7.0 / 36.0 - 1.7320508075688772 / 1080.0) * (18.0 / 11.0);
+constexpr double kTangHi = (7.0 / 36.0 + 1.7320508075688772 / 1080.0) * (18.0 / 11.0);
 
 struct FluxFixed { double v[FK_NFIX]; };
 
@@ -46,22 +47,15 @@ constexpr FluxFixed make_flux_fixed()
     FluxFixed t{};
     double* k = t.v;
     k[FK_ONE] = 1.0; k[FK_NZERO] = -0.0; k[FK_HALF] = 0.5; k[FK_MHALF] = -0.5; k[FK_2] = 2.0; k[FK_M2] = -2.0;
-    k[FK_3] = 3.0; k[FK_4] = 4.0; k[FK_5] = 5.0; k[FK_M3] = -3.0; k[FK_M4] = -4.0; k[FK_QUARTER] = 0.25;
-    k[FK_EIGHTH] = 0.125; k[FK_ERFC_TMAX] = 27.9;
+    k[FK_3] = 3.0; k[FK_4] = 4.0; k[FK_M4] = -4.0;
     const double gq = 0.28867513459481287;               // 1/(2 sqrt 3)
-    // the linear weights (d_lo, 11/18, d_hi) divided by 11/18 (the weights' normalisation
-    // cancels the common factor)
     k[FK_T13_3] = 13.0 / 3.0;
-    k[FK_DLO] = (7.0 / 36.0 - 1.7320508075688772 / 1080.0) * (18.0 / 11.0);
-    k[FK_DHI] = (7.0 / 36.0 + 1.7320508075688772 / 1080.0) * (18.0 / 11.0);
+    k[FK_DLO] = kTangLo;
+    k[FK_DHI] = kTangHi;
     k[FK_HG] = 0.5 * gq; k[FK_MHG] = -0.5 * gq;
-    // the quartic p(eta) through the five segment means (see SegmentRows::eq_derivs)
-    k[FK_A1T] = 8.0 / 12.0; k[FK_A2T] = -1.0 / 12.0; k[FK_S1T] = 13.0 / 9.0; k[FK_S2T] = -1.0 / 9.0;
-    k[FK_M0T] = -24.0 / 9.0;
-    k[FK_S1TT] = 16.0 / 12.0; k[FK_S2TT] = -1.0 / 12.0; k[FK_M0TT] = -30.0 / 12.0;
-    k[FK_M0N] = 1.0 - 6.0 / 4320.0; k[FK_S1N] = 4.0 / 4320.0; k[FK_S2N] = -1.0 / 4320.0;
-    k[FK_A1N] = 50.0 / 72.0; k[FK_A2N] = -7.0 / 72.0;
-    k[FK_C0P] = 0.28209479177387814; k[FK_C0M] = -0.28209479177387814;
+    // the quartic p(eta) through the five segment means (see SegmentRows::deriv_parts)
+    k[FK_M12TH] = -1.0 / 12.0; k[FK_M9TH] = -1.0 / 9.0; k[FK_M4320TH] = -1.0 / 4320.0; k[FK_M7_72] = -7.0 / 72.0;
+    k[FK_C1P] = 0.56418958354775628; k[FK_C1M] = -0.56418958354775628;
     k[FK_X32LN2] = 32.0 / 0.6931471805599453;             // 32 / ln 2
     k[FK_SHIFT] = 6755399441055744.0;                      // 1.5 * 2^52: rounds to an integer in the low bits
     k[FK_LN2HI] = 0.6931471805599453 / 32.0;               // ln 2 / 32 and the remainder of its rounding
@@ -91,10 +85,8 @@ __device__ __forceinline__ void flux_table_tile(double* t, const GridDev& G, dou
     t[FK_W3] = dt * dt * (1.0 / 6.0);
     t[FK_GAMMA] = G.gamma;
     t[FK_GM1] = G.gamma - 1.0;
-    t[FK_K] = G.K;
-    t[FK_K2] = G.K + 2.0;
-    t[FK_KK2] = G.K * (G.K + 2.0);
-    t[FK_INVK2] = __drcp_rn(G.K + 2.0);
+    t[FK_K1] = G.K + 1.0;
+    t[FK_K3] = G.K + 3.0;
     t[FK_K2INV2] = 2.0 * __drcp_rn(G.K + 2.0);
     t[FK_KHEAT] = 0.5 * (G.K + 4.0);
     t[FK_MU] = G.mu;
@@ -124,20 +116,39 @@ __device__ __forceinline__ void flux_table_tile(double* t, const GridDev& G, dou
 // final normalisation differ.  The weights are homogeneous in (e_k, Z) and in
 // (d_k), so the code carries 4 e_k = D_k^2 + 13/3 (second difference)^2 + 4 eps
 // (eps4 = 4 eps) and the linear weights divided by 11/18.
-// The caller passes A1 = v_1 - v_-1 and S1 = v_1 + v_-1, which the tangential
-// derivatives use too.
-__device__ __forceinline__ void tang_weno5_pair(const RegK& r, double vmm, double vm, double v0, double vp,
-                                                double vpp, double A1, double S1, double eps4, double& at_minus,
-                                                double& at_plus)
+// With the differences of the means, D_1 = A1 = v_1 - v_-1, D_0 = A1 - t0, D_2 = A1 - t1
+// (t0, t1 the third differences), so a point value is v_0 + (eta/2) (A1 - w_0 t0 - w_2 t1):
+// the weights enter through third differences alone, which is what the split form
+// (cgks_split.cuh) carries in pairs of FP32 where they are small beside the scale.
+struct TangDiffs { double A1, s1, t0, t1; };
+
+__device__ __forceinline__ void tang_diffs(const RegK& r, double vmm, double vm, double v0, double vp, double vpp,
+                                           TangDiffs& x)
 {
-    const double D0 = r.kfma(FK_3, v0, r.kfma(FK_M4, vm, vmm));
-    const double D1 = A1;
-    const double D2 = r.kfma(FK_4, vp, r.kfma(FK_M3, v0, -vpp));
-    const double s0 = r.kfma(FK_M2, vm, r.add(vmm, v0));
-    const double s1 = r.kfma(FK_M2, v0, S1);
-    const double s2 = r.kfma(FK_M2, vp, r.add(v0, vpp));
+    const double dA = r.sub(vm, vmm), dB = r.sub(v0, vm), dC = r.sub(vp, v0), dD = r.sub(vpp, vp);
+    x.s1 = r.sub(dC, dB);
+    x.t0 = r.sub(x.s1, r.sub(dB, dA));
+    x.t1 = r.sub(r.sub(dD, dC), x.s1);
+    x.A1 = r.add(dB, dC);
+}
+
+__device__ __forceinline__ void tang_weno5_pair(const RegK& r, double v0, const TangDiffs& x, double eps4,
+                                                int scale_hi, double& at_minus, double& at_plus)
+{
+#ifndef CGKS_OPCOUNT_HOST
+    if (split_scale_ok(scale_hi, eps4) && i_max(hi_abs(x.t0), hi_abs(x.t1)) < scale_hi + kTangThird * (1 << 20) &&
+        i_max(hi_abs(x.A1), hi_abs(x.s1)) < scale_hi + (1 << 20)) {
+        ff m, p;
+        tang_weno5_split(ff_from(x.A1), ff_from(x.s1), ff_from(x.t0), ff_from(x.t1), ff_from(eps4), CGKS_FF(kTangLo),
+                         CGKS_FF(kTangHi), m, p);
+        at_plus = r.kfma(FK_HG, r.sub(x.A1, r.add(d_from(p.h), d_from(p.l))), v0);
+        at_minus = r.kfma(FK_MHG, r.sub(x.A1, r.add(d_from(m.h), d_from(m.l))), v0);
+        return;
+    }
+#endif
+    const double D0 = r.sub(x.A1, x.t0), D2 = r.sub(x.A1, x.t1), s0 = r.sub(x.s1, x.t0), s2 = r.add(x.s1, x.t1);
     const double e0 = fma(D0, D0, fma(r.kmul(FK_T13_3, s0), s0, eps4));
-    const double e1 = fma(D1, D1, fma(r.kmul(FK_T13_3, s1), s1, eps4));
+    const double e1 = fma(x.A1, x.A1, fma(r.kmul(FK_T13_3, x.s1), x.s1, eps4));
     const double e2 = fma(D2, D2, fma(r.kmul(FK_T13_3, s2), s2, eps4));
     const double Z = fabs(r.sub(e0, e2));
     // (e_k + Z) times the other two = E + Z times the other two, E = e0 e1 e2
@@ -145,12 +156,12 @@ __device__ __forceinline__ void tang_weno5_pair(const RegK& r, double vmm, doubl
     const double P0 = fma(Z, e12, E);
     const double P1 = fma(Z, r.mul(e0, e2), E);
     const double P2 = fma(Z, r.mul(e0, e1), E);
-    const double Q0 = r.mul(P0, D0), Q1 = r.mul(P1, D1), Q2 = r.mul(P2, D2);
-    const double np = r.kfma(FK_DHI, Q2, r.kfma(FK_DLO, Q0, Q1)), dp = r.kfma(FK_DHI, P2, r.kfma(FK_DLO, P0, P1));
-    const double nm = r.kfma(FK_DLO, Q2, r.kfma(FK_DHI, Q0, Q1)), dm = r.kfma(FK_DLO, P2, r.kfma(FK_DHI, P0, P1));
+    const double Q0 = r.mul(P0, x.t0), Q2 = r.mul(P2, x.t1);
+    const double np = r.kfma(FK_DHI, Q2, r.kmul(FK_DLO, Q0)), dp = r.kfma(FK_DHI, P2, r.kfma(FK_DLO, P0, P1));
+    const double nm = r.kfma(FK_DLO, Q2, r.kmul(FK_DHI, Q0)), dm = r.kfma(FK_DLO, P2, r.kfma(FK_DHI, P0, P1));
     const double inv = r.rcp(r.mul(dp, dm));             // one reciprocal for both points
-    at_plus = r.kfma(FK_HG, r.mul(np, r.mul(dm, inv)), v0);
-    at_minus = r.kfma(FK_MHG, r.mul(nm, r.mul(dp, inv)), v0);
+    at_plus = r.kfma(FK_HG, fma(-np, r.mul(dm, inv), x.A1), v0);
+    at_minus = r.kfma(FK_MHG, fma(-nm, r.mul(dp, inv), x.A1), v0);
 }
 
 // Three means v_{-1..1}: two linear candidates with slopes v_0 - v_-1 and
@@ -170,10 +181,29 @@ __device__ __forceinline__ void tang_weno3_parts(const RegK& r, double vm, doubl
     den = r.add(n0, n1);
 }
 
+// One row's slope in the split form: false where the correction it carries is not
+// below 2^-11 of the scale (its relative error is about 2^-44).
+#ifndef CGKS_OPCOUNT_HOST
+__device__ __forceinline__ bool tang_weno3_small(const RegK& r, double vm, double v0, double vp, double eps,
+                                                 int scale_hi, double& slope)
+{
+    const double dm = r.sub(v0, vm), dp = r.sub(vp, v0), A = r.add(dp, dm), s = r.sub(dp, dm);
+    if (!(split_scale_ok(scale_hi, eps) && i_max(hi_abs(A), hi_abs(s)) < scale_hi + (1 << 20))) return false;
+    const ff c = tang_weno3_split(ff_from(A), ff_from(s), ff_from(eps));
+    const double ch = d_from(c.h);
+    slope = r.kmul(FK_HALF, r.sub(A, r.add(ch, d_from(c.l))));
+    return hi_abs(ch) < scale_hi + kTangSlope * (1 << 20);
+}
+#endif
+
 // the slopes of the left and right states' rows, with one reciprocal for both
 __device__ __forceinline__ void tang_weno3_slopes(const RegK& r, double lm, double l0, double lp, double rm,
-                                                  double r0, double rp, double eps, double& sl, double& sr)
+                                                  double r0, double rp, double eps, int scale_hi, double& sl,
+                                                  double& sr)
 {
+#ifndef CGKS_OPCOUNT_HOST
+    if (tang_weno3_small(r, lm, l0, lp, eps, scale_hi, sl) && tang_weno3_small(r, rm, r0, rp, eps, scale_hi, sr)) return;
+#endif
     double nl, dl, nr, dr;
     tang_weno3_parts(r, lm, l0, lp, eps, nl, dl);
     tang_weno3_parts(r, rm, r0, rp, eps, nr, dr);
@@ -192,7 +222,9 @@ __device__ __forceinline__ double exp_neg(const RegK& r, double x)
 #ifdef CGKS_OPCOUNT_HOST
     return cgks_opcount_exp(x);   // one exponential in the host operation count
 #endif
-    if (x < -700.0) return 0.0;
+#ifndef CGKS_OPCOUNT_HOST
+    if ((unsigned)d_hi(x) > 0xc085e000u) return 0.0;      // high word of -700
+#endif
     const double t = r.kfma(FK_X32LN2, x, r.k(FK_SHIFT));
     const double n = r.sub(t, r.k(FK_SHIFT));             // round(32 x / ln 2), exactly
     const int ni = (int)(unsigned)__double_as_longlong(t);
@@ -217,139 +249,139 @@ __device__ __forceinline__ double erfc_scaled(const RegK& r, double t, double e)
 #ifdef CGKS_OPCOUNT_HOST
     return cgks_opcount_erfc(t);   // one erfc in the host operation count
 #endif
-    const int k = (int)r.kmul(FK_4, fmin(t, r.k(FK_ERFC_TMAX)));
+#ifndef CGKS_OPCOUNT_HOST
+    // the piece and its centre in FP32 (a t on the border may take either piece)
+    const int k = (int)f_mul(4.0f, fminf(f_lead(t), 27.9f));
     const double* c = cgks_erfcx_coef[k];
-    const double z = r.sub(t, r.kfma(FK_QUARTER, (double)k, r.k(FK_EIGHTH)));
+    const double z = r.sub(t, d_from(f_fma(0.25f, f_int(k), 0.125f)));
     double v = c[0];
 #pragma unroll
     for (int m = 1; m <= CGKS_ERFCX_DEG; ++m) v = fma(v, z, c[m]);
     return r.mul(e, v);
+#endif
 }
 
-// the two lowest half-line u-moments of a Maxwellian with mean U and
-// sqrt(lambda) = sq: <u^0> = erfc(-+ s)/2, <u^1> = U <u^0> +- e^{-s^2}/(2 sqrt(pi lambda)),
-// s = U sqrt(lambda); SIDE = +1 for u > 0, -1 for u < 0
-template <int SIDE>
-__device__ __forceinline__ void half_moments01(const RegK& r, double U, double sq, double inv_sq, double& m0,
-                                               double& m1)
+// ------------------------------------------------------------------------
+// Sec. 2.1: half-line velocity moments of a Maxwellian per unit density, mean
+// (U, V), theta = p/rho = 1/(2 lambda), sqrt(lambda) = sq: m_n = <u^n> over u > 0
+// (side 0) or u < 0 (side 1), n = 0..3, and the signed density at u = 0,
+//   g = +-e^{-s^2} / sqrt(2 pi theta), s = U sqrt(lambda):
+//   m_0 = erfc(-+ s)/2,  m_1 = U m_0 + theta g,  m_{n+1} = U m_n + n theta m_{n-1}.
+struct HalfMoments { double m[4], g; };
+
+__device__ __forceinline__ void half_moments(const RegK& r, int side, double U, double theta, double th2, double sq,
+                                             HalfMoments& h)
 {
     const double s = r.mul(U, sq);
     const double e = exp_neg(r, -r.mul(s, s));
     const double hE = r.kmul(FK_HALF, erfc_scaled(r, fabs(s), e));    // erfc(|s|)/2
-    // SIDE +1: erfc(-s)/2 = 1 - erfc(s)/2 for s >= 0, erfc(|s|)/2 for s < 0; SIDE -1 mirrored
-    const bool pos = (SIDE > 0) ? (s >= 0.0) : (s < 0.0);
-    m0 = pos ? r.sub(r.one, hE) : hE;
-    m1 = fma(U, m0, r.kmul(SIDE > 0 ? FK_C0P : FK_C0M, r.mul(e, inv_sq)));
+    // u > 0: erfc(-s)/2 = 1 - erfc(s)/2 for s >= 0, erfc(|s|)/2 for s < 0; u < 0 mirrored
+#ifdef CGKS_OPCOUNT_HOST
+    const bool neg = s < 0.0;
+#else
+    const bool neg = d_hi(s) < 0;
+#endif
+    h.m[0] = (neg == (side != 0)) ? r.sub(r.one, hE) : hE;
+    h.g = r.kmul(side ? FK_C1M : FK_C1P, r.mul(e, sq));
+    h.m[1] = fma(U, h.m[0], r.mul(theta, h.g));
+    h.m[2] = fma(U, h.m[1], r.mul(theta, h.m[0]));
+    h.m[3] = fma(U, h.m[2], r.mul(th2, h.m[1]));
 }
 
-// ------------------------------------------------------------------------
-// Sec. 2.1: Maxwellian velocity moments.  theta = p/rho = 1/(2 lambda).
-struct Moments {
-    double u[7];     // <u^n>, n = 0..6 (whole line or half line)
-    double v[6];     // <v^n>, n = 0..5 (whole line); v[0] = 1 is never multiplied
-    double x1, x2;   // <xi^2>, <xi^4>
+// The slope terms of the half-line moments: <psi u (u a_n + v a_t)> (the flux part,
+// Th) and <psi (u a_n + v a_t)> (the interface-state part, Wsl), rho a_n and rho a_t
+// being the Maxwellian's relative slopes along the normal and the tangent (Sec. 2.1).
+// Since rho <phi a_n> is the normal derivative of rho <phi>, they are the
+// derivatives of the half-line moments rho <u^2 psi>, rho <u v psi> (and rho <u psi>,
+// rho <v psi>) along the conservative slopes, taken through the primitive variables:
+//   dm_n = n m_{n-1} dU + n(n-1)/2 m_{n-2} dtheta   (n >= 2),
+//   dm_1 = m_0 dU + g/2 dtheta,   dm_0 = g (dU - U/(2 theta) dtheta).
+// No micro-slope system is solved and moments to order 4 suffice (the form with
+// the micro-slope coefficients needs order 6 and half again the operations).  (R, A, B, C) = (rho', rho U', rho V',
+// rho theta').  Ar supplies the arithmetic (FP64 or split).
+template <class T> struct PrimSlope { T R, A, B, C; };
+
+template <class Ar, class T = typename Ar::T>
+__device__ __forceinline__ PrimSlope<T> prim_slope(const Ar& q, T U, T V, T hq2, T theta, const T b[4])
+{
+    PrimSlope<T> s;
+    s.R = b[0];
+    s.A = q.nmad(U, b[0], b[1]);
+    s.B = q.nmad(V, b[0], b[2]);
+    // e' = E' - (rho q^2/2)', e = rho theta / (gamma - 1)
+    const T de = q.nmad(hq2, b[0], q.nmad(V, s.B, q.nmad(U, s.A, b[3])));
+    s.C = q.nmad(theta, b[0], q.mul(q.gm1(), de));
+    return s;
+}
+
+template <class Ar, class T = typename Ar::T>
+__device__ __forceinline__ void slope_moments(const Ar& q, bool ne, T U, T V, T theta, T itheta, const T m[4], T g,
+                                              const T bn[4], const T bt[4], T Th[4], T Wsl[4])
+{
+    const T VV = q.mul(V, V), hq2 = q.half(q.mad(U, U, VV));
+    const PrimSlope<T> X = prim_slope(q, U, V, hq2, theta, bn), Y = prim_slope(q, U, V, hq2, theta, bt);
+    const T V2 = q.dbl(V), qt = q.mad(q.K1(), theta, VV), w = q.mad(q.K3(), theta, VV), v2 = q.add(VV, theta);
+    const T m4 = q.mad(U, m[3], q.mul(q.tri(theta), m[2]));
+    // y_n = (rho m_n)' along the normal (x) and the tangent (y)
+    auto y1 = [&](const PrimSlope<T>& s) { return q.mad(s.R, m[1], q.mad(s.A, m[0], q.mul(q.half(s.C), g))); };
+    auto y2 = [&](const PrimSlope<T>& s) { return q.mad(s.R, m[2], q.mad(q.dbl(s.A), m[1], q.mul(s.C, m[0]))); };
+    auto y3 = [&](const PrimSlope<T>& s) { return q.mad(s.R, m[3], q.tri(q.mad(s.A, m[2], q.mul(s.C, m[1])))); };
+    const T x2 = y2(X), x3 = y3(X), a1 = y1(Y), a2 = y2(Y), a3 = y3(Y);
+    const T x4 = q.mad(X.R, m4, q.dbl(q.mad(q.dbl(X.A), m[3], q.mul(q.tri(X.C), m[2]))));
+    const T xv = q.mad(V2, X.B, q.mul(q.K1(), X.C));                            // (V^2 + (K+1) theta)' rho
+    const T yv = q.mad(V, q.mad(V2, Y.B, q.mul(q.K3(), Y.C)), q.mul(Y.B, w));   // (V w)' rho
+    const T yt = q.mad(V2, Y.B, Y.C);                                           // (V^2 + theta)' rho
+    Th[0] = q.add(x2, q.mad(V, a1, q.mul(Y.B, m[1])));
+    Th[1] = q.add(x3, q.mad(V, a2, q.mul(Y.B, m[2])));
+    Th[2] = q.mad(V, x2, q.mad(X.B, m[2], q.mad(v2, a1, q.mul(m[1], yt))));
+    Th[3] = q.half(q.add(q.mad(m[2], xv, q.mad(qt, x2, x4)),
+                         q.mad(m[1], yv, q.mad(Y.B, m[3], q.mul(V, q.mad(w, a1, a3))))));
+    if (ne) {
+        const T x1 = y1(X);
+        const T a0 = q.mad(Y.R, m[0], q.mul(g, q.nmad(q.half(q.mul(U, itheta)), Y.C, Y.A)));
+        Wsl[0] = q.add(x1, q.mad(V, a0, q.mul(Y.B, m[0])));
+        Wsl[1] = q.add(x2, q.mad(V, a1, q.mul(Y.B, m[1])));
+        Wsl[2] = q.mad(V, x1, q.mad(X.B, m[1], q.mad(v2, a0, q.mul(m[0], yt))));
+        Wsl[3] = q.half(q.add(q.mad(m[1], xv, q.mad(qt, x1, x3)),
+                              q.mad(m[0], yv, q.mad(Y.B, m[2], q.mul(V, q.mad(w, a0, a2))))));
+    }
+}
+
+// FP64 arithmetic of slope_moments in the register forms
+struct Ar64 {
+    using T = double;
+    const RegK& r;
+    __device__ __forceinline__ double add(double a, double b) const { return r.add(a, b); }
+    __device__ __forceinline__ double sub(double a, double b) const { return r.sub(a, b); }
+    __device__ __forceinline__ double mul(double a, double b) const { return r.mul(a, b); }
+    __device__ __forceinline__ double mad(double a, double b, double c) const { return fma(a, b, c); }
+    __device__ __forceinline__ double nmad(double a, double b, double c) const { return fma(-a, b, c); }
+    __device__ __forceinline__ double half(double a) const { return r.kmul(FK_HALF, a); }
+    __device__ __forceinline__ double dbl(double a) const { return r.add(a, a); }
+    __device__ __forceinline__ double tri(double a) const { return r.kmul(FK_3, a); }
+    __device__ __forceinline__ double gm1() const { return r.k(FK_GM1); }
+    __device__ __forceinline__ double K1() const { return r.k(FK_K1); }
+    __device__ __forceinline__ double K3() const { return r.k(FK_K3); }
 };
 
-__device__ __forceinline__ void moments_tail(const RegK& r, Moments& m, double U, double V, double theta)
-{
-    const double t2 = r.add(theta, theta), t3 = r.kmul(FK_3, theta), t4 = r.kmul(FK_4, theta),
-                 t5 = r.kmul(FK_5, theta);
-    m.u[2] = fma(U, m.u[1], r.mul(theta, m.u[0]));
-    m.u[3] = fma(U, m.u[2], r.mul(t2, m.u[1]));
-    m.u[4] = fma(U, m.u[3], r.mul(t3, m.u[2]));
-    m.u[5] = fma(U, m.u[4], r.mul(t4, m.u[3]));
-    m.u[6] = fma(U, m.u[5], r.mul(t5, m.u[4]));
-    m.v[0] = 1.0;
-    m.v[1] = V;
-    m.v[2] = fma(V, V, theta);
-    m.v[3] = fma(V, m.v[2], r.mul(t2, V));
-    m.v[4] = fma(V, m.v[3], r.mul(t3, m.v[2]));
-    m.v[5] = fma(V, m.v[4], r.mul(t4, m.v[3]));
-    m.x1 = r.mul(r.k(FK_K), theta);
-    m.x2 = r.mul(r.mul(r.k(FK_KK2), theta), theta);
-}
-
-// <u^A psi> of a Maxwellian (whole-line v-moments, B = 0)
-template <int A>
-__device__ __forceinline__ void psi_u(const RegK& r, const Moments& m, double o[4])
-{
-    o[0] = m.u[A];
-    o[1] = m.u[A + 1];
-    o[2] = r.mul(m.u[A], m.v[1]);
-    o[3] = r.kmul(FK_HALF, fma(m.u[A], m.x1, fma(m.u[A], m.v[2], m.u[A + 2])));
-}
-
-// <psi u^A (u (a1 . psi) + v (a2 . psi))> for a Maxwellian, with a . psi =
-// a0 + a1 u + a2 v + a3 (u^2 + v^2 + xi^2)/2: the slope terms of the half-line
-// moments (A = 1: the flux part, A = 0: the interface-state part).  The
-// polynomial in the bracket, times u^A, is grouped by powers of v,
-//   v^0: a1_0 u + a1_1 u^2 + h1 u^3  (+ h1 u xi^2),  v^1: a2_0 + c12 u + h2 u^2  (+ h2 xi^2),
-//   v^2: a2_2 + h1 u,                v^3: h2,
-// (h = a_3/2, c12 = a1_2 + a2_1), so each psi component is a short sum of
-// products of the factorised u-, v- and xi-moments.
-// (a[3] holds h = a_3 / 2, as micro_slope returns it)
-template <int A>
-__device__ __forceinline__ void q_moments(const RegK& r, const Moments& m, const double a1[4], const double a2[4],
-                                          double o[4])
-{
-    const double h1 = a1[3], h2 = a2[3], c12 = r.add(a1[2], a2[1]);
-    // sums over u for the v^j groups at u-shift s2 (S_j) and the xi^2 parts (Z_j); S_3 = Z_1
-    double S0[3], S1[3], S2[3], Z0[3], Z1[3];
-#pragma unroll
-    for (int s2 = 0; s2 < 3; ++s2) {
-        Z0[s2] = r.mul(h1, m.u[A + 1 + s2]);
-        Z1[s2] = r.mul(h2, m.u[A + s2]);
-    }
-#pragma unroll
-    for (int s2 = 0; s2 < 3; ++s2) {
-        // h1 u[A+3] = Z0[2] and h2 u[A+2] = Z1[2] for the first shift
-        const double t0 = (s2 == 0) ? Z0[2] : r.mul(h1, m.u[A + 3 + s2]);
-        const double t1 = (s2 == 0) ? Z1[2] : r.mul(h2, m.u[A + 2 + s2]);
-        S0[s2] = fma(a1[1], m.u[A + 2 + s2], fma(a1[0], m.u[A + 1 + s2], t0));
-        S1[s2] = fma(c12, m.u[A + 1 + s2], fma(a2[0], m.u[A + s2], t1));
-        S2[s2] = fma(a2[2], m.u[A + s2], Z0[s2]);
-    }
-    const double x1 = m.x1, x2 = m.x2;
-    // sum_j v[j+sh] S_j[s2] + x1 (v[sh] Z0[s2] + v[sh+1] Z1[s2]), v[0] = 1
-    auto sum = [&](int s2, int sh) {
-        const double lo = (sh == 0) ? S0[s2] : r.mul(m.v[sh], S0[s2]);
-        const double z = (sh == 0) ? fma(m.v[1], Z1[s2], Z0[s2]) : fma(m.v[sh + 1], Z1[s2], r.mul(m.v[sh], Z0[s2]));
-        return fma(x1, z, fma(m.v[sh + 3], Z1[s2], fma(m.v[sh + 2], S2[s2], fma(m.v[sh + 1], S1[s2], lo))));
-    };
-    const double plain0 = fma(m.v[3], Z1[0], fma(m.v[2], S2[0], fma(m.v[1], S1[0], S0[0])));
-    const double xi0 = fma(m.v[1], Z1[0], Z0[0]);
-    o[0] = fma(x1, xi0, plain0);
-    o[1] = sum(1, 0);
-    o[2] = sum(0, 1);
-    o[3] = r.kmul(FK_HALF, fma(x2, xi0, fma(x1, plain0, r.add(sum(2, 0), sum(0, 2)))));
-}
-
-// micro-slope coefficients a with <psi psi^T> a = b for a Maxwellian
-// (closed form of the 4x4 moment system); a[3] receives h = a_3 / 2, the factor
-// q_moments uses (psi_4 carries 1/2)
-struct SlopeCtx { double U, V, Bm, inv_theta, c4; };
-
-__device__ __forceinline__ void slope_ctx(const RegK& r, double U, double V, double theta, double inv_theta,
-                                          SlopeCtx& s)
-{
-    s.U = U; s.V = V;
-    s.Bm = fma(U, U, fma(V, V, r.mul(r.k(FK_K2), theta)));
-    s.inv_theta = inv_theta;
-    s.c4 = r.mul(r.mul(inv_theta, inv_theta), r.k(FK_INVK2));
-}
-
-__device__ __forceinline__ void micro_slope(const RegK& r, const SlopeCtx& s, const double b[4], double a[4])
-{
-    const double R4 = fma(-s.Bm, b[0], r.add(b[3], b[3]));
-    const double R3 = fma(-s.V, b[0], b[2]);
-    const double R2 = fma(-s.U, b[0], b[1]);
-    const double a3 = r.mul(s.c4, r.kfma(FK_M2, fma(s.V, R3, r.mul(s.U, R2)), R4));
-    const double h = r.kmul(FK_HALF, a3);
-    a[2] = fma(-s.V, a3, r.mul(R3, s.inv_theta));
-    a[1] = fma(-s.U, a3, r.mul(R2, s.inv_theta));
-    a[0] = fma(-h, s.Bm, fma(-s.V, a[2], fma(-s.U, a[1], b[0])));
-    a[3] = h;
-}
+#if !defined(CGKS_OPCOUNT_HOST) || defined(CGKS_SPLIT_CHECK)
+// the same in pairs of FP32 (cgks_split.cuh)
+struct ArSplit {
+    using T = ff;
+    ff g1, k1, k3;
+    __device__ __forceinline__ ff add(ff a, ff b) const { return ff_add(a, b); }
+    __device__ __forceinline__ ff sub(ff a, ff b) const { return ff_sub(a, b); }
+    __device__ __forceinline__ ff mul(ff a, ff b) const { return ff_mul(a, b); }
+    __device__ __forceinline__ ff mad(ff a, ff b, ff c) const { return ff_add(ff_mul(a, b), c); }
+    __device__ __forceinline__ ff nmad(ff a, ff b, ff c) const { return ff_sub(c, ff_mul(a, b)); }
+    __device__ __forceinline__ ff half(ff a) const { return ff_scale(0.5f, a); }
+    __device__ __forceinline__ ff dbl(ff a) const { return ff_scale(2.0f, a); }
+    __device__ __forceinline__ ff tri(ff a) const { return ff_mulf(3.0f, a); }
+    __device__ __forceinline__ ff gm1() const { return g1; }
+    __device__ __forceinline__ ff K1() const { return k1; }
+    __device__ __forceinline__ ff K3() const { return k3; }
+};
+#endif
 
 // ------------------------------------------------------------------------
 // Euler time derivatives by Cauchy-Kowalevski in primitive variables.
@@ -364,91 +396,265 @@ __device__ __forceinline__ void micro_slope(const RegK& r, const SlopeCtx& s, co
 // (mu = tau p, bulk part 2/(K+2), heat conduction (K+4)/2 tau p grad(p/rho)).
 struct EulerTD { double Wt[4], Wtt[4], Ft[4], F[4], TNS[4]; };
 
+// the state, its primitive first derivatives and first time derivatives
+template <class T> struct EulerFirst {
+    T rho, U, V, ir, gir, hq2, e;               // gir = (gamma - 1) / rho, hq2 = (U^2 + V^2)/2
+    T rx, ry, Ux, Uy, Vx, Vy, ex, ey, Dv;       // Dv = U_x + V_y
+    T rt, Ut, Vt, et, uut;                      // uut = U U_t + V V_t
+};
+
+// W_tt from the first-order quantities and the conservative second derivatives
+template <class Ar, class T = typename Ar::T>
+__device__ __forceinline__ void euler_second(const Ar& q, const EulerFirst<T>& f, T gamma, const T Wxx[4],
+                                             const T Wxy[4], const T Wyy[4], T Wtt[4])
+{
+    const T rxx = Wxx[0], rxy = Wxy[0], ryy = Wyy[0], rx2 = q.dbl(f.rx), ry2 = q.dbl(f.ry);
+    // primitive second derivatives; KE = rho q^2 / 2: KE_xx = rho |u_x|^2 + u . m_xx - rho_xx q^2/2,
+    // KE_xy = rho u_x . u_y + u . m_xy - rho_xy q^2/2
+    const T Uxx = q.mul(q.nmad(f.U, rxx, q.nmad(f.Ux, rx2, Wxx[1])), f.ir);
+    const T Uxy = q.mul(q.nmad(f.U, rxy, q.nmad(f.Uy, f.rx, q.nmad(f.Ux, f.ry, Wxy[1]))), f.ir);
+    const T Uyy = q.mul(q.nmad(f.U, ryy, q.nmad(f.Uy, ry2, Wyy[1])), f.ir);
+    const T Vxx = q.mul(q.nmad(f.V, rxx, q.nmad(f.Vx, rx2, Wxx[2])), f.ir);
+    const T Vxy = q.mul(q.nmad(f.V, rxy, q.nmad(f.Vy, f.rx, q.nmad(f.Vx, f.ry, Wxy[2]))), f.ir);
+    const T Vyy = q.mul(q.nmad(f.V, ryy, q.nmad(f.Vy, ry2, Wyy[2])), f.ir);
+    auto ke = [&](const T W2[4], T a, T b, T c, T d) {   // rho (a b + c d) + u . m'' - rho'' q^2/2
+        return q.nmad(f.hq2, W2[0], q.mad(f.V, W2[2], q.mad(f.U, W2[1], q.mul(f.rho, q.mad(a, b, q.mul(c, d))))));
+    };
+    const T exx = q.sub(Wxx[3], ke(Wxx, f.Ux, f.Ux, f.Vx, f.Vx)), exy = q.sub(Wxy[3], ke(Wxy, f.Ux, f.Uy, f.Vx, f.Vy)),
+            eyy = q.sub(Wyy[3], ke(Wyy, f.Uy, f.Uy, f.Vy, f.Vy));
+    // mixed derivatives d/dx, d/dy of the (negated) first time derivatives
+    const T Dx = q.add(Uxx, Vxy), Dy = q.add(Uxy, Vyy);
+    const T nrxt = q.mad(f.rho, Dx, q.mad(f.rx, f.Dv, q.mad(f.V, rxy, q.mad(f.Vx, f.ry, q.mad(f.U, rxx, q.mul(f.Ux, f.rx))))));
+    const T nryt = q.mad(f.rho, Dy, q.mad(f.ry, f.Dv, q.mad(f.V, ryy, q.mad(f.Vy, f.ry, q.mad(f.U, rxy, q.mul(f.Uy, f.rx))))));
+    const T nUxt = q.mad(q.nmad(q.mul(f.ex, f.rx), f.ir, exx), f.gir, q.mad(f.V, Uxy, q.mad(f.Vx, f.Uy, q.mad(f.U, Uxx, q.mul(f.Ux, f.Ux)))));
+    const T nVyt = q.mad(q.nmad(q.mul(f.ey, f.ry), f.ir, eyy), f.gir, q.mad(f.V, Vyy, q.mad(f.Vy, f.Vy, q.mad(f.U, Vxy, q.mul(f.Uy, f.Vx)))));
+    const T nUyt = q.mad(q.nmad(q.mul(f.ex, f.ry), f.ir, exy), f.gir, q.mad(f.V, Uyy, q.mad(f.Vy, f.Uy, q.mad(f.U, Uxy, q.mul(f.Uy, f.Ux)))));
+    const T nVxt = q.mad(q.nmad(q.mul(f.ey, f.rx), f.ir, exy), f.gir, q.mad(f.V, Vxy, q.mad(f.Vx, f.Vy, q.mad(f.U, Vxx, q.mul(f.Ux, f.Vx)))));
+    const T next = q.mad(gamma, q.mad(f.e, Dx, q.mul(f.ex, f.Dv)), q.mad(f.V, exy, q.mad(f.Vx, f.ey, q.mad(f.U, exx, q.mul(f.Ux, f.ex)))));
+    const T neyt = q.mad(gamma, q.mad(f.e, Dy, q.mul(f.ey, f.Dv)), q.mad(f.V, eyy, q.mad(f.Vy, f.ey, q.mad(f.U, exy, q.mul(f.Uy, f.ex)))));
+    // second time derivatives (the mixed ones enter negated)
+    const T nDt = q.add(nUxt, nVyt);
+    const T rtt = q.mad(f.rho, nDt, q.nmad(f.rt, f.Dv, q.mad(f.V, nryt, q.nmad(f.Vt, f.ry, q.nmad(f.Ut, f.rx, q.mul(f.U, nrxt))))));
+    const T Utt = q.mad(q.mad(q.mul(f.ex, f.rt), f.ir, next), f.gir, q.mad(f.V, nUyt, q.nmad(f.Vt, f.Uy, q.nmad(f.Ut, f.Ux, q.mul(f.U, nUxt)))));
+    const T Vtt = q.mad(q.mad(q.mul(f.ey, f.rt), f.ir, neyt), f.gir, q.mad(f.V, nVyt, q.nmad(f.Vt, f.Vy, q.nmad(f.Ut, f.Vx, q.mul(f.U, nVxt)))));
+    const T ett = q.mad(gamma, q.nmad(f.et, f.Dv, q.mul(f.e, nDt)), q.mad(f.V, neyt, q.nmad(f.Vt, f.ey, q.nmad(f.Ut, f.ex, q.mul(f.U, next)))));
+    // back to conservative variables (E = e + KE)
+    const T rt2 = q.dbl(f.rt);
+    Wtt[0] = rtt;
+    Wtt[1] = q.mad(f.rho, Utt, q.mad(rt2, f.Ut, q.mul(rtt, f.U)));
+    Wtt[2] = q.mad(f.rho, Vtt, q.mad(rt2, f.Vt, q.mul(rtt, f.V)));
+    Wtt[3] = q.mad(f.rho, q.mad(f.V, Vtt, q.mad(f.Vt, f.Vt, q.mad(f.U, Utt, q.mul(f.Ut, f.Ut)))),
+                   q.mad(rt2, f.uut, q.mad(rtt, f.hq2, ett)));
+}
+
+#ifndef CGKS_OPCOUNT_HOST
+// W_tt in pairs of FP32: it enters the interface state as dt^2/8 W_tt and dt^2/6 W_tt,
+// second order in the changes over a time step.  False (nothing written) unless
+//   (a dt)^2 (sum of second derivatives + squared sum of first ones) < 2^-7
+// of the variables' scales rho, rho a, rho a^2 (a = |U| + |V| + 2 sqrt(theta)), so that
+// the pairs' rounding of W_tt (about 2^-45 of its largest term) stays below the last bit
+// of the state.
+__device__ __forceinline__ bool euler_second_split(const RegK& r, const EulerFirst<double>& f, double gamma,
+                                                   const double Wxx[4], const double Wxy[4], const double Wyy[4],
+                                                   double Wtt[4])
+{
+    EulerFirst<ff> g;
+    g.rho = ff_from(f.rho); g.U = ff_from(f.U); g.V = ff_from(f.V); g.ir = ff_from(f.ir); g.gir = ff_from(f.gir);
+    g.hq2 = ff_from(f.hq2); g.e = ff_from(f.e);
+    g.rx = ff_from(f.rx); g.ry = ff_from(f.ry); g.Ux = ff_from(f.Ux); g.Uy = ff_from(f.Uy);
+    g.Vx = ff_from(f.Vx); g.Vy = ff_from(f.Vy); g.ex = ff_from(f.ex); g.ey = ff_from(f.ey); g.Dv = ff_from(f.Dv);
+    g.rt = ff_from(f.rt); g.Ut = ff_from(f.Ut); g.Vt = ff_from(f.Vt); g.et = ff_from(f.et); g.uut = ff_from(f.uut);
+    ff xx[4], xy[4], yy[4], o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { xx[k] = ff_from(Wxx[k]); xy[k] = ff_from(Wxy[k]); yy[k] = ff_from(Wyy[k]); }
+    {
+        // theta = (gamma - 1) e / rho; e * gir
+        const float th = f_mul(g.e.h, g.gir.h), a = f_add(f_add(fabsf(g.U.h), fabsf(g.V.h)), f_mul(2.0f, f_mul(th, f_rsqrt(th))));
+        const float ia = f_rcp(a), ad = f_mul(a, f_lead(r.k(FK_DT))), ir = g.ir.h, ir1 = f_mul(ir, ia), ir2 = f_mul(ir1, ia);
+        // sums, not maxima: a NaN has to fail the comparison
+        auto m3 = [](ff a, ff b, ff c) { return f_add(f_add(fabsf(a.h), fabsf(b.h)), fabsf(c.h)); };
+        const float s2 = f_fma(m3(xx[3], xy[3], yy[3]), ir2,
+                               f_fma(f_add(m3(xx[1], xy[1], yy[1]), m3(xx[2], xy[2], yy[2])), ir1, f_mul(m3(xx[0], xy[0], yy[0]), ir)));
+        const float s1 = f_fma(f_add(fabsf(g.ex.h), fabsf(g.ey.h)), ir2,
+                               f_fma(f_add(m3(g.Ux, g.Uy, g.Vx), fabsf(g.Vy.h)), ia, f_mul(f_add(fabsf(g.rx.h), fabsf(g.ry.h)), ir)));
+        if (!(f_mul(f_mul(ad, ad), f_fma(s1, s1, s2)) < 1.0f / 128.0f)) return false;
+    }
+    euler_second(ArSplit{}, g, ff_from(gamma), xx, xy, yy, o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Wtt[k] = r.add(d_from(o[k].h), d_from(o[k].l));
+    return true;
+}
+#endif
+
 __device__ __forceinline__ void euler_time_derivs(const RegK& r, const double W[4], const double Wx[4],
                                                   const double Wy[4], const double Wxx[4], const double Wxy[4],
                                                   const double Wyy[4], double ir, double U, double V, double p,
                                                   double e, EulerTD& o)
 {
+    EulerFirst<double> f;
+    f.rho = W[0]; f.U = U; f.V = V; f.ir = ir; f.e = e;
     const double rho = W[0], m = W[1], E = W[3];
     // primitive first derivatives
-    const double rx = Wx[0], ry = Wy[0];
-    const double Ux = r.mul(fma(-U, rx, Wx[1]), ir), Uy = r.mul(fma(-U, ry, Wy[1]), ir);
-    const double Vx = r.mul(fma(-V, rx, Wx[2]), ir), Vy = r.mul(fma(-V, ry, Wy[2]), ir);
-    // kinetic energy KE = rho q^2 / 2: KE_x = u . m_x - rho_x q^2/2,
-    // KE_xx = rho |u_x|^2 + u . m_xx - rho_xx q^2/2, KE_xy = rho u_x . u_y + u . m_xy - rho_xy q^2/2
-    const double q2 = fma(U, U, r.mul(V, V));
-    const double hq2 = r.kmul(FK_HALF, q2);
-    const double KEx = fma(-hq2, rx, fma(V, Wx[2], r.mul(U, Wx[1])));
-    const double KEy = fma(-hq2, ry, fma(V, Wy[2], r.mul(U, Wy[1])));
-    const double ex = r.sub(Wx[3], KEx), ey = r.sub(Wy[3], KEy);
-    // primitive second derivatives
-    const double rxx = Wxx[0], rxy = Wxy[0], ryy = Wyy[0];
-    const double rx2 = r.add(rx, rx), ry2 = r.add(ry, ry);
-    const double Uxx = r.mul(fma(-U, rxx, fma(-Ux, rx2, Wxx[1])), ir);
-    const double Uxy = r.mul(fma(-U, rxy, fma(-Uy, rx, fma(-Ux, ry, Wxy[1]))), ir);
-    const double Uyy = r.mul(fma(-U, ryy, fma(-Uy, ry2, Wyy[1])), ir);
-    const double Vxx = r.mul(fma(-V, rxx, fma(-Vx, rx2, Wxx[2])), ir);
-    const double Vxy = r.mul(fma(-V, rxy, fma(-Vy, rx, fma(-Vx, ry, Wxy[2]))), ir);
-    const double Vyy = r.mul(fma(-V, ryy, fma(-Vy, ry2, Wyy[2])), ir);
-    const double KExx = fma(-hq2, rxx, fma(V, Wxx[2], fma(U, Wxx[1], r.mul(rho, fma(Ux, Ux, r.mul(Vx, Vx))))));
-    const double KExy = fma(-hq2, rxy, fma(V, Wxy[2], fma(U, Wxy[1], r.mul(rho, fma(Ux, Uy, r.mul(Vx, Vy))))));
-    const double KEyy = fma(-hq2, ryy, fma(V, Wyy[2], fma(U, Wyy[1], r.mul(rho, fma(Uy, Uy, r.mul(Vy, Vy))))));
-    const double exx = r.sub(Wxx[3], KExx), exy = r.sub(Wxy[3], KExy), eyy = r.sub(Wyy[3], KEyy);
+    f.rx = Wx[0]; f.ry = Wy[0];
+    f.Ux = r.mul(fma(-U, f.rx, Wx[1]), ir); f.Uy = r.mul(fma(-U, f.ry, Wy[1]), ir);
+    f.Vx = r.mul(fma(-V, f.rx, Wx[2]), ir); f.Vy = r.mul(fma(-V, f.ry, Wy[2]), ir);
+    // kinetic energy KE = rho q^2 / 2: KE_x = u . m_x - rho_x q^2/2
+    f.hq2 = r.kmul(FK_HALF, fma(U, U, r.mul(V, V)));
+    const double KEx = fma(-f.hq2, f.rx, fma(V, Wx[2], r.mul(U, Wx[1])));
+    const double KEy = fma(-f.hq2, f.ry, fma(V, Wy[2], r.mul(U, Wy[1])));
+    f.ex = r.sub(Wx[3], KEx); f.ey = r.sub(Wy[3], KEy);
     // first time derivatives (p_x / rho = e_x gir)
     const double gamma = r.k(FK_GAMMA);
-    const double gir = r.mul(r.k(FK_GM1), ir);
-    const double Dv = r.add(Ux, Vy);
-    const double rt = -fma(rho, Dv, fma(V, ry, r.mul(U, rx)));
-    const double Ut = -fma(ex, gir, fma(V, Uy, r.mul(U, Ux)));
-    const double Vt = -fma(ey, gir, fma(V, Vy, r.mul(U, Vx)));
-    const double et = -fma(r.mul(gamma, e), Dv, fma(V, ey, r.mul(U, ex)));
-    // mixed derivatives d/dx, d/dy of the first time derivatives
-    const double Dx = r.add(Uxx, Vxy), Dy = r.add(Uxy, Vyy);
-    const double rxt = -fma(rho, Dx, fma(rx, Dv, fma(V, rxy, fma(Vx, ry, fma(U, rxx, r.mul(Ux, rx))))));
-    const double ryt = -fma(rho, Dy, fma(ry, Dv, fma(V, ryy, fma(Vy, ry, fma(U, rxy, r.mul(Uy, rx))))));
-    const double Uxt = -fma(fma(-r.mul(ex, rx), ir, exx), gir, fma(V, Uxy, fma(Vx, Uy, fma(U, Uxx, r.mul(Ux, Ux)))));
-    const double Vyt = -fma(fma(-r.mul(ey, ry), ir, eyy), gir, fma(V, Vyy, fma(Vy, Vy, fma(U, Vxy, r.mul(Uy, Vx)))));
-    const double Uyt = -fma(fma(-r.mul(ex, ry), ir, exy), gir, fma(V, Uyy, fma(Vy, Uy, fma(U, Uxy, r.mul(Uy, Ux)))));
-    const double Vxt = -fma(fma(-r.mul(ey, rx), ir, exy), gir, fma(V, Vxy, fma(Vx, Vy, fma(U, Vxx, r.mul(Ux, Vx)))));
-    const double ext = -fma(gamma, fma(e, Dx, r.mul(ex, Dv)), fma(V, exy, fma(Vx, ey, fma(U, exx, r.mul(Ux, ex)))));
-    const double eyt = -fma(gamma, fma(e, Dy, r.mul(ey, Dv)), fma(V, eyy, fma(Vy, ey, fma(U, exy, r.mul(Uy, ex)))));
-    // second time derivatives
-    const double Dt = r.add(Uxt, Vyt);
-    const double rtt = -fma(rho, Dt, fma(rt, Dv, fma(V, ryt, fma(Vt, ry, fma(U, rxt, r.mul(Ut, rx))))));
-    const double Utt = -fma(fma(-r.mul(ex, rt), ir, ext), gir, fma(V, Uyt, fma(Vt, Uy, fma(U, Uxt, r.mul(Ut, Ux)))));
-    const double Vtt = -fma(fma(-r.mul(ey, rt), ir, eyt), gir, fma(V, Vyt, fma(Vt, Vy, fma(U, Vxt, r.mul(Ut, Vx)))));
-    const double ett = -fma(gamma, fma(e, Dt, r.mul(et, Dv)), fma(V, eyt, fma(Vt, ey, fma(U, ext, r.mul(Ut, ex)))));
-    // back to conservative variables (E = e + KE)
-    const double uut = fma(V, Vt, r.mul(U, Ut));
-    o.Wt[0] = rt;
-    o.Wt[1] = fma(rho, Ut, r.mul(rt, U));
-    o.Wt[2] = fma(rho, Vt, r.mul(rt, V));
-    o.Wt[3] = fma(rho, uut, fma(rt, hq2, et));
-    const double rt2 = r.add(rt, rt);
-    o.Wtt[0] = rtt;
-    o.Wtt[1] = fma(rho, Utt, fma(rt2, Ut, r.mul(rtt, U)));
-    o.Wtt[2] = fma(rho, Vtt, fma(rt2, Vt, r.mul(rtt, V)));
-    o.Wtt[3] = fma(rho, fma(V, Vtt, fma(Vt, Vt, fma(U, Utt, r.mul(Ut, Ut)))), fma(rt2, uut, fma(rtt, hq2, ett)));
+    f.gir = r.mul(r.k(FK_GM1), ir);
+    f.Dv = r.add(f.Ux, f.Vy);
+    f.rt = -fma(rho, f.Dv, fma(V, f.ry, r.mul(U, f.rx)));
+    f.Ut = -fma(f.ex, f.gir, fma(V, f.Uy, r.mul(U, f.Ux)));
+    f.Vt = -fma(f.ey, f.gir, fma(V, f.Vy, r.mul(U, f.Vx)));
+    f.et = -fma(r.mul(gamma, e), f.Dv, fma(V, f.ey, r.mul(U, f.ex)));
+    f.uut = fma(V, f.Vt, r.mul(U, f.Ut));
+    o.Wt[0] = f.rt;
+    o.Wt[1] = fma(rho, f.Ut, r.mul(f.rt, U));
+    o.Wt[2] = fma(rho, f.Vt, r.mul(f.rt, V));
+    o.Wt[3] = fma(rho, f.uut, fma(f.rt, f.hq2, f.et));
     // normal Euler flux and its time derivative
     const double Ep = r.add(E, p);
-    const double pt = r.mul(r.k(FK_GM1), et);
+    const double pt = r.mul(r.k(FK_GM1), f.et);
     o.F[0] = m;
     o.F[1] = fma(m, U, p);
     o.F[2] = r.mul(m, V);
     o.F[3] = r.mul(U, Ep);
     const double mt = o.Wt[1];
     o.Ft[0] = mt;
-    o.Ft[1] = fma(m, Ut, fma(mt, U, pt));
-    o.Ft[2] = fma(m, Vt, r.mul(mt, V));
-    o.Ft[3] = fma(U, r.add(o.Wt[3], pt), r.mul(Ut, Ep));
+    o.Ft[1] = fma(m, f.Ut, fma(mt, U, pt));
+    o.Ft[2] = fma(m, f.Vt, r.mul(mt, V));
+    o.Ft[3] = fma(U, r.add(o.Wt[3], pt), r.mul(f.Ut, Ep));
     // BGK Navier-Stokes flux per unit tau in the face-normal direction
-    const double sxx = r.mul(p, fma(-r.k(FK_K2INV2), Dv, r.add(Ux, Ux)));
-    const double sxy = r.mul(p, r.add(Uy, Vx));
-    const double thx = r.mul(fma(-r.mul(e, ir), rx, ex), gir);            // d/dx (p / rho)
+    const double sxx = r.mul(p, fma(-r.k(FK_K2INV2), f.Dv, r.add(f.Ux, f.Ux)));
+    const double sxy = r.mul(p, r.add(f.Uy, f.Vx));
+    const double thx = r.mul(fma(-r.mul(e, ir), f.rx, f.ex), f.gir);      // d/dx (p / rho)
     o.TNS[0] = 0.0;
     o.TNS[1] = sxx;
     o.TNS[2] = sxy;
     o.TNS[3] = fma(r.mul(r.k(FK_KHEAT), p), thx, fma(V, sxy, r.mul(U, sxx)));
+#ifndef CGKS_OPCOUNT_HOST
+    if (euler_second_split(r, f, gamma, Wxx, Wxy, Wyy, o.Wtt)) return;
+#endif
+    euler_second(Ar64{r}, f, gamma, Wxx, Wxy, Wyy, o.Wtt);
+}
+
+#ifndef CGKS_OPCOUNT_HOST
+// The slope moments in pairs of FP32.  They enter a face's flux through the weights
+// of order tau^2/dt and its state through h dt, a small correction where the
+// collision time is: false (nothing written) unless every weighted term is below
+// 2^-9 of the side's half-line flux of the same kind (a momentum's scale is the
+// normal momentum flux), so that the pairs' rounding stays below that flux's last
+// bit.  wth, wsl: the weights' magnitudes.
+
+template <class Src>
+__device__ __forceinline__ bool slope_moments_split(const RegK& r, const Src& src, int side, bool ne, double rho,
+                                                    double U, double V, double th, double sq, const HalfMoments& h,
+                                                    float wth, float wsl, ff Th[4], ff Wsl[4])
+{
+    const ff K1 = ff_from(r.k(FK_K1));
+    const ArSplit q{ff_from(r.k(FK_GM1)), K1, ff_add(K1, ff{2.0f, 0.0f})};
+    ff m[4], n[4], s[4], T[4], S[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = ff_from(h.m[k]);
+    src.ne_slopes_split(side, n, s);
+    const ff fV = ff_from(V), fth = ff_from(th);
+    const ff isq = ff_from(sq);
+    slope_moments(q, ne, ff_from(U), fV, fth, ff_scale(2.0f, ff_mul(isq, isq)), m, ff_from(h.g), n, s, T, S);
+    const float fr = f_lead(rho), qt = f_fma(fV.h, fV.h, f_mul(K1.h, fth.h)), f0 = f_mul(fr, fabsf(m[1].h)),
+                f1 = f_mul(fr, m[2].h), f3 = f_mul(f_mul(0.5f, fr), f_fma(fabsf(m[1].h), qt, fabsf(m[3].h)));
+    const float w = f_mul(512.0f, wth), v = f_mul(512.0f, wsl);
+    // sums, not maxima: a NaN has to fail the comparisons
+    bool ok = f0 > 1e-15f && f1 > 1e-15f && f3 > 1e-15f && f_mul(w, fabsf(T[0].h)) < f0 &&
+              f_mul(w, f_add(fabsf(T[1].h), fabsf(T[2].h))) < f1 && f_mul(w, fabsf(T[3].h)) < f3;
+    if (ne)
+        ok = ok && f_mul(v, fabsf(S[0].h)) < fr && f_mul(v, f_add(fabsf(S[1].h), fabsf(S[2].h))) < f0 &&
+             f_mul(v, fabsf(S[3].h)) < f_mul(f_mul(0.5f, fr), f_fma(m[0].h, qt, m[2].h));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Th[k] = ff_add(Th[k], T[k]);
+    if (ne)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) Wsl[k] = ff_add(Wsl[k], S[k]);
+    return ok;
+}
+#endif
+
+// the sums of both sides' half-line terms: fluxes Fh = <u psi>, states Wh = <psi> (where
+// the interface state needs them) and their slope terms Th, Wsl
+struct HalfSums { double Fh[4], Th[4], Wh[4], Wsl[4]; };
+
+// Side by side in a rolled loop: one copy of its instructions for both.  The slope terms
+// in pairs of FP32 first; where a side's do not qualify, the loop runs again with them in
+// FP64.
+template <class Src>
+__device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const double Wl[4], const double Wr[4],
+                                          double Ul, double Vl, double thl, double Ur, double Vr, double thr,
+                                          bool need_ne, float wth, float wsl, HalfSums& o)
+{
+#ifdef CGKS_OPCOUNT_HOST
+    bool split = false;
+#else
+    bool split = true;
+    ff Ts[4], Ss[4];
+#endif
+    for (;;) {
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { o.Fh[k] = 0.0; o.Th[k] = 0.0; o.Wh[k] = 0.0; o.Wsl[k] = 0.0; }
+#ifndef CGKS_OPCOUNT_HOST
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { Ts[k] = ff{0.0f, 0.0f}; Ss[k] = ff{0.0f, 0.0f}; }
+#endif
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            const double rho = side ? Wr[0] : Wl[0], U = side ? Ur : Ul, V = side ? Vr : Vl, th = side ? thr : thl;
+            HalfMoments h;
+            const double th2 = r.add(th, th);
+            const double sq = r.rsq(th2);                     // sqrt(lambda) = 1/sqrt(2 theta)
+            half_moments(r, side, U, th, th2, sq, h);
+            const double qt = fma(V, V, r.mul(r.k(FK_K1), th));       // <v^2 + xi^2>
+            o.Fh[0] = fma(rho, h.m[1], o.Fh[0]);
+            o.Fh[1] = fma(rho, h.m[2], o.Fh[1]);
+            o.Fh[2] = fma(rho, r.mul(V, h.m[1]), o.Fh[2]);
+            o.Fh[3] = fma(rho, r.kmul(FK_HALF, fma(h.m[1], qt, h.m[3])), o.Fh[3]);
+            if (need_ne) {
+                o.Wh[0] = fma(rho, h.m[0], o.Wh[0]);
+                o.Wh[1] = fma(rho, h.m[1], o.Wh[1]);
+                o.Wh[2] = fma(rho, r.mul(V, h.m[0]), o.Wh[2]);
+                o.Wh[3] = fma(rho, r.kmul(FK_HALF, fma(h.m[0], qt, h.m[2])), o.Wh[3]);
+            }
+#ifndef CGKS_OPCOUNT_HOST
+            if (split) {
+                ok &= slope_moments_split(r, src, side, need_ne, rho, U, V, th, sq, h, wth, wsl, Ts, Ss);
+                continue;
+            }
+#endif
+            double bn[4], bt[4], t[4], ws[4];
+            src.ne_slopes(side, bn, bt);
+            const double ith = need_ne ? r.mul(r.add(sq, sq), sq) : th;     // 1/theta = 2 lambda
+            slope_moments(Ar64{r}, need_ne, U, V, th, ith, h.m, h.g, bn, bt, t, ws);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) o.Th[k] = r.add(o.Th[k], t[k]);
+            if (need_ne)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(o.Wsl[k], ws[k]);
+        }
+        if (!split) return;
+#ifndef CGKS_OPCOUNT_HOST
+        if (ok) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) o.Th[k] = r.add(d_from(Ts[k].h), d_from(Ts[k].l));
+            if (need_ne)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(d_from(Ss[k].h), d_from(Ss[k].l));
+            return;
+        }
+#endif
+        split = false;
+    }
 }
 
 // ------------------------------------------------------------------------
@@ -457,9 +663,8 @@ __device__ __forceinline__ void euler_time_derivs(const RegK& r, const double W[
 // consumed, so that the 48 reconstructed quantities are never live at once:
 //   src.eq_value(W0)                          equilibrium state
 //   src.eq_derivs(W0n, W0t, W0nn, W0nt, W0tt)  its derivatives (face frame)
-//   src.ne_value(side, W, Wt)                 left (0) / right (1) state and its
-//                                             tangential derivative
-//   src.ne_normal(side, Wn)                   its normal derivative
+//   src.ne_value(side, W)                     left (0) / right (1) state
+//   src.ne_slopes(side, Wn, Wt)               its normal and tangential derivatives
 // The caller's table holds the grid's gamma, K and the time step.
 template <int STAGE, class Src>
 __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double Fb[4], double Ft[4], double Wm[4],
@@ -468,86 +673,52 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     // equilibrium state g0
     double W0[4];
     src.eq_value(W0);
-    const double ir0 = r.rcp(W0[0]);
+    const double ir0 = r.rcp3(W0[0]);
     const double U0 = r.mul(W0[1], ir0), V0 = r.mul(W0[2], ir0);
     const double e0 = r.kfma(FK_MHALF, fma(W0[2], V0, r.mul(W0[1], U0)), W0[3]);   // p0 / (gamma - 1)
     const double p0 = r.mul(r.k(FK_GM1), e0);
     // non-equilibrium states
-    double Wl[4], Wlt[4], Wr[4], Wrt[4];
-    src.ne_value(0, Wl, Wlt);
-    src.ne_value(1, Wr, Wrt);
-    const double irl = r.rcp(Wl[0]);
+    double Wl[4], Wr[4];
+    src.ne_value(0, Wl);
+    src.ne_value(1, Wr);
+    const double irl = r.rcp3(Wl[0]);
     const double Ul = r.mul(Wl[1], irl), Vl = r.mul(Wl[2], irl);
     const double pl = r.mul(r.k(FK_GM1), r.kfma(FK_MHALF, fma(Wl[2], Vl, r.mul(Wl[1], Ul)), Wl[3]));
-    const double irr = r.rcp(Wr[0]);
+    const double irr = r.rcp3(Wr[0]);
     const double Ur = r.mul(Wr[1], irr), Vr = r.mul(Wr[2], irr);
     const double pr = r.mul(r.k(FK_GM1), r.kfma(FK_MHALF, fma(Wr[2], Vr, r.mul(Wr[1], Ur)), Wr[3]));
-    const bool ok = (W0[0] > 0.0) && (p0 > 0.0) && (Wl[0] > 0.0) && (pl > 0.0) && (Wr[0] > 0.0) && (pr > 0.0);
+    const bool ok = positive(W0[0]) && positive(p0) && positive(Wl[0]) && positive(pl) && positive(Wr[0]) && positive(pr);
     const double thl = r.mul(pl, irl), thr = r.mul(pr, irr);
 
     // Sec. 4: collision time with pressure-jump enhancement; viscous flow: mu/p
     // with p the equilibrium pressure at the point
     const double mu = r.k(FK_MU), dt = r.k(FK_DT);
-    const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(pl, pr), r.rcp(r.add(pl, pr)))),
-                           mu > 0.0 ? r.mul(mu, r.rcp(p0)) : r.k(FK_EPSDT));
+    const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(pl, pr), r.rcp3(r.add(pl, pr)))),
+                           positive(mu) ? r.mul(mu, r.rcp3(p0)) : r.k(FK_EPSDT));
     // h = exp(-dt / (2 tau)) weights the non-equilibrium part of the interface state.
     // For dt > 80 tau, h < 4e-18: then 1 - h and 3 - h round to 1 and 3, and the
     // remaining h-terms change the window coefficients by under 2e-14 of a term
-    // that is itself O(tau^2), so h is taken as 0 without evaluating the exponential
+    // that is itself O(tau^2), so h is taken as 0 without evaluating the exponential.
+    // Below h = 1e-20 that part is under 1e-20 of the state it is added to: far below one
+    // ulp, so its velocity moments are not evaluated (the flux terms, weighted by O(tau),
+    // are).
     double h = 0.0;
-    if (tau > 0.0 && dt < 80.0 * tau) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp(tau)));
-    // below 1e-20 that part is under 1e-20 of the state it is added to: far below one ulp,
-    // so its velocity moments are not evaluated (the flux terms, weighted by O(tau), are)
+#ifdef CGKS_OPCOUNT_HOST
+    if (tau > 0.0 && dt < 80.0 * tau) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
     const bool need_ne = (STAGE == 1) && (h >= 1e-20);
+    const float wth = 0.0f, wsl = 0.0f;
+#else
+    const float ft = f_lead(tau), fdt = f_lead(dt);
+    if (ft > 0.0f && fdt < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
+    const bool need_ne = (STAGE == 1) && d_hi(h) >= 0x3bc79ca1;       // high word of 1e-20
+    // bounds of the slope terms' weights (FP32, for the choice of their arithmetic): beside F
+    // |b4| and |f4| dt/4 below are at most 4 tau (tau + h dt) / dt, beside W it is h dt
+    const float wsl = f_mul(fdt, f_lead(h));
+    const float wth = f_mul(f_mul(4.0f, f_mul(ft, f_add(ft, wsl))), f_lead(r.k(FK_IDT)));
+#endif
 
-    // half-line moments of g_l (u > 0) and g_r (u < 0)
-    double Fh[4], Th[4], Wh[4] = {0, 0, 0, 0}, Wsl[4] = {0, 0, 0, 0};
-    {
-        Moments ml;
-        const double th2 = r.add(thl, thl);
-        const double sq = rsqrt(th2);                     // sqrt(lambda_l) = 1/sqrt(2 theta)
-        const double ithl = r.mul(r.add(sq, sq), sq);     // 1/theta = 2 lambda_l
-        half_moments01<+1>(r, Ul, sq, r.mul(th2, sq), ml.u[0], ml.u[1]);
-        moments_tail(r, ml, Ul, Vl, thl);
-        SlopeCtx sl;
-        slope_ctx(r, Ul, Vl, thl, ithl, sl);
-        // micro-slopes of g_l: M^-1 (dW / rho); the 1/rho cancels against the rho in front
-        // of the slope moments, so M^-1 is applied to dW itself
-        double b1[4], a1[4], a2[4], o1[4], f[4];
-        src.ne_normal(0, b1);
-        micro_slope(r, sl, b1, a1);
-        micro_slope(r, sl, Wlt, a2);
-        psi_u<1>(r, ml, f);
-        q_moments<1>(r, ml, a1, a2, o1);
-        for (int k = 0; k < 4; ++k) { Fh[k] = r.mul(Wl[0], f[k]); Th[k] = o1[k]; }
-        if (need_ne) {
-            psi_u<0>(r, ml, f);
-            q_moments<0>(r, ml, a1, a2, o1);
-            for (int k = 0; k < 4; ++k) { Wh[k] = r.mul(Wl[0], f[k]); Wsl[k] = o1[k]; }
-        }
-    }
-    {
-        Moments mr;
-        const double th2 = r.add(thr, thr);
-        const double sq = rsqrt(th2);
-        const double ithr = r.mul(r.add(sq, sq), sq);
-        half_moments01<-1>(r, Ur, sq, r.mul(th2, sq), mr.u[0], mr.u[1]);
-        moments_tail(r, mr, Ur, Vr, thr);
-        SlopeCtx sr;
-        slope_ctx(r, Ur, Vr, thr, ithr, sr);
-        double b1[4], a1[4], a2[4], o1[4], f[4];
-        src.ne_normal(1, b1);
-        micro_slope(r, sr, b1, a1);
-        micro_slope(r, sr, Wrt, a2);
-        psi_u<1>(r, mr, f);
-        q_moments<1>(r, mr, a1, a2, o1);
-        for (int k = 0; k < 4; ++k) { Fh[k] = fma(Wr[0], f[k], Fh[k]); Th[k] = r.add(Th[k], o1[k]); }
-        if (need_ne) {
-            psi_u<0>(r, mr, f);
-            q_moments<0>(r, mr, a1, a2, o1);
-            for (int k = 0; k < 4; ++k) { Wh[k] = fma(Wr[0], f[k], Wh[k]); Wsl[k] = r.add(Wsl[k], o1[k]); }
-        }
-    }
+    HalfSums o;
+    half_sums(r, src, Wl, Wr, Ul, Vl, thl, Ur, Vr, thr, need_ne, wth, wsl, o);
 
     // Euler derivatives of the equilibrium state (W_t, W_tt, F, F_t), evaluated after the
     // half-line moments so that the two sets of intermediates are never live together
@@ -559,6 +730,7 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     }
 
     // tau-terms of g0: rho <(a_n u + a_t v) u psi> = TNS - F_t (the time part is the Euler F_t)
+    // window coefficients over [0, dt]
     const double idt = r.k(FK_IDT);
     const double omh = r.sub(r.one, h);
     const double ta = r.mul(tau, omh);                       // tau (1 - h)
@@ -570,8 +742,8 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     const double a = r.mul(tat, idt);
     const double b4 = r.mul(r.mul(tau, fma(-dh, r.sub(r.k(FK_2), h), tat)), idt);
     for (int k = 0; k < 4; ++k) {
-        const double dTh = (k == 0) ? -r.add(e.Ft[0], Th[0]) : r.sub(r.sub(e.TNS[k], e.Ft[k]), Th[k]);
-        const double dFh = r.sub(Fh[k], e.F[k]);
+        const double dTh = (k == 0) ? -r.add(e.Ft[0], o.Th[0]) : r.sub(r.sub(e.TNS[k], e.Ft[k]), o.Th[k]);
+        const double dFh = r.sub(o.Fh[k], e.F[k]);
         Ft[k] = fma(f4, dTh, fma(-g, dFh, e.Ft[k]));
         if (STAGE == 1) Fb[k] = fma(b4, dTh, (k == 0) ? fma(a, dFh, e.F[0]) : fma(-tau, e.TNS[k], fma(a, dFh, e.F[k])));
     }
@@ -582,8 +754,8 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
             Wm[k] = fma(r.k(FK_C8), e.Wtt[k], fma(hdt, e.Wt[k], W0[k]));
             Wb[k] = fma(r.k(FK_C6), e.Wtt[k], fma(dt, e.Wt[k], W0[k]));
             if (need_ne) {
-                Wm[k] = fma(h, fma(-hdt, e.Wt[k], r.sub(fma(-hdt, Wsl[k], Wh[k]), W0[k])), Wm[k]);
-                Wb[k] = fma(h2, fma(-dt, e.Wt[k], r.sub(fma(-dt, Wsl[k], Wh[k]), W0[k])), Wb[k]);
+                Wm[k] = fma(h, fma(-hdt, e.Wt[k], r.sub(fma(-hdt, o.Wsl[k], o.Wh[k]), W0[k])), Wm[k]);
+                Wb[k] = fma(h2, fma(-dt, e.Wt[k], r.sub(fma(-dt, o.Wsl[k], o.Wh[k]), W0[k])), Wb[k]);
             }
         }
     } else {

@@ -106,21 +106,30 @@ inline size_t face_doubles(int nx, int ny, int dim)
 struct TileRef { int grid, x0, y0, pad; };
 
 // tile shapes compiled into the library, in the public numbering of
-// cgks_set_tile_shape.  The flux kernel runs one face segment per thread and a
-// tile owns 2 TX TY segments (plus the grid's last faces on its edges), so
-// 16x8 (256), 16x16 (512), 24x16 and 32x12 (768) fill whole passes of
-// the 256-thread CTA; a tile's records must fit 227 KB of shared memory.
+// cgks_set_tile_shape.  The flux kernel runs one Gauss point of a face segment per
+// thread, 64 segments at a time per CTA of 128 threads; a tile owns 2 TX TY segments, its
+// records and the CTA's slices must fit 227 KB of shared memory.
 #define CGKS_FOR_EACH_TILE(X) X(16, 8) X(8, 16) X(32, 4) X(64, 1) X(16, 7) X(7, 16) X(14, 8) X(24, 8) \
     X(16, 14) X(20, 11) X(15, 15) X(22, 10) X(18, 12) X(20, 12) X(15, 16) X(17, 14) X(16, 16) X(24, 16) X(32, 12)
 #define CGKS_TILE_ENUM(w, h) TILE_##w##x##h,
 enum TileShape { CGKS_FOR_EACH_TILE(CGKS_TILE_ENUM) TILE_COUNT };
 #undef CGKS_TILE_ENUM
-#define CGKS_TILE_W(w, h) w,
-#define CGKS_TILE_H(w, h) h,
+// The tiles of a shape's queue: the shape itself, except that 8x16, the 2D default, is
+// worked on (queued and staged) as 8x4 strips of 64 segments, one pass of a CTA.  The
+// strips' records and slices take 49 KB, so three CTAs fit an SM; a small grid spreads
+// over twice the CTAs of 8x8 strips (64^2: stage-1 flux 75.8 -> 42.9 us; 2048^2: 18.4 ->
+// 17.8 ms).
+constexpr int work_w(int w, int) { return w; }
+constexpr int work_h(int w, int h) { return w == 8 && h == 16 ? 4 : h; }
+#define CGKS_TILE_W(w, h) work_w(w, h),
+#define CGKS_TILE_H(w, h) work_h(w, h),
 inline int tile_w(int s) { static const int v[TILE_COUNT] = {CGKS_FOR_EACH_TILE(CGKS_TILE_W)}; return v[s]; }
 inline int tile_h(int s) { static const int v[TILE_COUNT] = {CGKS_FOR_EACH_TILE(CGKS_TILE_H)}; return v[s]; }
 #undef CGKS_TILE_W
 #undef CGKS_TILE_H
+// the tiles of a grid for a shape, in queue order.  Along an axis that the tiles divide, one more
+// row of tiles holds the grid's last faces alone (they would cost the last tiles a second pass).
+std::vector<TileRef> make_tiles(int nx, int ny, int dim, int shape, int grid, bool last_faces = true);
 
 // the record kernel's CTA and chunk: one warp per FP64 unit of an SM, so that a
 // small grid's items spread over the SMs one warp per unit
@@ -141,12 +150,15 @@ inline int update_blocks(int nchunks, int nsm, int cpt = 1)
     const int cap = 8 * cpt * nsm;
     return nchunks < cap ? nchunks : cap;
 }
-// flux kernel: two resident CTAs of 128 threads per SM (one stages its tile
-// while the other computes)
-constexpr int kStageCtasPerSm = 2;
-inline int stage_blocks(int ntiles, int nsm)
+// flux kernel: resident CTAs of 128 threads per SM.  The 8x4 strips run three at 168
+// registers (250 B of spills in stage 1): with two CTAs the FP64 unit was 57 % busy, its
+// warps waiting for one another's FP64 and FP32 chains; four at 128 registers spill more
+// and are no faster (2048^2, stage 1: 21.4, 17.8, 18.3 ms with two, three, four).
+constexpr int stage_ctas(int tx, int ty) { return tx == 8 && ty == 4 ? 3 : 2; }
+inline int stage_blocks(int ntiles, int nsm, int shape)
 {
-    return ntiles < kStageCtasPerSm * nsm ? ntiles : kStageCtasPerSm * nsm;
+    const int cap = stage_ctas(tile_w(shape), tile_h(shape)) * nsm;
+    return ntiles < cap ? ntiles : cap;
 }
 
 // persistent grid of the record kernel: its resident CTAs (four per SM with

@@ -90,11 +90,10 @@ cgks_status setup_device(int dev, DeviceSymbols** out)
 
 // fills the descriptor, the tile queue and the record-kernel queue of this call
 // (kernel arguments carry the values, so no host buffer has to outlive the call)
-__global__ void noalloc_init_kernel(cgks::GridDev G, int tw, int th, int nchunks, int ncchunks)
+__global__ void noalloc_init_kernel(cgks::GridDev G, int tw, int th, int ntx, int ntiles, int nchunks, int ncchunks)
 {
-    const int ntx = (G.nx + tw - 1) / tw, nty = (G.ny + th - 1) / th;
     if (blockIdx.x == 0 && threadIdx.x == 0) g_desc = G;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntx * nty; t += gridDim.x * blockDim.x)
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x)
         g_tiles[t] = cgks::TileRef{0, (t % ntx) * tw, (t / ntx) * th, 0};
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nchunks; c += gridDim.x * blockDim.x)
         g_rchunks[c] = cgks::TileRef{0, cgks::kRecordChunk * c, 0, 0};
@@ -134,9 +133,11 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
         const int n = k < 2 ? prob->nx : prob->ny;
         if (prob->bc[k] == CGKS_BC_REFLECT && n < 2) return nfail(CGKS_E_INVAL, "a reflecting side needs >= 2 cells");
     }
-    const int shape = TILE_16x8;
+    const int shape = TILE_8x16;
     const int tw = tile_w(shape), th = tile_h(shape);
-    const long long ntiles = (long long)((prob->nx + tw - 1) / tw) * ((prob->ny + th - 1) / th);
+    // the queue of make_tiles: one more row of tiles along an axis that the tiles divide
+    const int ntx = prob->nx / tw + 1, nty = prob->ny / th + 1;
+    const long long ntiles = (long long)ntx * nty - (prob->nx % tw == 0 && prob->ny % th == 0 ? 1 : 0);
     if (ntiles > kMaxTiles) return nfail(CGKS_E_INVAL, "grid needs more tiles than CGKS_NOALLOC_MAX_TILES");
 
     int dev = 0, nsm = 1;
@@ -190,12 +191,12 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     const int nrc = (int)((items + kRecordChunk - 1) / kRecordChunk);
     const int ncc = (int)((cells + 255) / 256);
     const int work = nt > nrc ? nt : nrc;
-    noalloc_init_kernel<<<(work + 255) / 256, 256, 0, stream>>>(G, tw, th, nrc, ncc);
+    noalloc_init_kernel<<<(work + 255) / 256, 256, 0, stream>>>(G, tw, th, ntx, nt, nrc, ncc);
     NCK(cudaGetLastError());
     // control block starts from t, step 0, no error, state in the caller's buffer
     NCK(launch_set_ctrl(sym->ctrl, *t_inout, 0.0, -1, 1, stream));
     NCK(launch_cfl(sym->desc, 0, G, stream));
-    const int nblocks = stage_blocks(nt, nsm);
+    const int nblocks = stage_blocks(nt, nsm, shape);
     const int rblocks = record_blocks(nrc, nsm, cv);
     const int ublocks = update_blocks(ncc, nsm);
     for (int k = 0; k < nsteps; ++k) {

@@ -9,7 +9,7 @@
 
 namespace cgks {
 
-constexpr int kThreads = 128;
+constexpr int kThreads = 128, kPairs = kThreads / 2;
 
 template <int STAGE> struct FaceQ { static constexpr int n = (STAGE == 1) ? 16 : 8; };
 
@@ -37,199 +37,203 @@ struct StageLayout {
     static constexpr int NF = FaceQ<STAGE>::n;
     static constexpr int n_rx = RecGroups<TY, TX + 1>::n;
     static constexpr int n_ry = RecGroups<TX, TY + 1>::n;
-    // where it fits, a per-thread slice of 32 doubles holds the Gauss-point-independent
-    // parts of the tangential / normal derivatives of one segment (shared by its two points)
-    static constexpr int n_dc_full = 32 * kThreads;
-    static constexpr bool share =
-        kStageCtasPerSm * (sizeof(double) * (size_t)(n_rx + n_ry + n_dc_full) + 2048) <= 228 * 1024;
-    static constexpr int n_dc = share ? n_dc_full : 0;
-    static constexpr size_t bytes = sizeof(double) * (size_t)(n_rx + n_ry + n_dc);
+    // a slice per pair of threads: what the two Gauss points of its segment share
+    static constexpr int n_parts = 48 * kPairs;
+    static constexpr size_t bytes = sizeof(double) * (size_t)(n_rx + n_ry + n_parts);
 };
 
-// The face rows around one face segment (records of rows j-2..j+2 of one
-// face) and the reconstruction along the face at one Gauss point eta: the
-// WENO-Z point values (equilibrium over five rows, non-equilibrium slopes over
-// three) are computed once per segment for both points and carried in W0, sL,
-// sR; tangential derivatives of the equilibrium state and normal derivatives
-// come from the quartic / quadratic through the same line averages.
-template <bool SHARE>
-struct SegmentRows {
+// One Gauss point of a face segment: the face rows around it (records of rows
+// j-2..j+2 of one face) and the reconstruction along the face there.  The
+// segment's slice (segment_parts; part j of variable k at part[(kPartsVar k + j)
+// * stride]) holds what its two Gauss points share.
+enum { kPartsVar = 12, kParts = 4 * kPartsVar };   // 0..7: deriv_parts, 8, 9: W0 at eta = -g, +g, 10, 11: slopes of W_l, W_r
+
+struct SegmentPoint {
     RegK r;
     const double* rec;
     int pa, pb, pc, r0, rstride;
     double eta, iht;
-    double W0[4], sL[4], sR[4];   // WENO-Z values at this point, non-equilibrium slopes
-    const double* dc;             // SHARE: this thread's slice of the segment's derivative parts
+    int gp;                       // 0: eta = -g, 1: +g
+    const double* part;
+    int stride;
 
     __device__ __forceinline__ double at(int f, int k, int off) const
     {
         return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off);
     }
+    __device__ __forceinline__ double P(int k, int j) const { return part[(kPartsVar * k + j) * stride]; }
 
     __device__ __forceinline__ void eq_value(double W[4]) const
     {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) W[k] = W0[k];
+        for (int k = 0; k < 4; ++k) W[k] = P(k, 8 + gp);
     }
 
-    // The quartic through the segment means m_{j-2..j+2} (m0 the centre row), written
-    // with S1 = m_1 + m_-1, S2 = m_2 + m_-2, A1 = m_1 - m_-1, A2 = m_2 - m_-2:
-    //   p(eta)   = m0 - (S2 - 4 S1 + 6 m0)/4320 + eta (50 A1 - 7 A2)/72 + O(eta^2 - 1/12)
-    //   p'(eta)  = (8 A1 - A2)/12 + eta (13 S1 - S2 - 24 m0)/9 + O(eta^2 - 1/12)
-    //   p''(eta) = (16 S1 - S2 - 30 m0)/12 + eta (A2 - 2 A1)/2 + O(eta^2 - 1/12)
+    // The quartic through the segment means m_{j-2..j+2} (m0 the centre row): with A1 =
+    // m_1 - m_-1, the second difference s1, the sum ts and the difference td of the two
+    // third differences,
+    //   p(eta)   = m0 - td/4320 + eta (A1/2 - 7 ts/72) + O(eta^2 - 1/12)
+    //   p'(eta)  = A1/2 - ts/12 + eta (s1 - td/9) + O(eta^2 - 1/12)
+    //   p''(eta) = s1 - td/12 + eta ts/2 + O(eta^2 - 1/12)
     // (exact at the Gauss points eta = +-1/(2 sqrt 3), where eta^2 = 1/12)
     __device__ __forceinline__ void eq_derivs(double W0n[4], double W0t[4], double W0nn[4], double W0nt[4],
                                               double W0tt[4]) const
     {
         const double iht2 = r.mul(iht, iht);
-        if constexpr (SHARE) {
-            // the parts computed once per segment by seg_deriv_parts: value + eta * slope
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                auto P = [&](int j) { return dc[(8 * k + j) * kThreads]; };
-                W0t[k] = r.mul(fma(eta, P(1), P(0)), iht);
-                W0tt[k] = r.mul(fma(eta, P(3), P(2)), iht2);
-                W0n[k] = fma(eta, P(5), P(4));
-                W0nt[k] = r.mul(fma(eta, P(7), P(6)), iht);
-                W0nn[k] = at(RNN, k, 0);
-            }
-            return;
-        }
-        auto dp = [&](double m0, double S1, double S2, double A1, double A2) {   // p'(eta) / h_t
-            return r.mul(fma(eta, r.kfma(FK_S1T, S1, r.kfma(FK_S2T, S2, r.kmul(FK_M0T, m0))),
-                             r.kfma(FK_A1T, A1, r.kmul(FK_A2T, A2))), iht);
-        };
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            {
-                const double m0 = at(RV, k, 0), mp = at(RV, k, 1), mm = at(RV, k, -1);
-                const double m2p = at(RV, k, 2), m2m = at(RV, k, -2);
-                const double S1 = r.add(mp, mm), S2 = r.add(m2p, m2m), A1 = r.sub(mp, mm), A2 = r.sub(m2p, m2m);
-                W0t[k] = dp(m0, S1, S2, A1, A2);
-                W0tt[k] = r.mul(fma(eta, r.kfma(FK_HALF, A2, -A1),
-                                    r.kfma(FK_S1TT, S1, r.kfma(FK_S2TT, S2, r.kmul(FK_M0TT, m0)))), iht2);
-            }
-            {
-                const double m0 = at(RN, k, 0), mp = at(RN, k, 1), mm = at(RN, k, -1);
-                const double m2p = at(RN, k, 2), m2m = at(RN, k, -2);
-                const double S1 = r.add(mp, mm), S2 = r.add(m2p, m2m), A1 = r.sub(mp, mm), A2 = r.sub(m2p, m2m);
-                W0n[k] = fma(eta, r.kfma(FK_A1N, A1, r.kmul(FK_A2N, A2)),
-                             r.kfma(FK_M0N, m0, r.kfma(FK_S1N, S1, r.kmul(FK_S2N, S2))));
-                W0nt[k] = dp(m0, S1, S2, A1, A2);
-            }
+            W0t[k] = r.mul(fma(eta, P(k, 1), P(k, 0)), iht);
+            W0tt[k] = r.mul(fma(eta, P(k, 3), P(k, 2)), iht2);
+            W0n[k] = fma(eta, P(k, 5), P(k, 4));
+            W0nt[k] = r.mul(fma(eta, P(k, 7), P(k, 6)), iht);
             W0nn[k] = at(RNN, k, 0);
         }
     }
 
-    // the eta-independent parts of the quartic's derivatives above for variable k
-    // (rows m_{-2..2} of the values and of the normal derivatives), stored at dc
-    // (S1 = mp + mm and A1 = mp - mm come from the caller, which shares them with the WENO-Z values)
-    __device__ __forceinline__ static void seg_deriv_parts(const RegK& r, double* dc, double m2m, double S1, double A1,
-                                                           double m0, double m2p, double n2m, double nm, double n0,
-                                                           double np, double n2p)
-    {
-        const double S2 = r.add(m2p, m2m), A2 = r.sub(m2p, m2m);
-        dc[0 * kThreads] = r.kfma(FK_A1T, A1, r.kmul(FK_A2T, A2));
-        dc[1 * kThreads] = r.kfma(FK_S1T, S1, r.kfma(FK_S2T, S2, r.kmul(FK_M0T, m0)));
-        dc[2 * kThreads] = r.kfma(FK_S1TT, S1, r.kfma(FK_S2TT, S2, r.kmul(FK_M0TT, m0)));
-        dc[3 * kThreads] = r.kfma(FK_HALF, A2, -A1);
-        const double T1 = r.add(np, nm), T2 = r.add(n2p, n2m), B1 = r.sub(np, nm), B2 = r.sub(n2p, n2m);
-        dc[4 * kThreads] = r.kfma(FK_M0N, n0, r.kfma(FK_S1N, T1, r.kmul(FK_S2N, T2)));
-        dc[5 * kThreads] = r.kfma(FK_A1N, B1, r.kmul(FK_A2N, B2));
-        dc[6 * kThreads] = r.kfma(FK_A1T, B1, r.kmul(FK_A2T, B2));
-        dc[7 * kThreads] = r.kfma(FK_S1T, T1, r.kfma(FK_S2T, T2, r.kmul(FK_M0T, n0)));
-    }
-
-    __device__ __forceinline__ void ne_value(int side, double W[4], double Wt[4]) const
+    __device__ __forceinline__ void ne_value(int side, double W[4]) const
     {
         const int f = side ? RR : RL;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const double sl = side ? sR[k] : sL[k];
-            W[k] = fma(eta, sl, at(f, k, 0));
-            Wt[k] = r.mul(sl, iht);
-        }
+        for (int k = 0; k < 4; ++k) W[k] = fma(eta, P(k, 10 + side), at(f, k, 0));
     }
 
-    __device__ __forceinline__ void ne_normal(int side, double Wn[4]) const
+    __device__ __forceinline__ void ne_slopes(int side, double Wn[4], double Wt[4]) const
     {
         const int f = side ? RRN : RLN;
         const double he = r.kmul(FK_HALF, eta);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) Wn[k] = fma(he, r.sub(at(f, k, 1), at(f, k, -1)), at(f, k, 0));
+        for (int k = 0; k < 4; ++k) {
+            Wn[k] = fma(he, r.sub(at(f, k, 1), at(f, k, -1)), at(f, k, 0));
+            Wt[k] = r.mul(P(k, 10 + side), iht);
+        }
     }
+
+#ifndef CGKS_OPCOUNT_HOST
+    __device__ __forceinline__ void ne_slopes_split(int side, ff Wn[4], ff Wt[4]) const
+    {
+        const int f = side ? RRN : RLN;
+        const ff he = ff_from(r.kmul(FK_HALF, eta)), ih = ff_from(iht);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            Wn[k] = ff_add(ff_mul(he, ff_sub(ff_from(at(f, k, 1)), ff_from(at(f, k, -1)))), ff_from(at(f, k, 0)));
+            Wt[k] = ff_mul(ff_from(P(k, 10 + side)), ih);
+        }
+    }
+#endif
 };
 
-// One face segment of the flux kernel: the nonlinear point values along the face
-// at both Gauss points, then the gas-kinetic evaluation at each point, Gauss-
-// averaged (weight 1/2) with the stage's time factors into acc (face frame;
-// stage 1: the W* and R flux combinations and the interface states W(dt/2),
-// W(dt); stage 2: dt^2/3 F_t and dt^2/3 W_tt).  rec, pa, pb, pc, r0, rstride
-// locate the segment's face rows in the tile's records; dc is this thread's
-// slice for the Gauss-point-independent derivative parts (SHARE).  PARK: the
-// first point's sums are stored at park[q * park_stride] (the segment's own
-// output slots) while the second point is evaluated, and read back after it,
-// which frees their registers (the same values, the same bits).  Returns
-// false if a state was non-physical.
-template <int STAGE, bool SHARE, bool PARK = false>
-__device__ __forceinline__ bool segment_results(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
-                                                int rstride, double iht, double* dc, double acc[FaceQ<STAGE>::n],
-                                                double* park = nullptr, size_t park_stride = 0)
+// the eta-independent parts of the quartic's derivatives for one variable (differences x
+// of the values, rows n_{-2..2} of the normal derivatives), part j at p[j * stride]
+__device__ __forceinline__ void deriv_parts(const RegK& r, double* p, int stride, const TangDiffs& x, double n2m,
+                                            double nm, double n0, double np, double n2p)
 {
-    constexpr int NF = FaceQ<STAGE>::n;
-    constexpr double gq = 0.28867513459481287;   // 1/(2 sqrt 3): Gauss points at +-gq
-    const double weps = r.k(FK_WEPS), weps4 = r.k(FK_WEPS4);
-    bool bad = false;
-#pragma unroll
-    for (int q = 0; q < NF; ++q) acc[q] = 0.0;
-    // the nonlinear values along the face: both Gauss points at once
-    double W0m[4], W0p[4], sL[4], sR[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        auto R = [&](int f, int off) { return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off); };
-        const double m2m = R(RV, -2), mm = R(RV, -1), m0 = R(RV, 0), mp = R(RV, 1), m2p = R(RV, 2);
-        const double S1 = r.add(mp, mm), A1 = r.sub(mp, mm);
-        tang_weno5_pair(r, m2m, mm, m0, mp, m2p, A1, S1, weps4, W0m[k], W0p[k]);
-        if constexpr (SHARE)
-            SegmentRows<true>::seg_deriv_parts(r, dc + 8 * k * kThreads, m2m, S1, A1, m0, m2p, R(RN, -2), R(RN, -1),
-                                               R(RN, 0), R(RN, 1), R(RN, 2));
-        tang_weno3_slopes(r, R(RL, -1), R(RL, 0), R(RL, 1), R(RR, -1), R(RR, 0), R(RR, 1), weps, sL[k], sR[k]);
+    {
+        const double ts = r.add(x.t0, x.t1), td = r.sub(x.t1, x.t0);
+        p[0 * stride] = r.kfma(FK_M12TH, ts, r.kmul(FK_HALF, x.A1));
+        p[1 * stride] = r.kfma(FK_M9TH, td, x.s1);
+        p[2 * stride] = r.kfma(FK_M12TH, td, x.s1);
+        p[3 * stride] = r.kmul(FK_HALF, ts);
     }
+    const double B1 = r.sub(np, nm), hB = r.kmul(FK_HALF, B1), s1 = r.kfma(FK_M2, n0, r.add(np, nm));
+    const double ts = r.kfma(FK_M2, B1, r.sub(n2p, n2m));
+    const double td = r.kfma(FK_M4, s1, r.kfma(FK_M2, n0, r.add(n2p, n2m)));
+    p[4 * stride] = r.kfma(FK_M4320TH, td, n0);
+    p[5 * stride] = r.kfma(FK_M7_72, ts, hB);
+    p[6 * stride] = r.kfma(FK_M12TH, ts, hB);
+    p[7 * stride] = r.kfma(FK_M9TH, td, s1);
+}
+
+// What the Gauss points of a segment share, for variables k0..k1-1: the nonlinear values
+// along the face at both points, the non-equilibrium slopes, the derivatives' parts.  A
+// rolled loop: unrolled, its instructions alone outgrow the instruction cache.
+__device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
+                                              int rstride, int k0, int k1, double* part, int stride)
+{
+    const double weps = r.k(FK_WEPS), weps4 = r.k(FK_WEPS4);
+    auto R = [&](int f, int k, int off) { return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off); };
+#ifndef CGKS_OPCOUNT_HOST
+    // scales (high words): the smallest of the three states' densities and energies; a
+    // momentum also against sqrt(rho E)
+    const int sc0 = i_min(i_min(hi_abs(R(RV, 0, 0)), hi_abs(R(RL, 0, 0))), hi_abs(R(RR, 0, 0)));
+    const int sc3 = i_min(i_min(hi_abs(R(RV, 3, 0)), hi_abs(R(RL, 3, 0))), hi_abs(R(RR, 3, 0)));
+#endif
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+        double* p = part + kPartsVar * k * stride;
+        const double m0 = R(RV, k, 0);
+        TangDiffs x;
+        tang_diffs(r, R(RV, k, -2), R(RV, k, -1), m0, R(RV, k, 1), R(RV, k, 2), x);
+#ifdef CGKS_OPCOUNT_HOST
+        const int sc = 0;
+#else
+        const int sc = k == 0 ? sc0 : k == 3 ? sc3 : i_max(hi_abs(m0), (sc0 >> 1) + (sc3 >> 1));
+#endif
+        tang_weno5_pair(r, m0, x, weps4, sc, p[8 * stride], p[9 * stride]);
+        deriv_parts(r, p, stride, x, R(RN, k, -2), R(RN, k, -1), R(RN, k, 0), R(RN, k, 1), R(RN, k, 2));
+        tang_weno3_slopes(r, R(RL, k, -1), R(RL, k, 0), R(RL, k, 1), R(RR, k, -1), R(RR, k, 0), R(RR, k, 1), weps, sc,
+                          p[10 * stride], p[11 * stride]);
+    }
+}
+
+// The results of one Gauss point (stage 1: Fb, Ft, Wm, Wb; stage 2: Ft, Wtt in a, b).
+template <int STAGE> struct PointResult { double a[4], b[4], c[4], d[4]; };
+
+template <int STAGE>
+__device__ __forceinline__ bool segment_point(const SegmentPoint& src, PointResult<STAGE>& o)
+{
+    if constexpr (STAGE == 1) return gks_point<1>(src.r, src, o.a, o.b, o.c, o.d, o.d);
+    else return gks_point<2>(src.r, src, o.c, o.a, o.c, o.d, o.b);
+}
+
+// Variable k of a segment's results (face frame) from the sums of its two points' results:
+// the Gauss weight 1/2 times the stage's time factors; stage 1: the W* and R flux
+// combinations and the interface states W(dt/2), W(dt); stage 2: dt^2/3 F_t, dt^2/3 W_tt.
+// put(q, value): result group q.
+template <int STAGE, class Put>
+__device__ __forceinline__ void gauss_average(const RegK& r, double a, double b, double c, double d, Put put)
+{
+    if constexpr (STAGE == 1) {
+        put(0, r.kfma(FK_W1B, b, r.kmul(FK_W1A, a)));
+        put(1, r.kfma(FK_W2B, b, r.kmul(FK_W2A, a)));
+        put(2, r.kmul(FK_HALF, c));
+        put(3, r.kmul(FK_HALF, d));
+    } else {
+        put(0, r.kmul(FK_W3, a));
+        put(1, r.kmul(FK_W3, b));
+    }
+}
+
+// One face segment by one thread (the flux kernel gives each Gauss point a thread of its
+// own, the same operations): parts, both points, the average into acc (face frame).
+// Returns false if a state was non-physical.
+template <int STAGE>
+__device__ __forceinline__ bool segment_results(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
+                                                int rstride, double iht, double* part, int stride,
+                                                double acc[FaceQ<STAGE>::n])
+{
+    constexpr double gq = 0.28867513459481287;   // 1/(2 sqrt 3): Gauss points at +-gq
+    segment_parts(r, rec, pa, pb, pc, r0, rstride, 0, 4, part, stride);
+    PointResult<STAGE> s;
+    bool ok = true;
 #pragma unroll 1
     for (int gp = 0; gp < 2; ++gp) {
-        const double eta = gp ? gq : -gq;
-        const SegmentRows<SHARE> src{r, rec, pa, pb, pc, r0, rstride, eta, iht,
-                                     {gp ? W0p[0] : W0m[0], gp ? W0p[1] : W0m[1], gp ? W0p[2] : W0m[2],
-                                      gp ? W0p[3] : W0m[3]},
-                                     {sL[0], sL[1], sL[2], sL[3]}, {sR[0], sR[1], sR[2], sR[3]}, dc};
-        double Fb[4], Ft[4], Wm[4], Wb[4], Wtt[4];
-        bad |= !gks_point<STAGE>(r, src, Fb, Ft, Wm, Wb, Wtt);
-        if (PARK && gp == 1) {
+        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? gq : -gq, iht, gp, part, stride};
+        PointResult<STAGE> o;
+        ok &= segment_point<STAGE>(src, o);
 #pragma unroll
-            for (int q = 0; q < NF; ++q) acc[q] = park[q * park_stride];
-        }
-        // Gauss average (weight 1/2 per point) times the stage's time factors
-        if (STAGE == 1) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                acc[k] = r.kfma(FK_W1B, Ft[k], r.kfma(FK_W1A, Fb[k], acc[k]));
-                acc[4 + k] = r.kfma(FK_W2B, Ft[k], r.kfma(FK_W2A, Fb[k], acc[4 + k]));
-                acc[8 + k] = r.kfma(FK_HALF, Wm[k], acc[8 + k]);
-                acc[12 + k] = r.kfma(FK_HALF, Wb[k], acc[12 + k]);
+        for (int k = 0; k < 4; ++k) {
+            s.a[k] = gp ? r.add(s.a[k], o.a[k]) : o.a[k];
+            s.b[k] = gp ? r.add(s.b[k], o.b[k]) : o.b[k];
+            if (STAGE == 1) {
+                s.c[k] = gp ? r.add(s.c[k], o.c[k]) : o.c[k];
+                s.d[k] = gp ? r.add(s.d[k], o.d[k]) : o.d[k];
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                acc[k] = r.kfma(FK_W3, Ft[k], acc[k]);
-                acc[4 + k] = r.kfma(FK_W3, Wtt[k], acc[4 + k]);
-            }
-        }
-        if (PARK && gp == 0) {
-#pragma unroll
-            for (int q = 0; q < NF; ++q) park[q * park_stride] = acc[q];
         }
     }
-    return !bad;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        gauss_average<STAGE>(r, s.a[k], s.b[k], s.c[k], s.d[k], [&](int q, double v) { acc[4 * q + k] = v; });
+    return ok;
 }
 
 }  // namespace cgks

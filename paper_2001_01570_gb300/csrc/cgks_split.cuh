@@ -37,6 +37,7 @@ CGKS_SPLIT_FN float f_sub(float a, float b) { return __fsub_rn(a, b); }
 CGKS_SPLIT_FN float f_mul(float a, float b) { return __fmul_rn(a, b); }
 CGKS_SPLIT_FN float f_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 CGKS_SPLIT_FN float f_rcp(float a) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a)); return y; }
+CGKS_SPLIT_FN float f_rsqrt(float a) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a)); return y; }
 CGKS_SPLIT_FN float f_bits(uint32_t b) { return __uint_as_float(b); }
 CGKS_SPLIT_FN uint32_t f_word(float a) { return __float_as_uint(a); }
 CGKS_SPLIT_FN float f_int(int i) { return __int2float_rn(i); }
@@ -44,6 +45,7 @@ CGKS_SPLIT_FN int d_hi(double x) { return __double2hiint(x); }
 CGKS_SPLIT_FN int d_lo(double x) { return __double2loint(x); }
 CGKS_SPLIT_FN double d_make(int hi, int lo) { return __hiloint2double(hi, lo); }
 CGKS_SPLIT_FN int i_max(int a, int b) { return max(a, b); }
+CGKS_SPLIT_FN int i_min(int a, int b) { return min(a, b); }
 #else
 #define CGKS_SPLIT_FN inline
 inline float f_add(float a, float b) { return a + b; }
@@ -51,6 +53,7 @@ inline float f_sub(float a, float b) { return a - b; }
 inline float f_mul(float a, float b) { return a * b; }
 inline float f_fma(float a, float b, float c) { return ::fmaf(a, b, c); }
 inline float f_rcp(float a) { return 1.0f / a; }
+inline float f_rsqrt(float a) { return 1.0f / ::sqrtf(a); }
 inline float f_bits(uint32_t b) { float a; memcpy(&a, &b, 4); return a; }
 inline uint32_t f_word(float a) { uint32_t b; memcpy(&b, &a, 4); return b; }
 inline float f_int(int i) { return (float)i; }
@@ -66,6 +69,7 @@ inline CGKS_HOST_DOUBLE d_make(int hi, int lo)
     return x;
 }
 inline int i_max(int a, int b) { return a > b ? a : b; }
+inline int i_min(int a, int b) { return a < b ? a : b; }
 #endif
 
 struct ff { float h, l; };
@@ -89,6 +93,14 @@ CGKS_SPLIT_FN ff ff_from(double x)
     r.h = f_bits(hb | sgn);
     r.l = f_mul(f_int((int)(lo & 0x1fffffffu)), f_bits(sc | sgn));
     return r;
+}
+
+// the leading 24 bits of x as a float (truncated; zero below 2^-126)
+CGKS_SPLIT_FN float f_lead(double x)
+{
+    const uint32_t hi = (uint32_t)d_hi(x);
+    const uint32_t t = (uint32_t)i_max((int)(hi & 0x7fffffffu) - (896 << 20), 0);
+    return f_bits((hi & 0x80000000u) | (t << 3));
 }
 
 // a float as a double (zero and denormals give zero), integer operations
@@ -235,15 +247,56 @@ CGKS_SPLIT_FN void weno_side_split(const DiffData& x, ff eps, ff& dval, ff& dslo
 // differences' magnitudes (and s3's) against the variable's scale, compared as
 // the high words of FP64 numbers (for finite non-negative values their order is
 // the values'; NaN and infinity compare above everything).  scale_hi: high word
-// of the variable's scale; the ranges 2^-40..2^30 of the scale and 2^-46..2^30 of
-// eps keep every FP32 intermediate normal where it counts.
+// of the variable's scale; the ranges 2^-30..2^25 of the scale and of eps keep every
+// FP32 intermediate normal where it counts.
 constexpr int kHiOne = 1023 << 20;   // high word of 1.0; one binary order is 1 << 20
 CGKS_SPLIT_FN int hi_abs(double x) { return d_hi(x) & 0x7fffffff; }
+CGKS_SPLIT_FN bool split_scale_ok(int scale_hi, double eps)
+{
+    return scale_hi >= kHiOne - (30 << 20) && scale_hi < kHiOne + (25 << 20) && d_hi(eps) >= kHiOne - (30 << 20) &&
+           d_hi(eps) < kHiOne + (25 << 20);
+}
 CGKS_SPLIT_FN bool split_ok(int scale_hi, double eps, double w, double t, double u, double p, double q, double s3)
 {
     const int m3 = i_max(i_max(i_max(hi_abs(w), hi_abs(t)), hi_abs(u)), i_max(hi_abs(p), hi_abs(q)));
-    return scale_hi >= kHiOne - (40 << 20) && scale_hi < kHiOne + (30 << 20) && d_hi(eps) >= kHiOne - (46 << 20) &&
-           d_hi(eps) < kHiOne + (30 << 20) && m3 < scale_hi - (7 << 20) && hi_abs(s3) < scale_hi;
+    return split_scale_ok(scale_hi, eps) && m3 < scale_hi - (7 << 20) && hi_abs(s3) < scale_hi;
+}
+
+// ------------------------------------------------------------------------
+// The nonlinear values along a face (cgks_flux.cuh) as corrections; taken where the third
+// differences (the slope's correction) are below these powers of two of the scale.
+constexpr int kTangThird = -6, kTangSlope = -11;
+
+// Five means: D1 - sum_k w_k D_k = w_0 t0 + w_2 t1 at both Gauss points, from D1, the
+// centre's second difference s1, the third differences t0, t1 and 4 x epsilon; dlo,
+// dhi: the linear weights over the centre's.
+CGKS_SPLIT_FN void tang_weno5_split(ff D1, ff s1, ff t0, ff t1, ff eps4, ff dlo, ff dhi, ff& minus, ff& plus)
+{
+    const ff c133 = CGKS_FF(13.0 / 3.0);
+    auto e = [&](ff D, ff s) { return ff_addp(ff_addp(ff_sqr(D), ff_mul(c133, ff_sqr(s))), eps4); };
+    const ff e0 = e(ff_sub(D1, t0), ff_sub(s1, t0)), e1 = e(D1, s1), e2 = e(ff_sub(D1, t1), ff_add(s1, t1));
+    ff Z = ff_sub(e0, e2);
+    if (Z.h < 0.0f) Z = ff_neg(Z);
+    const ff one = ff{1.0f, 0.0f};
+    const ff a0 = ff_addp(one, ff_mul(Z, ff_rcp(e0))), a1 = ff_addp(one, ff_mul(Z, ff_rcp(e1))),
+             a2 = ff_addp(one, ff_mul(Z, ff_rcp(e2)));
+    const ff l0 = ff_mul(dlo, a0), h0 = ff_mul(dhi, a0), l2 = ff_mul(dlo, a2), h2 = ff_mul(dhi, a2);
+    const ff dp = ff_addp(ff_addp(l0, h2), a1), dm = ff_addp(ff_addp(h0, l2), a1);
+    plus = ff_mul(ff_add(ff_mul(l0, t0), ff_mul(h2, t1)), ff_rcp(dp));
+    minus = ff_mul(ff_add(ff_mul(h0, t0), ff_mul(l2, t1)), ff_rcp(dm));
+}
+
+// Three means, slopes dm, dp to the neighbours, A = dp + dm, s = dp - dm: the nonlinear
+// slope is (A - c) / 2 with c = Z sA s / (2 e0 e1 + Z (e0 + e1)), Z = |sA|: all of one
+// sign below, so c keeps the pairs' relative accuracy.
+CGKS_SPLIT_FN ff tang_weno3_split(ff A, ff s, ff eps)
+{
+    const ff dm = ff_scale(0.5f, ff_sub(A, s)), dp = ff_scale(0.5f, ff_add(A, s));
+    const ff e0 = ff_addp(ff_sqr(dm), eps), e1 = ff_addp(ff_sqr(dp), eps);
+    const ff sA = ff_mul(s, A);
+    const ff Z = sA.h < 0.0f ? ff_neg(sA) : sA;
+    const ff den = ff_addp(ff_scale(2.0f, ff_mul(e0, e1)), ff_mul(Z, ff_addp(e0, e1)));
+    return ff_mul(ff_mul(ff_mul(Z, sA), s), ff_rcp(den));
 }
 
 }  // namespace cgks

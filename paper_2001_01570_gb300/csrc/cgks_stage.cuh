@@ -8,17 +8,24 @@
 //   phase 1  stage the face-row records the tile needs (its faces on its rows
 //            and two rows either side) with asynchronous copies
 //   phase 2  per face segment the tile owns (the x- and y-faces on the low side
-//            of its cells, plus the grid's last face where the tile ends on the
-//            grid's edge, so every face is evaluated once), at two Gauss points:
-//            WENO-Z point values along the face over rows j-2..j+2
-//            (equilibrium) and j-1..j+1 (non-equilibrium states, with their
-//            tangential slopes); tangential derivatives of the equilibrium state
-//            and normal derivatives from the quartic / quadratic through the same
-//            line averages (their Gauss-point-independent parts once per
-//            segment); the gas-kinetic evaluation at each point; the Gauss
-//            average, weighted by the stage's time factors, written to the face
-//            results (stage 1: the W* and R flux combinations and the interface
-//            states W(dt/2), W(dt); stage 2: dt^2/3 F_t and dt^2/3 W_tt)
+//            of its cells; the grid's last faces have tiles of their own, so every
+//            face is evaluated once) a pair of lanes.  Together they compute what
+//            its two Gauss points share, two variables each, into the pair's slice
+//            of shared memory: WENO-Z point values along the face over rows
+//            j-2..j+2 (equilibrium) and j-1..j+1 (non-equilibrium states, with
+//            their tangential slopes) and the parts of the quartic through the same
+//            line averages.  Then each lane evaluates one point; their results are
+//            exchanged by shuffles, averaged, weighted by the stage's time factors
+//            and written to the face results, two variables per lane (stage 1: the
+//            W* and R flux combinations and the interface states W(dt/2), W(dt);
+//            stage 2: dt^2/3 F_t and dt^2/3 W_tt)
+// What bounds it: the FP64 unit (68 cycles per warp instruction) with FP32 issue beside
+// it; about 1,000 FP64 instructions and 18,000 others per warp and 32 segments.  One
+// thread per segment ran both points in turn with the first one's sums and the shared
+// parts in registers (255 of them, 1.8 KB of spills once the FP32 pairs came in); one
+// thread per point needs 168 and halves the chain of dependent instructions that a small
+// grid waits for.  Measured per launch, stage 1 / 2: 2048^2 27.66 / 25.41 -> 17.8 / 14.4
+// ms, 512^2 1.93 / 1.77 -> 1.14 / 0.94 ms, 64^2 155 / 138 -> 43 / 38 us.
 // Coefficients (fixed, and the tile's grid and dt) come from the shared-memory
 // table of cgks_flux.cuh; all arithmetic is in the register-only DFMA forms.
 // The kernel is persistent: CTAs stride over a flattened tile queue that may
@@ -34,7 +41,7 @@ namespace cgks {
 static __constant__ FluxFixed kFluxFixed = make_flux_fixed();
 
 template <int TX, int TY, int STAGE>
-__global__ void __launch_bounds__(kThreads, kStageCtasPerSm)
+__global__ void __launch_bounds__(kThreads, stage_ctas(TX, TY))
 stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tiles, int ntiles,
              const int* __restrict__ dcount)
 {
@@ -43,7 +50,7 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
     extern __shared__ double smem[];
     double* rx = smem;                  // x-face records, RecGroups<TY, TX+1>
     double* ry = rx + L::n_rx;          // y-face records, RecGroups<TX, TY+1>
-    double* dc = ry + L::n_ry + threadIdx.x;   // [32][kThreads] when L::share
+    double* part = ry + L::n_ry + (threadIdx.x >> 1);   // [kParts][kPairs]: this pair's slice
     __shared__ double s_fk[FK_N];       // coefficient table (fixed part, then the tile's grid and dt)
     __shared__ int s_skip;
     // the queue length (a kernel argument, or in device memory for a server's patched queue) is
@@ -119,22 +126,16 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
 
         // ---------------- phase 2: face segments, two Gauss points each
         bool bad = false;
-        // the tile's own faces: x-faces x0..x0+TX-1 and y-faces y0..y0+TY-1 of its
-        // cells, plus the last face of the grid where the tile ends on the grid's
-        // edge; every face is evaluated by exactly one tile
-        const int xe = (x0 + TX == nx) ? TY : 0, ye = (!dim1 && y0 + TY == ny) ? TX : 0;
-        const int nseg = (dim1 ? TX * TY : 2 * TX * TY) + xe + ye;
+        // the tile's own faces: x-faces x0..x0+TX-1 and y-faces y0..y0+TY-1 (a tile with
+        // x0 = nx or y0 = ny has the grid's last faces alone); every face is evaluated by
+        // exactly one tile
+        const int nseg = dim1 ? TX * TY : 2 * TX * TY;
         const size_t nfx = (size_t)ny * (nx + 1), nfy = (size_t)(ny + 1) * nx;
-        for (int item = tid; item < nseg; item += kThreads) {
-            int fl, jl, il, gl;
-            bool xo;
-            if (item < TX * TY) { xo = true; fl = item % TX; jl = item / TX; }
-            else if (!dim1 && item < 2 * TX * TY) { xo = false; const int it = item - TX * TY; il = it % TX; gl = it / TX; }
-            else {
-                const int it = item - (dim1 ? TX * TY : 2 * TX * TY);
-                if (it < xe) { xo = true; fl = TX; jl = it; }
-                else { xo = false; il = it - xe; gl = TY; }
-            }
+        const int gp = tid & 1;
+        const unsigned pair = 3u << (tid & 30);         // the two lanes of this pair
+        for (int item = tid >> 1; item < nseg; item += kPairs) {
+            const bool xo = item < TX * TY;
+            const int it = xo ? item : item - TX * TY, fl = it % TX, jl = it / TX;   // cell of the tile
             const double* rec;
             int pa, pb, pc, r0, rstride;
             double* out;
@@ -145,10 +146,10 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
                 r0 = jl * (TX + 1) + fl; rstride = TX + 1;
                 out = G.facex; ostride = nfx; oidx = (size_t)(y0 + jl) * (nx + 1) + x0 + fl;
             } else {
-                if (!((y0 + gl <= ny) && (x0 + il < nx))) continue;
+                if (!((y0 + jl <= ny) && (x0 + fl < nx))) continue;
                 rec = ry; pa = RecGroups<TX, TY + 1>::pa; pb = RecGroups<TX, TY + 1>::pb; pc = RecGroups<TX, TY + 1>::pc;
-                r0 = il * (TY + 1) + gl; rstride = TY + 1;
-                out = G.facey; ostride = nfy; oidx = (size_t)(y0 + gl) * nx + x0 + il;
+                r0 = fl * (TY + 1) + jl; rstride = TY + 1;
+                out = G.facey; ostride = nfy; oidx = (size_t)(y0 + jl) * nx + x0 + fl;
             }
             // the segment's record window (rows -2..2 of group A, -1..1 of group B, 0 of group C)
             // and its output index
@@ -156,21 +157,29 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
                                     oidx < ostride,
                                 G.ctrl))
                 continue;
-            const double iht = r.k(xo ? FK_IDY : FK_IDX);
-            double acc[NF];
-            // stage 2 parks the first Gauss point's sums in the output slots: its register
-            // allocation then spills nothing (measured: 26.3 -> 25.5 ms on 2048^2); stage 1
-            // runs faster with them in registers
-            bad |= !segment_results<STAGE, L::share, STAGE == 2>(r, rec, pa, pb, pc, r0, rstride, iht, dc, acc,
-                                                                  out + oidx, ostride);
-            // back to the physical frame (y-faces: swap momentum components)
+            __syncwarp(pair);   // the slice's reads of the segment before
+            // the pair's lanes compute two variables' parts each, then a Gauss point each
+            segment_parts(r, rec, pa, pb, pc, r0, rstride, 2 * gp, 2 * gp + 2, part, kPairs);
+            __syncwarp(pair);
+            constexpr double gq = 0.28867513459481287;
+            const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? gq : -gq, r.k(xo ? FK_IDY : FK_IDX), gp, part,
+                                   kPairs};
+            PointResult<STAGE> o;
+            bad |= !segment_point<STAGE>(src, o);
+            // each lane averages and writes two variables: the other lane's sums for them come by
+            // shuffle
+            auto sum = [&](const double v[4], int m) {
+                const double mine = gp ? v[2 + m] : v[m], theirs = gp ? v[m] : v[2 + m];
+                return r.add(mine, __shfl_xor_sync(pair, theirs, 1));
+            };
 #pragma unroll
-            for (int q = 0; q < NF; q += 4) {
-                const int k1 = xo ? 1 : 2, k2 = xo ? 2 : 1;
-                out[(q + 0) * ostride + oidx] = acc[q + 0];
-                out[(q + k1) * ostride + oidx] = acc[q + 1];
-                out[(q + k2) * ostride + oidx] = acc[q + 2];
-                out[(q + 3) * ostride + oidx] = acc[q + 3];
+            for (int m = 0; m < 2; ++m) {
+                const double a = sum(o.a, m), b = sum(o.b, m);
+                double c = 0.0, d = 0.0;
+                if (STAGE == 1) { c = sum(o.c, m); d = sum(o.d, m); }
+                // back to the physical frame (y-faces: swap momentum components)
+                const int k = 2 * gp + m, kp = (k == 1 || k == 2) && !xo ? 3 - k : k;
+                gauss_average<STAGE>(r, a, b, c, d, [&](int q, double v) { out[(4 * q + kp) * ostride + oidx] = v; });
             }
         }
         if (bad) atomicOr(&G.ctrl->status, (int)CGKS_E_NONPHYSICAL);
@@ -216,15 +225,16 @@ cudaError_t launch_stage_t(const GridDev* grids, const TileRef* tiles, int ntile
 
 // The launcher and shared-memory size of one tile shape (one translation unit
 // per shape, so the shapes compile in parallel).
-#define CGKS_STAGE_INSTANCE(TX, TY)                                                                         \
+#define CGKS_STAGE_INSTANCE(W, H) CGKS_STAGE_INSTANCE_(W, H, work_w(W, H), work_h(W, H))
+#define CGKS_STAGE_INSTANCE_(W, H, TX, TY)                                                                  \
     static_assert(StageLayout<TX, TY, 1>::bytes + 64 <= 227 * 1024, "stage-1 tile exceeds shared memory");  \
-    cudaError_t launch_stage_##TX##x##TY(int stage, const GridDev* grids, const TileRef* tiles, int ntiles,  \
+    cudaError_t launch_stage_##W##x##H(int stage, const GridDev* grids, const TileRef* tiles, int ntiles,  \
                                          int nblocks, cudaStream_t st, const int* dcount)                   \
     {                                                                                                       \
         return stage == 1 ? launch_stage_t<TX, TY, 1>(grids, tiles, ntiles, nblocks, st, dcount)            \
                           : launch_stage_t<TX, TY, 2>(grids, tiles, ntiles, nblocks, st, dcount);           \
     }                                                                                                       \
-    size_t smem_##TX##x##TY(int stage)                                                                      \
+    size_t smem_##W##x##H(int stage)                                                                      \
     {                                                                                                       \
         return stage == 1 ? StageLayout<TX, TY, 1>::bytes : StageLayout<TX, TY, 2>::bytes;                  \
     }

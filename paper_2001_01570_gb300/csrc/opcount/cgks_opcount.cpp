@@ -180,7 +180,7 @@ bool tile_segments(const RegK& r, const GridDev& G, int x0, int y0, const std::v
         }
         const Real iht = r.k(xo ? FK_IDY : FK_IDX);
         Real acc[NF];
-        ok &= segment_results<STAGE, true>(r, rec, pa, pb, pc, r0, rstride, iht, dc.data(), acc);
+        ok &= segment_results<STAGE>(r, rec, pa, pb, pc, r0, rstride, iht, dc.data(), 1, acc);
         for (int q = 0; q < NF; q += 4) {
             const int k1 = xo ? 1 : 2, k2 = xo ? 2 : 1;
             out[(q + 0) * ostride + oidx] = acc[q + 0];
@@ -279,7 +279,7 @@ struct HostStep {
     {
         GridDev& G = g.G;
         const int nx = G.nx, ny = G.ny;
-        std::vector<Real> rx, ry, dc(32 * kThreads, Real(0.0));
+        std::vector<Real> rx, ry, dc(kParts, Real(0.0));
         const int nrec = record_rows(nx, ny, 2);
         bool ok = true;
         unsigned long long scratch[3 * cgks_oc::K_N];

@@ -10,6 +10,7 @@
 #include <random>
 
 #define CGKS_OPCOUNT_HOST 1   // the plain FP64 forms of the device headers
+#define CGKS_SPLIT_CHECK 1    // and the pairs' arithmetic beside them
 inline double cgks_opcount_rcp(double x) { return 1.0 / x; }
 inline double cgks_opcount_exp(double x) { return std::exp(x); }
 inline double cgks_opcount_erfc(double x) { return std::erfc(x); }
@@ -25,10 +26,11 @@ inline double __longlong_as_double(long long b) { double x; memcpy(&x, &b, 8); r
 template <class T> inline T __ldg(const T* p) { return *p; }
 inline int min(int a, int b) { return a < b ? a : b; }
 inline int max(int a, int b) { return a > b ? a : b; }
+#include "cgks_split.cuh"
 #include "cgks_device.cuh"
 #include "cgks_internal.h"
 #include "cgks_records.cuh"
-#include "cgks_split.cuh"
+#include "cgks_flux.cuh"
 
 using namespace cgks;
 typedef long double Q;
@@ -151,9 +153,159 @@ static void check_pairs()
     printf("pairs 0 0 0 %.4e %.4e %.4e %.4e\n", worst, exact, back, std::fabs(val(ff_from(0.0))) + std::fabs(d_from(0.0f)));
 }
 
+// arithmetic of slope_moments and euler_second in long double
+struct ArLD {
+    using T = Q;
+    Q g1, k1, k3;
+    Q add(Q a, Q b) const { return a + b; }
+    Q sub(Q a, Q b) const { return a - b; }
+    Q mul(Q a, Q b) const { return a * b; }
+    Q mad(Q a, Q b, Q c) const { return a * b + c; }
+    Q nmad(Q a, Q b, Q c) const { return c - a * b; }
+    Q half(Q a) const { return a / 2; }
+    Q dbl(Q a) const { return a + a; }
+    Q tri(Q a) const { return 3 * a; }
+    Q gm1() const { return g1; }
+    Q K1() const { return k1; }
+    Q K3() const { return k3; }
+};
+
+struct FluxTable {
+    double t[FK_N];
+    RegK r;
+    FluxTable()
+    {
+        const FluxFixed f = make_flux_fixed();
+        for (int i = 0; i < FK_N; ++i) t[i] = 0.0;
+        for (int i = 0; i < FK_NFIX; ++i) t[i] = f.v[i];
+        t[FK_GM1] = 0.4; t[FK_GAMMA] = 1.4; t[FK_K1] = 4.0; t[FK_K3] = 6.0;
+        r = RegK{t, 1.0, -0.0};
+    }
+};
+
+// the two point values and the slope along a face, from five (three) means of a smooth function
+static void check_tangential(int lev)
+{
+    const FluxTable F;
+    const RegK& r = F.r;
+    std::mt19937_64 g(5 + lev);
+    std::uniform_real_distribution<double> u(0.0, 1.0);
+    const double eps = 1e-6, hg = 0.5 * 0.28867513459481287;
+    Stat s5, s3;
+    const long rows = 20000;
+    for (long it = 0; it < rows; ++it) {
+        const double base = 0.5 + u(g), amp = std::ldexp(1.0, -lev), k1 = 0.2 + u(g), k2 = 0.2 + 2.0 * u(g), p1 = 6.28 * u(g), p2 = 6.28 * u(g);
+        double v[5];
+        for (int c = 0; c < 5; ++c) v[c] = base + amp * (std::sin(k1 * c + p1) + 0.5 * std::sin(k2 * c + p2));
+        TangDiffs x;
+        tang_diffs(r, v[0], v[1], v[2], v[3], v[4], x);
+        const int sc = hi_abs(v[2]);
+        if (i_max(hi_abs(x.t0), hi_abs(x.t1)) < sc + kTangThird * (1 << 20)) {
+            double om, op;
+            tang_weno5_pair(r, v[2], x, 4.0 * eps, 0, om, op);
+            ff m, p;
+            tang_weno5_split(ff_from(x.A1), ff_from(x.s1), ff_from(x.t0), ff_from(x.t1), ff_from(4.0 * eps), CGKS_FF(kTangLo), CGKS_FF(kTangHi), m, p);
+            const double nm = fma(-hg, x.A1 - val(m), v[2]), np = fma(hg, x.A1 - val(p), v[2]);
+            const Q V[5] = {v[0], v[1], v[2], v[3], v[4]}, D[3] = {3 * V[2] - 4 * V[1] + V[0], V[3] - V[1], 4 * V[3] - V[4] - 3 * V[2]};
+            Q e[3];
+            for (int k = 0; k < 3; ++k) { const Q s2 = V[k] - 2 * V[k + 1] + V[k + 2]; e[k] = D[k] * D[k] + 13 * s2 * s2 / 3 + 4 * (Q)eps; }
+            const Q Z = std::fabs(e[0] - e[2]);
+            Q ref[2];
+            for (int side = 0; side < 2; ++side) {
+                const Q w[3] = {side ? (Q)kTangLo : (Q)kTangHi, 1, side ? (Q)kTangHi : (Q)kTangLo};
+                Q n = 0, d = 0;
+                for (int k = 0; k < 3; ++k) { const Q a = w[k] * (1 + Z / e[k]); n += a * D[k]; d += a; }
+                ref[side] = V[2] + (side ? (Q)hg : -(Q)hg) * n / d;
+            }
+            s5.add(std::max(err(nm, ref[0]), err(np, ref[1])), std::max(err(om, ref[0]), err(op, ref[1])));
+        }
+        {
+            const double dm = v[2] - v[1], dp = v[3] - v[2], A = dp + dm, s = dp - dm;
+            const ff c = tang_weno3_split(ff_from(A), ff_from(s), ff_from(eps));
+            if (hi_abs(d_from(c.h)) < sc + kTangSlope * (1 << 20)) {
+                double n, d;
+                tang_weno3_parts(r, v[1], v[2], v[3], eps, n, d);
+                const Q a = (Q)v[2] - v[1], b = (Q)v[3] - v[2], e0 = a * a + (Q)eps, e1 = b * b + (Q)eps, z = std::fabs(e0 - e1);
+                const Q w0 = 1 + z / e0, w1 = 1 + z / e1, ref = (w0 * a + w1 * b) / (w0 + w1);
+                s3.add(err(0.5 * (A - val(c)), ref), err(n / d, ref));
+            }
+        }
+    }
+    s5.print("tang_value", lev, rows);
+    s3.print("tang_slope", lev, rows);
+}
+
+// slope moments and W_tt against long double, relative to the size of their terms
+static void check_moments()
+{
+    const FluxTable F;
+    std::mt19937_64 g(17);
+    std::uniform_real_distribution<double> u(-1.0, 1.0);
+    const ArLD ql{(Q)0.4, 4, 6};
+    const ArSplit qs{ff_from(0.4), ff_from(4.0), ff_from(6.0)};
+    const Ar64 q64{F.r};
+    Stat st, se;
+    const long rows = 20000;
+    for (long it = 0; it < rows; ++it) {
+        const double U = 1.5 * u(g), V = 1.5 * u(g), th = 0.3 + std::fabs(u(g)), sq = std::sqrt(0.5 / th);
+        const int side = it & 1;
+        double m[4], bn[4], bt[4];
+        m[0] = 0.5 * std::erfc((side ? 1 : -1) * U * sq);
+        const double gd = (side ? -1 : 1) * std::exp(-U * U * sq * sq) * sq / std::sqrt(M_PI);
+        m[1] = U * m[0] + th * gd; m[2] = U * m[1] + th * m[0]; m[3] = U * m[2] + 2 * th * m[1];
+        for (int k = 0; k < 4; ++k) { bn[k] = u(g); bt[k] = u(g); }
+        Q Lm[4], Ln[4], Lt[4], T[4], W[4];
+        double T64[4], W64[4];
+        ff Sm[4], Sn[4], St[4], Ts[4], Ws[4];
+        for (int k = 0; k < 4; ++k) {
+            Lm[k] = m[k]; Ln[k] = bn[k]; Lt[k] = bt[k];
+            Sm[k] = ff_from(m[k]); Sn[k] = ff_from(bn[k]); St[k] = ff_from(bt[k]);
+        }
+        const double ith = 1.0 / th;
+        slope_moments(ql, true, (Q)U, (Q)V, (Q)th, (Q)ith, Lm, (Q)gd, Ln, Lt, T, W);
+        slope_moments(q64, true, U, V, th, ith, m, gd, bn, bt, T64, W64);
+        slope_moments(qs, true, ff_from(U), ff_from(V), ff_from(th), ff_from(ith), Sm, ff_from(gd), Sn, St, Ts, Ws);
+        double size = 0.0, a = 0.0, b = 0.0;
+        for (int k = 0; k < 4; ++k) size += std::fabs(bn[k]) + std::fabs(bt[k]);
+        size *= std::pow(1.0 + U * U + V * V + th, 2);
+        for (int k = 0; k < 4; ++k) {
+            a = std::max(a, std::max(err(val(Ts[k]), T[k]), err(val(Ws[k]), W[k])));
+            b = std::max(b, std::max(err(T64[k], T[k]), err(W64[k], W[k])));
+        }
+        st.add(a / size, b / size);
+
+        EulerFirst<double> f;
+        double* fd = (double*)&f;
+        for (size_t i = 0; i < sizeof f / sizeof(double); ++i) fd[i] = u(g);
+        f.rho = 0.5 + std::fabs(u(g)); f.U = U; f.V = V; f.ir = 1.0 / f.rho; f.gir = 0.4 * f.ir; f.hq2 = 0.5 * (U * U + V * V); f.e = f.rho * th / 0.4;
+        EulerFirst<Q> fl;
+        EulerFirst<ff> fs;
+        for (size_t i = 0; i < sizeof f / sizeof(double); ++i) { ((Q*)&fl)[i] = fd[i]; ((ff*)&fs)[i] = ff_from(fd[i]); }
+        double w2[3][4], o64[4], sec = 0.0;
+        Q l2[3][4], ol[4];
+        ff s2[3][4], os[4];
+        for (int d = 0; d < 3; ++d)
+            for (int k = 0; k < 4; ++k) { w2[d][k] = u(g); l2[d][k] = w2[d][k]; s2[d][k] = ff_from(w2[d][k]); sec += std::fabs(w2[d][k]); }
+        euler_second(ql, fl, (Q)1.4, l2[0], l2[1], l2[2], ol);
+        euler_second(q64, f, 1.4, w2[0], w2[1], w2[2], o64);
+        euler_second(qs, fs, ff_from(1.4), s2[0], s2[1], s2[2], os);
+        const double sp = 1.0 + std::fabs(U) + std::fabs(V) + 2.0 * std::sqrt(th);
+        double first = 0.0;
+        for (size_t i = 0; i < sizeof f / sizeof(double); ++i) first += std::fabs(fd[i]);
+        const double sz = sp * sp * sp * sp * (sec + first * first) * (1.0 + f.rho) * (1.0 + f.ir);
+        a = b = 0.0;
+        for (int k = 0; k < 4; ++k) { a = std::max(a, err(val(os[k]), ol[k])); b = std::max(b, err(o64[k], ol[k])); }
+        se.add(a / sz, b / sz);
+    }
+    st.print("slope_moments", 0, rows);
+    se.print("euler_second", 0, rows);
+}
+
 int main()
 {
     check_pairs();
+    for (int lev : {2, 4, 6, 9, 14}) check_tangential(lev);
+    check_moments();
     for (double base : {1.0, 0.0})
         for (int lev : {1, 3, 5, 8, 12, 20}) { check_rows<8>(lev, base, 1.0); check_rows<6>(lev, base, 1.0); }
     return 0;

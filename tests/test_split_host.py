@@ -40,3 +40,24 @@ def test_split_rows_are_as_exact_as_fp64(lines, what, base):
         assert taken > 0
         assert mx <= 2.0 ** -51, (what, lev, mx)
         assert mx <= mx64 + 2.0 ** -54 and rms <= rms64 + 2.0 ** -54, (what, lev, mx, mx64, rms, rms64)
+
+
+@pytest.mark.parametrize("what", ["tang_value", "tang_slope"])
+def test_split_values_along_a_face_are_as_exact_as_fp64(lines, what):
+    """The same bounds: third differences of at most 2^-6 of the scale times the Gauss points' 0.14,
+    slope corrections of at most 2^-11."""
+    rows = [ln for ln in lines if ln[0] == what]
+    assert len(rows) == 5 and rows[-1][2] == rows[-1][3]
+    for _, lev, taken, total, mx, mx64, rms, rms64 in rows:
+        assert taken > 0 and mx <= 2.0 ** -51, (what, lev, mx)
+        assert mx <= mx64 + 2.0 ** -54 and rms <= rms64 + 2.0 ** -54, (what, lev, mx, mx64, rms, rms64)
+
+
+@pytest.mark.parametrize("what", ["slope_moments", "euler_second"])
+def test_split_moments_and_time_derivatives_hold_41_bits_of_their_terms(lines, what):
+    """Up to 140 pair operations of 2^-47 each on terms no larger than the size they are measured
+    against: 2^-40 at the very worst; random signs leave far less.  The kernel takes them only where
+    their weight is below 2^-7 of the quantity they are added to."""
+    (_, _, n, total, mx, mx64, rms, _), = [ln for ln in lines if ln[0] == what]
+    assert n == total and mx <= 2.0 ** -41 and rms <= 2.0 ** -46
+    assert mx64 <= 2.0 ** -49
