@@ -211,7 +211,7 @@ cgks_status cgks_create(const cgks_problem* prob, void* cuda_stream, cgks_solver
     std::vector<TileRef> tiles = make_tiles(s->nx, s->ny, prob->dim, s->shape, 0);
     s->ntiles = (int)tiles.size();
     if (e == cudaSuccess) e = cudaMalloc(&s->d_tiles, tiles.size() * sizeof(TileRef));
-    std::vector<TileRef> rchunks = record_chunks(s->nx, s->ny, prob->dim, prob->recon_vars, 0);
+    std::vector<TileRef> rchunks = record_chunks(s->nx, s->ny, prob->dim, 0);
     s->nrchunks = (int)rchunks.size();
     if (e == cudaSuccess) e = cudaMalloc(&s->d_rchunks, rchunks.size() * sizeof(TileRef));
     std::vector<TileRef> cchunks = cell_chunks(s->nx, s->ny, 0);
@@ -345,7 +345,7 @@ static cgks_status enqueue_steps(cgks_solver* s, int nsteps, long* launches, boo
 {
     const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
-    const int rblocks = record_blocks(s->nrchunks, s->nsm, cv);
+    const int rblocks = record_blocks(s->nrchunks, s->nsm);
     const int ublocks = update_blocks(s->ncchunks, s->nsm, 4);
     const int fblocks = s->nftiles < s->nsm ? s->nftiles : s->nsm;
     for (int k = 0; k < nsteps; ++k) {
@@ -440,7 +440,7 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
     for (auto& e : ev) CK(cudaEventCreate(&e));
     const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
-    const int rblocks = record_blocks(s->nrchunks, s->nsm, cv);
+    const int rblocks = record_blocks(s->nrchunks, s->nsm);
     const int ublocks = update_blocks(s->ncchunks, s->nsm, 4);
     for (int k = 0; k < nsteps; ++k) {
         cudaEvent_t* e = &ev[(size_t)k * (NK + 1)];

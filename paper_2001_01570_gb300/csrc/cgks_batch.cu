@@ -142,7 +142,7 @@ cudaError_t BatchEngine::set_members(const std::vector<std::pair<int, GridDev>>&
             const std::vector<TileRef> t = make_tiles(G.nx, G.ny, G.dim, s, slot);
             q[s].insert(q[s].end(), t.begin(), t.end());
         }
-        std::vector<TileRef> r = record_chunks(G.nx, G.ny, G.dim, G.recon_vars, slot);
+        std::vector<TileRef> r = record_chunks(G.nx, G.ny, G.dim, slot);
         q[TILE_COUNT + G.recon_vars].insert(q[TILE_COUNT + G.recon_vars].end(), r.begin(), r.end());
         std::vector<TileRef> c = cell_chunks(G.nx, G.ny, slot);
         q[TILE_COUNT + 2].insert(q[TILE_COUNT + 2].end(), c.begin(), c.end());
@@ -206,7 +206,7 @@ cudaError_t BatchEngine::capture(int cand)
         for (int stage = 1; stage <= 2; ++stage) {
             for (int v = 0; v < 2 && e1 == cudaSuccess; ++v)
                 e1 = launch_records(stage, v, d_grids_, d_q_[TILE_COUNT + v], (int)cap_[TILE_COUNT + v],
-                                    record_blocks(1 << 30, nsm_, v), cap, cnt + TILE_COUNT + v);
+                                    record_blocks(1 << 30, nsm_), cap, cnt + TILE_COUNT + v);
             if (e1 == cudaSuccess)
                 e1 = launch_stage(c.shape, stage, d_grids_, d_q_[c.shape], (int)cap_[c.shape],
                                   stage_blocks(1 << 30, nsm_, c.shape), cap, cnt + c.shape);

@@ -95,6 +95,11 @@ __host__ __device__ inline int record_rows(int nx, int ny, int dim)
 {
     return (nx + 1) * (ny + 4) + (dim == 2 ? (ny + 1) * (nx + 4) : 0);
 }
+// rows a record kernel works on: in 1D the grid's only row (j = 0) is all its flux kernel reads
+__host__ __device__ inline int record_work_rows(int nx, int ny, int dim)
+{
+    return dim == 2 ? record_rows(nx, ny, dim) : nx + 1;
+}
 inline size_t record_doubles(int nx, int ny, int dim) { return (size_t)28 * record_rows(nx, ny, dim); }
 // per face up to 16 results (stage 1: two flux combinations, two interface states)
 inline size_t face_doubles(int nx, int ny, int dim)
@@ -135,8 +140,9 @@ std::vector<TileRef> make_tiles(int nx, int ny, int dim, int shape, int grid, bo
 // small grid's items spread over the SMs one warp per unit
 constexpr int kRecordChunk = 128;
 // the record kernel's work queue: chunks of kRecordChunk (record, variable) items of one
-// grid (one record per item in characteristic mode); TileRef.x0 is the first item
-std::vector<TileRef> record_chunks(int nx, int ny, int dim, int recon_vars, int grid);
+// grid (one row of four lanes per four items in characteristic mode); TileRef.x0 is the
+// first item
+std::vector<TileRef> record_chunks(int nx, int ny, int dim, int grid);
 // the update kernel's work queue: chunks of 256 cells of one grid (TileRef.x0
 // is the first cell)
 std::vector<TileRef> cell_chunks(int nx, int ny, int grid);
@@ -161,11 +167,10 @@ inline int stage_blocks(int ntiles, int nsm, int shape)
     return ntiles < cap ? ntiles : cap;
 }
 
-// persistent grid of the record kernel: its resident CTAs (four per SM with
-// conservative variables, two with characteristic ones), at most one per chunk
-inline int record_blocks(int nchunks, int nsm, int char_vars)
+// persistent grid of the record kernel: its resident CTAs (four per SM), at most one per chunk
+inline int record_blocks(int nchunks, int nsm)
 {
-    const int cap = (char_vars ? 2 : 4) * nsm;
+    const int cap = 4 * nsm;
     return nchunks < cap ? nchunks : cap;
 }
 

@@ -187,7 +187,7 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     }
     const int nt = (int)ntiles;
     const int cv = prob->recon_vars;
-    const long long items = (long long)(cv ? 1 : 4) * record_rows(prob->nx, prob->ny, 2);
+    const long long items = 4LL * record_rows(prob->nx, prob->ny, 2);
     const int nrc = (int)((items + kRecordChunk - 1) / kRecordChunk);
     const int ncc = (int)((cells + 255) / 256);
     const int work = nt > nrc ? nt : nrc;
@@ -197,7 +197,7 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     NCK(launch_set_ctrl(sym->ctrl, *t_inout, 0.0, -1, 1, stream));
     NCK(launch_cfl(sym->desc, 0, G, stream));
     const int nblocks = stage_blocks(nt, nsm, shape);
-    const int rblocks = record_blocks(nrc, nsm, cv);
+    const int rblocks = record_blocks(nrc, nsm);
     const int ublocks = update_blocks(ncc, nsm);
     for (int k = 0; k < nsteps; ++k) {
         NCK(launch_begin_step(sym->desc, 1, stream));

@@ -18,7 +18,7 @@ namespace cgks {
 __constant__ ReconTab kReconTab = make_recon_tab();
 
 // CHAR = 0: conservative variables, one (record, variable) per thread;
-// CHAR = 1: characteristic variables, one record (all four variables) per thread.
+// CHAR = 1: characteristic variables, one (record, field) per lane of a quad.
 // The reconstruction order is per grid (a uniform branch per chunk).
 // Bound by the FP64 unit and FP32 issue together: about 55 FP64 instructions of 68
 // cycles per warp (differences, linear reconstruction, the sums that bring the
@@ -26,10 +26,13 @@ __constant__ ReconTab kReconTab = make_recon_tab();
 // pair (cgks_split.cuh); rows that fail split_ok take 240 more FP64 instructions.
 // Measured per stage on the 2048^2 vortex: 15.73 ms with the pair in FP64, 4.08 ms;
 // 512^2: 1.010 -> 0.333 ms; 97x61 (three warps per FP64 unit): 44.5 -> 17.5 us.
+// Characteristic mode with a thread per row ran 600 FP64 instructions and four WENO-Z pairs
+// in one chain (401 cells in 1D: 78 us; a lane per field, and only the grid's own row of the
+// five a 1D stencil would take: 41 us; 200x50: 99 -> 89 us, most of it rows at shocks).
 // CTAs of 128 threads, four per SM: one of 256 left a small grid's items on half
 // of the SMs (100 cells in 1D: 24.7 us; spread over twice the CTAs: 20.9).
 template <int STAGE, int CHAR>
-__global__ void __launch_bounds__(kRecordChunk, CHAR ? 2 : 4) records_kernel(const GridDev* __restrict__ grids,
+__global__ void __launch_bounds__(kRecordChunk, 4) records_kernel(const GridDev* __restrict__ grids,
                                                                     const TileRef* __restrict__ chunks, int nchunks,
                                                                     const int* __restrict__ dcount)
 {
@@ -45,24 +48,24 @@ __global__ void __launch_bounds__(kRecordChunk, CHAR ? 2 : 4) records_kernel(con
         if (G.ctrl->done) continue;
         const double* __restrict__ src = (STAGE == 1) ? G.buf[G.ctrl->par] : G.ws;
         const size_t PL = (size_t)G.nx * G.ny;
-        const int nrec = record_rows(G.nx, G.ny, G.dim);
+        const int nrec = record_work_rows(G.nx, G.ny, G.dim);
         const int item = tr.x0 + (int)threadIdx.x;
+        if (item >= 4 * nrec) continue;
         if (!CHAR) {
-            if (item >= 4 * nrec) continue;
             const int k = item / nrec;
             if (G.order == 6) cons_row<6>(RegK{s_tab + RK_N, one, nzero}, G, src, PL, item - k * nrec, k);
             else cons_row<8>(RegK{s_tab, one, nzero}, G, src, PL, item - k * nrec, k);
         } else {
-            if (item >= nrec) continue;
-            if (G.order == 6) char_row<6>(RegK{s_tab + RK_N, one, nzero}, G, src, PL, item);
-            else char_row<8>(RegK{s_tab, one, nzero}, G, src, PL, item);
+            const unsigned quad = 0xfu << (threadIdx.x & 28);
+            if (G.order == 6) char_row_quad<6>(RegK{s_tab + RK_N, one, nzero}, G, src, PL, item >> 2, item & 3, quad);
+            else char_row_quad<8>(RegK{s_tab, one, nzero}, G, src, PL, item >> 2, item & 3, quad);
         }
     }
 }
 
-std::vector<TileRef> record_chunks(int nx, int ny, int dim, int recon_vars, int grid)
+std::vector<TileRef> record_chunks(int nx, int ny, int dim, int grid)
 {
-    const long long items = (long long)(recon_vars ? 1 : 4) * record_rows(nx, ny, dim);
+    const long long items = 4LL * record_work_rows(nx, ny, dim);
     std::vector<TileRef> c;
     for (long long s = 0; s < items; s += kRecordChunk) c.push_back(TileRef{grid, (int)s, 0, 0});
     return c;

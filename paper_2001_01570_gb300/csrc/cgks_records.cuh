@@ -51,6 +51,7 @@ __device__ __forceinline__ RowRef row_ref(const GridDev& G, int r)
 {
     RowRef q;
     const int nx = G.nx, ny = G.ny;
+    if (G.dim == 1) r += 2 * (nx + 1);      // the grid's only row: no neighbours along the faces are read
     const int nrx = (nx + 1) * (ny + 4);
     q.xo = r < nrx;
     if (q.xo) {
@@ -185,71 +186,88 @@ __device__ __forceinline__ int scale_of(int k, double b, double c, double rho, d
 }
 #endif
 
-// The arithmetic of one record in characteristic variables: all four variables
-// from the stencil cells' values Qa[var][cell] and h times normal gradients
-// Sa[var][cell] (face frame), written through out(field, k, value).
+// The linear part of one variable's record (values Q, h times normal gradients S), through
+// out(field, k, value).
 template <int ORDER, class Out>
-__device__ __forceinline__ void char_record(const RegK& r, double gamma, const double Qa[4][4], const double Sa[4][4],
-                                            double ih, double weno_eps, bool inner, Out out)
+__device__ __forceinline__ void linear_fields(const RegK& r, const double Q[4], const double S[4], double ih, int k,
+                                              Out out)
+{
+    double v, hvx, h2vxx;
+#ifdef CGKS_OPCOUNT_HOST
+    linear_recon_rk<ORDER>(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], v, hvx, h2vxx);
+#else
+    RowDiffs x;
+    row_diffs_rk(r, Q, S, x);
+    linear_diff_rk<ORDER>(r, Q[1], r.kmul(RK_HALF, x.d2), x, v, hvx, h2vxx);
+#endif
+    out(RV, k, v);
+    out(RN, k, r.mul(hvx, ih));
+    out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
+}
+
+// Characteristic variables: the basis at the mean of the two cells sharing the face ...
+__device__ __forceinline__ void char_basis(const RegK& r, double gamma, const double Qa[4][4], double& rho, CharState& cs)
 {
     double Wref[4];
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) Wref[kk] = r.mul(0.5, r.add(Qa[kk][1], Qa[kk][2]));
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        double v, hvx, h2vxx;
-#ifdef CGKS_OPCOUNT_HOST
-        linear_recon_rk<ORDER>(r, Qa[k][0], Qa[k][1], Qa[k][2], Qa[k][3], Sa[k][0], Sa[k][1], Sa[k][2], Sa[k][3], v,
-                               hvx, h2vxx);
-#else
-        RowDiffs x;
-        row_diffs_rk(r, Qa[k], Sa[k], x);
-        linear_diff_rk<ORDER>(r, Qa[k][1], r.kmul(RK_HALF, x.d2), x, v, hvx, h2vxx);
-#endif
-        out(RV, k, v);
-        out(RN, k, r.mul(hvx, ih));
-        out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
-    }
-    if (!inner) return;
-    // project on the left eigenvectors of the normal flux Jacobian at the
-    // mean of the two cells sharing the face, WENO-Z per field, map back
-    CharState cs;
     char_state(r, Wref, gamma, cs);
-    double cvl[4], csl[4], cvr[4], csr[4];
+    rho = Wref[0];
+}
+
+// ... and field m: projected on its left eigenvector, WENO-Z, slopes per unit length.
+// w[0..3]: left and right value, left and right slope.
+template <int ORDER>
+__device__ __forceinline__ void char_field(const RegK& r, const CharState& cs, double rho, int m, const double Qa[4][4],
+                                           const double Sa[4][4], double ih, double weno_eps, double w[4])
+{
+    double l[4], Q[4], S[4];
+    char_left_row(r, cs, m, l);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
+        S[c] = char_project(r, m, l, Sa[0][c], Sa[1][c], Sa[2][c], Sa[3][c]);
+    }
+#ifdef CGKS_OPCOUNT_HOST
+    weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, w[0], w[2], w[1], w[3]);
+#else
+    // every characteristic field is measured against the density, whose dimension it has
+    RowDiffs x;
+    row_diffs_rk(r, Q, S, x);
+    weno_pair_row<ORDER>(r, Q, S, x, r.kmul(RK_HALF, x.d2), weno_eps, hi_abs(rho), w[0], w[2], w[1], w[3]);
+#endif
+    w[2] = r.mul(w[2], ih);
+    w[3] = r.mul(w[3], ih);
+}
+
+// The arithmetic of one record in characteristic variables by one thread: all four
+// variables from the stencil cells' values Qa[var][cell] and h times normal gradients
+// Sa[var][cell] (face frame), written through out(field, k, value).  (The record kernel
+// gives each field a lane of its own, the same operations.)
+template <int ORDER, class Out>
+__device__ __forceinline__ void char_record(const RegK& r, double gamma, const double Qa[4][4], const double Sa[4][4],
+                                            double ih, double weno_eps, bool inner, Out out)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) linear_fields<ORDER>(r, Qa[k], Sa[k], ih, k, out);
+    if (!inner) return;
+    CharState cs;
+    double rho, w[4][4], o4[4];
+    char_basis(r, gamma, Qa, rho, cs);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        double l[4], Q[4], S[4];
-        char_left_row(r, cs, m, l);
+        double v[4];
+        char_field<ORDER>(r, cs, rho, m, Qa, Sa, ih, weno_eps, v);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
-            S[c] = char_project(r, m, l, Sa[0][c], Sa[1][c], Sa[2][c], Sa[3][c]);
-        }
-#ifdef CGKS_OPCOUNT_HOST
-        weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, cvl[m], csl[m], cvr[m], csr[m]);
-#else
-        // every characteristic field is measured against the density, whose dimension it has
-        RowDiffs x;
-        row_diffs_rk(r, Q, S, x);
-        weno_pair_row<ORDER>(r, Q, S, x, r.kmul(RK_HALF, x.d2), weno_eps, hi_abs(Wref[0]), cvl[m], csl[m], cvr[m],
-                             csr[m]);
-#endif
-        csl[m] = r.mul(csl[m], ih);
-        csr[m] = r.mul(csr[m], ih);
+        for (int q = 0; q < 4; ++q) w[q][m] = v[q];
     }
-    double o4[4];
-    char_to_cons(r, cs, cvl, o4);
+    const int fields[4] = {RL, RR, RLN, RRN};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) out(RL, k, o4[k]);
-    char_to_cons(r, cs, cvr, o4);
+    for (int q = 0; q < 4; ++q) {
+        char_to_cons(r, cs, w[q], o4);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) out(RR, k, o4[k]);
-    char_to_cons(r, cs, csl, o4);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) out(RLN, k, o4[k]);
-    char_to_cons(r, cs, csr, o4);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) out(RRN, k, o4[k]);
+        for (int k = 0; k < 4; ++k) out(fields[q], k, o4[k]);
+    }
 }
 
 // Conservative variables: variable k of face row `row`.
@@ -293,14 +311,10 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
 
-// Characteristic variables: all four variables of face row `row`.
-template <int ORDER>
-__device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
-                                         int row)
+// the stencil cells of a row, all four variables in the face frame
+__device__ __forceinline__ void char_stencil(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+                                             const RowRef& q, double Qa[4][4], double Sa[4][4])
 {
-    const RowRef q = row_ref(G, row);
-    if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
-    double Qa[4][4], Sa[4][4];
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
         const int pk = q.xo ? kk : ((kk == 1) ? 2 : (kk == 2) ? 1 : kk);
@@ -311,11 +325,66 @@ __device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const 
             Sa[kk][c] = r.mul(q.h, cell_value(G, src, PL, i, j, q.gn + pk));
         }
     }
+}
+
+// Characteristic variables: all four variables of face row `row` by one thread (the host
+// count) ...
+template <int ORDER>
+__device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+                                         int row)
+{
+    const RowRef q = row_ref(G, row);
+    if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
+    double Qa[4][4], Sa[4][4];
+    char_stencil(r, G, src, PL, q, Qa, Sa);
     double* o = q.base + q.idx;
     const size_t st = q.stride;
     char_record<ORDER>(r, G.gamma, Qa, Sa, q.ih, G.weno_eps, q.inner,
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
+
+#ifndef CGKS_OPCOUNT_HOST
+// ... or by four lanes (a quad of a warp), lane m with variable m of the linear fields and
+// field m of the WENO-Z step; the four fields' results are transposed by shuffles, and
+// lane m brings quantity m (left, right value, left, right slope) back to conservative
+// variables.  One thread per row ran the four fields in turn: 600 FP64 instructions in
+// one chain and 254 registers.
+template <int ORDER>
+__device__ __forceinline__ void char_row_quad(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+                                              int row, int m, unsigned quad)
+{
+    const RowRef q = row_ref(G, row);
+    if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
+    double Qa[4][4], Sa[4][4], Qm[4], Sm[4];
+    char_stencil(r, G, src, PL, q, Qa, Sa);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        Qm[c] = m == 0 ? Qa[0][c] : m == 1 ? Qa[1][c] : m == 2 ? Qa[2][c] : Qa[3][c];
+        Sm[c] = m == 0 ? Sa[0][c] : m == 1 ? Sa[1][c] : m == 2 ? Sa[2][c] : Sa[3][c];
+    }
+    double* o = q.base + q.idx;
+    const size_t st = q.stride;
+    linear_fields<ORDER>(r, Qm, Sm, q.ih, m, [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
+    if (!q.inner) return;                     // the same for the quad's lanes (one row)
+    CharState cs;
+    double rho, w[4], t[4], o4[4];
+    char_basis(r, G.gamma, Qa, rho, cs);
+    char_field<ORDER>(r, cs, rho, m, Qa, Sa, q.ih, G.weno_eps, w);
+    // t[j] = field j of quantity m: step s sends quantity m ^ s to lane m ^ s
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int j = m ^ s;
+        const double mine = j == 0 ? w[0] : j == 1 ? w[1] : j == 2 ? w[2] : w[3];
+        const double got = __shfl_xor_sync(quad, mine, s);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = i == j ? got : t[i];
+    }
+    char_to_cons(r, cs, t, o4);
+    const int f = m == 0 ? RL : m == 1 ? RR : m == 2 ? RLN : RRN;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[(f * 4 + k) * st] = o4[k];
+}
+#endif
 
 
 }  // namespace cgks

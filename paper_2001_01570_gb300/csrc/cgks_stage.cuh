@@ -77,7 +77,6 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
         __syncthreads();
         if (s_skip) continue;
         const int nx = G.nx, ny = G.ny, x0 = tr.x0, y0 = tr.y0;
-        const bool dim1 = (G.dim == 1);
 
         // ---------------- phase 1: the tile's face-row records (the record kernel
         // wrote them for every face row of the grid): x-faces x0..x0+TX on rows
@@ -90,12 +89,12 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
             // group g of one orientation: plane p of the group is global plane p0 + p, its
             // local row q is record row base + q (records carry two ghost rows first)
             auto stage = [&](unsigned sbase, int sofs, int np, int plane, int F, int p0, const double* g, size_t gs,
-                             int gfaces, int row0, int face0, int nface_max, int row_max, bool on, int nsmem) {
+                             int gfaces, int row0, int face0, int nface_max, int row_max, int nsmem) {
                 const int n = np * plane;
                 for (int idx = tid; idx < n; idx += kThreads) {
                     const int p = idx / plane, rem = idx - p * plane;
                     const int q = rem / F, fc = rem - q * F;
-                    bool valid = on && (face0 + fc <= nface_max) && (row0 + q <= row_max);
+                    bool valid = (face0 + fc <= nface_max) && (row0 + q <= row_max);
                     if (!CGKS_IN_BOUNDS(sofs + idx < nsmem, G.ctrl)) continue;
                     if (valid)
                         valid = CGKS_IN_BOUNDS(row0 + q >= 0 && face0 + fc >= 0 &&
@@ -111,15 +110,14 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
             using RX = RecGroups<TY, TX + 1>;
             using RY = RecGroups<TX, TY + 1>;
             // x-faces: record rows y0 + 2 + (own row); group A starts two rows earlier, B one
-            stage(sbx, 0, 8, RX::pa, TX + 1, 0, G.recx, sx, nx + 1, y0, x0, nx, ny + 3, true, RX::n);
-            stage(sbx, 8 * RX::pa, 16, RX::pb, TX + 1, 4 * RL, G.recx, sx, nx + 1, y0 + 1, x0, nx, ny + 3, true, RX::n);
+            stage(sbx, 0, 8, RX::pa, TX + 1, 0, G.recx, sx, nx + 1, y0, x0, nx, ny + 3, RX::n);
+            stage(sbx, 8 * RX::pa, 16, RX::pb, TX + 1, 4 * RL, G.recx, sx, nx + 1, y0 + 1, x0, nx, ny + 3, RX::n);
             stage(sbx, 8 * RX::pa + 16 * RX::pb, 4, RX::pc, TX + 1, 4 * RNN, G.recx, sx, nx + 1, y0 + 2, x0, nx, ny + 3,
-                  true, RX::n);
-            stage(sby, 0, 8, RY::pa, TY + 1, 0, G.recy, sy, ny + 1, x0, y0, ny, nx + 3, !dim1, RY::n);
-            stage(sby, 8 * RY::pa, 16, RY::pb, TY + 1, 4 * RL, G.recy, sy, ny + 1, x0 + 1, y0, ny, nx + 3, !dim1,
-                  RY::n);
+                  RX::n);
+            stage(sby, 0, 8, RY::pa, TY + 1, 0, G.recy, sy, ny + 1, x0, y0, ny, nx + 3, RY::n);
+            stage(sby, 8 * RY::pa, 16, RY::pb, TY + 1, 4 * RL, G.recy, sy, ny + 1, x0 + 1, y0, ny, nx + 3, RY::n);
             stage(sby, 8 * RY::pa + 16 * RY::pb, 4, RY::pc, TY + 1, 4 * RNN, G.recy, sy, ny + 1, x0 + 2, y0, ny, nx + 3,
-                  !dim1, RY::n);
+                  RY::n);
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
         __syncthreads();
@@ -129,7 +127,7 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
         // the tile's own faces: x-faces x0..x0+TX-1 and y-faces y0..y0+TY-1 (a tile with
         // x0 = nx or y0 = ny has the grid's last faces alone); every face is evaluated by
         // exactly one tile
-        const int nseg = dim1 ? TX * TY : 2 * TX * TY;
+        constexpr int nseg = 2 * TX * TY;
         const size_t nfx = (size_t)ny * (nx + 1), nfy = (size_t)(ny + 1) * nx;
         const int gp = tid & 1;
         const unsigned pair = 3u << (tid & 30);         // the two lanes of this pair
