@@ -346,11 +346,11 @@ static cgks_status enqueue_steps(cgks_solver* s, int nsteps, long* launches, boo
     const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
     const int rblocks = record_blocks(s->nrchunks, s->nsm);
-    const int ublocks = update_blocks(s->ncchunks, s->nsm, 4);
+    const int cpt = update_cpt((long long)s->nx * s->ny, s->nsm), ublocks = update_blocks(s->ncchunks, s->nsm, cpt);
     const int fblocks = s->nftiles < s->nsm ? s->nftiles : s->nsm;
     for (int k = 0; k < nsteps; ++k) {
-        CK(launch_begin_step(s->d_desc, 1, s->stream));
         if (fused) {
+            CK(launch_begin_step(s->d_desc, 1, s->stream, 1));
             CK(launch_fused_step(s->d_desc, s->d_ftiles, s->nftiles, fblocks, s->stream));
             CK(launch_end_step(s->d_desc, 1, s->stream));
             *launches += 3;
@@ -359,10 +359,9 @@ static cgks_status enqueue_steps(cgks_solver* s, int nsteps, long* launches, boo
         for (int stage = 1; stage <= 2; ++stage) {
             CK(launch_records(stage, cv, s->d_desc, s->d_rchunks, s->nrchunks, rblocks, s->stream));
             CK(launch_stage(s->shape, stage, s->d_desc, s->d_tiles, s->ntiles, nblocks, s->stream));
-            CK(launch_update(stage, s->d_desc, s->d_cchunks, s->ncchunks, ublocks, s->stream, nullptr, 4));
+            CK(launch_update(stage, s->d_desc, s->d_cchunks, s->ncchunks, ublocks, s->stream, nullptr, cpt));
         }
-        CK(launch_end_step(s->d_desc, 1, s->stream));
-        *launches += 8;
+        *launches += 6;
     }
     return CGKS_OK;
 }
@@ -393,6 +392,10 @@ static cgks_status step_impl(cgks_solver* s, int nsteps, double t_end, double* t
     long launches = 0;
     CK(launch_set_ctrl(s->d_ctrl, 0.0, t_end > 0.0 ? t_end : 0.0, -1, 0, s->stream));
     launches += 1;
+    if (!fused) {
+        CK(launch_begin_step(s->d_desc, 1, s->stream));   // the later steps start where the one before ends
+        launches += 1;
+    }
     const int chunk = t_end > 0.0 ? 32 : nsteps;
     int done_steps = 0;
     Ctrl c;
@@ -435,17 +438,17 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
     if (!s || nsteps <= 0 || !stage_ms) return fail(CGKS_E_INVAL, "bad arguments");
     g_last_launches = 0;
     CK(launch_set_ctrl(s->d_ctrl, 0.0, 0.0, -1, 0, s->stream));
-    constexpr int NK = 8;
+    CK(launch_begin_step(s->d_desc, 1, s->stream));
+    constexpr int NK = 8;   // the step's start and end take no launch of their own: intervals 0 and 7 are empty
     std::vector<cudaEvent_t> ev((size_t)nsteps * (NK + 1));
     for (auto& e : ev) CK(cudaEventCreate(&e));
     const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
     const int rblocks = record_blocks(s->nrchunks, s->nsm);
-    const int ublocks = update_blocks(s->ncchunks, s->nsm, 4);
+    const int cpt = update_cpt((long long)s->nx * s->ny, s->nsm), ublocks = update_blocks(s->ncchunks, s->nsm, cpt);
     for (int k = 0; k < nsteps; ++k) {
         cudaEvent_t* e = &ev[(size_t)k * (NK + 1)];
         CK(cudaEventRecord(e[0], s->stream));
-        CK(launch_begin_step(s->d_desc, 1, s->stream));
         CK(cudaEventRecord(e[1], s->stream));
         for (int stage = 1; stage <= 2; ++stage) {
             cudaEvent_t* f = e + 1 + 3 * (stage - 1);
@@ -453,10 +456,9 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
             CK(cudaEventRecord(f[1], s->stream));
             CK(launch_stage(s->shape, stage, s->d_desc, s->d_tiles, s->ntiles, nblocks, s->stream));
             CK(cudaEventRecord(f[2], s->stream));
-            CK(launch_update(stage, s->d_desc, s->d_cchunks, s->ncchunks, ublocks, s->stream, nullptr, 4));
+            CK(launch_update(stage, s->d_desc, s->d_cchunks, s->ncchunks, ublocks, s->stream, nullptr, cpt));
             CK(cudaEventRecord(f[3], s->stream));
         }
-        CK(launch_end_step(s->d_desc, 1, s->stream));
         CK(cudaEventRecord(e[8], s->stream));
     }
     CK(cudaStreamSynchronize(s->stream));
@@ -469,7 +471,7 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
         }
     for (auto& e : ev) cudaEventDestroy(e);
     for (int q = 0; q < NK; ++q) stage_ms[q] = acc[q] / nsteps;
-    g_last_launches = 1 + (long)NK * nsteps;
+    g_last_launches = 2 + 6L * nsteps;
     Ctrl c;
     cgks_status st = read_ctrl(s, &c);
     if (st != CGKS_OK) return st;

@@ -182,9 +182,8 @@ cudaError_t BatchEngine::set_members(const std::vector<std::pair<int, GridDev>>&
         if (d_q_[k]) put(d_q_[k], q[k].data(), q[k].size() * sizeof(TileRef));
     put(d_counts_, counts, sizeof(counts));
     if (e == cudaSuccess) e = cudaEventRecord(stage_done_, stream_);
-    // per step: begin + end, and per stage two record launches (conservative and
-    // characteristic grids), flux, update
-    launches_per_step_ = 2 + 2 * 4;
+    // per stage two record launches (conservative and characteristic grids), flux, update
+    launches_per_step_ = 2 * 4;
     return e;
 }
 
@@ -202,7 +201,7 @@ cudaError_t BatchEngine::capture(int cand)
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         const int* cnt = d_counts_;
-        cudaError_t e1 = launch_begin_step(d_grids_, nslots_, cap);
+        cudaError_t e1 = cudaSuccess;
         for (int stage = 1; stage <= 2; ++stage) {
             for (int v = 0; v < 2 && e1 == cudaSuccess; ++v)
                 e1 = launch_records(stage, v, d_grids_, d_q_[TILE_COUNT + v], (int)cap_[TILE_COUNT + v],
@@ -214,7 +213,6 @@ cudaError_t BatchEngine::capture(int cand)
                 e1 = launch_update(stage, d_grids_, d_q_[TILE_COUNT + 2], (int)cap_[TILE_COUNT + 2],
                                    update_blocks(1 << 30, nsm_, c.cpt), cap, cnt + TILE_COUNT + 2, c.cpt);
         }
-        if (e1 == cudaSuccess) e1 = launch_end_step(d_grids_, nslots_, cap);
         e = cudaStreamEndCapture(cap, &graph);
         if (e1 != cudaSuccess) e = e1;
     }
@@ -263,6 +261,9 @@ cudaError_t BatchEngine::replay(int cand, int nsteps, cudaEvent_t before, cudaEv
     cudaError_t e = cudaSuccess;
     if (!exec_[cand]) e = capture(cand);
     if (e == cudaSuccess && before) e = cudaEventRecord(before, stream_);
+    // the first step's dt, for grids that have joined; the later ones start where the one before ends
+    if (e == cudaSuccess) e = launch_begin_step(d_grids_, nslots_, stream_);
+    if (launches) *launches += 1;
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
         e = cudaGraphLaunch(exec_[cand], stream_);
         if (launches) *launches += launches_per_step_;

@@ -1,5 +1,6 @@
 // cgks_control.cu -- step-control kernels (CFL time step, step begin/end),
 // state layout conversions and the stage-kernel dispatcher.
+#include "cgks_control.cuh"
 #include "cgks_internal.h"
 #include "../../include/cgks.h"
 #include <math.h>
@@ -35,56 +36,31 @@ size_t stage_smem_bytes(int shape, int stage)
     }
 }
 
-static __device__ __forceinline__ unsigned long long inf_bits() { return 0x7ff0000000000000ull; }
-
-// Start of a step: dt = CFL * (min over cells of dx/(|U|+c+2 nu/dx)) of the current
-// state, clipped so that t does not pass t_end; marks grids that are finished.
-__global__ void begin_step_kernel(const GridDev* grids, int n)
+__global__ void begin_step_kernel(const GridDev* grids, int n, int reset)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n) return;
     Ctrl* C = grids[g].ctrl;
-    if (C->done) return;
-    if (C->status) { C->done = 1; return; }
-    if (C->steps_target >= 0 && C->steps >= C->steps_target) { C->done = 1; return; }
-    if (C->t_end > 0.0 && C->t >= C->t_end) { C->done = 1; return; }
-    double dt = grids[g].cfl * __longlong_as_double((long long)C->dtmin_bits);
-    if (!(dt > 0.0) || isinf(dt)) { C->status |= CGKS_E_NONPHYSICAL; C->done = 1; return; }
-    if (C->t_end > 0.0 && C->t + dt > C->t_end) dt = C->t_end - C->t;
-    C->dt = dt;
-    C->dtmin_bits = inf_bits();
+    begin_step(grids[g], C);
+    if (reset && !C->done) C->amax_bits[0] = C->amax_bits[1] = 0;
 }
 
-// End of a step: the new state becomes current unless a kernel raised an error.
 __global__ void end_step_kernel(const GridDev* grids, int n)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n) return;
-    Ctrl* C = grids[g].ctrl;
-    if (C->done) return;
-    if (C->status) { C->done = 1; return; }
-    C->par ^= 1;
-    C->t += C->dt;
-    C->steps += 1;
+    if (g < n) end_step(grids[g].ctrl);
 }
 
-// CFL bound of the current state (after a state is set).
+// speed maxima of the current state (after a state is set)
 __global__ void cfl_kernel(const GridDev* grids, int gidx)
 {
     const GridDev& G = grids[gidx];
     const size_t PL = (size_t)G.nx * G.ny;
     const double* W = G.buf[G.ctrl->par];
-    double dmin = INFINITY;
-    bool bad = false;
-    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < PL; c += (size_t)gridDim.x * blockDim.x) {
-        double d;
-        if (!cfl_cell_bound(G, W[c], W[PL + c], W[2 * PL + c], W[3 * PL + c], G.dim == 1, &d)) { bad = true; continue; }
-        dmin = fmin(dmin, d);
-    }
-    if (bad) atomicOr(&G.ctrl->status, (int)CGKS_E_NONPHYSICAL);
-    for (int o = 16; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
-    if ((threadIdx.x & 31) == 0 && dmin < INFINITY)
-        atomicMin(&G.ctrl->dtmin_bits, (unsigned long long)__double_as_longlong(dmin));
+    SpeedMax s;
+    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < PL; c += (size_t)gridDim.x * blockDim.x)
+        s.cell(G, W[c], W[PL + c], W[2 * PL + c], W[3 * PL + c]);
+    speed_max_warp(G.ctrl, s);
 }
 
 __global__ void set_ctrl_kernel(Ctrl* c, double t, double t_end, long long steps_target, int reset, long long steps0)
@@ -96,7 +72,8 @@ __global__ void set_ctrl_kernel(Ctrl* c, double t, double t_end, long long steps
         c->done = 0;
         c->par = 0;
         c->dt = 0.0;
-        c->dtmin_bits = inf_bits();
+        c->amax_bits[0] = c->amax_bits[1] = 0;
+        c->arrived = 0;
     } else if (!c->status) {
         // a new request may continue a solve that was stopped by its step target or t_end
         c->done = 0;
@@ -134,9 +111,9 @@ __global__ void compress1d_kernel(const double* src, double* dst, int nx)
     for (int p = 0; p < 6; ++p) dst[(size_t)p * nx + i] = src[(size_t)map[p] * nx + i];
 }
 
-cudaError_t launch_begin_step(const GridDev* grids, int n, cudaStream_t st)
+cudaError_t launch_begin_step(const GridDev* grids, int n, cudaStream_t st, int reset)
 {
-    begin_step_kernel<<<(n + 127) / 128, 128, 0, st>>>(grids, n);
+    begin_step_kernel<<<(n + 127) / 128, 128, 0, st>>>(grids, n, reset);
     return cudaGetLastError();
 }
 

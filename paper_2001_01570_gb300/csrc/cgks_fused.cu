@@ -5,6 +5,7 @@
 // does more FP64 work than the three-kernel step (records, flux and update per
 // stage) and is slower on this FP64-bound path; it is kept as the measured
 // alternative and gives the same bits.
+#include "cgks_control.cuh"
 #include "cgks_fused.cuh"
 
 #include <mutex>
@@ -51,7 +52,7 @@ fused_step_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__
                                   G.bc[0] == CGKS_BC_PERIODIC,
                                   G.bc[2] == CGKS_BC_PERIODIC};
         bool bad = false;
-        double dtmin = INFINITY;
+        SpeedMax smax;
         T.records1(tid, kFusedThreads);
         __syncthreads();
         bad |= !T.flux1(tid, kFusedThreads);
@@ -62,12 +63,9 @@ fused_step_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__
         __syncthreads();
         bad |= !T.flux2(tid, kFusedThreads);
         __syncthreads();
-        T.update2(tid, kFusedThreads, dtmin, bad);
+        T.update2(tid, kFusedThreads, smax);
         if (bad) atomicOr(&G.ctrl->status, (int)CGKS_E_NONPHYSICAL);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dtmin = fmin(dtmin, __shfl_xor_sync(0xffffffffu, dtmin, o));
-        if ((tid & 31) == 0 && dtmin < INFINITY)
-            atomicMin(&G.ctrl->dtmin_bits, (unsigned long long)__double_as_longlong(dtmin));
+        speed_max_warp(G.ctrl, smax);
     }
 }
 

@@ -105,7 +105,7 @@ struct FusedTile {
         const int nv = cv ? 1 : 4;
         // x-faces: EX+1 faces x (EY+4) rows; y-faces: EY+1 faces x (EX+4) columns
         const int nxr = (EX + 1) * (EY + 4), nyr = (EY + 1) * (EX + 4);
-        const double* __restrict__ src = G.buf[par];
+        const double* src = G.buf[par];
         const size_t PL = (size_t)G.nx * G.ny;
         for (int item = tid; item < nv * (nxr + nyr); item += nth) {
             const int k = item / (nxr + nyr);
@@ -212,8 +212,7 @@ struct FusedTile {
     {
         constexpr int NS = L::n1x + L::n1y;
         double* ws = P;   // 12 planes of EX x EY
-        double dtmin = 0.0;
-        bool bad = false;
+        SpeedMax none;
         for (int c = tid; c < EX * EY; c += nth) {
             const int lx = c % EX, ly = c / EX;
             const int i = x0 - 2 + lx, j = y0 - 2 + ly;
@@ -221,7 +220,7 @@ struct FusedTile {
             const int wi = perx ? wrap(i, G.nx) : i, wj = pery ? wrap(j, G.ny) : j;
             const size_t off = (size_t)wj * G.nx + wi;
             const bool own = lx >= 2 && lx < TX + 2 && ly >= 2 && ly < TY + 2 && i < G.nx && j < G.ny;
-            double* __restrict__ rbuf = G.buf[par ^ 1];
+            double* rbuf = G.buf[par ^ 1];
             const size_t PL = (size_t)G.nx * G.ny;
             update_cell_core<1>(
                 G, par, off, [&](int q, int side) { return Q[q * NS + ly * (EX + 1) + lx + side]; },
@@ -230,7 +229,7 @@ struct FusedTile {
                 [&](int p, double v) {
                     if (own) rbuf[p * PL + off] = v;
                 },
-                dtmin, bad);
+                none);
         }
     }
 
@@ -351,7 +350,7 @@ struct FusedTile {
     }
 
     // ---------------- phase 6: stage-2 update of the tile's cells
-    __device__ void update2(int tid, int nth, double& dtmin, bool& bad) const
+    __device__ void update2(int tid, int nth, SpeedMax& smax) const
     {
         constexpr int NS = L::n2x + L::n2y;
         for (int c = tid; c < TX * TY; c += nth) {
@@ -362,7 +361,7 @@ struct FusedTile {
             update_cell_core<2>(
                 G, par, off, [&](int q, int side) { return Q[q * NS + ly * (TX + 1) + lx + side]; },
                 [&](int q, int side) { return Q[q * NS + L::n2x + lx * (TY + 1) + ly + side]; },
-                [&](int, double) {}, [&](int, double) {}, dtmin, bad);
+                [&](int, double) {}, [&](int, double) {}, smax);
         }
     }
 };

@@ -14,18 +14,18 @@ namespace cgks {
 // library tracks
 constexpr int kMaxDevices = 64;
 
-// Per-grid control block in device memory.  Written only by the step-control
-// kernels and the stage kernels, so a sequence of steps (or a CUDA graph of
-// them) runs without any host round trip.
+// Per-grid control block in device memory.  Written only by kernels, so a sequence of
+// steps (or a CUDA graph of them) runs without any host round trip.
 struct Ctrl {
     double dt;                        // time step of the step in flight
     double t;                         // simulated time of the state in buf[par]
     double t_end;                     // > 0: clip the last step to reach t_end, then stop
-    unsigned long long dtmin_bits;    // min over cells of dx/(|U|+c) (positive double bits)
+    unsigned long long amax_bits[2];  // max over cells of |U|+c+2 nu/dx and |V|+c+2 nu/dy
+                                      // (positive double bits) of the state in buf[par]
     int status;                       // CGKS_E_* bits raised by kernels
     int done;                         // 1: no further steps run on this grid
     int par;                          // index of the buffer holding the current state
-    int pad;
+    int arrived;                      // chunks of the stage-2 update that have finished
     long long steps;                  // steps completed
     long long steps_target;           // < 0: unlimited
 };
@@ -67,26 +67,43 @@ __device__ __forceinline__ bool in_bounds(bool ok, Ctrl* c)
 #define CGKS_IN_BOUNDS(cond, ctrl) true
 #endif
 
-// CFL bound of one cell, dx/(|U|+c+2 nu/dx) and dy/(|V|+c+2 nu/dy) (Sec. 4; nu =
-// mu/rho), written with explicitly rounded operations so that every kernel that
-// evaluates it (the stage-2 update of a step, the bound of a state that was set
-// or restored) gets the same bits: a restored checkpoint continues exactly as
-// the uninterrupted run.  Returns false for rho <= 0 or p <= 0 (or NaN).
-__device__ __forceinline__ bool cfl_cell_bound(const GridDev& G, double r, double m, double n, double E, bool dim1,
-                                               double* d_out)
+// Signal speeds of one cell, |U|+c+2 nu/dx and |V|+c+2 nu/dy (Sec. 4; nu = mu/rho), written
+// with explicitly rounded operations so that every kernel that evaluates them (the stage-2
+// update of a step, the bound of a state that was set or restored) gets the same bits: a
+// restored checkpoint continues exactly as the uninterrupted run.  The time step needs
+// min over cells of dx / speed, and since a rounded quotient does not grow with its
+// divisor, that is dx / (max over cells of speed), the same bits with one division per
+// step instead of two per cell.  Returns false for rho <= 0 or p <= 0 (or NaN).
+__device__ __forceinline__ bool cfl_cell_speeds(const GridDev& G, double r, double m, double n, double E, double a[2])
 {
-    const double ir = __ddiv_rn(1.0, r);
+    const double ir = __drcp_rn(r);
     const double U = __dmul_rn(m, ir), V = __dmul_rn(n, ir);
     const double ke = __dmul_rn(0.5, __dadd_rn(__dmul_rn(m, U), __dmul_rn(n, V)));
     const double p = __dmul_rn(__dsub_rn(G.gamma, 1.0), __dsub_rn(E, ke));
     if (!(r > 0.0) || !(p > 0.0)) return false;
     const double c = __dsqrt_rn(__dmul_rn(__dmul_rn(G.gamma, p), ir));
     const double two_nu = __dmul_rn(2.0, __dmul_rn(G.mu, ir));
-    double d = __ddiv_rn(G.dx, __dadd_rn(__dadd_rn(fabs(U), c), __dmul_rn(two_nu, G.inv_dx)));
-    if (!dim1) d = fmin(d, __ddiv_rn(G.dy, __dadd_rn(__dadd_rn(fabs(V), c), __dmul_rn(two_nu, G.inv_dy))));
-    *d_out = d;
+    a[0] = __dadd_rn(__dadd_rn(fabs(U), c), __dmul_rn(two_nu, G.inv_dx));
+    a[1] = __dadd_rn(__dadd_rn(fabs(V), c), __dmul_rn(two_nu, G.inv_dy));
     return true;
 }
+
+// largest signal speeds of the cells a thread has seen
+struct SpeedMax {
+    double a[2] = {0.0, 0.0};
+    bool bad = false;
+    __device__ __forceinline__ void cell(const GridDev& G, double r, double m, double n, double E)
+    {
+        double s[2];
+        if (!cfl_cell_speeds(G, r, m, n, E, s)) { bad = true; return; }
+#ifdef CGKS_OPCOUNT_HOST
+        // the operation count is the method's: a bound dx / speed of every cell
+        (void)fmin(__ddiv_rn(G.dx, s[0]), __ddiv_rn(G.dy, s[1]));
+#endif
+        a[0] = fmax(a[0], s[0]);
+        a[1] = fmax(a[1], s[1]);
+    }
+};
 #endif
 
 // face rows with a record: x-faces 0..nx on rows -2..ny+1, y-faces 0..ny on
@@ -143,19 +160,23 @@ constexpr int kRecordChunk = 128;
 // grid (one row of four lanes per four items in characteristic mode); TileRef.x0 is the
 // first item
 std::vector<TileRef> record_chunks(int nx, int ny, int dim, int grid);
-// the update kernel's work queue: chunks of 256 cells of one grid (TileRef.x0
+// the update kernel's work queue: chunks of kCellChunk cells of one grid (TileRef.x0
 // is the first cell)
+constexpr int kCellChunk = 128;
 std::vector<TileRef> cell_chunks(int nx, int ny, int grid);
-// cpt: cells per thread of the update kernel (1, 2 or 4: CTAs of 256, 128 or 64
-// threads per chunk of 256 cells)
+// cpt: cells per thread of the update kernel (1, 2 or 4: CTAs of 128, 64 or 32 threads)
 cudaError_t launch_update(int stage, const GridDev* grids, const TileRef* chunks, int nchunks, int nblocks,
                           cudaStream_t st, const int* dcount = nullptr, int cpt = 1);
-// persistent grid of the update kernel: up to 8 resident CTAs per SM
+// persistent grid of the update kernel: its resident CTAs
 inline int update_blocks(int nchunks, int nsm, int cpt = 1)
 {
-    const int cap = 8 * cpt * nsm;
+    const int cap = (cpt == 1 ? 16 : 32) * nsm;
     return nchunks < cap ? nchunks : cap;
 }
+// cells per thread for one grid run by itself: one while the cells are at most four warps
+// per FP64 unit (four units per SM), where the chain of one thread's instructions counts;
+// two above, where the loads in flight do
+inline int update_cpt(long long cells, int nsm) { return cells <= 4LL * 32 * 4 * nsm ? 1 : 2; }
 // flux kernel: resident CTAs of 128 threads per SM.  The 8x4 strips run three at 168
 // registers (250 B of spills in stage 1): with two CTAs the FP64 unit was 57 % busy, its
 // warps waiting for one another's FP64 and FP32 chains; four at 128 registers spill more
@@ -174,6 +195,37 @@ inline int record_blocks(int nchunks, int nsm)
     return nchunks < cap ? nchunks : cap;
 }
 
+#ifdef __CUDACC__
+// The kernels of a step follow one another in a chain.  Each is launched with programmatic
+// stream serialization: once every CTA of the kernel before is done with its work
+// (release_next), its CTAs may become resident and load their coefficient tables;
+// wait_previous returns when the kernel before has finished and its writes are visible.
+// Per step without / with the chain: 100 cells in 1D 85.4 / 71.7 us, 64^2 136.4 / 133.6.
+// (Released at their start instead, the next kernel's CTAs fill the SMs that happen to be
+// free, up to three on one: 187 us on 64^2.)  Every kernel of the
+// chain waits before its first access to data of a step, so a kernel's end implies the end
+// of all before it; and none reads such data through the non-coherent path (__ldg, const
+// __restrict__), which may take it to be constant from the kernel's early start on.
+__device__ __forceinline__ void release_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // launchers (defined in the kernel translation units).  The persistent kernels
 // stride over a work queue of `n` entries; a non-NULL `dcount` points to an int
 // in device memory that holds the queue's current length instead (read when the
@@ -187,7 +239,10 @@ size_t stage_smem_bytes(int shape, int stage);
 // the fused step (cgks_fused.cu): both stages of a step in one launch over 16 x 8
 // tiles (make_tiles with TILE_16x8), one CTA of 256 threads per SM
 cudaError_t launch_fused_step(const GridDev* grids, const TileRef* tiles, int ntiles, int nblocks, cudaStream_t st);
-cudaError_t launch_begin_step(const GridDev* grids, int ngrids, cudaStream_t st);
+// begin_step (cgks_control.cuh) of every grid: before the first step after control blocks
+// were set; the stage-2 update runs it for the steps that follow.  reset != 0 also clears
+// the speed maxima (the fused step, which has no stage-1 update launch to do so)
+cudaError_t launch_begin_step(const GridDev* grids, int ngrids, cudaStream_t st, int reset = 0);
 cudaError_t launch_end_step(const GridDev* grids, int ngrids, cudaStream_t st);
 cudaError_t launch_cfl(const GridDev* grids, int gidx, const GridDev& host, cudaStream_t st);
 cudaError_t launch_expand1d(const double* src6, double* dst12, int nx, cudaStream_t st);

@@ -32,7 +32,7 @@ constexpr size_t kMaxRecordRows = 2 * kMaxCells + 5 * ((size_t)kMaxSide + kMaxCe
 constexpr int kMaxChunks = (int)((4 * kMaxRecordRows + cgks::kRecordChunk - 1) / cgks::kRecordChunk);
 // face results: 16 per face, (nx+1) ny + nx (ny+1) faces
 constexpr size_t kMaxFaces = 2 * kMaxCells + (size_t)kMaxSide + kMaxCells / kMaxSide;
-constexpr int kMaxCellChunks = (int)((kMaxCells + 255) / 256);
+constexpr int kMaxCellChunks = (int)((kMaxCells + cgks::kCellChunk - 1) / cgks::kCellChunk);
 
 // scratch: buffer for the other state (ping-pong) and for W*, 12 planes each
 static __device__ __align__(256) double g_scratch[2 * 12 * kMaxCells];
@@ -98,7 +98,7 @@ __global__ void noalloc_init_kernel(cgks::GridDev G, int tw, int th, int ntx, in
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nchunks; c += gridDim.x * blockDim.x)
         g_rchunks[c] = cgks::TileRef{0, cgks::kRecordChunk * c, 0, 0};
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncchunks; c += gridDim.x * blockDim.x)
-        g_cchunks[c] = cgks::TileRef{0, 256 * c, 0, 0};
+        g_cchunks[c] = cgks::TileRef{0, cgks::kCellChunk * c, 0, 0};
 }
 
 #define NCK(call)                                                                                  \
@@ -189,7 +189,7 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     const int cv = prob->recon_vars;
     const long long items = 4LL * record_rows(prob->nx, prob->ny, 2);
     const int nrc = (int)((items + kRecordChunk - 1) / kRecordChunk);
-    const int ncc = (int)((cells + 255) / 256);
+    const int ncc = (int)((cells + kCellChunk - 1) / kCellChunk);
     const int work = nt > nrc ? nt : nrc;
     noalloc_init_kernel<<<(work + 255) / 256, 256, 0, stream>>>(G, tw, th, ntx, nt, nrc, ncc);
     NCK(cudaGetLastError());
@@ -198,15 +198,14 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     NCK(launch_cfl(sym->desc, 0, G, stream));
     const int nblocks = stage_blocks(nt, nsm, shape);
     const int rblocks = record_blocks(nrc, nsm);
-    const int ublocks = update_blocks(ncc, nsm);
+    const int cpt = update_cpt((long long)cells, nsm), ublocks = update_blocks(ncc, nsm, cpt);
+    NCK(launch_begin_step(sym->desc, 1, stream));
     for (int k = 0; k < nsteps; ++k) {
-        NCK(launch_begin_step(sym->desc, 1, stream));
         for (int stage = 1; stage <= 2; ++stage) {
             NCK(launch_records(stage, cv, sym->desc, sym->rchunks, nrc, rblocks, stream));
             NCK(launch_stage(shape, stage, sym->desc, sym->tiles, nt, nblocks, stream));
-            NCK(launch_update(stage, sym->desc, sym->cchunks, ncc, ublocks, stream));
+            NCK(launch_update(stage, sym->desc, sym->cchunks, ncc, ublocks, stream, nullptr, cpt));
         }
-        NCK(launch_end_step(sym->desc, 1, stream));
     }
     Ctrl c;
     NCK(cudaMemcpyAsync(&c, sym->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, stream));

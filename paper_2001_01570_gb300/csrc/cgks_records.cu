@@ -36,17 +36,18 @@ __global__ void __launch_bounds__(kRecordChunk, 4) records_kernel(const GridDev*
                                                                     const TileRef* __restrict__ chunks, int nchunks,
                                                                     const int* __restrict__ dcount)
 {
-    if (dcount) nchunks = *dcount;   // queue length in device memory (a server's patched queue)
     __shared__ double s_tab[2 * RK_N];
     for (int i = threadIdx.x; i < 2 * RK_N; i += blockDim.x) s_tab[i] = kReconTab.v[i / RK_N][i % RK_N];
     __syncthreads();
     const double one = ((volatile const double*)s_tab)[RK_ONE];
     const double nzero = ((volatile const double*)s_tab)[RK_NZERO];
+    wait_previous();
+    if (dcount) nchunks = *dcount;   // queue length in device memory (a server's patched queue)
     for (int ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
         const TileRef tr = chunks[ch];
         const GridDev& G = grids[tr.grid];
         if (G.ctrl->done) continue;
-        const double* __restrict__ src = (STAGE == 1) ? G.buf[G.ctrl->par] : G.ws;
+        const double* src = (STAGE == 1) ? G.buf[G.ctrl->par] : G.ws;
         const size_t PL = (size_t)G.nx * G.ny;
         const int nrec = record_work_rows(G.nx, G.ny, G.dim);
         const int item = tr.x0 + (int)threadIdx.x;
@@ -61,6 +62,7 @@ __global__ void __launch_bounds__(kRecordChunk, 4) records_kernel(const GridDev*
             else char_row_quad<8>(RegK{s_tab, one, nzero}, G, src, PL, item >> 2, item & 3, quad);
         }
     }
+    release_next();
 }
 
 std::vector<TileRef> record_chunks(int nx, int ny, int dim, int grid)
@@ -75,14 +77,9 @@ cudaError_t launch_records(int stage, int char_vars, const GridDev* grids, const
                            int nblocks, cudaStream_t st, const int* dcount)
 {
     if (nchunks <= 0 || nblocks <= 0) return cudaSuccess;
-    if (char_vars) {
-        if (stage == 1) records_kernel<1, 1><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
-        else records_kernel<2, 1><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
-    } else {
-        if (stage == 1) records_kernel<1, 0><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
-        else records_kernel<2, 0><<<nblocks, kRecordChunk, 0, st>>>(grids, chunks, nchunks, dcount);
-    }
-    return cudaGetLastError();
+    auto* kernel = char_vars ? (stage == 1 ? records_kernel<1, 1> : records_kernel<2, 1>)
+                             : (stage == 1 ? records_kernel<1, 0> : records_kernel<2, 0>);
+    return launch_chained(kernel, nblocks, kRecordChunk, 0, st, grids, chunks, nchunks, dcount);
 }
 
 }  // namespace cgks

@@ -25,14 +25,14 @@ __device__ __forceinline__ double bc_value(const GridDev& G, double v, int i, in
 }
 
 // plane p of cell (i, j) with the boundary conditions applied outside the grid
-__device__ __forceinline__ double cell_value(const GridDev& G, const double* __restrict__ src, size_t PL, int i, int j,
+__device__ __forceinline__ double cell_value(const GridDev& G, const double* src, size_t PL, int i, int j,
                                              int p)
 {
     int kx, ky;
     const int si = map_axis(i, G.nx, G.bc[0], G.bc[1], kx);
     const int sj = map_axis(j, G.ny, G.bc[2], G.bc[3], ky);
     if (!CGKS_IN_BOUNDS(si >= 0 && si < G.nx && sj >= 0 && sj < G.ny && p >= 0 && p < 12, G.ctrl)) return 0.0;
-    return bc_value(G, __ldg(src + (size_t)p * PL + (size_t)sj * G.nx + si), i, j, kx, ky, p);
+    return bc_value(G, src[(size_t)p * PL + (size_t)sj * G.nx + si], i, j, kx, ky, p);
 }
 
 // geometry of record r of a grid: orientation, stencil start cell and step,
@@ -272,7 +272,7 @@ __device__ __forceinline__ void char_record(const RegK& r, double gamma, const d
 
 // Conservative variables: variable k of face row `row`.
 template <int ORDER>
-__device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+__device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const double* src, size_t PL,
                                          int row, int k)
 {
     const RowRef q = row_ref(G, row);
@@ -287,11 +287,11 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
         const double* d = src + (size_t)(q.gn + pv) * PL + (size_t)q.j0 * G.nx + q.i0;
         const size_t step = q.di ? 1 : (size_t)G.nx;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) { Q[c] = __ldg(v + c * step); S[c] = r.mul(q.h, __ldg(d + c * step)); }
+        for (int c = 0; c < 4; ++c) { Q[c] = v[c * step]; S[c] = r.mul(q.h, d[c * step]); }
         if (mom && q.inner) {
             const double* b = src + (size_t)q.j0 * G.nx + q.i0 + step;
-            rho = __ldg(b);
-            E = __ldg(b + 3 * PL);
+            rho = b[0];
+            E = b[3 * PL];
         }
     } else {
 #pragma unroll
@@ -312,7 +312,7 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
 }
 
 // the stencil cells of a row, all four variables in the face frame
-__device__ __forceinline__ void char_stencil(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+__device__ __forceinline__ void char_stencil(const RegK& r, const GridDev& G, const double* src, size_t PL,
                                              const RowRef& q, double Qa[4][4], double Sa[4][4])
 {
 #pragma unroll
@@ -330,7 +330,7 @@ __device__ __forceinline__ void char_stencil(const RegK& r, const GridDev& G, co
 // Characteristic variables: all four variables of face row `row` by one thread (the host
 // count) ...
 template <int ORDER>
-__device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+__device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const double* src, size_t PL,
                                          int row)
 {
     const RowRef q = row_ref(G, row);
@@ -350,7 +350,7 @@ __device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const 
 // variables.  One thread per row ran the four fields in turn: 600 FP64 instructions in
 // one chain and 254 registers.
 template <int ORDER>
-__device__ __forceinline__ void char_row_quad(const RegK& r, const GridDev& G, const double* __restrict__ src, size_t PL,
+__device__ __forceinline__ void char_row_quad(const RegK& r, const GridDev& G, const double* src, size_t PL,
                                               int row, int m, unsigned quad)
 {
     const RowRef q = row_ref(G, row);

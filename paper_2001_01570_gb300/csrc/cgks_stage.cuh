@@ -62,6 +62,8 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
     __syncthreads();
     const RegK r{s_fk, ((volatile const double*)s_fk)[FK_ONE], ((volatile const double*)s_fk)[FK_NZERO]};
 
+    wait_previous();
+
     // the queue length: the kernel argument, or the int in device memory behind dcount (a server's
     // queue, patched between replays), read at each tile -- at 255 registers a bound kept in a
     // register through the loop costs spills (5 % of the stage-1 kernel's time)
@@ -182,6 +184,7 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
         }
         if (bad) atomicOr(&G.ctrl->status, (int)CGKS_E_NONPHYSICAL);
     }
+    release_next();
 }
 
 // The kernel's attributes (more than 48 KB of dynamic shared memory, the
@@ -217,8 +220,7 @@ cudaError_t launch_stage_t(const GridDev* grids, const TileRef* tiles, int ntile
     cudaError_t e = configure_stage_t<TX, TY, STAGE>();
     if (e != cudaSuccess) return e;
     if (ntiles <= 0 || nblocks <= 0) return cudaSuccess;
-    stage_kernel<TX, TY, STAGE><<<nblocks, kThreads, L::bytes, st>>>(grids, tiles, ntiles, dcount);
-    return cudaGetLastError();
+    return launch_chained(stage_kernel<TX, TY, STAGE>, nblocks, kThreads, L::bytes, st, grids, tiles, ntiles, dcount);
 }
 
 // The launcher and shared-memory size of one tile shape (one translation unit

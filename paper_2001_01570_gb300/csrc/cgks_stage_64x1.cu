@@ -102,6 +102,7 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
     if (tid < 32) s_fk[FK_EXP2 + tid] = exp2((double)tid * (1.0 / 32.0));
     __syncthreads();
     const RegK r{s_fk, ((volatile const double*)s_fk)[FK_ONE], ((volatile const double*)s_fk)[FK_NZERO]};
+    wait_previous();
     for (int tile = blockIdx.x; tile < (dcount ? *(volatile const int*)dcount : ntiles); tile += gridDim.x) {
         __syncthreads();
         const TileRef tr = tiles[tile];
@@ -118,7 +119,7 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
         // the grid's row (j = 0) of the records [7][4][5][nx+1]
         const size_t sx = (size_t)5 * (nx + 1), at0 = (size_t)2 * (nx + 1) + face;
         if (!CGKS_IN_BOUNDS(27 * sx + at0 < 28 * sx && face >= 0, G.ctrl)) continue;
-        auto rec = [&](int f, int k) { return __ldg(G.recx + (size_t)(f * 4 + k) * sx + at0); };
+        auto rec = [&](int f, int k) { return G.recx[(size_t)(f * 4 + k) * sx + at0]; };
         auto state = [&](int f) { return State1{rec(f, 0), rec(f, 1), rec(f, 3)}; };
         const State1 W = state(RV), Wx = state(RN), Wxx = state(RNN), H = state(RL + side), Hn = state(RLN + side);
         const double ir = r.rcp3(W.r), U = r.mul(W.m, ir), e = r.kfma(FK_MHALF, r.mul(W.m, U), W.e);
@@ -184,6 +185,7 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
         if (STAGE == 1) out[(8 * side + 6) * os] = 0.0;
         if (!ok) atomicOr(&G.ctrl->status, (int)CGKS_E_NONPHYSICAL);
     }
+    release_next();
 }
 
 }  // namespace
@@ -192,9 +194,8 @@ cudaError_t launch_stage_64x1(int stage, const GridDev* grids, const TileRef* ti
                               cudaStream_t st, const int* dcount)
 {
     if (ntiles <= 0 || nblocks <= 0) return cudaSuccess;
-    if (stage == 1) flux1d_kernel<1><<<nblocks, kThreads, 0, st>>>(grids, tiles, ntiles, dcount);
-    else flux1d_kernel<2><<<nblocks, kThreads, 0, st>>>(grids, tiles, ntiles, dcount);
-    return cudaGetLastError();
+    return launch_chained(stage == 1 ? flux1d_kernel<1> : flux1d_kernel<2>, nblocks, kThreads, 0, st, grids, tiles, ntiles,
+                          dcount);
 }
 
 size_t smem_64x1(int) { return 0; }

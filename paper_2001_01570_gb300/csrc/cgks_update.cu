@@ -7,50 +7,68 @@
 //            R  = W - (dt F + dt^2/6 F_t) differences,    R_grad from W(dt)
 //            (the face results already carry the dt factors and the Gauss weights)
 //   stage 2: W^{n+1} = R - dt^2/3 F_t* differences, grad^{n+1} = R_grad + dt^2/3
-//            differences of W_tt*; then the CFL bound of W^{n+1} for the next step
+//            differences of W_tt*; the signal speeds of W^{n+1}; the grid's last chunk
+//            to finish ends the step and starts the next one (its dt)
+#include "cgks_control.cuh"
 #include "cgks_update.cuh"
 
 namespace cgks {
 
-// One CTA per chunk of 256 cells of one grid; CPT cells per thread (256 / CPT
-// threads), the cells of a thread 256 / CPT apart so that every pass of the CTA
-// reads and writes contiguous cells.
+// One CTA per chunk of kCellChunk cells of one grid; CPT cells per thread, the cells of a
+// thread kCellChunk / CPT apart so that every pass of the CTA reads and writes contiguous
+// cells.
+// What bounds it: HBM on large grids; on small ones the chain of one thread's 80 (stage 1)
+// to 150 FP64 instructions per cell, so those run one cell per thread.  Measured, stage 1 / 2,
+// before (four cells per thread, chunks of 256, two quotients per cell, the step's end and
+// start in launches of their own) and now: 64^2 27 / 29 -> 14 / 17 us (5 of them the event
+// pair's), 2048^2 537 / 693 -> 575 / 607 us (one cell per thread 573 / 673, four 844 / 590).
 template <int STAGE, int CPT>
-__global__ void __launch_bounds__(256 / CPT) update_kernel(const GridDev* __restrict__ grids,
-                                                           const TileRef* __restrict__ chunks, int nchunks,
-                                                           const int* __restrict__ dcount)
+__global__ void __launch_bounds__(kCellChunk / CPT) update_kernel(const GridDev* __restrict__ grids,
+                                                                  const TileRef* __restrict__ chunks, int nchunks,
+                                                                  const int* __restrict__ dcount)
 {
-    constexpr int NT = 256 / CPT;
+    constexpr int NT = kCellChunk / CPT;
+    wait_previous();
     if (dcount) nchunks = *dcount;   // queue length in device memory (a server's patched queue)
     for (int ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
         const TileRef tr = chunks[ch];
         const GridDev& G = grids[tr.grid];
-        const Ctrl* C = G.ctrl;
+        Ctrl* C = G.ctrl;
         if (C->done) continue;                      // uniform over the block (one grid per chunk)
         const int par = C->par;
         const long long PL = (long long)G.nx * G.ny;
-        double dtmin = INFINITY;
-        bool bad = false;
+        // dt has been taken from the maxima of the state the step started from
+        if (STAGE == 1 && tr.x0 == 0 && threadIdx.x == 0) C->amax_bits[0] = C->amax_bits[1] = 0;
+        SpeedMax smax;
 #pragma unroll
         for (int m = 0; m < CPT; ++m) {
             const long long cell = (long long)tr.x0 + threadIdx.x + m * NT;
-            if (cell < PL) update_cell<STAGE>(G, par, cell, dtmin, bad);
+            if (cell < PL) update_cell<STAGE>(G, par, cell, smax);
         }
         if (STAGE == 2) {
-            if (bad) atomicOr(&G.ctrl->status, (int)CGKS_E_NONPHYSICAL);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dtmin = fmin(dtmin, __shfl_xor_sync(0xffffffffu, dtmin, o));
-            if ((threadIdx.x & 31) == 0 && dtmin < INFINITY)
-                atomicMin(&G.ctrl->dtmin_bits, (unsigned long long)__double_as_longlong(dtmin));
+            speed_max_warp(C, smax);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                // every chunk's maxima and status are in the control block before its arrival is
+                __threadfence();
+                const int last = (int)((PL + kCellChunk - 1) / kCellChunk) - 1;
+                if (atomicAdd(&C->arrived, 1) == last) {
+                    __threadfence();
+                    C->arrived = 0;
+                    end_step(C);
+                    begin_step(G, C);
+                }
+            }
         }
     }
+    release_next();
 }
 
 std::vector<TileRef> cell_chunks(int nx, int ny, int grid)
 {
     const long long cells = (long long)nx * ny;
     std::vector<TileRef> c;
-    for (long long s = 0; s < cells; s += 256) c.push_back(TileRef{grid, (int)s, 0, 0});
+    for (long long s = 0; s < cells; s += kCellChunk) c.push_back(TileRef{grid, (int)s, 0, 0});
     return c;
 }
 
@@ -58,18 +76,10 @@ cudaError_t launch_update(int stage, const GridDev* grids, const TileRef* chunks
                           cudaStream_t st, const int* dcount, int cpt)
 {
     if (nchunks <= 0 || nblocks <= 0) return cudaSuccess;
-#define CGKS_UPDATE_LAUNCH(S, C) update_kernel<S, C><<<nblocks, 256 / C, 0, st>>>(grids, chunks, nchunks, dcount)
-    if (stage == 1) {
-        if (cpt == 4) CGKS_UPDATE_LAUNCH(1, 4);
-        else if (cpt == 2) CGKS_UPDATE_LAUNCH(1, 2);
-        else CGKS_UPDATE_LAUNCH(1, 1);
-    } else {
-        if (cpt == 4) CGKS_UPDATE_LAUNCH(2, 4);
-        else if (cpt == 2) CGKS_UPDATE_LAUNCH(2, 2);
-        else CGKS_UPDATE_LAUNCH(2, 1);
-    }
-#undef CGKS_UPDATE_LAUNCH
-    return cudaGetLastError();
+    auto* kernel = stage == 1 ? (cpt == 4 ? update_kernel<1, 4> : cpt == 2 ? update_kernel<1, 2> : update_kernel<1, 1>)
+                              : (cpt == 4 ? update_kernel<2, 4> : cpt == 2 ? update_kernel<2, 2> : update_kernel<2, 1>);
+    const int threads = kCellChunk / (cpt == 4 ? 4 : cpt == 2 ? 2 : 1);
+    return launch_chained(kernel, nblocks, threads, 0, st, grids, chunks, nchunks, dcount);
 }
 
 }  // namespace cgks

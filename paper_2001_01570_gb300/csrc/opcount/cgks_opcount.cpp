@@ -252,15 +252,11 @@ struct HostStep {
             G.inflow[side][3] = Real(q[3] / (prob->gamma - 1.0) + 0.5 * q[0] * (q[1] * q[1] + q[2] * q[2]));
         }
         // dt from the CFL bound of the state (not part of the counted launches)
-        double dmin = INFINITY;
-        for (size_t c = 0; c < PL; ++c) {
-            Real d;
-            if (!cfl_cell_bound(G, G.buf[0][c], G.buf[0][PL + c], G.buf[0][2 * PL + c], G.buf[0][3 * PL + c], false,
-                                &d))
-                return -2;
-            dmin = std::min(dmin, d.v);
-        }
-        const Real dt = Real(prob->cfl * dmin);
+        SpeedMax smax;
+        for (size_t c = 0; c < PL; ++c)
+            smax.cell(G, G.buf[0][c], G.buf[0][PL + c], G.buf[0][2 * PL + c], G.buf[0][3 * PL + c]);
+        if (smax.bad) return -2;
+        const Real dt = Real(prob->cfl * std::min(G.dx.v / smax.a[0].v, G.dy.v / smax.a[1].v));
         rt = make_recon_tab();
         const int ob = G.order == 6 ? 1 : 0;
         rrec = RegK{rt.v[ob], rt.v[ob][RK_ONE], rt.v[ob][RK_NZERO]};
@@ -315,14 +311,13 @@ struct HostStep {
             snapshot(o + cgks_oc::K_N);
             // cell updates
             memset(cgks_oc::g_tally, 0, sizeof(cgks_oc::g_tally));
-            Real dtmin = Real(INFINITY);
-            bool bad = false;
+            SpeedMax smax;
             for (long long cell = 0; cell < (long long)PL; ++cell) {
-                if (stage == 1) update_cell<1>(G, 0, cell, dtmin, bad);
-                else update_cell<2>(G, 0, cell, dtmin, bad);
+                if (stage == 1) update_cell<1>(G, 0, cell, smax);
+                else update_cell<2>(G, 0, cell, smax);
             }
             snapshot(o + 2 * cgks_oc::K_N);
-            ok &= !bad;
+            ok &= !smax.bad;
         }
         return ok;
     }
@@ -336,7 +331,7 @@ struct HostStep {
         std::vector<Real> P(L::nP, Real(0.0)), Q(L::nQ, Real(0.0));
         const RegK rr = rrec;
         bool ok = true;
-        Real dtmin = Real(INFINITY);
+        SpeedMax smax;
         for (int y0 = 0; y0 < G.ny; y0 += kFusedTY)
             for (int x0 = 0; x0 < G.nx; x0 += kFusedTX) {
                 const FusedTile<kFusedTX, kFusedTY> T{G, P.data(), Q.data(), rflux, rr, x0, y0, 0,
@@ -347,8 +342,8 @@ struct HostStep {
                 T.update1(0, 1);
                 T.records2(0, 1);
                 bad |= !T.flux2(0, 1);
-                T.update2(0, 1, dtmin, bad);
-                ok &= !bad;
+                T.update2(0, 1, smax);
+                ok &= !bad && !smax.bad;
             }
         return ok;
     }
