@@ -133,19 +133,8 @@ __device__ __forceinline__ void tang_diffs(const RegK& r, double vmm, double vm,
 }
 
 __device__ __forceinline__ void tang_weno5_pair(const RegK& r, double v0, const TangDiffs& x, double eps4,
-                                                int scale_hi, double& at_minus, double& at_plus)
+                                                double& at_minus, double& at_plus)
 {
-#ifndef CGKS_OPCOUNT_HOST
-    if (split_scale_ok(scale_hi, eps4) && i_max(hi_abs(x.t0), hi_abs(x.t1)) < scale_hi + kTangThird * (1 << 20) &&
-        i_max(hi_abs(x.A1), hi_abs(x.s1)) < scale_hi + (1 << 20)) {
-        ff m, p;
-        tang_weno5_split(ff_from(x.A1), ff_from(x.s1), ff_from(x.t0), ff_from(x.t1), ff_from(eps4), CGKS_FF(kTangLo),
-                         CGKS_FF(kTangHi), m, p);
-        at_plus = r.kfma(FK_HG, r.sub(x.A1, r.add(d_from(p.h), d_from(p.l))), v0);
-        at_minus = r.kfma(FK_MHG, r.sub(x.A1, r.add(d_from(m.h), d_from(m.l))), v0);
-        return;
-    }
-#endif
     const double D0 = r.sub(x.A1, x.t0), D2 = r.sub(x.A1, x.t1), s0 = r.sub(x.s1, x.t0), s2 = r.add(x.s1, x.t1);
     const double e0 = fma(D0, D0, fma(r.kmul(FK_T13_3, s0), s0, eps4));
     const double e1 = fma(x.A1, x.A1, fma(r.kmul(FK_T13_3, x.s1), x.s1, eps4));
@@ -241,9 +230,27 @@ __device__ __forceinline__ double exp_neg(const RegK& r, double x)
 
 // ------------------------------------------------------------------------
 // erfc(t) for t >= 0 from e = exp(-t^2): e * erfcx(t), erfcx from the piecewise
-// polynomials of cgks_erfcx_table.h (relative error ~2e-16); 11 FMAs instead
-// of a full erfc evaluation, since the half-line moments need e anyway.  Past
-// t = 27.3 e underflows to 0; a NaN t selects the last piece and stays NaN.
+// polynomials of cgks_erfcx_table.h (relative error ~2e-16) instead of a full erfc
+// evaluation, since the half-line moments need e anyway.  Past t = 27.3 e underflows to 0;
+// a NaN t selects the last piece and stays NaN.  With |z| <= 1/8 the terms from z^3 on are
+// below 2^-10 of the value, so Horner's steps down to the z^3 coefficient run in pairs of
+// FP32 (their 2^-46 is 2^-56 of the value) and only the last three in FP64.
+#ifndef CGKS_OPCOUNT_HOST
+constexpr int kErfcxPairs = CGKS_ERFCX_DEG - 2;      // coefficients of z^11 .. z^3
+struct ErfcxPairs { float2 c[CGKS_ERFCX_PIECES][kErfcxPairs]; };
+constexpr ErfcxPairs make_erfcx_pairs()
+{
+    ErfcxPairs t{};
+    for (int k = 0; k < CGKS_ERFCX_PIECES; ++k)
+        for (int m = 0; m < kErfcxPairs; ++m) {
+            const double x = cgks_erfcx_coef[k][m];
+            t.c[k][m].x = (float)x;
+            t.c[k][m].y = (float)(x - (double)(float)x);
+        }
+    return t;
+}
+static __device__ const ErfcxPairs kErfcxTab = make_erfcx_pairs();
+#endif
 __device__ __forceinline__ double erfc_scaled(const RegK& r, double t, double e)
 {
 #ifdef CGKS_OPCOUNT_HOST
@@ -254,9 +261,20 @@ __device__ __forceinline__ double erfc_scaled(const RegK& r, double t, double e)
     const int k = (int)f_mul(4.0f, fminf(f_lead(t), 27.9f));
     const double* c = cgks_erfcx_coef[k];
     const double z = r.sub(t, d_from(f_fma(0.25f, f_int(k), 0.125f)));
-    double v = c[0];
+    const float2* cp = kErfcxTab.c[k];
+    const ff zf = ff_from(z);
+    ff w{cp[0].x, cp[0].y};
 #pragma unroll
-    for (int m = 1; m <= CGKS_ERFCX_DEG; ++m) v = fma(v, z, c[m]);
+    for (int m = 1; m < kErfcxPairs; ++m) {
+        // c + w z, the coefficient the larger addend
+        const ff p = ff_mul(w, zf);
+        const float2 a = cp[m];
+        const float s = f_add(a.x, p.h);
+        w = ff{s, f_add(f_sub(p.h, f_sub(s, a.x)), f_add(a.y, p.l))};
+    }
+    double v = r.add(d_from(w.h), d_from(w.l));
+#pragma unroll
+    for (int m = kErfcxPairs; m <= CGKS_ERFCX_DEG; ++m) v = fma(v, z, c[m]);
     return r.mul(e, v);
 #endif
 }
@@ -454,9 +472,9 @@ __device__ __forceinline__ void euler_second(const Ar& q, const EulerFirst<T>& f
 // of the variables' scales rho, rho a, rho a^2 (a = |U| + |V| + 2 sqrt(theta)), so that
 // the pairs' rounding of W_tt (about 2^-45 of its largest term) stays below the last bit
 // of the state.
-__device__ __forceinline__ bool euler_second_split(const RegK& r, const EulerFirst<double>& f, double gamma,
-                                                   const double Wxx[4], const double Wxy[4], const double Wyy[4],
-                                                   double Wtt[4])
+template <class Src>
+__device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src, const EulerFirst<double>& f,
+                                                   double gamma, double Wtt[4])
 {
     EulerFirst<ff> g;
     g.rho = ff_from(f.rho); g.U = ff_from(f.U); g.V = ff_from(f.V); g.ir = ff_from(f.ir); g.gir = ff_from(f.gir);
@@ -465,8 +483,7 @@ __device__ __forceinline__ bool euler_second_split(const RegK& r, const EulerFir
     g.Vx = ff_from(f.Vx); g.Vy = ff_from(f.Vy); g.ex = ff_from(f.ex); g.ey = ff_from(f.ey); g.Dv = ff_from(f.Dv);
     g.rt = ff_from(f.rt); g.Ut = ff_from(f.Ut); g.Vt = ff_from(f.Vt); g.et = ff_from(f.et); g.uut = ff_from(f.uut);
     ff xx[4], xy[4], yy[4], o[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) { xx[k] = ff_from(Wxx[k]); xy[k] = ff_from(Wxy[k]); yy[k] = ff_from(Wyy[k]); }
+    src.eq_second_split(xx, xy, yy);
     {
         // theta = (gamma - 1) e / rho; e * gir
         const float th = f_mul(g.e.h, g.gir.h), a = f_add(f_add(fabsf(g.U.h), fabsf(g.V.h)), f_mul(2.0f, f_mul(th, f_rsqrt(th))));
@@ -486,11 +503,12 @@ __device__ __forceinline__ bool euler_second_split(const RegK& r, const EulerFir
 }
 #endif
 
-__device__ __forceinline__ void euler_time_derivs(const RegK& r, const double W[4], const double Wx[4],
-                                                  const double Wy[4], const double Wxx[4], const double Wxy[4],
-                                                  const double Wyy[4], double ir, double U, double V, double p,
-                                                  double e, EulerTD& o)
+template <class Src>
+__device__ __forceinline__ void euler_time_derivs(const RegK& r, const Src& src, const double W[4], double ir, double U,
+                                                  double V, double p, double e, EulerTD& o)
 {
+    double Wx[4], Wy[4];
+    src.eq_first(Wx, Wy);
     EulerFirst<double> f;
     f.rho = W[0]; f.U = U; f.V = V; f.ir = ir; f.e = e;
     const double rho = W[0], m = W[1], E = W[3];
@@ -537,8 +555,10 @@ __device__ __forceinline__ void euler_time_derivs(const RegK& r, const double W[
     o.TNS[2] = sxy;
     o.TNS[3] = fma(r.mul(r.k(FK_KHEAT), p), thx, fma(V, sxy, r.mul(U, sxx)));
 #ifndef CGKS_OPCOUNT_HOST
-    if (euler_second_split(r, f, gamma, Wxx, Wxy, Wyy, o.Wtt)) return;
+    if (euler_second_split(r, src, f, gamma, o.Wtt)) return;
 #endif
+    double Wxx[4], Wxy[4], Wyy[4];
+    src.eq_second(Wxx, Wxy, Wyy);
     euler_second(Ar64{r}, f, gamma, Wxx, Wxy, Wyy, o.Wtt);
 }
 
@@ -662,7 +682,8 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
 // Inputs of one Gauss point are pulled from the caller's loader when they are
 // consumed, so that the 48 reconstructed quantities are never live at once:
 //   src.eq_value(W0)                          equilibrium state
-//   src.eq_derivs(W0n, W0t, W0nn, W0nt, W0tt)  its derivatives (face frame)
+//   src.eq_first(W0n, W0t)                    its derivatives (face frame) ...
+//   src.eq_second(W0nn, W0nt, W0tt)           ... and second derivatives
 //   src.ne_value(side, W)                     left (0) / right (1) state
 //   src.ne_slopes(side, Wn, Wt)               its normal and tangential derivatives
 // The caller's table holds the grid's gamma, K and the time step.
@@ -723,11 +744,7 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     // Euler derivatives of the equilibrium state (W_t, W_tt, F, F_t), evaluated after the
     // half-line moments so that the two sets of intermediates are never live together
     EulerTD e;
-    {
-        double W0n[4], W0t[4], W0nn[4], W0nt[4], W0tt[4];
-        src.eq_derivs(W0n, W0t, W0nn, W0nt, W0tt);
-        euler_time_derivs(r, W0, W0n, W0t, W0nn, W0nt, W0tt, ir0, U0, V0, p0, e0, e);
-    }
+    euler_time_derivs(r, src, W0, ir0, U0, V0, p0, e0, e);
 
     // tau-terms of g0: rho <(a_n u + a_t v) u psi> = TNS - F_t (the time part is the Euler F_t)
     // window coefficients over [0, dt]

@@ -42,11 +42,30 @@ struct StageLayout {
     static constexpr size_t bytes = sizeof(double) * (size_t)(n_rx + n_ry + n_parts);
 };
 
+// The quartic through the segment means m_{j-2..j+2} (m0 the centre row): with A1 = m_1 -
+// m_-1, the second difference s1, the sum ts and the difference td of the two third
+// differences,
+//   p(eta)   = m0 - td/4320 + eta (A1/2 - 7 ts/72) + O(eta^2 - 1/12)
+//   p'(eta)  = A1/2 - ts/12 + eta (s1 - td/9) + O(eta^2 - 1/12)
+//   p''(eta) = s1 - td/12 + eta ts/2 + O(eta^2 - 1/12)
+// (exact at the Gauss points eta = +-1/(2 sqrt 3), where eta^2 = 1/12)
+__device__ __forceinline__ double quartic_v0(const RegK& r, double m0, const TangDiffs& x) { return r.kfma(FK_M4320TH, r.sub(x.t1, x.t0), m0); }
+__device__ __forceinline__ double quartic_v1(const RegK& r, const TangDiffs& x) { return r.kfma(FK_M7_72, r.add(x.t0, x.t1), r.kmul(FK_HALF, x.A1)); }
+__device__ __forceinline__ double quartic_t0(const RegK& r, const TangDiffs& x) { return r.kfma(FK_M12TH, r.add(x.t0, x.t1), r.kmul(FK_HALF, x.A1)); }
+__device__ __forceinline__ double quartic_t1(const RegK& r, const TangDiffs& x) { return r.kfma(FK_M9TH, r.sub(x.t1, x.t0), x.s1); }
+__device__ __forceinline__ double quartic_tt0(const RegK& r, const TangDiffs& x) { return r.kfma(FK_M12TH, r.sub(x.t1, x.t0), x.s1); }
+__device__ __forceinline__ double quartic_tt1(const RegK& r, const TangDiffs& x) { return r.kmul(FK_HALF, r.add(x.t0, x.t1)); }
+
 // One Gauss point of a face segment: the face rows around it (records of rows
 // j-2..j+2 of one face) and the reconstruction along the face there.  The
 // segment's slice (segment_parts; part j of variable k at part[(kPartsVar k + j)
 // * stride]) holds what its two Gauss points share.
-enum { kPartsVar = 12, kParts = 4 * kPartsVar };   // 0..7: deriv_parts, 8, 9: W0 at eta = -g, +g, 10, 11: slopes of W_l, W_r
+// Parts of a variable: W0, its tangential slope per unit eta and its normal derivative at
+// eta = -g and +g; the slopes of W_l and W_r; as pairs of FP32 what the second derivatives
+// need (d2/deta2 = PTT0 + eta PTT1, d2/dn deta = PNT0 + eta PNT1; the host operation
+// count keeps them in FP64).
+enum { PV = 0, PT = 2, PN = 4, PS = 6, PTT0 = 8, PTT1, PNT0, PNT1, kPartsVar, kParts = 4 * kPartsVar };
+constexpr double kGauss = 0.28867513459481287;   // 1/(2 sqrt 3): Gauss points at +-kGauss
 
 struct SegmentPoint {
     RegK r;
@@ -66,35 +85,56 @@ struct SegmentPoint {
     __device__ __forceinline__ void eq_value(double W[4]) const
     {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) W[k] = P(k, 8 + gp);
+        for (int k = 0; k < 4; ++k) W[k] = P(k, PV + gp);
     }
 
-    // The quartic through the segment means m_{j-2..j+2} (m0 the centre row): with A1 =
-    // m_1 - m_-1, the second difference s1, the sum ts and the difference td of the two
-    // third differences,
-    //   p(eta)   = m0 - td/4320 + eta (A1/2 - 7 ts/72) + O(eta^2 - 1/12)
-    //   p'(eta)  = A1/2 - ts/12 + eta (s1 - td/9) + O(eta^2 - 1/12)
-    //   p''(eta) = s1 - td/12 + eta ts/2 + O(eta^2 - 1/12)
-    // (exact at the Gauss points eta = +-1/(2 sqrt 3), where eta^2 = 1/12)
-    __device__ __forceinline__ void eq_derivs(double W0n[4], double W0t[4], double W0nn[4], double W0nt[4],
-                                              double W0tt[4]) const
+    __device__ __forceinline__ void eq_first(double W0n[4], double W0t[4]) const
+    {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            W0n[k] = P(k, PN + gp);
+            W0t[k] = r.mul(P(k, PT + gp), iht);
+        }
+    }
+
+    // the second derivatives in FP64, from the rows
+    __device__ __forceinline__ void eq_second(double W0nn[4], double W0nt[4], double W0tt[4]) const
     {
         const double iht2 = r.mul(iht, iht);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            W0t[k] = r.mul(fma(eta, P(k, 1), P(k, 0)), iht);
-            W0tt[k] = r.mul(fma(eta, P(k, 3), P(k, 2)), iht2);
-            W0n[k] = fma(eta, P(k, 5), P(k, 4));
-            W0nt[k] = r.mul(fma(eta, P(k, 7), P(k, 6)), iht);
             W0nn[k] = at(RNN, k, 0);
+#ifdef CGKS_OPCOUNT_HOST
+            W0tt[k] = r.mul(fma(eta, P(k, PTT1), P(k, PTT0)), iht2);
+            W0nt[k] = r.mul(fma(eta, P(k, PNT1), P(k, PNT0)), iht);
+#else
+            TangDiffs x;
+            tang_diffs(r, at(RV, k, -2), at(RV, k, -1), at(RV, k, 0), at(RV, k, 1), at(RV, k, 2), x);
+            W0tt[k] = r.mul(fma(eta, quartic_tt1(r, x), quartic_tt0(r, x)), iht2);
+            tang_diffs(r, at(RN, k, -2), at(RN, k, -1), at(RN, k, 0), at(RN, k, 1), at(RN, k, 2), x);
+            W0nt[k] = r.mul(fma(eta, quartic_t1(r, x), quartic_t0(r, x)), iht);
+#endif
         }
     }
+
+#ifndef CGKS_OPCOUNT_HOST
+    __device__ __forceinline__ void eq_second_split(ff W0nn[4], ff W0nt[4], ff W0tt[4]) const
+    {
+        const ff ih = ff_from(iht), ih2 = ff_mul(ih, ih), et = gp ? CGKS_FF(kGauss) : CGKS_FF(-kGauss);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            W0tt[k] = ff_mul(ff_add(ff_unpack(P(k, PTT0)), ff_mul(et, ff_unpack(P(k, PTT1)))), ih2);
+            W0nt[k] = ff_mul(ff_add(ff_unpack(P(k, PNT0)), ff_mul(et, ff_unpack(P(k, PNT1)))), ih);
+            W0nn[k] = ff_from(at(RNN, k, 0));
+        }
+    }
+#endif
 
     __device__ __forceinline__ void ne_value(int side, double W[4]) const
     {
         const int f = side ? RR : RL;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) W[k] = fma(eta, P(k, 10 + side), at(f, k, 0));
+        for (int k = 0; k < 4; ++k) W[k] = fma(eta, P(k, PS + side), at(f, k, 0));
     }
 
     __device__ __forceinline__ void ne_slopes(int side, double Wn[4], double Wt[4]) const
@@ -104,7 +144,7 @@ struct SegmentPoint {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             Wn[k] = fma(he, r.sub(at(f, k, 1), at(f, k, -1)), at(f, k, 0));
-            Wt[k] = r.mul(P(k, 10 + side), iht);
+            Wt[k] = r.mul(P(k, PS + side), iht);
         }
     }
 
@@ -116,38 +156,18 @@ struct SegmentPoint {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             Wn[k] = ff_add(ff_mul(he, ff_sub(ff_from(at(f, k, 1)), ff_from(at(f, k, -1)))), ff_from(at(f, k, 0)));
-            Wt[k] = ff_mul(ff_from(P(k, 10 + side)), ih);
+            Wt[k] = ff_mul(ff_from(P(k, PS + side)), ih);
         }
     }
 #endif
 };
 
-// the eta-independent parts of the quartic's derivatives for one variable (differences x
-// of the values, rows n_{-2..2} of the normal derivatives), part j at p[j * stride]
-__device__ __forceinline__ void deriv_parts(const RegK& r, double* p, int stride, const TangDiffs& x, double n2m,
-                                            double nm, double n0, double np, double n2p)
-{
-    {
-        const double ts = r.add(x.t0, x.t1), td = r.sub(x.t1, x.t0);
-        p[0 * stride] = r.kfma(FK_M12TH, ts, r.kmul(FK_HALF, x.A1));
-        p[1 * stride] = r.kfma(FK_M9TH, td, x.s1);
-        p[2 * stride] = r.kfma(FK_M12TH, td, x.s1);
-        p[3 * stride] = r.kmul(FK_HALF, ts);
-    }
-    const double B1 = r.sub(np, nm), hB = r.kmul(FK_HALF, B1), s1 = r.kfma(FK_M2, n0, r.add(np, nm));
-    const double ts = r.kfma(FK_M2, B1, r.sub(n2p, n2m));
-    const double td = r.kfma(FK_M4, s1, r.kfma(FK_M2, n0, r.add(n2p, n2m)));
-    p[4 * stride] = r.kfma(FK_M4320TH, td, n0);
-    p[5 * stride] = r.kfma(FK_M7_72, ts, hB);
-    p[6 * stride] = r.kfma(FK_M12TH, ts, hB);
-    p[7 * stride] = r.kfma(FK_M9TH, td, s1);
-}
-
-// What the Gauss points of a segment share, for variables k0..k1-1: the nonlinear values
-// along the face at both points, the non-equilibrium slopes, the derivatives' parts.  A
-// rolled loop: unrolled, its instructions alone outgrow the instruction cache.
+// What the Gauss points of a segment share, for variables k0..k1-1.  Corrections in
+// pairs of FP32 where the rows' differences are small beside the variable's scale (ihn:
+// inverse spacing along the normal, for the derivative rows' differences), else in FP64.
+// A rolled loop: unrolled, its instructions alone outgrow the instruction cache.
 __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
-                                              int rstride, int k0, int k1, double* part, int stride)
+                                              int rstride, double ihn, int k0, int k1, double* part, int stride)
 {
     const double weps = r.k(FK_WEPS), weps4 = r.k(FK_WEPS4);
     auto R = [&](int f, int k, int off) { return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off); };
@@ -160,18 +180,75 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
 #pragma unroll 1
     for (int k = k0; k < k1; ++k) {
         double* p = part + kPartsVar * k * stride;
-        const double m0 = R(RV, k, 0);
-        TangDiffs x;
-        tang_diffs(r, R(RV, k, -2), R(RV, k, -1), m0, R(RV, k, 1), R(RV, k, 2), x);
-#ifdef CGKS_OPCOUNT_HOST
-        const int sc = 0;
-#else
-        const int sc = k == 0 ? sc0 : k == 3 ? sc3 : i_max(hi_abs(m0), (sc0 >> 1) + (sc3 >> 1));
+        int sc = 0;
+        bool split = false;
+        const double m0 = R(RV, k, 0), n0 = R(RN, k, 0);
+#ifndef CGKS_OPCOUNT_HOST
+        sc = k == 0 ? sc0 : k == 3 ? sc3 : i_max(hi_abs(m0), (sc0 >> 1) + (sc3 >> 1));
+        {
+            const double vm = R(RV, k, -1), vp = R(RV, k, 1), nm = R(RN, k, -1), np = R(RN, k, 1);
+            const double va = r.sub(vm, R(RV, k, -2)), vb = r.sub(m0, vm), vc = r.sub(vp, m0), vd = r.sub(R(RV, k, 2), vp);
+            const double na = r.sub(nm, R(RN, k, -2)), nb = r.sub(n0, nm), nc = r.sub(np, n0), nd = r.sub(R(RN, k, 2), np);
+            const QuarticParts v = quartic_split(ff_from(va), ff_from(vb), ff_from(vc), ff_from(vd));
+            const int m1 = i_max(i_max(hi_abs(va), hi_abs(vb)), i_max(hi_abs(vc), hi_abs(vd)));
+            const int mn = i_max(i_max(hi_abs(na), hi_abs(nb)), i_max(hi_abs(nc), hi_abs(nd)));
+            const int lim = sc + kTangFirst * (1 << 20);
+            split = split_scale_ok(sc, weps4) && m1 < lim && mn < lim + i_min(hi_abs(ihn), kHiOne + (60 << 20)) - kHiOne &&
+                    i_max(f_abs_word(v.t0.h), f_abs_word(v.t1.h)) < f_scale_word(sc) + kTangThird * (1 << 23);
+            if (split) {
+                const ff g = CGKS_FF(kGauss), m12 = CGKS_FF(-1.0 / 12.0), c9 = CGKS_FF(1.0 / 9.0);
+                auto sum = [&](double base, ff c) { return r.add(base, r.add(d_from(c.h), d_from(c.l))); };
+                const double A1 = r.sub(vp, vm);
+                ff lo, hi;
+                tang_weno5_split(v.A, v.s, v.t0, v.t1, ff_from(weps4), CGKS_FF(kTangLo), CGKS_FF(kTangHi), lo, hi);
+                p[(PV + 0) * stride] = r.kfma(FK_MHG, sum(A1, ff_neg(lo)), m0);
+                p[(PV + 1) * stride] = r.kfma(FK_HG, sum(A1, ff_neg(hi)), m0);
+                // the quartic of SegmentPoint: slope A1/2 - ts/12 + eta (s - td/9), second derivative
+                // s - td/12 + eta ts/2, value + eta (A1/2 - 7 ts/72) - td/4320
+                const ff x = ff_mul(m12, v.ts), y = ff_mul(g, ff_sub(v.s, ff_mul(c9, v.td)));
+                const double hA = r.kmul(FK_HALF, A1);
+                p[(PT + 0) * stride] = sum(hA, ff_sub(x, y));
+                p[(PT + 1) * stride] = sum(hA, ff_add(x, y));
+                p[PTT0 * stride] = ff_pack(ff_add(v.s, ff_mul(m12, v.td)));
+                p[PTT1 * stride] = ff_pack(ff_scale(0.5f, v.ts));
+                const QuarticParts n = quartic_split(ff_from(na), ff_from(nb), ff_from(nc), ff_from(nd));
+                const ff hB = ff_scale(0.5f, n.A), u = ff_mul(CGKS_FF(-1.0 / 4320.0), n.td),
+                         w = ff_mul(g, ff_add(hB, ff_mul(CGKS_FF(-7.0 / 72.0), n.ts)));
+                p[(PN + 0) * stride] = sum(n0, ff_sub(u, w));
+                p[(PN + 1) * stride] = sum(n0, ff_add(u, w));
+                p[PNT0 * stride] = ff_pack(ff_add(hB, ff_mul(m12, n.ts)));
+                p[PNT1 * stride] = ff_pack(ff_sub(n.s, ff_mul(c9, n.td)));
+            }
+        }
 #endif
-        tang_weno5_pair(r, m0, x, weps4, sc, p[8 * stride], p[9 * stride]);
-        deriv_parts(r, p, stride, x, R(RN, k, -2), R(RN, k, -1), R(RN, k, 0), R(RN, k, 1), R(RN, k, 2));
+        if (!split) {
+            TangDiffs x;
+            tang_diffs(r, R(RV, k, -2), R(RV, k, -1), m0, R(RV, k, 1), R(RV, k, 2), x);
+            tang_weno5_pair(r, m0, x, weps4, p[(PV + 0) * stride], p[(PV + 1) * stride]);
+            const double t0 = quartic_t0(r, x), gt = r.mul(kGauss, quartic_t1(r, x));
+            p[(PT + 0) * stride] = r.sub(t0, gt);
+            p[(PT + 1) * stride] = r.add(t0, gt);
+#ifdef CGKS_OPCOUNT_HOST
+            p[PTT0 * stride] = quartic_tt0(r, x);
+            p[PTT1 * stride] = quartic_tt1(r, x);
+#else
+            p[PTT0 * stride] = ff_pack(ff_from(quartic_tt0(r, x)));
+            p[PTT1 * stride] = ff_pack(ff_from(quartic_tt1(r, x)));
+#endif
+            tang_diffs(r, R(RN, k, -2), R(RN, k, -1), n0, R(RN, k, 1), R(RN, k, 2), x);
+            const double v0 = quartic_v0(r, n0, x), gv = r.mul(kGauss, quartic_v1(r, x));
+            p[(PN + 0) * stride] = r.sub(v0, gv);
+            p[(PN + 1) * stride] = r.add(v0, gv);
+#ifdef CGKS_OPCOUNT_HOST
+            p[PNT0 * stride] = quartic_t0(r, x);
+            p[PNT1 * stride] = quartic_t1(r, x);
+#else
+            p[PNT0 * stride] = ff_pack(ff_from(quartic_t0(r, x)));
+            p[PNT1 * stride] = ff_pack(ff_from(quartic_t1(r, x)));
+#endif
+        }
         tang_weno3_slopes(r, R(RL, k, -1), R(RL, k, 0), R(RL, k, 1), R(RR, k, -1), R(RR, k, 0), R(RR, k, 1), weps, sc,
-                          p[10 * stride], p[11 * stride]);
+                          p[(PS + 0) * stride], p[(PS + 1) * stride]);
     }
 }
 
@@ -208,16 +285,15 @@ __device__ __forceinline__ void gauss_average(const RegK& r, double a, double b,
 // Returns false if a state was non-physical.
 template <int STAGE>
 __device__ __forceinline__ bool segment_results(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
-                                                int rstride, double iht, double* part, int stride,
+                                                int rstride, double ihn, double iht, double* part, int stride,
                                                 double acc[FaceQ<STAGE>::n])
 {
-    constexpr double gq = 0.28867513459481287;   // 1/(2 sqrt 3): Gauss points at +-gq
-    segment_parts(r, rec, pa, pb, pc, r0, rstride, 0, 4, part, stride);
+    segment_parts(r, rec, pa, pb, pc, r0, rstride, ihn, 0, 4, part, stride);
     PointResult<STAGE> s;
     bool ok = true;
 #pragma unroll 1
     for (int gp = 0; gp < 2; ++gp) {
-        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? gq : -gq, iht, gp, part, stride};
+        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, iht, gp, part, stride};
         PointResult<STAGE> o;
         ok &= segment_point<STAGE>(src, o);
 #pragma unroll

@@ -111,6 +111,10 @@ CGKS_SPLIT_FN double d_from(float a)
     return d_make((int)hi, m < 0x00800000u ? 0 : (int)(b << 29));
 }
 
+// a pair in the 64 bits of a double
+CGKS_SPLIT_FN double ff_pack(ff a) { return d_make((int)f_word(a.h), (int)f_word(a.l)); }
+CGKS_SPLIT_FN ff ff_unpack(double x) { return ff{f_bits((uint32_t)d_hi(x)), f_bits((uint32_t)d_lo(x))}; }
+
 CGKS_SPLIT_FN ff ff_neg(ff a) { return ff{-a.h, -a.l}; }
 // renormalise (|h| >= |l|)
 CGKS_SPLIT_FN ff ff_norm(float h, float l)
@@ -263,9 +267,29 @@ CGKS_SPLIT_FN bool split_ok(int scale_hi, double eps, double w, double t, double
 }
 
 // ------------------------------------------------------------------------
-// The nonlinear values along a face (cgks_flux.cuh) as corrections; taken where the third
-// differences (the slope's correction) are below these powers of two of the scale.
-constexpr int kTangThird = -6, kTangSlope = -11;
+// The values and derivatives along a face (cgks_segment.cuh) as corrections; taken where the
+// first and third differences (the slope's correction) are below these powers of two of
+// the scale.
+constexpr int kTangFirst = -3, kTangThird = -6, kTangSlope = -11;
+
+// The quartic through five means from the four differences a..d of neighbours: the
+// centre's difference A = b + c, second difference s, the third differences t0, t1, their
+// sum ts and difference td.
+struct QuarticParts { ff A, s, t0, t1, ts, td; };
+CGKS_SPLIT_FN QuarticParts quartic_split(ff a, ff b, ff c, ff d)
+{
+    QuarticParts q;
+    q.A = ff_add(b, c);
+    q.s = ff_sub(c, b);
+    q.t0 = ff_sub(q.s, ff_sub(b, a));
+    q.t1 = ff_sub(ff_sub(d, c), q.s);
+    q.ts = ff_add(q.t0, q.t1);
+    q.td = ff_sub(q.t1, q.t0);
+    return q;
+}
+// a float's bits for a scale's high word (within split_scale_ok's range)
+CGKS_SPLIT_FN int f_scale_word(int scale_hi) { return (scale_hi - (896 << 20)) << 3; }
+CGKS_SPLIT_FN int f_abs_word(float x) { return (int)(f_word(x) & 0x7fffffffu); }
 
 // Five means: D1 - sum_k w_k D_k = w_0 t0 + w_2 t1 at both Gauss points, from D1, the
 // centre's second difference s1, the third differences t0, t1 and 4 x epsilon; dlo,

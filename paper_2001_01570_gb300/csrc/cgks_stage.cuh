@@ -159,10 +159,9 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
                 continue;
             __syncwarp(pair);   // the slice's reads of the segment before
             // the pair's lanes compute two variables' parts each, then a Gauss point each
-            segment_parts(r, rec, pa, pb, pc, r0, rstride, 2 * gp, 2 * gp + 2, part, kPairs);
+            segment_parts(r, rec, pa, pb, pc, r0, rstride, r.k(xo ? FK_IDX : FK_IDY), 2 * gp, 2 * gp + 2, part, kPairs);
             __syncwarp(pair);
-            constexpr double gq = 0.28867513459481287;
-            const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? gq : -gq, r.k(xo ? FK_IDY : FK_IDX), gp, part,
+            const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, r.k(xo ? FK_IDY : FK_IDX), gp, part,
                                    kPairs};
             PointResult<STAGE> o;
             bad |= !segment_point<STAGE>(src, o);

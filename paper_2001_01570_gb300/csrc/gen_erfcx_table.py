@@ -61,7 +61,7 @@ def main():
              "#pragma once",
              f"#define CGKS_ERFCX_PIECES {NPIECE}",
              f"#define CGKS_ERFCX_DEG {DEG}",
-             f"__device__ const double cgks_erfcx_coef[{NPIECE}][{DEG + 1}] = {{"]
+             f"static constexpr __device__ double cgks_erfcx_coef[{NPIECE}][{DEG + 1}] = {{"]
     for c, co in pieces:
         lines.append("    {" + ", ".join(repr(float(co[m])) for m in range(DEG, -1, -1)) + "},")
     lines.append("};")

@@ -200,12 +200,15 @@ static void check_tangential(int lev)
         TangDiffs x;
         tang_diffs(r, v[0], v[1], v[2], v[3], v[4], x);
         const int sc = hi_abs(v[2]);
-        if (i_max(hi_abs(x.t0), hi_abs(x.t1)) < sc + kTangThird * (1 << 20)) {
+        const ff da = ff_from(v[1] - v[0]), db = ff_from(v[2] - v[1]), dc = ff_from(v[3] - v[2]), dd = ff_from(v[4] - v[3]);
+        const QuarticParts q = quartic_split(da, db, dc, dd);
+        if (std::max(std::max(hi_abs(v[1] - v[0]), hi_abs(v[2] - v[1])), std::max(hi_abs(v[3] - v[2]), hi_abs(v[4] - v[3]))) < sc + kTangFirst * (1 << 20) &&
+            i_max(hi_abs(x.t0), hi_abs(x.t1)) < sc + kTangThird * (1 << 20)) {
             double om, op;
-            tang_weno5_pair(r, v[2], x, 4.0 * eps, 0, om, op);
+            tang_weno5_pair(r, v[2], x, 4.0 * eps, om, op);
             ff m, p;
-            tang_weno5_split(ff_from(x.A1), ff_from(x.s1), ff_from(x.t0), ff_from(x.t1), ff_from(4.0 * eps), CGKS_FF(kTangLo), CGKS_FF(kTangHi), m, p);
-            const double nm = fma(-hg, x.A1 - val(m), v[2]), np = fma(hg, x.A1 - val(p), v[2]);
+            tang_weno5_split(q.A, q.s, q.t0, q.t1, ff_from(4.0 * eps), CGKS_FF(kTangLo), CGKS_FF(kTangHi), m, p);
+            const double A1 = v[3] - v[1], nm = fma(-hg, A1 - val(m), v[2]), np = fma(hg, A1 - val(p), v[2]);
             const Q V[5] = {v[0], v[1], v[2], v[3], v[4]}, D[3] = {3 * V[2] - 4 * V[1] + V[0], V[3] - V[1], 4 * V[3] - V[4] - 3 * V[2]};
             Q e[3];
             for (int k = 0; k < 3; ++k) { const Q s2 = V[k] - 2 * V[k + 1] + V[k + 2]; e[k] = D[k] * D[k] + 13 * s2 * s2 / 3 + 4 * (Q)eps; }
