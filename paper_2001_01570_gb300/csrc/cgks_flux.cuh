@@ -33,6 +33,8 @@ enum FluxK {
     FK_W1A, FK_W1B, FK_W2A, FK_W2B, FK_W3,          // Gauss-average weights of the face results
     FK_GAMMA, FK_GM1, FK_K1, FK_K3, FK_K2INV2, FK_KHEAT, FK_MU,
     FK_IDX, FK_IDY, FK_WEPS, FK_WEPS4,
+    // the same as pairs of FP32 (ff_pack): gamma, gamma - 1, K + 1, K + 3, inverse spacings, epsilons
+    FK_PGAMMA, FK_PGM1, FK_PK1, FK_PK3, FK_PIDX, FK_PIDY, FK_PWEPS, FK_PWEPS4,
     FK_N
 };
 
@@ -94,6 +96,16 @@ __device__ __forceinline__ void flux_table_tile(double* t, const GridDev& G, dou
     t[FK_IDY] = G.inv_dy;
     t[FK_WEPS] = G.weno_eps;
     t[FK_WEPS4] = 4.0 * G.weno_eps;
+#ifndef CGKS_OPCOUNT_HOST
+    t[FK_PGAMMA] = ff_pack(ff_from(G.gamma));
+    t[FK_PGM1] = ff_pack(ff_from(t[FK_GM1]));
+    t[FK_PK1] = ff_pack(ff_from(t[FK_K1]));
+    t[FK_PK3] = ff_pack(ff_from(t[FK_K3]));
+    t[FK_PIDX] = ff_pack(ff_from(G.inv_dx));
+    t[FK_PIDY] = ff_pack(ff_from(G.inv_dy));
+    t[FK_PWEPS] = ff_pack(ff_from(G.weno_eps));
+    t[FK_PWEPS4] = ff_pack(ff_from(t[FK_WEPS4]));
+#endif
 }
 
 // ------------------------------------------------------------------------
@@ -178,7 +190,7 @@ __device__ __forceinline__ bool tang_weno3_small(const RegK& r, double vm, doubl
 {
     const double dm = r.sub(v0, vm), dp = r.sub(vp, v0), A = r.add(dp, dm), s = r.sub(dp, dm);
     if (!(split_scale_ok(scale_hi, eps) && i_max(hi_abs(A), hi_abs(s)) < scale_hi + (1 << 20))) return false;
-    const ff c = tang_weno3_split(ff_from(A), ff_from(s), ff_from(eps));
+    const ff c = tang_weno3_split(ff_from(A), ff_from(s), ff_unpack(r.k(FK_PWEPS)));
     const double ch = d_from(c.h);
     slope = r.kmul(FK_HALF, r.sub(A, r.add(ch, d_from(c.l))));
     return hi_abs(ch) < scale_hi + kTangSlope * (1 << 20);
@@ -383,15 +395,15 @@ struct Ar64 {
 };
 
 #if !defined(CGKS_OPCOUNT_HOST) || defined(CGKS_SPLIT_CHECK)
-// the same in pairs of FP32 (cgks_split.cuh)
+// the same in pairs of FP32 (cgks_split.cuh), not renormalised: the results' weights leave room
 struct ArSplit {
     using T = ff;
     ff g1, k1, k3;
-    __device__ __forceinline__ ff add(ff a, ff b) const { return ff_add(a, b); }
-    __device__ __forceinline__ ff sub(ff a, ff b) const { return ff_sub(a, b); }
+    __device__ __forceinline__ ff add(ff a, ff b) const { return ff_addp(a, b); }
+    __device__ __forceinline__ ff sub(ff a, ff b) const { return ff_addp(a, ff_neg(b)); }
     __device__ __forceinline__ ff mul(ff a, ff b) const { return ff_mul(a, b); }
-    __device__ __forceinline__ ff mad(ff a, ff b, ff c) const { return ff_add(ff_mul(a, b), c); }
-    __device__ __forceinline__ ff nmad(ff a, ff b, ff c) const { return ff_sub(c, ff_mul(a, b)); }
+    __device__ __forceinline__ ff mad(ff a, ff b, ff c) const { return ff_addp(ff_mul(a, b), c); }
+    __device__ __forceinline__ ff nmad(ff a, ff b, ff c) const { return ff_addp(c, ff_neg(ff_mul(a, b))); }
     __device__ __forceinline__ ff half(ff a) const { return ff_scale(0.5f, a); }
     __device__ __forceinline__ ff dbl(ff a) const { return ff_scale(2.0f, a); }
     __device__ __forceinline__ ff tri(ff a) const { return ff_mulf(3.0f, a); }
@@ -474,7 +486,7 @@ __device__ __forceinline__ void euler_second(const Ar& q, const EulerFirst<T>& f
 // of the state.
 template <class Src>
 __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src, const EulerFirst<double>& f,
-                                                   double gamma, double Wtt[4])
+                                                   double Wtt[4])
 {
     EulerFirst<ff> g;
     g.rho = ff_from(f.rho); g.U = ff_from(f.U); g.V = ff_from(f.V); g.ir = ff_from(f.ir); g.gir = ff_from(f.gir);
@@ -496,7 +508,7 @@ __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src
                                f_fma(f_add(m3(g.Ux, g.Uy, g.Vx), fabsf(g.Vy.h)), ia, f_mul(f_add(fabsf(g.rx.h), fabsf(g.ry.h)), ir)));
         if (!(f_mul(f_mul(ad, ad), f_fma(s1, s1, s2)) < 1.0f / 128.0f)) return false;
     }
-    euler_second(ArSplit{}, g, ff_from(gamma), xx, xy, yy, o);
+    euler_second(ArSplit{}, g, ff_unpack(r.k(FK_PGAMMA)), xx, xy, yy, o);
 #pragma unroll
     for (int k = 0; k < 4; ++k) Wtt[k] = r.add(d_from(o[k].h), d_from(o[k].l));
     return true;
@@ -555,7 +567,7 @@ __device__ __forceinline__ void euler_time_derivs(const RegK& r, const Src& src,
     o.TNS[2] = sxy;
     o.TNS[3] = fma(r.mul(r.k(FK_KHEAT), p), thx, fma(V, sxy, r.mul(U, sxx)));
 #ifndef CGKS_OPCOUNT_HOST
-    if (euler_second_split(r, src, f, gamma, o.Wtt)) return;
+    if (euler_second_split(r, src, f, o.Wtt)) return;
 #endif
     double Wxx[4], Wxy[4], Wyy[4];
     src.eq_second(Wxx, Wxy, Wyy);
@@ -575,8 +587,8 @@ __device__ __forceinline__ bool slope_moments_split(const RegK& r, const Src& sr
                                                     double U, double V, double th, double sq, const HalfMoments& h,
                                                     float wth, float wsl, ff Th[4], ff Wsl[4])
 {
-    const ff K1 = ff_from(r.k(FK_K1));
-    const ArSplit q{ff_from(r.k(FK_GM1)), K1, ff_add(K1, ff{2.0f, 0.0f})};
+    const ff K1 = ff_unpack(r.k(FK_PK1));
+    const ArSplit q{ff_unpack(r.k(FK_PGM1)), K1, ff_unpack(r.k(FK_PK3))};
     ff m[4], n[4], s[4], T[4], S[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) m[k] = ff_from(h.m[k]);

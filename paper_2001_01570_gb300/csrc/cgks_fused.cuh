@@ -194,8 +194,7 @@ struct FusedTile {
             if (!CGKS_IN_BOUNDS(r0 >= 0 && r0 + 4 * rstride < pa && r0 + 2 * rstride < pb && r0 < pc, G.ctrl)) continue;
             double acc[16];
             double part[kParts];
-            bad |= !segment_results<1>(rf, rec, pa, pb, pc, r0, rstride, rf.k(xo ? FK_IDX : FK_IDY),
-                                       rf.k(xo ? FK_IDY : FK_IDX), part, 1, acc);
+            bad |= !segment_results<1>(rf, rec, pa, pb, pc, r0, rstride, xo, part, 1, acc);
 #pragma unroll
             for (int qq = 0; qq < 16; qq += 4) {
                 const int k1 = xo ? 1 : 2, k2 = xo ? 2 : 1;
@@ -337,8 +336,7 @@ struct FusedTile {
             if (!CGKS_IN_BOUNDS(r0 >= 0 && r0 + 4 * rstride < pa && r0 + 2 * rstride < pb && r0 < pc, G.ctrl)) continue;
             double acc[8];
             double part[kParts];
-            bad |= !segment_results<2>(rf, rec, pa, pb, pc, r0, rstride, rf.k(xo ? FK_IDX : FK_IDY),
-                                       rf.k(xo ? FK_IDY : FK_IDX), part, 1, acc);
+            bad |= !segment_results<2>(rf, rec, pa, pb, pc, r0, rstride, xo, part, 1, acc);
 #pragma unroll
             for (int qq = 0; qq < 8; qq += 4) {
                 const int k1 = xo ? 1 : 2, k2 = xo ? 2 : 1;

@@ -75,6 +75,7 @@ struct SegmentPoint {
     int gp;                       // 0: eta = -g, 1: +g
     const double* part;
     int stride;
+    int ihp;                      // table index of iht as a pair
 
     __device__ __forceinline__ double at(int f, int k, int off) const
     {
@@ -120,11 +121,11 @@ struct SegmentPoint {
 #ifndef CGKS_OPCOUNT_HOST
     __device__ __forceinline__ void eq_second_split(ff W0nn[4], ff W0nt[4], ff W0tt[4]) const
     {
-        const ff ih = ff_from(iht), ih2 = ff_mul(ih, ih), et = gp ? CGKS_FF(kGauss) : CGKS_FF(-kGauss);
+        const ff ih = ff_unpack(r.k(ihp)), ih2 = ff_mul(ih, ih), et = gp ? CGKS_FF(kGauss) : CGKS_FF(-kGauss);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            W0tt[k] = ff_mul(ff_add(ff_unpack(P(k, PTT0)), ff_mul(et, ff_unpack(P(k, PTT1)))), ih2);
-            W0nt[k] = ff_mul(ff_add(ff_unpack(P(k, PNT0)), ff_mul(et, ff_unpack(P(k, PNT1)))), ih);
+            W0tt[k] = ff_mul(ff_addp(ff_unpack(P(k, PTT0)), ff_mul(et, ff_unpack(P(k, PTT1)))), ih2);
+            W0nt[k] = ff_mul(ff_addp(ff_unpack(P(k, PNT0)), ff_mul(et, ff_unpack(P(k, PNT1)))), ih);
             W0nn[k] = ff_from(at(RNN, k, 0));
         }
     }
@@ -152,10 +153,10 @@ struct SegmentPoint {
     __device__ __forceinline__ void ne_slopes_split(int side, ff Wn[4], ff Wt[4]) const
     {
         const int f = side ? RRN : RLN;
-        const ff he = ff_from(r.kmul(FK_HALF, eta)), ih = ff_from(iht);
+        const ff he = gp ? CGKS_FF(0.5 * kGauss) : CGKS_FF(-0.5 * kGauss), ih = ff_unpack(r.k(ihp));
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            Wn[k] = ff_add(ff_mul(he, ff_sub(ff_from(at(f, k, 1)), ff_from(at(f, k, -1)))), ff_from(at(f, k, 0)));
+            Wn[k] = ff_addp(ff_mul(he, ff_addp(ff_from(at(f, k, 1)), ff_neg(ff_from(at(f, k, -1))))), ff_from(at(f, k, 0)));
             Wt[k] = ff_mul(ff_from(P(k, PS + side)), ih);
         }
     }
@@ -200,7 +201,7 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
                 auto sum = [&](double base, ff c) { return r.add(base, r.add(d_from(c.h), d_from(c.l))); };
                 const double A1 = r.sub(vp, vm);
                 ff lo, hi;
-                tang_weno5_split(v.A, v.s, v.t0, v.t1, ff_from(weps4), CGKS_FF(kTangLo), CGKS_FF(kTangHi), lo, hi);
+                tang_weno5_split(v.A, v.s, v.t0, v.t1, ff_unpack(r.k(FK_PWEPS4)), CGKS_FF(kTangLo), CGKS_FF(kTangHi), lo, hi);
                 p[(PV + 0) * stride] = r.kfma(FK_MHG, sum(A1, ff_neg(lo)), m0);
                 p[(PV + 1) * stride] = r.kfma(FK_HG, sum(A1, ff_neg(hi)), m0);
                 // the quartic of SegmentPoint: slope A1/2 - ts/12 + eta (s - td/9), second derivative
@@ -285,15 +286,17 @@ __device__ __forceinline__ void gauss_average(const RegK& r, double a, double b,
 // Returns false if a state was non-physical.
 template <int STAGE>
 __device__ __forceinline__ bool segment_results(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
-                                                int rstride, double ihn, double iht, double* part, int stride,
+                                                int rstride, bool xo, double* part, int stride,
                                                 double acc[FaceQ<STAGE>::n])
 {
-    segment_parts(r, rec, pa, pb, pc, r0, rstride, ihn, 0, 4, part, stride);
+    const double iht = r.k(xo ? FK_IDY : FK_IDX);
+    const int ihp = xo ? FK_PIDY : FK_PIDX;
+    segment_parts(r, rec, pa, pb, pc, r0, rstride, r.k(xo ? FK_IDX : FK_IDY), 0, 4, part, stride);
     PointResult<STAGE> s;
     bool ok = true;
 #pragma unroll 1
     for (int gp = 0; gp < 2; ++gp) {
-        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, iht, gp, part, stride};
+        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, iht, gp, part, stride, ihp};
         PointResult<STAGE> o;
         ok &= segment_point<STAGE>(src, o);
 #pragma unroll

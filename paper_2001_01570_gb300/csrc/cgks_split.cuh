@@ -122,7 +122,9 @@ CGKS_SPLIT_FN ff ff_norm(float h, float l)
     const float s = f_add(h, l);
     return ff{s, f_sub(l, f_sub(s, h))};
 }
-// a + b without renormalisation: for addends of one sign
+// a + b without renormalisation: for addends of one sign, and where a result's rounding need
+// only be small beside its addends (after a cancellation l may be as large as h, and the
+// products below leave out l times l)
 CGKS_SPLIT_FN ff ff_addp(ff a, ff b)
 {
     const float s = f_add(a.h, b.h), t = f_sub(s, a.h);

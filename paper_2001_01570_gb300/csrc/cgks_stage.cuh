@@ -162,7 +162,7 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
             segment_parts(r, rec, pa, pb, pc, r0, rstride, r.k(xo ? FK_IDX : FK_IDY), 2 * gp, 2 * gp + 2, part, kPairs);
             __syncwarp(pair);
             const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, r.k(xo ? FK_IDY : FK_IDX), gp, part,
-                                   kPairs};
+                                   kPairs, xo ? FK_PIDY : FK_PIDX};
             PointResult<STAGE> o;
             bad |= !segment_point<STAGE>(src, o);
             // each lane averages and writes two variables: the other lane's sums for them come by

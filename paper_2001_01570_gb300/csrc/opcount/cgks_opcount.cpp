@@ -178,9 +178,8 @@ bool tile_segments(const RegK& r, const GridDev& G, int x0, int y0, const std::v
             r0 = il * (TY + 1) + gl; rstride = TY + 1;
             out = G.facey; ostride = nfy; oidx = (size_t)(y0 + gl) * nx + x0 + il;
         }
-        const Real iht = r.k(xo ? FK_IDY : FK_IDX);
         Real acc[NF];
-        ok &= segment_results<STAGE>(r, rec, pa, pb, pc, r0, rstride, r.k(xo ? FK_IDX : FK_IDY), iht, dc.data(), 1, acc);
+        ok &= segment_results<STAGE>(r, rec, pa, pb, pc, r0, rstride, xo, dc.data(), 1, acc);
         for (int q = 0; q < NF; q += 4) {
             const int k1 = xo ? 1 : 2, k2 = xo ? 2 : 1;
             out[(q + 0) * ostride + oidx] = acc[q + 0];
