@@ -288,20 +288,30 @@ cgks_status cgks_destroy(cgks_solver* s)
     return CGKS_OK;
 }
 
+// whether this solver's kernels may read and write device planes at p directly: memory of its
+// own device, aligned (a copy takes any other)
+static bool kernel_access(const cgks_solver* s, const void* p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return a.type == cudaMemoryTypeDevice && a.device == s->device && ((uintptr_t)p & 7) == 0;
+}
+
 static cgks_status set_state_impl(cgks_solver* s, const double* planes, int on_device, double t, long long steps)
 {
     if (!s || !planes) return fail(CGKS_E_INVAL, "NULL argument");
     if (steps < 0) return fail(CGKS_E_INVAL, "steps must be >= 0");
     const size_t PL = (size_t)s->nx * s->ny;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CK(launch_set_ctrl(s->d_ctrl, t, 0.0, -1, 1, s->stream, steps));
     if (s->prob.dim == 1) {
-        CK(cudaMemcpyAsync(s->d_stage1d, planes, 6 * PL * sizeof(double), kind, s->stream));
-        CK(launch_expand1d(s->d_stage1d, s->host_desc.buf[0], s->nx, s->stream));
+        const bool direct = on_device && kernel_access(s, planes);
+        if (!direct) CK(cudaMemcpyAsync(s->d_stage1d, planes, 6 * PL * sizeof(double), kind, s->stream));
+        CK(launch_set_state_1d(s->d_desc, direct ? planes : s->d_stage1d, t, steps, s->stream));
     } else {
+        CK(launch_set_ctrl(s->d_ctrl, t, 0.0, -1, 1, s->stream, steps));
         CK(cudaMemcpyAsync(s->host_desc.buf[0], planes, 12 * PL * sizeof(double), kind, s->stream));
+        CK(launch_cfl(s->d_desc, 0, s->host_desc, s->stream));
     }
-    CK(launch_cfl(s->d_desc, 0, s->host_desc, s->stream));
     if (!on_device) CK(cudaStreamSynchronize(s->stream));
     return CGKS_OK;
 }
@@ -320,16 +330,20 @@ cgks_status cgks_get_state(cgks_solver* s, double* planes, int on_device, double
 {
     if (!s) return fail(CGKS_E_INVAL, "solver is NULL");
     Ctrl c;
+    const size_t PL = (size_t)s->nx * s->ny;
+    // device planes: a kernel picks the buffer, so one synchronisation serves the planes and the
+    // control block
+    const bool direct = planes && on_device && kernel_access(s, planes);
+    if (direct) CK(launch_get_state(s->d_desc, s->host_desc, planes, s->stream));
     cgks_status st = read_ctrl(s, &c);
     if (st != CGKS_OK) return st;
     if (t) *t = c.t;
     if (steps) *steps = (long)c.steps;
-    if (planes) {
-        const size_t PL = (size_t)s->nx * s->ny;
+    if (planes && !direct) {
         const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         const double* cur = s->host_desc.buf[c.par & 1];
         if (s->prob.dim == 1) {
-            CK(launch_compress1d(cur, s->d_stage1d, s->nx, s->stream));
+            CK(launch_get_state(s->d_desc, s->host_desc, s->d_stage1d, s->stream));
             CK(cudaMemcpyAsync(planes, s->d_stage1d, 6 * PL * sizeof(double), kind, s->stream));
         } else {
             CK(cudaMemcpyAsync(planes, cur, 12 * PL * sizeof(double), kind, s->stream));

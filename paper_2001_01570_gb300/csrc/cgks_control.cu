@@ -63,7 +63,8 @@ __global__ void cfl_kernel(const GridDev* grids, int gidx)
     speed_max_warp(G.ctrl, s);
 }
 
-__global__ void set_ctrl_kernel(Ctrl* c, double t, double t_end, long long steps_target, int reset, long long steps0)
+__device__ __forceinline__ void set_ctrl(Ctrl* c, double t, double t_end, long long steps_target, int reset,
+                                         long long steps0)
 {
     if (reset) {
         c->t = t;
@@ -82,6 +83,11 @@ __global__ void set_ctrl_kernel(Ctrl* c, double t, double t_end, long long steps
     c->steps_target = steps_target;
 }
 
+__global__ void set_ctrl_kernel(Ctrl* c, double t, double t_end, long long steps_target, int reset, long long steps0)
+{
+    set_ctrl(c, t, t_end, steps_target, reset, steps0);
+}
+
 // a batch call continues every grid of the batch that has no error: no step
 // target, no end time
 __global__ void batch_resume_kernel(const GridDev* grids, int n)
@@ -94,21 +100,45 @@ __global__ void batch_resume_kernel(const GridDev* grids, int n)
     c->steps_target = -1;
 }
 
-// 1D planes (rho, rhoU, rhoE, their x-gradients) <-> the internal 2D layout
-__global__ void expand1d_kernel(const double* src, double* dst, int nx)
+// The state of a 1D grid (6 planes: rho, rhoU, rhoE, their x-gradients) into the internal
+// 2D layout, with the control block of a solve that starts there and the state's speed
+// maxima: one CTA, one launch (a batch of small grids is set one by one).
+__global__ void __launch_bounds__(256) set_state_1d_kernel(const GridDev* grids, const double* src, double t,
+                                                           long long steps0)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nx) return;
-    const int map[12] = {0, 1, -1, 2, 3, 4, -1, 5, -1, -1, -1, -1};
-    for (int p = 0; p < 12; ++p) dst[(size_t)p * nx + i] = map[p] < 0 ? 0.0 : src[(size_t)map[p] * nx + i];
+    const GridDev& G = grids[0];
+    Ctrl* C = G.ctrl;
+    if (threadIdx.x == 0) {
+        set_ctrl(C, t, 0.0, -1, 1, steps0);
+        __threadfence_block();
+    }
+    __syncthreads();
+    const int nx = G.nx;
+    double* dst = G.buf[0];
+    SpeedMax s;
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+        double v[6];
+#pragma unroll
+        for (int p = 0; p < 6; ++p) v[p] = src[(size_t)p * nx + i];
+        const int map[12] = {0, 1, -1, 2, 3, 4, -1, 5, -1, -1, -1, -1};
+#pragma unroll
+        for (int p = 0; p < 12; ++p) dst[(size_t)p * nx + i] = map[p] < 0 ? 0.0 : v[map[p]];
+        s.cell(G, v[0], v[1], 0.0, v[2]);
+    }
+    speed_max_warp(C, s);
 }
 
-__global__ void compress1d_kernel(const double* src, double* dst, int nx)
+// The current state, whichever buffer holds it, as the caller's planes.
+__global__ void get_state_kernel(const GridDev* grids, double* dst)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nx) return;
+    const GridDev& G = grids[0];
+    const double* src = G.buf[G.ctrl->par & 1];
+    const size_t PL = (size_t)G.nx * G.ny, n = (G.dim == 1 ? 6 : 12) * PL;
     const int map[6] = {0, 1, 3, 4, 5, 7};
-    for (int p = 0; p < 6; ++p) dst[(size_t)p * nx + i] = src[(size_t)map[p] * nx + i];
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t p = i / PL;
+        dst[i] = src[G.dim == 1 ? (size_t)map[p] * PL + (i - p * PL) : i];
+    }
 }
 
 cudaError_t launch_begin_step(const GridDev* grids, int n, cudaStream_t st, int reset)
@@ -145,15 +175,17 @@ cudaError_t launch_batch_resume(const GridDev* grids, int n, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_expand1d(const double* src6, double* dst12, int nx, cudaStream_t st)
+cudaError_t launch_set_state_1d(const GridDev* grids, const double* src, double t, long long steps0, cudaStream_t st)
 {
-    expand1d_kernel<<<(nx + 255) / 256, 256, 0, st>>>(src6, dst12, nx);
+    set_state_1d_kernel<<<1, 256, 0, st>>>(grids, src, t, steps0);
     return cudaGetLastError();
 }
 
-cudaError_t launch_compress1d(const double* src12, double* dst6, int nx, cudaStream_t st)
+cudaError_t launch_get_state(const GridDev* grids, const GridDev& host, double* dst, cudaStream_t st)
 {
-    compress1d_kernel<<<(nx + 255) / 256, 256, 0, st>>>(src12, dst6, nx);
+    const size_t n = (size_t)(host.dim == 1 ? 6 : 12) * host.nx * host.ny;
+    const size_t blocks = (n + 255) / 256;
+    get_state_kernel<<<(int)(blocks < 1216 ? blocks : 1216), 256, 0, st>>>(grids, dst);
     return cudaGetLastError();
 }
 

@@ -245,8 +245,10 @@ cudaError_t launch_fused_step(const GridDev* grids, const TileRef* tiles, int nt
 cudaError_t launch_begin_step(const GridDev* grids, int ngrids, cudaStream_t st, int reset = 0);
 cudaError_t launch_end_step(const GridDev* grids, int ngrids, cudaStream_t st);
 cudaError_t launch_cfl(const GridDev* grids, int gidx, const GridDev& host, cudaStream_t st);
-cudaError_t launch_expand1d(const double* src6, double* dst12, int nx, cudaStream_t st);
-cudaError_t launch_compress1d(const double* src12, double* dst6, int nx, cudaStream_t st);
+// grids[0]'s state from 6 device planes (1D), with its control block reset; its current state
+// to device planes
+cudaError_t launch_set_state_1d(const GridDev* grids, const double* src, double t, long long steps0, cudaStream_t st);
+cudaError_t launch_get_state(const GridDev* grids, const GridDev& host, double* dst, cudaStream_t st);
 // reset != 0: the control block starts a solve at time t with `steps0` steps
 // already taken (0 for a new solve, the checkpoint's count on a restore)
 cudaError_t launch_set_ctrl(Ctrl* c, double t, double t_end, long long steps_target, int reset, cudaStream_t st,
