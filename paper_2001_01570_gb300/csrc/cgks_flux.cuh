@@ -480,7 +480,7 @@ __device__ __forceinline__ void euler_second(const Ar& q, const EulerFirst<T>& f
 #ifndef CGKS_OPCOUNT_HOST
 // W_tt in pairs of FP32: it enters the interface state as dt^2/8 W_tt and dt^2/6 W_tt,
 // second order in the changes over a time step.  False (nothing written) unless
-//   (a dt)^2 (sum of second derivatives + squared sum of first ones) < 2^-7
+//   (a dt)^2 (sum of second derivatives + squared sum of first ones) < 2^-6
 // of the variables' scales rho, rho a, rho a^2 (a = |U| + |V| + 2 sqrt(theta)), so that
 // the pairs' rounding of W_tt (about 2^-45 of its largest term) stays below the last bit
 // of the state.
@@ -506,7 +506,7 @@ __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src
                                f_fma(f_add(m3(xx[1], xy[1], yy[1]), m3(xx[2], xy[2], yy[2])), ir1, f_mul(m3(xx[0], xy[0], yy[0]), ir)));
         const float s1 = f_fma(f_add(fabsf(g.ex.h), fabsf(g.ey.h)), ir2,
                                f_fma(f_add(m3(g.Ux, g.Uy, g.Vx), fabsf(g.Vy.h)), ia, f_mul(f_add(fabsf(g.rx.h), fabsf(g.ry.h)), ir)));
-        if (!(f_mul(f_mul(ad, ad), f_fma(s1, s1, s2)) < 1.0f / 128.0f)) return false;
+        if (!(f_mul(f_mul(ad, ad), f_fma(s1, s1, s2)) < 1.0f / 64.0f)) return false;
     }
     euler_second(ArSplit{}, g, ff_unpack(r.k(FK_PGAMMA)), xx, xy, yy, o);
 #pragma unroll
@@ -578,7 +578,7 @@ __device__ __forceinline__ void euler_time_derivs(const RegK& r, const Src& src,
 // The slope moments in pairs of FP32.  They enter a face's flux through the weights
 // of order tau^2/dt and its state through h dt, a small correction where the
 // collision time is: false (nothing written) unless every weighted term is below
-// 2^-9 of the side's half-line flux of the same kind (a momentum's scale is the
+// 2^-7 of the side's half-line flux of the same kind (a momentum's scale is the
 // normal momentum flux), so that the pairs' rounding stays below that flux's last
 // bit.  wth, wsl: the weights' magnitudes.
 
@@ -598,7 +598,7 @@ __device__ __forceinline__ bool slope_moments_split(const RegK& r, const Src& sr
     slope_moments(q, ne, ff_from(U), fV, fth, ff_scale(2.0f, ff_mul(isq, isq)), m, ff_from(h.g), n, s, T, S);
     const float fr = f_lead(rho), qt = f_fma(fV.h, fV.h, f_mul(K1.h, fth.h)), f0 = f_mul(fr, fabsf(m[1].h)),
                 f1 = f_mul(fr, m[2].h), f3 = f_mul(f_mul(0.5f, fr), f_fma(fabsf(m[1].h), qt, fabsf(m[3].h)));
-    const float w = f_mul(512.0f, wth), v = f_mul(512.0f, wsl);
+    const float w = f_mul(128.0f, wth), v = f_mul(128.0f, wsl);
     // sums, not maxima: a NaN has to fail the comparisons
     bool ok = f0 > 1e-15f && f1 > 1e-15f && f3 > 1e-15f && f_mul(w, fabsf(T[0].h)) < f0 &&
               f_mul(w, f_add(fabsf(T[1].h), fabsf(T[2].h))) < f1 && f_mul(w, fabsf(T[3].h)) < f3;
