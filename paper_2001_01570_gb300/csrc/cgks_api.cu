@@ -357,7 +357,6 @@ cgks_status cgks_get_state(cgks_solver* s, double* planes, int on_device, double
 
 static cgks_status enqueue_steps(cgks_solver* s, int nsteps, long* launches, bool fused)
 {
-    const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
     const int rblocks = record_blocks(s->nrchunks, s->nsm);
     const int cpt = update_cpt((long long)s->nx * s->ny, s->nsm), ublocks = update_blocks(s->ncchunks, s->nsm, cpt);
@@ -372,7 +371,8 @@ static cgks_status enqueue_steps(cgks_solver* s, int nsteps, long* launches, boo
         }
         for (int stage = 1; stage <= 2; ++stage) {
             CK(launch_records(stage, cv, s->d_desc, s->d_rchunks, s->nrchunks, rblocks, s->stream));
-            CK(launch_stage(s->shape, stage, s->d_desc, s->d_tiles, s->ntiles, nblocks, s->stream));
+            CK(launch_stage(s->shape, stage, s->d_desc, s->d_tiles, s->ntiles,
+                            stage_blocks(s->ntiles, s->nsm, s->shape), s->stream));
             CK(launch_update(stage, s->d_desc, s->d_cchunks, s->ncchunks, ublocks, s->stream, nullptr, cpt));
         }
         *launches += 6;
@@ -456,7 +456,6 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
     constexpr int NK = 8;   // the step's start and end take no launch of their own: intervals 0 and 7 are empty
     std::vector<cudaEvent_t> ev((size_t)nsteps * (NK + 1));
     for (auto& e : ev) CK(cudaEventCreate(&e));
-    const int nblocks = stage_blocks(s->ntiles, s->nsm, s->shape);
     const int cv = s->prob.recon_vars;
     const int rblocks = record_blocks(s->nrchunks, s->nsm);
     const int cpt = update_cpt((long long)s->nx * s->ny, s->nsm), ublocks = update_blocks(s->ncchunks, s->nsm, cpt);
@@ -468,7 +467,8 @@ cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8])
             cudaEvent_t* f = e + 1 + 3 * (stage - 1);
             CK(launch_records(stage, cv, s->d_desc, s->d_rchunks, s->nrchunks, rblocks, s->stream));
             CK(cudaEventRecord(f[1], s->stream));
-            CK(launch_stage(s->shape, stage, s->d_desc, s->d_tiles, s->ntiles, nblocks, s->stream));
+            CK(launch_stage(s->shape, stage, s->d_desc, s->d_tiles, s->ntiles,
+                            stage_blocks(s->ntiles, s->nsm, s->shape), s->stream));
             CK(cudaEventRecord(f[2], s->stream));
             CK(launch_update(stage, s->d_desc, s->d_cchunks, s->ncchunks, ublocks, s->stream, nullptr, cpt));
             CK(cudaEventRecord(f[3], s->stream));

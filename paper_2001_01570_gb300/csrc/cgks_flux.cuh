@@ -14,6 +14,11 @@
 
 namespace cgks {
 
+// A branch that the compiler may not turn into predicated instructions: those occupy the
+// FP64 unit whether their predicate holds or not (the interface state's non-equilibrium
+// terms, skipped by almost every warp, cost stage 1 a ninth of its FP64 instructions so).
+#define CGKS_BRANCH(cond) _Pragma("unroll 1") for (bool go_ = (cond); go_; go_ = false)
+
 // Layout of the flux kernel's shared-memory table.  Fixed constants first
 // (copied from kFluxFixed), then the values of the tile's grid and time step
 // (written by the CTA's first thread at the start of each tile).
@@ -366,7 +371,8 @@ __device__ __forceinline__ void slope_moments(const Ar& q, bool ne, T U, T V, T 
     Th[2] = q.mad(V, x2, q.mad(X.B, m[2], q.mad(v2, a1, q.mul(m[1], yt))));
     Th[3] = q.half(q.add(q.mad(m[2], xv, q.mad(qt, x2, x4)),
                          q.mad(m[1], yv, q.mad(Y.B, m[3], q.mul(V, q.mad(w, a1, a3))))));
-    if (ne) {
+    CGKS_BRANCH(ne)
+    {
         const T x1 = y1(X);
         const T a0 = q.mad(Y.R, m[0], q.mul(g, q.nmad(q.half(q.mul(U, itheta)), Y.C, Y.A)));
         Wsl[0] = q.add(x1, q.mad(V, a0, q.mul(Y.B, m[0])));
@@ -652,7 +658,8 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
             o.Fh[1] = fma(rho, h.m[2], o.Fh[1]);
             o.Fh[2] = fma(rho, r.mul(V, h.m[1]), o.Fh[2]);
             o.Fh[3] = fma(rho, r.kmul(FK_HALF, fma(h.m[1], qt, h.m[3])), o.Fh[3]);
-            if (need_ne) {
+            CGKS_BRANCH(need_ne)
+            {
                 o.Wh[0] = fma(rho, h.m[0], o.Wh[0]);
                 o.Wh[1] = fma(rho, h.m[1], o.Wh[1]);
                 o.Wh[2] = fma(rho, r.mul(V, h.m[0]), o.Wh[2]);
@@ -666,22 +673,22 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
 #endif
             double bn[4], bt[4], t[4], ws[4];
             src.ne_slopes(side, bn, bt);
-            const double ith = need_ne ? r.mul(r.add(sq, sq), sq) : th;     // 1/theta = 2 lambda
+            const double ith = r.mul(r.add(sq, sq), sq);     // 1/theta = 2 lambda
             slope_moments(Ar64{r}, need_ne, U, V, th, ith, h.m, h.g, bn, bt, t, ws);
 #pragma unroll
             for (int k = 0; k < 4; ++k) o.Th[k] = r.add(o.Th[k], t[k]);
-            if (need_ne)
+            CGKS_BRANCH(need_ne)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(o.Wsl[k], ws[k]);
+            for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(o.Wsl[k], ws[k]);
         }
         if (!split) return;
 #ifndef CGKS_OPCOUNT_HOST
         if (ok) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) o.Th[k] = r.add(d_from(Ts[k].h), d_from(Ts[k].l));
-            if (need_ne)
+            CGKS_BRANCH(need_ne)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(d_from(Ss[k].h), d_from(Ss[k].l));
+            for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(d_from(Ss[k].h), d_from(Ss[k].l));
             return;
         }
 #endif
@@ -726,8 +733,9 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     // Sec. 4: collision time with pressure-jump enhancement; viscous flow: mu/p
     // with p the equilibrium pressure at the point
     const double mu = r.k(FK_MU), dt = r.k(FK_DT);
-    const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(pl, pr), r.rcp3(r.add(pl, pr)))),
-                           positive(mu) ? r.mul(mu, r.rcp3(p0)) : r.k(FK_EPSDT));
+    double tau0 = r.k(FK_EPSDT);
+    CGKS_BRANCH(positive(mu)) tau0 = r.mul(mu, r.rcp3(p0));
+    const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(pl, pr), r.rcp3(r.add(pl, pr)))), tau0);
     // h = exp(-dt / (2 tau)) weights the non-equilibrium part of the interface state.
     // For dt > 80 tau, h < 4e-18: then 1 - h and 3 - h round to 1 and 3, and the
     // remaining h-terms change the window coefficients by under 2e-14 of a term
@@ -742,7 +750,7 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     const float wth = 0.0f, wsl = 0.0f;
 #else
     const float ft = f_lead(tau), fdt = f_lead(dt);
-    if (ft > 0.0f && fdt < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
+    CGKS_BRANCH(ft > 0.0f && fdt < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
     const bool need_ne = (STAGE == 1) && d_hi(h) >= 0x3bc79ca1;       // high word of 1e-20
     // bounds of the slope terms' weights (FP32, for the choice of their arithmetic): beside F
     // |b4| and |f4| dt/4 below are at most 4 tau (tau + h dt) / dt, beside W it is h dt
@@ -778,11 +786,15 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     }
     if (STAGE == 1) {
         // interface state W(t) = W0 + t W_t + t^2/2 W_tt + e^{-t/tau} [W_ne(t) - W0 - t W_t]
-        const double hdt = r.k(FK_HDT), h2 = r.mul(h, h);
+        const double hdt = r.k(FK_HDT);
         for (int k = 0; k < 4; ++k) {
             Wm[k] = fma(r.k(FK_C8), e.Wtt[k], fma(hdt, e.Wt[k], W0[k]));
             Wb[k] = fma(r.k(FK_C6), e.Wtt[k], fma(dt, e.Wt[k], W0[k]));
-            if (need_ne) {
+        }
+        CGKS_BRANCH(need_ne)
+        {
+            const double h2 = r.mul(h, h);
+            for (int k = 0; k < 4; ++k) {
                 Wm[k] = fma(h, fma(-hdt, e.Wt[k], r.sub(fma(-hdt, o.Wsl[k], o.Wh[k]), W0[k])), Wm[k]);
                 Wb[k] = fma(h2, fma(-dt, e.Wt[k], r.sub(fma(-dt, o.Wsl[k], o.Wh[k]), W0[k])), Wb[k]);
             }

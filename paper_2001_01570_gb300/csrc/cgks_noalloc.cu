@@ -196,14 +196,13 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     // control block starts from t, step 0, no error, state in the caller's buffer
     NCK(launch_set_ctrl(sym->ctrl, *t_inout, 0.0, -1, 1, stream));
     NCK(launch_cfl(sym->desc, 0, G, stream));
-    const int nblocks = stage_blocks(nt, nsm, shape);
     const int rblocks = record_blocks(nrc, nsm);
     const int cpt = update_cpt((long long)cells, nsm), ublocks = update_blocks(ncc, nsm, cpt);
     NCK(launch_begin_step(sym->desc, 1, stream));
     for (int k = 0; k < nsteps; ++k) {
         for (int stage = 1; stage <= 2; ++stage) {
             NCK(launch_records(stage, cv, sym->desc, sym->rchunks, nrc, rblocks, stream));
-            NCK(launch_stage(shape, stage, sym->desc, sym->tiles, nt, nblocks, stream));
+            NCK(launch_stage(shape, stage, sym->desc, sym->tiles, nt, stage_blocks(nt, nsm, shape), stream));
             NCK(launch_update(stage, sym->desc, sym->cchunks, ncc, ublocks, stream, nullptr, cpt));
         }
     }

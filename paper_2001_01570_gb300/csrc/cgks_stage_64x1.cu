@@ -46,7 +46,8 @@ __device__ __forceinline__ void half_1d(const RegK& r, int side, const State1& W
     o.T.r = y2;
     o.T.m = y3;
     o.T.e = r.kmul(FK_HALF, fma(m2, xv, fma(qt, y2, y4)));
-    if (ne) {
+    CGKS_BRANCH(ne)
+    {
         const double y1 = fma(R, m1, fma(A, m0, r.mul(r.kmul(FK_HALF, C), h.g)));
         o.W.r = r.mul(W.r, m0);
         o.W.m = o.F.r;
@@ -130,11 +131,12 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
         // collision time and its weight, as gks_point (the other side's pressure by shuffle)
         const double po = __shfl_xor_sync(pair, ph, 1);
         const double mu = r.k(FK_MU), dt = r.k(FK_DT);
-        const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(ph, po), r.rcp3(r.add(ph, po)))),
-                               positive(mu) ? r.mul(mu, r.rcp3(p)) : r.k(FK_EPSDT));
+        double tau0 = r.k(FK_EPSDT);
+        CGKS_BRANCH(positive(mu)) tau0 = r.mul(mu, r.rcp3(p));
+        const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(ph, po), r.rcp3(r.add(ph, po)))), tau0);
         double h = 0.0;
         const float ft = f_lead(tau);
-        if (ft > 0.0f && f_lead(dt) < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
+        CGKS_BRANCH(ft > 0.0f && f_lead(dt) < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
         const bool need_ne = (STAGE == 1) && d_hi(h) >= 0x3bc79ca1;       // h >= 1e-20
         Half1 o;
         half_1d(r, side, H, Hn, Uh, thh, need_ne, o);
@@ -145,7 +147,7 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
         };
         both(o.F);
         both(o.T);
-        if (need_ne) { both(o.W); both(o.S); }        // tau is the pair's, so need_ne is too
+        CGKS_BRANCH(need_ne) { both(o.W); both(o.S); }        // tau is the pair's, so need_ne is too
         Euler1 E;
         euler_1d(r, W, Wx, Wxx, ir, U, p, e, E);
         // window coefficients over [0, dt] (gks_point)
@@ -164,7 +166,8 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
             if (STAGE == 1) {
                 const double fb = fma(b4, dTh, fma(-tau, TNS, fma(a, dFh, F))), fb2 = r.add(fb, fb);
                 double wm = fma(r.k(FK_C8), Wtt, fma(hdt, Wt, W0)), wb = fma(r.k(FK_C6), Wtt, fma(dt, Wt, W0));
-                if (need_ne) {
+                CGKS_BRANCH(need_ne)
+                {
                     wm = fma(h, fma(-hdt, Wt, r.sub(fma(-hdt, Ws, Wh), W0)), wm);
                     wb = fma(h2, fma(-dt, Wt, r.sub(fma(-dt, Ws, Wh), W0)), wb);
                 }
