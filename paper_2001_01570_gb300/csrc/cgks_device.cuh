@@ -369,13 +369,14 @@ struct CharState { double U, V, c, H, q2, b1, b2, ic; };
 // the characteristic path gets the same bits)
 __device__ __forceinline__ void char_state(const RegK& r, const double W[4], double gamma, CharState& s)
 {
-    const double ir = __drcp_rn(W[0]), gm1 = r.sub(gamma, r.one);
+    const double ir = r.rcp3(W[0]), gm1 = r.sub(gamma, r.one);
     s.U = r.mul(W[1], ir);
     s.V = r.mul(W[2], ir);
     s.q2 = fma(s.V, s.V, r.mul(s.U, s.U));
     const double p = r.mul(gm1, fma(r.mul(-0.5, W[0]), s.q2, W[3]));
-    s.c = __dsqrt_rn(r.mul(r.mul(gamma, p), ir));
-    s.ic = __drcp_rn(s.c);
+    const double c2 = r.mul(r.mul(gamma, p), ir);
+    s.ic = r.rsq(c2);
+    s.c = r.mul(c2, s.ic);
     s.H = r.mul(r.add(W[3], p), ir);
     s.b2 = r.mul(r.mul(gm1, s.ic), s.ic);
     s.b1 = r.mul(r.mul(0.5, s.b2), s.q2);

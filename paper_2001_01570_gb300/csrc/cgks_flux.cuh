@@ -37,7 +37,7 @@ enum FluxK {
     FK_DT = FK_NFIX2, FK_IDT, FK_4IDT2, FK_HDT, FK_MHDT, FK_EPSDT, FK_CTAUDT, FK_C8, FK_C6,
     FK_W1A, FK_W1B, FK_W2A, FK_W2B, FK_W3,          // Gauss-average weights of the face results
     FK_GAMMA, FK_GM1, FK_K1, FK_K3, FK_K2INV2, FK_KHEAT, FK_MU,
-    FK_IDX, FK_IDY, FK_WEPS, FK_WEPS4,
+    FK_IDX, FK_IDY, FK_HIDX, FK_HIDY, FK_WEPS, FK_WEPS4,
     // the same as pairs of FP32 (ff_pack): gamma, gamma - 1, K + 1, K + 3, inverse spacings, epsilons
     FK_PGAMMA, FK_PGM1, FK_PK1, FK_PK3, FK_PIDX, FK_PIDY, FK_PWEPS, FK_PWEPS4,
     FK_N
@@ -99,6 +99,8 @@ __device__ __forceinline__ void flux_table_tile(double* t, const GridDev& G, dou
     t[FK_MU] = G.mu;
     t[FK_IDX] = G.inv_dx;
     t[FK_IDY] = G.inv_dy;
+    t[FK_HIDX] = 0.5 * G.inv_dx;
+    t[FK_HIDY] = 0.5 * G.inv_dy;
     t[FK_WEPS] = G.weno_eps;
     t[FK_WEPS4] = 4.0 * G.weno_eps;
 #ifndef CGKS_OPCOUNT_HOST
@@ -187,22 +189,22 @@ __device__ __forceinline__ void tang_weno3_parts(const RegK& r, double vm, doubl
     den = r.add(n0, n1);
 }
 
-// One row's slope in the split form: false where the correction it carries is not
+// Twice one row's slope in the split form: false where the correction it carries is not
 // below 2^-11 of the scale (its relative error is about 2^-44).
 #ifndef CGKS_OPCOUNT_HOST
 __device__ __forceinline__ bool tang_weno3_small(const RegK& r, double vm, double v0, double vp, double eps,
-                                                 int scale_hi, double& slope)
+                                                 int scale_hi, double& slope2)
 {
     const double dm = r.sub(v0, vm), dp = r.sub(vp, v0), A = r.add(dp, dm), s = r.sub(dp, dm);
     if (!(split_scale_ok(scale_hi, eps) && i_max(hi_abs(A), hi_abs(s)) < scale_hi + (1 << 20))) return false;
     const ff c = tang_weno3_split(ff_from(A), ff_from(s), ff_unpack(r.k(FK_PWEPS)));
     const double ch = d_from(c.h);
-    slope = r.kmul(FK_HALF, r.sub(A, r.add(ch, d_from(c.l))));
+    slope2 = r.sub(A, r.add(ch, d_from(c.l)));
     return hi_abs(ch) < scale_hi + kTangSlope * (1 << 20);
 }
 #endif
 
-// the slopes of the left and right states' rows, with one reciprocal for both
+// twice the slopes of the left and right states' rows, with one reciprocal for both
 __device__ __forceinline__ void tang_weno3_slopes(const RegK& r, double lm, double l0, double lp, double rm,
                                                   double r0, double rp, double eps, int scale_hi, double& sl,
                                                   double& sr)
@@ -214,8 +216,8 @@ __device__ __forceinline__ void tang_weno3_slopes(const RegK& r, double lm, doub
     tang_weno3_parts(r, lm, l0, lp, eps, nl, dl);
     tang_weno3_parts(r, rm, r0, rp, eps, nr, dr);
     const double inv = r.rcp(r.mul(dl, dr));
-    sl = r.mul(nl, r.mul(dr, inv));
-    sr = r.mul(nr, r.mul(dl, inv));
+    sl = r.mul(r.add(nl, nl), r.mul(dr, inv));
+    sr = r.mul(r.add(nr, nr), r.mul(dl, inv));
 }
 
 // ------------------------------------------------------------------------

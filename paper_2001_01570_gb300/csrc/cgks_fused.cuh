@@ -151,15 +151,15 @@ struct FusedTile {
                 if (G.order == 6) cons_record<6>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
                 else cons_record<8>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
             } else {
-                double Qa[4][4], Sa[4][4];
+                double Qa[4][4], Na[4][4];
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                     const int pk = xo ? kk : ((kk == 1) ? 2 : (kk == 2) ? 1 : kk);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) { Qa[kk][c] = cell(c, pk); Sa[kk][c] = rr.mul(h, cell(c, gn + pk)); }
+                    for (int c = 0; c < 4; ++c) { Qa[kk][c] = cell(c, pk); Na[kk][c] = cell(c, gn + pk); }
                 }
-                if (G.order == 6) char_record<6>(rr, G.gamma, Qa, Sa, ih, G.weno_eps, inner, out);
-                else char_record<8>(rr, G.gamma, Qa, Sa, ih, G.weno_eps, inner, out);
+                if (G.order == 6) char_record<6>(rr, G.gamma, Qa, Na, h, ih, G.weno_eps, inner, out);
+                else char_record<8>(rr, G.gamma, Qa, Na, h, ih, G.weno_eps, inner, out);
             }
         }
     }
@@ -295,15 +295,15 @@ struct FusedTile {
                 if (G.order == 6) cons_record<6>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
                 else cons_record<8>(rr, Qv, S, ih, G.weno_eps, inner, k, sc, out);
             } else {
-                double Qa[4][4], Sa[4][4];
+                double Qa[4][4], Na[4][4];
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                     const int pk = xo ? kk : ((kk == 1) ? 2 : (kk == 2) ? 1 : kk);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) { Qa[kk][c] = cell(c, pk); Sa[kk][c] = rr.mul(h, cell(c, gn + pk)); }
+                    for (int c = 0; c < 4; ++c) { Qa[kk][c] = cell(c, pk); Na[kk][c] = cell(c, gn + pk); }
                 }
-                if (G.order == 6) char_record<6>(rr, G.gamma, Qa, Sa, ih, G.weno_eps, inner, out);
-                else char_record<8>(rr, G.gamma, Qa, Sa, ih, G.weno_eps, inner, out);
+                if (G.order == 6) char_record<6>(rr, G.gamma, Qa, Na, h, ih, G.weno_eps, inner, out);
+                else char_record<8>(rr, G.gamma, Qa, Na, h, ih, G.weno_eps, inner, out);
             }
         }
     }

@@ -186,13 +186,15 @@ __device__ __forceinline__ int scale_of(int k, double b, double c, double rho, d
 }
 #endif
 
-// The linear part of one variable's record (values Q, h times normal gradients S), through
+// The linear part of one variable's record (values Q, normal gradients N), through
 // out(field, k, value).
 template <int ORDER, class Out>
-__device__ __forceinline__ void linear_fields(const RegK& r, const double Q[4], const double S[4], double ih, int k,
-                                              Out out)
+__device__ __forceinline__ void linear_fields(const RegK& r, const double Q[4], const double N[4], double h, double ih,
+                                              int k, Out out)
 {
-    double v, hvx, h2vxx;
+    double v, hvx, h2vxx, S[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) S[c] = r.mul(h, N[c]);
 #ifdef CGKS_OPCOUNT_HOST
     linear_recon_rk<ORDER>(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], v, hvx, h2vxx);
 #else
@@ -219,14 +221,14 @@ __device__ __forceinline__ void char_basis(const RegK& r, double gamma, const do
 // w[0..3]: left and right value, left and right slope.
 template <int ORDER>
 __device__ __forceinline__ void char_field(const RegK& r, const CharState& cs, double rho, int m, const double Qa[4][4],
-                                           const double Sa[4][4], double ih, double weno_eps, double w[4])
+                                           const double Na[4][4], double h, double ih, double weno_eps, double w[4])
 {
     double l[4], Q[4], S[4];
     char_left_row(r, cs, m, l);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
-        S[c] = char_project(r, m, l, Sa[0][c], Sa[1][c], Sa[2][c], Sa[3][c]);
+        S[c] = r.mul(h, char_project(r, m, l, Na[0][c], Na[1][c], Na[2][c], Na[3][c]));
     }
 #ifdef CGKS_OPCOUNT_HOST
     weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, w[0], w[2], w[1], w[3]);
@@ -241,15 +243,15 @@ __device__ __forceinline__ void char_field(const RegK& r, const CharState& cs, d
 }
 
 // The arithmetic of one record in characteristic variables by one thread: all four
-// variables from the stencil cells' values Qa[var][cell] and h times normal gradients
-// Sa[var][cell] (face frame), written through out(field, k, value).  (The record kernel
+// variables from the stencil cells' values Qa[var][cell] and normal gradients
+// Na[var][cell] (face frame), written through out(field, k, value).  (The record kernel
 // gives each field a lane of its own, the same operations.)
 template <int ORDER, class Out>
-__device__ __forceinline__ void char_record(const RegK& r, double gamma, const double Qa[4][4], const double Sa[4][4],
-                                            double ih, double weno_eps, bool inner, Out out)
+__device__ __forceinline__ void char_record(const RegK& r, double gamma, const double Qa[4][4], const double Na[4][4],
+                                            double h, double ih, double weno_eps, bool inner, Out out)
 {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) linear_fields<ORDER>(r, Qa[k], Sa[k], ih, k, out);
+    for (int k = 0; k < 4; ++k) linear_fields<ORDER>(r, Qa[k], Na[k], h, ih, k, out);
     if (!inner) return;
     CharState cs;
     double rho, w[4][4], o4[4];
@@ -257,7 +259,7 @@ __device__ __forceinline__ void char_record(const RegK& r, double gamma, const d
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         double v[4];
-        char_field<ORDER>(r, cs, rho, m, Qa, Sa, ih, weno_eps, v);
+        char_field<ORDER>(r, cs, rho, m, Qa, Na, h, ih, weno_eps, v);
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[q][m] = v[q];
     }
@@ -312,8 +314,8 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
 }
 
 // the stencil cells of a row, all four variables in the face frame
-__device__ __forceinline__ void char_stencil(const RegK& r, const GridDev& G, const double* src, size_t PL,
-                                             const RowRef& q, double Qa[4][4], double Sa[4][4])
+__device__ __forceinline__ void char_stencil(const GridDev& G, const double* src, size_t PL,
+                                             const RowRef& q, double Qa[4][4], double Na[4][4])
 {
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
@@ -322,7 +324,7 @@ __device__ __forceinline__ void char_stencil(const RegK& r, const GridDev& G, co
         for (int c = 0; c < 4; ++c) {
             const int i = q.i0 + c * q.di, j = q.j0 + c * q.dj;
             Qa[kk][c] = cell_value(G, src, PL, i, j, pk);
-            Sa[kk][c] = r.mul(q.h, cell_value(G, src, PL, i, j, q.gn + pk));
+            Na[kk][c] = cell_value(G, src, PL, i, j, q.gn + pk);
         }
     }
 }
@@ -335,11 +337,11 @@ __device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const 
 {
     const RowRef q = row_ref(G, row);
     if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
-    double Qa[4][4], Sa[4][4];
-    char_stencil(r, G, src, PL, q, Qa, Sa);
+    double Qa[4][4], Na[4][4];
+    char_stencil(G, src, PL, q, Qa, Na);
     double* o = q.base + q.idx;
     const size_t st = q.stride;
-    char_record<ORDER>(r, G.gamma, Qa, Sa, q.ih, G.weno_eps, q.inner,
+    char_record<ORDER>(r, G.gamma, Qa, Na, q.h, q.ih, G.weno_eps, q.inner,
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
 
@@ -355,21 +357,21 @@ __device__ __forceinline__ void char_row_quad(const RegK& r, const GridDev& G, c
 {
     const RowRef q = row_ref(G, row);
     if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
-    double Qa[4][4], Sa[4][4], Qm[4], Sm[4];
-    char_stencil(r, G, src, PL, q, Qa, Sa);
+    double Qa[4][4], Na[4][4], Qm[4], Nm[4];
+    char_stencil(G, src, PL, q, Qa, Na);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         Qm[c] = m == 0 ? Qa[0][c] : m == 1 ? Qa[1][c] : m == 2 ? Qa[2][c] : Qa[3][c];
-        Sm[c] = m == 0 ? Sa[0][c] : m == 1 ? Sa[1][c] : m == 2 ? Sa[2][c] : Sa[3][c];
+        Nm[c] = m == 0 ? Na[0][c] : m == 1 ? Na[1][c] : m == 2 ? Na[2][c] : Na[3][c];
     }
     double* o = q.base + q.idx;
     const size_t st = q.stride;
-    linear_fields<ORDER>(r, Qm, Sm, q.ih, m, [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
+    linear_fields<ORDER>(r, Qm, Nm, q.h, q.ih, m, [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
     if (!q.inner) return;                     // the same for the quad's lanes (one row)
     CharState cs;
     double rho, w[4], t[4], o4[4];
     char_basis(r, G.gamma, Qa, rho, cs);
-    char_field<ORDER>(r, cs, rho, m, Qa, Sa, q.ih, G.weno_eps, w);
+    char_field<ORDER>(r, cs, rho, m, Qa, Na, q.h, q.ih, G.weno_eps, w);
     // t[j] = field j of quantity m: step s sends quantity m ^ s to lane m ^ s
 #pragma unroll
     for (int s = 0; s < 4; ++s) {

@@ -37,9 +37,14 @@ struct StageLayout {
     static constexpr int NF = FaceQ<STAGE>::n;
     static constexpr int n_rx = RecGroups<TY, TX + 1>::n;
     static constexpr int n_ry = RecGroups<TX, TY + 1>::n;
+    static constexpr int n_rec = n_rx + n_ry;
     // a slice per pair of threads: what the two Gauss points of its segment share
     static constexpr int n_parts = 48 * kPairs;
-    static constexpr size_t bytes = sizeof(double) * (size_t)(n_rx + n_ry + n_parts);
+    // record buffers: two where the shape's CTAs still fit an SM (static shared memory and
+    // the 1 KB the system takes per CTA included)
+    static constexpr int buffers =
+        stage_ctas(TX, TY) * (sizeof(double) * (size_t)(2 * n_rec + n_parts) + 2560) <= 228 * 1024 ? 2 : 1;
+    static constexpr size_t bytes = sizeof(double) * (size_t)(buffers * n_rec + n_parts);
 };
 
 // The quartic through the segment means m_{j-2..j+2} (m0 the centre row): with A1 = m_1 -
@@ -60,8 +65,8 @@ __device__ __forceinline__ double quartic_tt1(const RegK& r, const TangDiffs& x)
 // j-2..j+2 of one face) and the reconstruction along the face there.  The
 // segment's slice (segment_parts; part j of variable k at part[(kPartsVar k + j)
 // * stride]) holds what its two Gauss points share.
-// Parts of a variable: W0, its tangential slope per unit eta and its normal derivative at
-// eta = -g and +g; the slopes of W_l and W_r; as pairs of FP32 what the second derivatives
+// Parts of a variable: W0, twice its tangential slope per unit eta and its normal derivative
+// at eta = -g and +g; twice the slopes of W_l and W_r; as pairs of FP32 what the second derivatives
 // need (d2/deta2 = PTT0 + eta PTT1, d2/dn deta = PNT0 + eta PNT1; the host operation
 // count keeps them in FP64).
 enum { PV = 0, PT = 2, PN = 4, PS = 6, PTT0 = 8, PTT1, PNT0, PNT1, kPartsVar, kParts = 4 * kPartsVar };
@@ -71,7 +76,7 @@ struct SegmentPoint {
     RegK r;
     const double* rec;
     int pa, pb, pc, r0, rstride;
-    double eta, iht;
+    double eta, iht, hiht;        // inverse spacing along the face and its half
     int gp;                       // 0: eta = -g, 1: +g
     const double* part;
     int stride;
@@ -94,7 +99,7 @@ struct SegmentPoint {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             W0n[k] = P(k, PN + gp);
-            W0t[k] = r.mul(P(k, PT + gp), iht);
+            W0t[k] = r.mul(P(k, PT + gp), hiht);
         }
     }
 
@@ -134,8 +139,9 @@ struct SegmentPoint {
     __device__ __forceinline__ void ne_value(int side, double W[4]) const
     {
         const int f = side ? RR : RL;
+        const double heta = r.k(gp ? FK_HG : FK_MHG);   // eta / 2
 #pragma unroll
-        for (int k = 0; k < 4; ++k) W[k] = fma(eta, P(k, PS + side), at(f, k, 0));
+        for (int k = 0; k < 4; ++k) W[k] = fma(heta, P(k, PS + side), at(f, k, 0));
     }
 
     __device__ __forceinline__ void ne_slopes(int side, double Wn[4], double Wt[4]) const
@@ -145,7 +151,7 @@ struct SegmentPoint {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             Wn[k] = fma(he, r.sub(at(f, k, 1), at(f, k, -1)), at(f, k, 0));
-            Wt[k] = r.mul(P(k, PS + side), iht);
+            Wt[k] = r.mul(P(k, PS + side), hiht);
         }
     }
 
@@ -153,7 +159,7 @@ struct SegmentPoint {
     __device__ __forceinline__ void ne_slopes_split(int side, ff Wn[4], ff Wt[4]) const
     {
         const int f = side ? RRN : RLN;
-        const ff he = gp ? CGKS_FF(0.5 * kGauss) : CGKS_FF(-0.5 * kGauss), ih = ff_unpack(r.k(ihp));
+        const ff he = gp ? CGKS_FF(0.5 * kGauss) : CGKS_FF(-0.5 * kGauss), ih = ff_scale(0.5f, ff_unpack(r.k(ihp)));
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             Wn[k] = ff_addp(ff_mul(he, ff_addp(ff_from(at(f, k, 1)), ff_neg(ff_from(at(f, k, -1))))), ff_from(at(f, k, 0)));
@@ -206,10 +212,9 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
                 p[(PV + 1) * stride] = r.kfma(FK_HG, sum(A1, ff_neg(hi)), m0);
                 // the quartic of SegmentPoint: slope A1/2 - ts/12 + eta (s - td/9), second derivative
                 // s - td/12 + eta ts/2, value + eta (A1/2 - 7 ts/72) - td/4320
-                const ff x = ff_mul(m12, v.ts), y = ff_mul(g, ff_sub(v.s, ff_mul(c9, v.td)));
-                const double hA = r.kmul(FK_HALF, A1);
-                p[(PT + 0) * stride] = sum(hA, ff_sub(x, y));
-                p[(PT + 1) * stride] = sum(hA, ff_add(x, y));
+                const ff x = ff_mul(CGKS_FF(-1.0 / 6.0), v.ts), y = ff_mul(CGKS_FF(2.0 * kGauss), ff_sub(v.s, ff_mul(c9, v.td)));
+                p[(PT + 0) * stride] = sum(A1, ff_sub(x, y));
+                p[(PT + 1) * stride] = sum(A1, ff_add(x, y));
                 p[PTT0 * stride] = ff_pack(ff_add(v.s, ff_mul(m12, v.td)));
                 p[PTT1 * stride] = ff_pack(ff_scale(0.5f, v.ts));
                 const QuarticParts n = quartic_split(ff_from(na), ff_from(nb), ff_from(nc), ff_from(nd));
@@ -226,9 +231,9 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
             TangDiffs x;
             tang_diffs(r, R(RV, k, -2), R(RV, k, -1), m0, R(RV, k, 1), R(RV, k, 2), x);
             tang_weno5_pair(r, m0, x, weps4, p[(PV + 0) * stride], p[(PV + 1) * stride]);
-            const double t0 = quartic_t0(r, x), gt = r.mul(kGauss, quartic_t1(r, x));
-            p[(PT + 0) * stride] = r.sub(t0, gt);
-            p[(PT + 1) * stride] = r.add(t0, gt);
+            const double t0 = quartic_t0(r, x), t2 = r.add(t0, t0), gt = r.mul(2.0 * kGauss, quartic_t1(r, x));
+            p[(PT + 0) * stride] = r.sub(t2, gt);
+            p[(PT + 1) * stride] = r.add(t2, gt);
 #ifdef CGKS_OPCOUNT_HOST
             p[PTT0 * stride] = quartic_tt0(r, x);
             p[PTT1 * stride] = quartic_tt1(r, x);
@@ -296,7 +301,8 @@ __device__ __forceinline__ bool segment_results(const RegK& r, const double* rec
     bool ok = true;
 #pragma unroll 1
     for (int gp = 0; gp < 2; ++gp) {
-        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, iht, gp, part, stride, ihp};
+        const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, iht, r.k(xo ? FK_HIDY : FK_HIDX), gp, part,
+                               stride, ihp};
         PointResult<STAGE> o;
         ok &= segment_point<STAGE>(src, o);
 #pragma unroll

@@ -6,7 +6,8 @@
 //
 // One CTA owns a TX x TY tile of cells of one grid and runs, in shared memory:
 //   phase 1  stage the face-row records the tile needs (its faces on its rows
-//            and two rows either side) with asynchronous copies
+//            and two rows either side) with asynchronous copies, for the CTA's
+//            next tile while it works on this one where two buffers fit
 //   phase 2  per face segment the tile owns (the x- and y-faces on the low side
 //            of its cells; the grid's last faces have tiles of their own, so every
 //            face is evaluated once) a pair of lanes.  Together they compute what
@@ -48,13 +49,9 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
     using L = StageLayout<TX, TY, STAGE>;
     constexpr int NF = L::NF;
     extern __shared__ double smem[];
-    double* rx = smem;                  // x-face records, RecGroups<TY, TX+1>
-    double* ry = rx + L::n_rx;          // y-face records, RecGroups<TX, TY+1>
-    double* part = ry + L::n_ry + (threadIdx.x >> 1);   // [kParts][kPairs]: this pair's slice
+    double* part = smem + L::buffers * L::n_rec + (threadIdx.x >> 1);   // [kParts][kPairs]: this pair's slice
     __shared__ double s_fk[FK_N];       // coefficient table (fixed part, then the tile's grid and dt)
     __shared__ int s_skip;
-    // the queue length (a kernel argument, or in device memory for a server's patched queue) is
-    // kept in shared memory: at 255 registers a loop bound in a register costs spills
     const int tid = threadIdx.x;
 
     for (int i = tid; i < FK_NFIX; i += kThreads) s_fk[i] = kFluxFixed.v[i];
@@ -64,65 +61,77 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
 
     wait_previous();
 
-    // the queue length: the kernel argument, or the int in device memory behind dcount (a server's
-    // queue, patched between replays), read at each tile -- at 255 registers a bound kept in a
-    // register through the loop costs spills (5 % of the stage-1 kernel's time)
-    for (int tile = blockIdx.x; tile < (dcount ? *(volatile const int*)dcount : ntiles); tile += gridDim.x) {
-        __syncthreads();
+    // ---------------- phase 1: a tile's face-row records (the record kernel wrote them for
+    // every face row of the grid) into buffer `buf`: x-faces x0..x0+TX on rows y0-2..y0+TY+1,
+    // y-faces y0..y0+TY on columns x0-2..x0+TX+1, each field on the rows it is read on; rows
+    // beyond the grid's last ghost row are zero and unused.  Asynchronous 8-byte copies,
+    // zero-filled where invalid.
+    auto issue = [&](int tile, int buf) {
         const TileRef tr = tiles[tile];
         const GridDev& G = grids[tr.grid];
+        const int nx = G.nx, ny = G.ny, x0 = tr.x0, y0 = tr.y0;
+        const size_t sx = (size_t)(ny + 4) * (nx + 1), sy = (size_t)(nx + 4) * (ny + 1);
+        const unsigned sbx = (unsigned)__cvta_generic_to_shared(smem + buf * L::n_rec), sby = sbx + 8u * L::n_rx;
+        // group g of one orientation: plane p of the group is global plane p0 + p, its
+        // local row q is record row base + q (records carry two ghost rows first)
+        auto stage = [&](unsigned sbase, int sofs, int np, int plane, int F, int p0, const double* g, size_t gs,
+                         int gfaces, int row0, int face0, int nface_max, int row_max, int nsmem) {
+            const int n = np * plane;
+            for (int idx = tid; idx < n; idx += kThreads) {
+                const int p = idx / plane, rem = idx - p * plane;
+                const int q = rem / F, fc = rem - q * F;
+                bool valid = (face0 + fc <= nface_max) && (row0 + q <= row_max);
+                if (!CGKS_IN_BOUNDS(sofs + idx < nsmem, G.ctrl)) continue;
+                if (valid)
+                    valid = CGKS_IN_BOUNDS(row0 + q >= 0 && face0 + fc >= 0 &&
+                                               (size_t)(p0 + p) * gs + (size_t)(row0 + q) * gfaces + face0 + fc <
+                                                   28 * gs,
+                                           G.ctrl);
+                const double* src = valid ? g + (size_t)(p0 + p) * gs + (size_t)(row0 + q) * gfaces + face0 + fc
+                                          : G.recx;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(sbase + 8u * (unsigned)(sofs + idx)),
+                             "l"(src), "r"(valid ? 8 : 0) : "memory");
+            }
+        };
+        using RX = RecGroups<TY, TX + 1>;
+        using RY = RecGroups<TX, TY + 1>;
+        // x-faces: record rows y0 + 2 + (own row); group A starts two rows earlier, B one
+        stage(sbx, 0, 8, RX::pa, TX + 1, 0, G.recx, sx, nx + 1, y0, x0, nx, ny + 3, RX::n);
+        stage(sbx, 8 * RX::pa, 16, RX::pb, TX + 1, 4 * RL, G.recx, sx, nx + 1, y0 + 1, x0, nx, ny + 3, RX::n);
+        stage(sbx, 8 * RX::pa + 16 * RX::pb, 4, RX::pc, TX + 1, 4 * RNN, G.recx, sx, nx + 1, y0 + 2, x0, nx, ny + 3,
+              RX::n);
+        stage(sby, 0, 8, RY::pa, TY + 1, 0, G.recy, sy, ny + 1, x0, y0, ny, nx + 3, RY::n);
+        stage(sby, 8 * RY::pa, 16, RY::pb, TY + 1, 4 * RL, G.recy, sy, ny + 1, x0 + 1, y0, ny, nx + 3, RY::n);
+        stage(sby, 8 * RY::pa + 16 * RY::pb, 4, RY::pc, TY + 1, 4 * RNN, G.recy, sy, ny + 1, x0 + 2, y0, ny, nx + 3,
+              RY::n);
+    };
+    // the queue length: the kernel argument, or the int in device memory behind dcount (a server's
+    // queue, patched between replays), read at each tile
+    auto length = [&] { return dcount ? *(volatile const int*)dcount : ntiles; };
+
+    // with two buffers the next tile's records are copied while this one's are used
+    if (L::buffers == 2 && (int)blockIdx.x < length()) issue(blockIdx.x, 0);
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < length(); tile += gridDim.x) {
+        __syncthreads();                              // the tile before is finished: table and buffer are free
+        const TileRef tr = tiles[tile];
+        const GridDev& G = grids[tr.grid];
+        if (L::buffers == 1) issue(tile, 0);
         if (tid == 0) {
             const Ctrl* C = G.ctrl;
             s_skip = C->done;
             if (!C->done) flux_table_tile(s_fk, G, C->dt);
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
+        const double* rx = smem + buf * L::n_rec;     // x-face records, RecGroups<TY, TX+1>
+        const double* ry = rx + L::n_rx;              // y-face records, RecGroups<TX, TY+1>
+        if (L::buffers == 2) {
+            if (tile + (int)gridDim.x < length()) issue(tile + gridDim.x, buf ^ 1);
+            buf ^= 1;
+        }
         if (s_skip) continue;
         const int nx = G.nx, ny = G.ny, x0 = tr.x0, y0 = tr.y0;
-
-        // ---------------- phase 1: the tile's face-row records (the record kernel
-        // wrote them for every face row of the grid): x-faces x0..x0+TX on rows
-        // y0-2..y0+TY+1, y-faces y0..y0+TY on columns x0-2..x0+TX+1, each field on
-        // the rows it is read on; rows beyond the grid's last ghost row are zero
-        // and unused.  Asynchronous 8-byte copies, zero-filled where invalid.
-        {
-            const size_t sx = (size_t)(ny + 4) * (nx + 1), sy = (size_t)(nx + 4) * (ny + 1);
-            const unsigned sbx = (unsigned)__cvta_generic_to_shared(rx), sby = (unsigned)__cvta_generic_to_shared(ry);
-            // group g of one orientation: plane p of the group is global plane p0 + p, its
-            // local row q is record row base + q (records carry two ghost rows first)
-            auto stage = [&](unsigned sbase, int sofs, int np, int plane, int F, int p0, const double* g, size_t gs,
-                             int gfaces, int row0, int face0, int nface_max, int row_max, int nsmem) {
-                const int n = np * plane;
-                for (int idx = tid; idx < n; idx += kThreads) {
-                    const int p = idx / plane, rem = idx - p * plane;
-                    const int q = rem / F, fc = rem - q * F;
-                    bool valid = (face0 + fc <= nface_max) && (row0 + q <= row_max);
-                    if (!CGKS_IN_BOUNDS(sofs + idx < nsmem, G.ctrl)) continue;
-                    if (valid)
-                        valid = CGKS_IN_BOUNDS(row0 + q >= 0 && face0 + fc >= 0 &&
-                                                   (size_t)(p0 + p) * gs + (size_t)(row0 + q) * gfaces + face0 + fc <
-                                                       28 * gs,
-                                               G.ctrl);
-                    const double* src = valid ? g + (size_t)(p0 + p) * gs + (size_t)(row0 + q) * gfaces + face0 + fc
-                                              : G.recx;
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(sbase + 8u * (unsigned)(sofs + idx)),
-                                 "l"(src), "r"(valid ? 8 : 0) : "memory");
-                }
-            };
-            using RX = RecGroups<TY, TX + 1>;
-            using RY = RecGroups<TX, TY + 1>;
-            // x-faces: record rows y0 + 2 + (own row); group A starts two rows earlier, B one
-            stage(sbx, 0, 8, RX::pa, TX + 1, 0, G.recx, sx, nx + 1, y0, x0, nx, ny + 3, RX::n);
-            stage(sbx, 8 * RX::pa, 16, RX::pb, TX + 1, 4 * RL, G.recx, sx, nx + 1, y0 + 1, x0, nx, ny + 3, RX::n);
-            stage(sbx, 8 * RX::pa + 16 * RX::pb, 4, RX::pc, TX + 1, 4 * RNN, G.recx, sx, nx + 1, y0 + 2, x0, nx, ny + 3,
-                  RX::n);
-            stage(sby, 0, 8, RY::pa, TY + 1, 0, G.recy, sy, ny + 1, x0, y0, ny, nx + 3, RY::n);
-            stage(sby, 8 * RY::pa, 16, RY::pb, TY + 1, 4 * RL, G.recy, sy, ny + 1, x0 + 1, y0, ny, nx + 3, RY::n);
-            stage(sby, 8 * RY::pa + 16 * RY::pb, 4, RY::pc, TY + 1, 4 * RNN, G.recy, sy, ny + 1, x0 + 2, y0, ny, nx + 3,
-                  RY::n);
-            asm volatile("cp.async.wait_all;" ::: "memory");
-        }
-        __syncthreads();
 
         // ---------------- phase 2: face segments, two Gauss points each
         bool bad = false;
@@ -161,8 +170,8 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
             // the pair's lanes compute two variables' parts each, then a Gauss point each
             segment_parts(r, rec, pa, pb, pc, r0, rstride, r.k(xo ? FK_IDX : FK_IDY), 2 * gp, 2 * gp + 2, part, kPairs);
             __syncwarp(pair);
-            const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, r.k(xo ? FK_IDY : FK_IDX), gp, part,
-                                   kPairs, xo ? FK_PIDY : FK_PIDX};
+            const SegmentPoint src{r, rec, pa, pb, pc, r0, rstride, gp ? kGauss : -kGauss, r.k(xo ? FK_IDY : FK_IDX),
+                                   r.k(xo ? FK_HIDY : FK_HIDX), gp, part, kPairs, xo ? FK_PIDY : FK_PIDX};
             PointResult<STAGE> o;
             bad |= !segment_point<STAGE>(src, o);
             // each lane averages and writes two variables: the other lane's sums for them come by
