@@ -313,18 +313,35 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
 
-// the stencil cells of a row, all four variables in the face frame
-__device__ __forceinline__ void char_stencil(const GridDev& G, const double* src, size_t PL,
-                                             const RowRef& q, double Qa[4][4], double Na[4][4])
+// the stencil cells of a row, all four variables in the face frame.  Outside the grid the
+// boundary mapping is one per cell, not per value: 32 copies of it (cell_value) outgrew the
+// instruction cache (200x50: half of the warps' time went to waiting for instructions).
+__device__ __forceinline__ void char_stencil(const GridDev& G, const double* src, size_t PL, const RowRef& q,
+                                             double Qa[4][4], double Na[4][4])
 {
+    const int i3 = q.i0 + 3 * q.di, j3 = q.j0 + 3 * q.dj;
+    const int p1 = q.xo ? 1 : 2, p2 = q.xo ? 2 : 1;         // planes of the normal and tangential momentum
+    const bool inside = q.i0 >= 0 && q.j0 >= 0 && i3 < G.nx && j3 < G.ny;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        const int pk = q.xo ? kk : ((kk == 1) ? 2 : (kk == 2) ? 1 : kk);
+    for (int c = 0; c < 4; ++c) {
+        const int i = q.i0 + c * q.di, j = q.j0 + c * q.dj;
+        int kx = 0, ky = 0, si = i, sj = j;
+        if (!inside) {
+            si = map_axis(i, G.nx, G.bc[0], G.bc[1], kx);
+            sj = map_axis(j, G.ny, G.bc[2], G.bc[3], ky);
+            if (!CGKS_IN_BOUNDS(si >= 0 && si < G.nx && sj >= 0 && sj < G.ny, G.ctrl)) si = sj = 0;
+        }
+        const double* v = src + (size_t)sj * G.nx + si;
+        const double* n = v + (size_t)q.gn * PL;
+        Qa[0][c] = v[0]; Qa[1][c] = v[p1 * PL]; Qa[2][c] = v[p2 * PL]; Qa[3][c] = v[3 * PL];
+        Na[0][c] = n[0]; Na[1][c] = n[p1 * PL]; Na[2][c] = n[p2 * PL]; Na[3][c] = n[3 * PL];
+        if (kx | ky) {
+            const int pk[4] = {0, p1, p2, 3};
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int i = q.i0 + c * q.di, j = q.j0 + c * q.dj;
-            Qa[kk][c] = cell_value(G, src, PL, i, j, pk);
-            Na[kk][c] = cell_value(G, src, PL, i, j, q.gn + pk);
+            for (int k = 0; k < 4; ++k) {
+                Qa[k][c] = bc_value(G, Qa[k][c], i, j, kx, ky, pk[k]);
+                Na[k][c] = bc_value(G, Na[k][c], i, j, kx, ky, q.gn + pk[k]);
+            }
         }
     }
 }
