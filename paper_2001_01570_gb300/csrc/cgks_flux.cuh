@@ -72,48 +72,76 @@ constexpr FluxFixed make_flux_fixed()
     return t;
 }
 
-// per-tile entries of the table for a grid and its time step
+// the table's entries for a grid and its time step, in four parts of about equal length
+// for a warp each (one thread's chain took 4,300 cycles, the longest part's takes a third)
+__device__ __forceinline__ void flux_table_part(double* t, const GridDev& G, double dt, int part)
+{
+    if (part == 0) {
+        t[FK_DT] = dt;
+        t[FK_HDT] = 0.5 * dt;
+        t[FK_MHDT] = -0.5 * dt;
+        t[FK_EPSDT] = G.eps_tau * dt;
+        t[FK_CTAUDT] = G.c_tau * dt;
+        t[FK_C8] = 0.125 * dt * dt;
+        // stage 1: half of (dt/2, dt^2/8) and of (dt, dt^2/6) per Gauss point; stage 2: half of dt^2/3
+        t[FK_W1A] = 0.25 * dt;
+        t[FK_W1B] = dt * dt * (1.0 / 16.0);
+        t[FK_W2A] = 0.5 * dt;
+        t[FK_W2B] = dt * dt * (1.0 / 12.0);
+        t[FK_W3] = dt * dt * (1.0 / 6.0);
+    } else if (part == 1) {
+        t[FK_IDT] = __drcp_rn(dt);
+        t[FK_4IDT2] = 4.0 * __drcp_rn(dt * dt);
+        t[FK_GAMMA] = G.gamma;
+        t[FK_MU] = G.mu;
+        t[FK_IDX] = G.inv_dx;
+        t[FK_IDY] = G.inv_dy;
+        t[FK_HIDX] = 0.5 * G.inv_dx;
+        t[FK_HIDY] = 0.5 * G.inv_dy;
+    } else if (part == 2) {
+        t[FK_C6] = dt * dt / 6.0;
+        t[FK_GM1] = G.gamma - 1.0;
+        t[FK_K1] = G.K + 1.0;
+        t[FK_K3] = G.K + 3.0;
+        t[FK_K2INV2] = 2.0 * __drcp_rn(G.K + 2.0);
+        t[FK_KHEAT] = 0.5 * (G.K + 4.0);
+        t[FK_WEPS] = G.weno_eps;
+        t[FK_WEPS4] = 4.0 * G.weno_eps;
+    } else {
+#ifndef CGKS_OPCOUNT_HOST
+        t[FK_PGAMMA] = ff_pack(ff_from(G.gamma));
+        t[FK_PGM1] = ff_pack(ff_from(G.gamma - 1.0));
+        t[FK_PK1] = ff_pack(ff_from(G.K + 1.0));
+        t[FK_PK3] = ff_pack(ff_from(G.K + 3.0));
+        t[FK_PIDX] = ff_pack(ff_from(G.inv_dx));
+        t[FK_PIDY] = ff_pack(ff_from(G.inv_dy));
+        t[FK_PWEPS] = ff_pack(ff_from(G.weno_eps));
+        t[FK_PWEPS4] = ff_pack(ff_from(4.0 * G.weno_eps));
+#endif
+    }
+}
+
 __device__ __forceinline__ void flux_table_tile(double* t, const GridDev& G, double dt)
 {
-    t[FK_DT] = dt;
-    t[FK_IDT] = __drcp_rn(dt);
-    t[FK_4IDT2] = 4.0 * __drcp_rn(dt * dt);
-    t[FK_HDT] = 0.5 * dt;
-    t[FK_MHDT] = -0.5 * dt;
-    t[FK_EPSDT] = G.eps_tau * dt;
-    t[FK_CTAUDT] = G.c_tau * dt;
-    t[FK_C8] = 0.125 * dt * dt;
-    t[FK_C6] = dt * dt / 6.0;
-    // stage 1: half of (dt/2, dt^2/8) and of (dt, dt^2/6) per Gauss point; stage 2: half of dt^2/3
-    t[FK_W1A] = 0.25 * dt;
-    t[FK_W1B] = dt * dt * (1.0 / 16.0);
-    t[FK_W2A] = 0.5 * dt;
-    t[FK_W2B] = dt * dt * (1.0 / 12.0);
-    t[FK_W3] = dt * dt * (1.0 / 6.0);
-    t[FK_GAMMA] = G.gamma;
-    t[FK_GM1] = G.gamma - 1.0;
-    t[FK_K1] = G.K + 1.0;
-    t[FK_K3] = G.K + 3.0;
-    t[FK_K2INV2] = 2.0 * __drcp_rn(G.K + 2.0);
-    t[FK_KHEAT] = 0.5 * (G.K + 4.0);
-    t[FK_MU] = G.mu;
-    t[FK_IDX] = G.inv_dx;
-    t[FK_IDY] = G.inv_dy;
-    t[FK_HIDX] = 0.5 * G.inv_dx;
-    t[FK_HIDY] = 0.5 * G.inv_dy;
-    t[FK_WEPS] = G.weno_eps;
-    t[FK_WEPS4] = 4.0 * G.weno_eps;
-#ifndef CGKS_OPCOUNT_HOST
-    t[FK_PGAMMA] = ff_pack(ff_from(G.gamma));
-    t[FK_PGM1] = ff_pack(ff_from(t[FK_GM1]));
-    t[FK_PK1] = ff_pack(ff_from(t[FK_K1]));
-    t[FK_PK3] = ff_pack(ff_from(t[FK_K3]));
-    t[FK_PIDX] = ff_pack(ff_from(G.inv_dx));
-    t[FK_PIDY] = ff_pack(ff_from(G.inv_dy));
-    t[FK_PWEPS] = ff_pack(ff_from(G.weno_eps));
-    t[FK_PWEPS4] = ff_pack(ff_from(t[FK_WEPS4]));
-#endif
+    for (int part = 0; part < 4; ++part) flux_table_part(t, G, dt, part);
 }
+
+#ifndef CGKS_OPCOUNT_HOST
+// The table for the grid of a CTA's next tile (four warps, between two barriers): `held` is
+// the grid that it holds.  dt and `done` are fixed for the launch, so consecutive tiles of one
+// grid share it; made anew for each tile it took the first warp, and with it one of the SM's four
+// FP64 units, 75 instructions beside the some 800 of a tile's fluxes.
+__device__ __forceinline__ void flux_table_grid(double* t, const GridDev& G, int grid, int& held, int& skip)
+{
+    if (grid == held) return;
+    held = grid;
+    if (threadIdx.x & 31) return;
+    const Ctrl* C = G.ctrl;
+    const int done = C->done;
+    if (threadIdx.x == 0) skip = done;
+    if (!done) flux_table_part(t, G, C->dt, (int)(threadIdx.x >> 5));
+}
+#endif
 
 // ------------------------------------------------------------------------
 // Nonlinear point values along a face (2D): WENO-Z over the line averages of

@@ -111,17 +111,13 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
 
     // with two buffers the next tile's records are copied while this one's are used
     if (L::buffers == 2 && (int)blockIdx.x < length()) issue(blockIdx.x, 0);
-    int buf = 0;
+    int buf = 0, held = -1;
     for (int tile = blockIdx.x; tile < length(); tile += gridDim.x) {
         __syncthreads();                              // the tile before is finished: table and buffer are free
         const TileRef tr = tiles[tile];
         const GridDev& G = grids[tr.grid];
         if (L::buffers == 1) issue(tile, 0);
-        if (tid == 0) {
-            const Ctrl* C = G.ctrl;
-            s_skip = C->done;
-            if (!C->done) flux_table_tile(s_fk, G, C->dt);
-        }
+        flux_table_grid(s_fk, G, tr.grid, held, s_skip);
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         const double* rx = smem + buf * L::n_rec;     // x-face records, RecGroups<TY, TX+1>

@@ -104,15 +104,12 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
     __syncthreads();
     const RegK r{s_fk, ((volatile const double*)s_fk)[FK_ONE], ((volatile const double*)s_fk)[FK_NZERO]};
     wait_previous();
+    int held = -1;
     for (int tile = blockIdx.x; tile < (dcount ? *(volatile const int*)dcount : ntiles); tile += gridDim.x) {
         __syncthreads();
         const TileRef tr = tiles[tile];
         const GridDev& G = grids[tr.grid];
-        if (tid == 0) {
-            const Ctrl* C = G.ctrl;
-            s_skip = C->done;
-            if (!C->done) flux_table_tile(s_fk, G, C->dt);
-        }
+        flux_table_grid(s_fk, G, tr.grid, held, s_skip);
         __syncthreads();
         if (s_skip) continue;
         const int face = tr.x0 + (tid >> 1), nx = G.nx;

@@ -24,9 +24,24 @@ __device__ __forceinline__ void update_cell_core(const GridDev& G, int par, size
     const size_t PL = (size_t)G.nx * G.ny;
     double* rbuf = G.buf[par ^ 1];
     const double idx_ = G.inv_dx, idy_ = G.inv_dy;
+    // a variable's face results are all read before its first output is written: the compiler
+    // keeps a read that follows a write where it is, one memory latency each
+    constexpr int NQ = STAGE == 1 ? 4 : 2;
+    double x[NQ][2], y[NQ][2];
+    int k0 = 0;
+    auto read = [&](int k) {
+        k0 = k;
+#pragma unroll
+        for (int n = 0; n < NQ; ++n)
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                x[n][s] = FX(4 * n + k, s);
+                y[n][s] = FY(4 * n + k, s);
+            }
+    };
     // high - low of face result q along x and y
-    auto dX = [&](int q) { return __dsub_rn(FX(q, 1), FX(q, 0)); };
-    auto dY = [&](int q) { return __dsub_rn(FY(q, 1), FY(q, 0)); };
+    auto dX = [&](int q) { return __dsub_rn(x[(q - k0) / 4][1], x[(q - k0) / 4][0]); };
+    auto dY = [&](int q) { return __dsub_rn(y[(q - k0) / 4][1], y[(q - k0) / 4][0]); };
     // a - dX/h_x - dY/h_y
     auto div = [&](double a, int q) { return fma(-dY(q), idy_, fma(-dX(q), idx_, a)); };
     if (STAGE == 1) {
@@ -34,6 +49,7 @@ __device__ __forceinline__ void update_cell_core(const GridDev& G, int par, size
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const double W = src[k * PL + off];
+            read(k);
             ws_out(k, div(W, k));
             ws_out(4 + k, __dmul_rn(dX(8 + k), idx_));
             ws_out(8 + k, __dmul_rn(dY(8 + k), idy_));
@@ -45,11 +61,12 @@ __device__ __forceinline__ void update_cell_core(const GridDev& G, int par, size
         double Wn[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const double R = rbuf[k * PL + off];
+            const double R = rbuf[k * PL + off], Rx = rbuf[(4 + k) * PL + off], Ry = rbuf[(8 + k) * PL + off];
+            read(k);
             Wn[k] = div(R, k);
             rbuf[k * PL + off] = Wn[k];
-            rbuf[(4 + k) * PL + off] = fma(dX(4 + k), idx_, rbuf[(4 + k) * PL + off]);
-            rbuf[(8 + k) * PL + off] = fma(dY(4 + k), idy_, rbuf[(8 + k) * PL + off]);
+            rbuf[(4 + k) * PL + off] = fma(dX(4 + k), idx_, Rx);
+            rbuf[(8 + k) * PL + off] = fma(dY(4 + k), idy_, Ry);
         }
         smax.cell(G, Wn[0], Wn[1], Wn[2], Wn[3]);   // for the next step's CFL bound (Sec. 4)
     }
