@@ -38,14 +38,14 @@ __device__ __forceinline__ int map_axis(int i, int n, int bclo, int bchi, int& k
     kind = 0;
     if (i < 0) {
         const int m = -1 - i;
-        if (bclo == CGKS_BC_PERIODIC) { int r = i % n; return r < 0 ? r + n : r; }
+        if (bclo == CGKS_BC_PERIODIC) { int r = i + n; if (r < 0) { r = i % n; r = r < 0 ? r + n : r; } return r; }
         if (bclo == CGKS_BC_REFLECT) { kind = 1; return min(m, n - 1); }
         if (bclo == CGKS_BC_INFLOW) { kind = 2; return 0; }
         kind = 3; return 0;
     }
     if (i >= n) {
         const int m = i - n;
-        if (bchi == CGKS_BC_PERIODIC) return i % n;
+        if (bchi == CGKS_BC_PERIODIC) return m < n ? m : i % n;
         if (bchi == CGKS_BC_REFLECT) { kind = 1; return max(n - 1 - m, 0); }
         if (bchi == CGKS_BC_INFLOW) { kind = 2; return n - 1; }
         kind = 3; return n - 1;

@@ -71,6 +71,45 @@ __device__ __forceinline__ RowRef row_ref(const GridDev& G, int r)
     return q;
 }
 
+// The four stencil cells of a row: where each one's values are read (its source cell inside
+// the grid) and the boundary transforms along x and y.  The index across the row is the same
+// for the four, so it is mapped once, and all of a row's values are read before the first is
+// transformed: mapping and reading value by value (ten, in characteristic mode 32 copies of
+// the mapping, one memory latency each) took 12,000 of a boundary row's 19,000 cycles, and
+// the copies outgrew the instruction cache.
+struct Stencil {
+    size_t at[4];
+    int kn[4], kt;          // transform kinds along and across the row
+    bool ghost;             // some cell lies outside the grid
+    __device__ __forceinline__ int kind(int c) const { return kn[c] | kt; }
+    // plane p of cell c from the value v of its source cell
+    __device__ __forceinline__ double value(const GridDev& G, const RowRef& q, int c, double v, int p) const
+    {
+        return bc_value(G, v, q.i0 + c * q.di, q.j0 + c * q.dj, q.xo ? kn[c] : kt, q.xo ? kt : kn[c], p);
+    }
+};
+
+__device__ __forceinline__ void map_stencil(const GridDev& G, const RowRef& q, Stencil& s)
+{
+    const int i3 = q.i0 + 3 * q.di, j3 = q.j0 + 3 * q.dj;
+    s.ghost = !(q.i0 >= 0 && q.j0 >= 0 && i3 < G.nx && j3 < G.ny);
+    s.kt = 0;
+    const size_t step = q.di ? 1 : (size_t)G.nx, base = (size_t)q.j0 * G.nx + q.i0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) { s.at[c] = base + c * step; s.kn[c] = 0; }
+    if (!s.ghost) return;
+    const int bn = q.xo ? 0 : 2, bt = 2 - bn;           // the axes' boundary conditions
+    const int nn = q.xo ? G.nx : G.ny, nt = q.xo ? G.ny : G.nx;
+    int st = map_axis(q.xo ? q.j0 : q.i0, nt, G.bc[bt], G.bc[bt + 1], s.kt);
+    if (!CGKS_IN_BOUNDS(st >= 0 && st < nt, G.ctrl)) st = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        int sn = map_axis((q.xo ? q.i0 : q.j0) + c, nn, G.bc[bn], G.bc[bn + 1], s.kn[c]);
+        if (!CGKS_IN_BOUNDS(sn >= 0 && sn < nn, G.ctrl)) sn = 0;
+        s.at[c] = q.xo ? (size_t)st * G.nx + sn : (size_t)sn * G.nx + st;
+    }
+}
+
 // Coefficient table of the register-form reconstruction, one block per order
 // (index 0: the 8th-order scheme, 1: the 6th-order variant); copied to shared
 // memory by each CTA.
@@ -281,67 +320,53 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
     if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
     const int pv = q.xo ? k : ((k == 1) ? 2 : (k == 2) ? 1 : k);   // face frame: normal momentum first
     double Q[4], S[4], rho = 0.0, E = 0.0;   // rho, E: cell b's, where a momentum's scale needs them
-    const bool mom = k == 1 || k == 2;
-    const int i3 = q.i0 + 3 * q.di, j3 = q.j0 + 3 * q.dj;
-    if (q.i0 >= 0 && q.j0 >= 0 && i3 < G.nx && j3 < G.ny) {
-        // stencil inside the grid: no boundary mapping
-        const double* v = src + (size_t)pv * PL + (size_t)q.j0 * G.nx + q.i0;
-        const double* d = src + (size_t)(q.gn + pv) * PL + (size_t)q.j0 * G.nx + q.i0;
-        const size_t step = q.di ? 1 : (size_t)G.nx;
+    Stencil c4;
+    map_stencil(G, q, c4);
+    const double *v = src + (size_t)pv * PL, *d = src + (size_t)(q.gn + pv) * PL;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) { Q[c] = v[c * step]; S[c] = r.mul(q.h, d[c * step]); }
-        if (mom && q.inner) {
-            const double* b = src + (size_t)q.j0 * G.nx + q.i0 + step;
-            rho = b[0];
-            E = b[3 * PL];
-        }
-    } else {
+    for (int c = 0; c < 4; ++c) { Q[c] = v[c4.at[c]]; S[c] = d[c4.at[c]]; }
+    const bool mom = (k == 1 || k == 2) && q.inner;
+    if (mom) { rho = src[c4.at[1]]; E = src[3 * PL + c4.at[1]]; }
+    if (c4.ghost) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const int i = q.i0 + c * q.di, j = q.j0 + c * q.dj;
-            Q[c] = cell_value(G, src, PL, i, j, pv);
-            S[c] = r.mul(q.h, cell_value(G, src, PL, i, j, q.gn + pv));
+            if (!c4.kind(c)) continue;
+            Q[c] = c4.value(G, q, c, Q[c], pv);
+            S[c] = c4.value(G, q, c, S[c], q.gn + pv);
         }
-        if (mom && q.inner) {
-            rho = cell_value(G, src, PL, q.i0 + q.di, q.j0 + q.dj, 0);
-            E = cell_value(G, src, PL, q.i0 + q.di, q.j0 + q.dj, 3);
-        }
+        if (mom && c4.kind(1)) { rho = c4.value(G, q, 1, rho, 0); E = c4.value(G, q, 1, E, 3); }
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) S[c] = r.mul(q.h, S[c]);
     double* o = q.base + q.idx;
     const size_t st = q.stride;
     cons_record<ORDER>(r, Q, S, q.ih, G.weno_eps, q.inner, k, scale_of(k, Q[1], Q[2], rho, E),
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
 
-// the stencil cells of a row, all four variables in the face frame.  Outside the grid the
-// boundary mapping is one per cell, not per value: 32 copies of it (cell_value) outgrew the
-// instruction cache (200x50: half of the warps' time went to waiting for instructions).
+// the stencil cells of a row, all four variables in the face frame
 __device__ __forceinline__ void char_stencil(const GridDev& G, const double* src, size_t PL, const RowRef& q,
                                              double Qa[4][4], double Na[4][4])
 {
-    const int i3 = q.i0 + 3 * q.di, j3 = q.j0 + 3 * q.dj;
     const int p1 = q.xo ? 1 : 2, p2 = q.xo ? 2 : 1;         // planes of the normal and tangential momentum
-    const bool inside = q.i0 >= 0 && q.j0 >= 0 && i3 < G.nx && j3 < G.ny;
+    Stencil c4;
+    map_stencil(G, q, c4);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const int i = q.i0 + c * q.di, j = q.j0 + c * q.dj;
-        int kx = 0, ky = 0, si = i, sj = j;
-        if (!inside) {
-            si = map_axis(i, G.nx, G.bc[0], G.bc[1], kx);
-            sj = map_axis(j, G.ny, G.bc[2], G.bc[3], ky);
-            if (!CGKS_IN_BOUNDS(si >= 0 && si < G.nx && sj >= 0 && sj < G.ny, G.ctrl)) si = sj = 0;
-        }
-        const double* v = src + (size_t)sj * G.nx + si;
+        const double* v = src + c4.at[c];
         const double* n = v + (size_t)q.gn * PL;
         Qa[0][c] = v[0]; Qa[1][c] = v[p1 * PL]; Qa[2][c] = v[p2 * PL]; Qa[3][c] = v[3 * PL];
         Na[0][c] = n[0]; Na[1][c] = n[p1 * PL]; Na[2][c] = n[p2 * PL]; Na[3][c] = n[3 * PL];
-        if (kx | ky) {
-            const int pk[4] = {0, p1, p2, 3};
+    }
+    if (!c4.ghost) return;
+    const int pk[4] = {0, p1, p2, 3};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                Qa[k][c] = bc_value(G, Qa[k][c], i, j, kx, ky, pk[k]);
-                Na[k][c] = bc_value(G, Na[k][c], i, j, kx, ky, q.gn + pk[k]);
-            }
+    for (int c = 0; c < 4; ++c) {
+        if (!c4.kind(c)) continue;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            Qa[k][c] = c4.value(G, q, c, Qa[k][c], pk[k]);
+            Na[k][c] = c4.value(G, q, c, Na[k][c], q.gn + pk[k]);
         }
     }
 }
