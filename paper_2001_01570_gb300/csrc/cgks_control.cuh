@@ -11,7 +11,8 @@ namespace cgks {
 // current state, clipped so that t does not pass t_end; marks a grid that is finished.  A
 // function of the control block alone that it leaves valid: running it again before the
 // step gives the same dt.
-__device__ __forceinline__ void begin_step(const GridDev& G, volatile Ctrl* C)
+template <class C_>
+__device__ __forceinline__ void begin_step(const GridDev& G, C_* C)
 {
     if (C->done) return;
     if (C->status) { C->done = 1; return; }
@@ -26,13 +27,27 @@ __device__ __forceinline__ void begin_step(const GridDev& G, volatile Ctrl* C)
 }
 
 // End of a step: the new state becomes current unless a kernel raised an error.
-__device__ __forceinline__ void end_step(volatile Ctrl* C)
+template <class C_>
+__device__ __forceinline__ void end_step(C_* C)
 {
     if (C->done) return;
     if (C->status) { C->done = 1; return; }
     C->par ^= 1;
     C->t += C->dt;
     C->steps += 1;
+}
+
+// The end of a step and the start of the next, the control block read once: as field after
+// field between their branches the reads took a memory latency each (with the rest of the last
+// chunk's end 9,400 cycles).
+__device__ __forceinline__ void turn_step(const GridDev& G, volatile Ctrl* C)
+{
+    Ctrl c;
+    c.dt = C->dt; c.t = C->t; c.t_end = C->t_end; c.amax_bits[0] = C->amax_bits[0]; c.amax_bits[1] = C->amax_bits[1];
+    c.status = C->status; c.done = C->done; c.par = C->par; c.steps = C->steps; c.steps_target = C->steps_target;
+    end_step(&c);
+    begin_step(G, &c);
+    C->dt = c.dt; C->t = c.t; C->status = c.status; C->done = c.done; C->par = c.par; C->steps = c.steps;
 }
 
 // A warp's speed maxima into the grid's control block (positive doubles compare as their
@@ -42,7 +57,10 @@ __device__ __forceinline__ void speed_max_warp(Ctrl* C, SpeedMax& s)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int d = 0; d < 2; ++d) s.a[d] = fmax(s.a[d], __shfl_xor_sync(0xffffffffu, s.a[d], o));
+        for (int d = 0; d < 2; ++d) {   // as integers, off the FP64 unit
+            const long long v = __double_as_longlong(s.a[d]);
+            s.a[d] = __longlong_as_double(max(v, __shfl_xor_sync(0xffffffffu, v, o)));
+        }
     if ((threadIdx.x & 31) == 0)
 #pragma unroll
         for (int d = 0; d < 2; ++d) {

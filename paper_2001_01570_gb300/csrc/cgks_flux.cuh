@@ -31,7 +31,7 @@ enum FluxK {
     FK_X32LN2, FK_SHIFT, FK_LN2HI, FK_LN2LO,         // exponential: argument reduction
     FK_P2, FK_P3, FK_P4, FK_P5, FK_P6,               // exponential: 1/k! of the Taylor polynomial
     FK_NFIX,
-    FK_EXP2 = FK_NFIX,                               // 2^(j/32), j = 0..31 (computed per CTA)
+    FK_EXP2 = FK_NFIX,                               // 2^(j/32), j = 0..31
     FK_NFIX2 = FK_EXP2 + 32,
     // per grid and tile
     FK_DT = FK_NFIX2, FK_IDT, FK_4IDT2, FK_HDT, FK_MHDT, FK_EPSDT, FK_CTAUDT, FK_C8, FK_C6,
@@ -47,7 +47,7 @@ enum FluxK {
 constexpr double kTangLo = (7.0 / 36.0 - 1.7320508075688772 / 1080.0) * (18.0 / 11.0);
 constexpr double kTangHi = (7.0 / 36.0 + 1.7320508075688772 / 1080.0) * (18.0 / 11.0);
 
-struct FluxFixed { double v[FK_NFIX]; };
+struct FluxFixed { double v[FK_NFIX2]; };
 
 constexpr FluxFixed make_flux_fixed()
 {
@@ -69,6 +69,16 @@ constexpr FluxFixed make_flux_fixed()
     k[FK_LN2LO] = 2.3190468138462996e-17 / 32.0;
     k[FK_P2] = 1.0 / 2.0; k[FK_P3] = 1.0 / 6.0; k[FK_P4] = 1.0 / 24.0; k[FK_P5] = 1.0 / 120.0;
     k[FK_P6] = 1.0 / 720.0;
+    const double e2[32] = {                                // 2^(j/32)
+        1.0, 1.0218971486541166, 1.0442737824274138, 1.0671404006768237,
+        1.0905077326652577, 1.1143867425958924, 1.1387886347566916, 1.1637248587775775,
+        1.189207115002721, 1.215247359980469, 1.241857812073484, 1.2690509571917332,
+        1.2968395546510096, 1.3252366431597413, 1.3542555469368927, 1.383909881963832,
+        1.4142135623730951, 1.4451808069770467, 1.4768261459394993, 1.5091644275934228,
+        1.5422108254079407, 1.5759808451078865, 1.6104903319492543, 1.6457554781539649,
+        1.681792830507429, 1.7186192981224779, 1.7562521603732995, 1.7947090750031072,
+        1.8340080864093424, 1.8741676341103, 1.9152065613971474, 1.9571441241754002};
+    for (int j = 0; j < 32; ++j) k[FK_EXP2 + j] = e2[j];
     return t;
 }
 

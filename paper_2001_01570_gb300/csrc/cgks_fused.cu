@@ -12,8 +12,8 @@
 
 namespace cgks {
 
-static __constant__ FluxFixed kFusedFluxFixed = make_flux_fixed();
-static __constant__ ReconTab kFusedReconTab = make_recon_tab();
+static __device__ const FluxFixed kFusedFluxFixed = make_flux_fixed();
+static __device__ const ReconTab kFusedReconTab = make_recon_tab();
 
 template <int TX, int TY>
 __global__ void __launch_bounds__(kFusedThreads, 1)
@@ -25,8 +25,7 @@ fused_step_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__
     __shared__ double s_rk[2 * RK_N];
     __shared__ int s_skip;
     const int tid = threadIdx.x;
-    for (int i = tid; i < FK_NFIX; i += kFusedThreads) s_fk[i] = kFusedFluxFixed.v[i];
-    if (tid < 32) s_fk[FK_EXP2 + tid] = exp2((double)tid * (1.0 / 32.0));
+    for (int i = tid; i < FK_NFIX2; i += kFusedThreads) s_fk[i] = kFusedFluxFixed.v[i];
     for (int i = tid; i < 2 * RK_N; i += kFusedThreads) s_rk[i] = kFusedReconTab.v[i / RK_N][i % RK_N];
     __syncthreads();
     const double one = ((volatile const double*)s_fk)[FK_ONE], nzero = ((volatile const double*)s_fk)[FK_NZERO];

@@ -15,7 +15,8 @@
 
 namespace cgks {
 
-__constant__ ReconTab kReconTab = make_recon_tab();
+// in global memory: lanes that read different words of constant memory are served one by one
+static __device__ const ReconTab kReconTab = make_recon_tab();
 
 // CHAR = 0: conservative variables, one (record, variable) per thread;
 // CHAR = 1: characteristic variables, one (record, field) per lane of a quad.

@@ -39,7 +39,9 @@
 
 namespace cgks {
 
-static __constant__ FluxFixed kFluxFixed = make_flux_fixed();
+// (in global memory: lanes that read different words of constant memory are served one by one, which
+// with 2^(j/32) computed per CTA took 2,300 cycles at the start of every launch)
+static __device__ const FluxFixed kFluxFixed = make_flux_fixed();
 
 template <int TX, int TY, int STAGE>
 __global__ void __launch_bounds__(kThreads, stage_ctas(TX, TY))
@@ -54,8 +56,7 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
     __shared__ int s_skip;
     const int tid = threadIdx.x;
 
-    for (int i = tid; i < FK_NFIX; i += kThreads) s_fk[i] = kFluxFixed.v[i];
-    if (tid < 32) s_fk[FK_EXP2 + tid] = exp2((double)tid * (1.0 / 32.0));
+    for (int i = tid; i < FK_NFIX2; i += kThreads) s_fk[i] = kFluxFixed.v[i];
     __syncthreads();
     const RegK r{s_fk, ((volatile const double*)s_fk)[FK_ONE], ((volatile const double*)s_fk)[FK_NZERO]};
 

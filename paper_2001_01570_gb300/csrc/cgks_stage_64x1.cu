@@ -16,7 +16,7 @@
 
 namespace cgks {
 
-static __constant__ FluxFixed kFluxFixed1d = make_flux_fixed();
+static __device__ const FluxFixed kFluxFixed1d = make_flux_fixed();
 
 namespace {
 
@@ -99,8 +99,7 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
     __shared__ int s_skip;
     const int tid = threadIdx.x, side = tid & 1;
     const unsigned pair = 3u << (tid & 30);
-    for (int i = tid; i < FK_NFIX; i += kThreads) s_fk[i] = kFluxFixed1d.v[i];
-    if (tid < 32) s_fk[FK_EXP2 + tid] = exp2((double)tid * (1.0 / 32.0));
+    for (int i = tid; i < FK_NFIX2; i += kThreads) s_fk[i] = kFluxFixed1d.v[i];
     __syncthreads();
     const RegK r{s_fk, ((volatile const double*)s_fk)[FK_ONE], ((volatile const double*)s_fk)[FK_NZERO]};
     wait_previous();

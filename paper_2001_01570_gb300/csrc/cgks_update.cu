@@ -55,8 +55,7 @@ __global__ void __launch_bounds__(kCellChunk / CPT) update_kernel(const GridDev*
                 if (atomicAdd(&C->arrived, 1) == last) {
                     __threadfence();
                     C->arrived = 0;
-                    end_step(C);
-                    begin_step(G, C);
+                    turn_step(G, C);
                 }
             }
         }
