@@ -133,10 +133,7 @@ __device__ __forceinline__ bool positive(double x)
 // each starting with 1.0 and -0.0.  Indices are offsets within a block.
 enum ReconK {
     RK_ONE = 0, RK_NZERO,
-    RK_LV,          // linear value: (a+d), (b+c), (A-D), (B-C)
-    RK_LS = RK_LV + 4,    // linear h*slope: (c-b), (d-a), (A+D), (B+C)
-    RK_LC = RK_LS + 4,    // linear h^2*curvature: ((b+c)-(a+d)), (A-D), (B-C)
-    RK_E0 = RK_LC + 3,    // smoothness indicators e0..e6 (beta_k + eps)
+    RK_E0,                // smoothness indicators e0..e6 (beta_k + eps)
     RK_E1 = RK_E0 + 3, RK_E2 = RK_E1 + 6, RK_E3 = RK_E2 + 6, RK_E4 = RK_E3 + 3, RK_E5 = RK_E4 + 3,
     RK_E6 = RK_E5 + 10,
     RK_Z = RK_E6 + 10,    // Z_ref: 3, -2
@@ -161,36 +158,15 @@ enum ReconK {
 // to the face (no A, D terms):
 //   P5 = ((a+d) + 29 (b+c))/60 + (B-C)/5,  h P5_x = 9 (c-b)/4 + (d-a)/36 - 2 (B+C)/3,
 //   h^2 P5_xx = ((b+c) - (a+d))/4 - 3 (B-C)/2.
-// The coefficients come from the table block of the grid's order.
-template <int ORDER>
-__device__ __forceinline__ void linear_recon_rk(const RegK& r, double a, double b, double c, double d,
-                                                double A, double B, double C, double D,
-                                                double& v, double& hvx, double& h2vxx)
-{
-    const double ad = r.add(a, d), bc = r.add(b, c), BmC = r.sub(B, C);
-    const double cb = r.sub(c, b), da = r.sub(d, a), BpC = r.add(B, C), diff = r.sub(bc, ad);
-    if constexpr (ORDER == 6) {
-        v = r.kfma(RK_LV + 0, ad, r.kfma(RK_LV + 1, bc, r.kmul(RK_LV + 3, BmC)));
-        hvx = r.kfma(RK_LS + 0, cb, r.kfma(RK_LS + 1, da, r.kmul(RK_LS + 3, BpC)));
-        h2vxx = r.kfma(RK_LC + 0, diff, r.kmul(RK_LC + 2, BmC));
-    } else {
-        const double AmD = r.sub(A, D), ApD = r.add(A, D);
-        v = r.kfma(RK_LV + 0, ad, r.kfma(RK_LV + 1, bc, r.kfma(RK_LV + 2, AmD, r.kmul(RK_LV + 3, BmC))));
-        hvx = r.kfma(RK_LS + 0, cb, r.kfma(RK_LS + 1, da, r.kfma(RK_LS + 2, ApD, r.kmul(RK_LS + 3, BpC))));
-        h2vxx = r.kfma(RK_LC + 1, AmD, r.kfma(RK_LC + 2, BmC, diff));
-    }
-}
-
-#ifndef CGKS_OPCOUNT_HOST   // the host operation count takes the plain forms
-// The same reconstruction in differences of the stencil data (the notation of
-// cgks_split.cuh; 8th order: t + u = s3 + s4 - 2((d1-A) + (D-d3)) and so on):
+// Evaluated in differences of the stencil data (the notation of cgks_split.cuh, t + u =
+// s3 + s4 - 2((d1-A) + (D-d3)) and so on; coefficients from the table block of the grid's order):
 //   P7       = b + d2/2 - (s3+s4)/12 + (t+u)/140 + 17(p-q)/70
 //   h P7_x   = d2 - 10w/27 - (t-u)/72 - 11(p+q)/12
 //   h^2 P7_xx = (s3+s4)/2 - (t+u)/8 - 9(p-q)/4
 // (order 6: -(s3+s4)/12 + (p-q)/5;  -11w/36 - 2(p+q)/3;  (s3+s4)/2 - 3(p-q)/2).
 // The sums of order-one values cancel exactly in the differences, so the value is
 // one rounding from exact (largest error over random smooth rows 0.11e-15 against
-// 0.36e-15 of the form above) and the operations are fewer: the differences are
+// 0.36e-15 of the forms above) and the operations are fewer: the differences are
 // shared with the nonlinear part.
 struct RowDiffs { double d1, d2, d3, s3, s4, w, t, u, p, q; };
 
@@ -221,7 +197,6 @@ __device__ __forceinline__ void linear_diff_rk(const RegK& r, double b, double h
     }
     v = r.add(b, y);
 }
-#endif
 
 // ------------------------------------------------------------------------
 // Sec. 3.3: nonlinear compact reconstruction.  With d1 = b-a, d2 = c-b,

@@ -122,17 +122,6 @@ constexpr ReconTab make_recon_tab()
         double* k = t.v[o];
         const bool six = (o == 1);
         k[RK_ONE] = 1.0; k[RK_NZERO] = -0.0;
-        if (six) {
-            k[RK_LV + 0] = 1.0 / 60.0; k[RK_LV + 1] = 29.0 / 60.0; k[RK_LV + 2] = 0.0; k[RK_LV + 3] = 0.2;
-            k[RK_LS + 0] = 2.25; k[RK_LS + 1] = 1.0 / 36.0; k[RK_LS + 2] = 0.0; k[RK_LS + 3] = -2.0 / 3.0;
-            k[RK_LC + 0] = 0.25; k[RK_LC + 1] = 0.0; k[RK_LC + 2] = -1.5;
-        } else {
-            k[RK_LV + 0] = 25.0 / 420.0; k[RK_LV + 1] = 185.0 / 420.0; k[RK_LV + 2] = 6.0 / 420.0;
-            k[RK_LV + 3] = 102.0 / 420.0;
-            k[RK_LS + 0] = 270.0 / 108.0; k[RK_LS + 1] = 14.0 / 108.0; k[RK_LS + 2] = -3.0 / 108.0;
-            k[RK_LS + 3] = -99.0 / 108.0;
-            k[RK_LC + 0] = 1.0; k[RK_LC + 1] = -0.25; k[RK_LC + 2] = -2.25;
-        }
         k[RK_HALF] = 0.5; k[RK_MHALF] = -0.5; k[RK_M2] = -2.0; k[RK_M6TH] = -1.0 / 6.0;
         k[RK_DV + 0] = -1.0 / 12.0; k[RK_DV + 1] = six ? 0.2 : 17.0 / 70.0; k[RK_DV + 2] = six ? 0.0 : 1.0 / 140.0;
         k[RK_DS + 0] = six ? -11.0 / 36.0 : -10.0 / 27.0; k[RK_DS + 1] = six ? -2.0 / 3.0 : -11.0 / 12.0;
@@ -184,14 +173,10 @@ __device__ __forceinline__ void cons_record(const RegK& r, const double Q[4], co
                                             double weno_eps, bool inner, int k, int scale_hi, Out out)
 {
     double v, hvx, h2vxx;
-#ifdef CGKS_OPCOUNT_HOST
-    linear_recon_rk<ORDER>(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], v, hvx, h2vxx);
-#else
     RowDiffs x;
     row_diffs_rk(r, Q, S, x);
     const double hd2 = r.kmul(RK_HALF, x.d2);
     linear_diff_rk<ORDER>(r, Q[1], hd2, x, v, hvx, h2vxx);
-#endif
     out(RV, k, v);
     out(RN, k, r.mul(hvx, ih));
     out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
@@ -234,13 +219,9 @@ __device__ __forceinline__ void linear_fields(const RegK& r, const double Q[4], 
     double v, hvx, h2vxx, S[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) S[c] = r.mul(h, N[c]);
-#ifdef CGKS_OPCOUNT_HOST
-    linear_recon_rk<ORDER>(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], v, hvx, h2vxx);
-#else
     RowDiffs x;
     row_diffs_rk(r, Q, S, x);
     linear_diff_rk<ORDER>(r, Q[1], r.kmul(RK_HALF, x.d2), x, v, hvx, h2vxx);
-#endif
     out(RV, k, v);
     out(RN, k, r.mul(hvx, ih));
     out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
