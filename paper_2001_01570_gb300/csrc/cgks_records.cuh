@@ -110,6 +110,26 @@ __device__ __forceinline__ void map_stencil(const GridDev& G, const RowRef& q, S
     }
 }
 
+// one cell of the stencil, for the lane that reads it alone
+struct StencilCell {
+    size_t at;
+    int kn, kt;
+    __device__ __forceinline__ double value(const GridDev& G, const RowRef& q, int c, double v, int p) const
+    {
+        return bc_value(G, v, q.i0 + c * q.di, q.j0 + c * q.dj, q.xo ? kn : kt, q.xo ? kt : kn, p);
+    }
+};
+
+__device__ __forceinline__ void map_cell(const GridDev& G, const RowRef& q, int c, StencilCell& s)
+{
+    const int i = q.i0 + c * q.di, j = q.j0 + c * q.dj;
+    int kx, ky, si = map_axis(i, G.nx, G.bc[0], G.bc[1], kx), sj = map_axis(j, G.ny, G.bc[2], G.bc[3], ky);
+    if (!CGKS_IN_BOUNDS(si >= 0 && si < G.nx && sj >= 0 && sj < G.ny, G.ctrl)) si = sj = 0;
+    s.at = (size_t)sj * G.nx + si;
+    s.kn = q.xo ? kx : ky;
+    s.kt = q.xo ? ky : kx;
+}
+
 // Coefficient table of the register-form reconstruction, one block per order
 // (index 0: the 8th-order scheme, 1: the 6th-order variant); copied to shared
 // memory by each CTA.
@@ -227,29 +247,15 @@ __device__ __forceinline__ void linear_fields(const RegK& r, const double Q[4], 
     out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
 }
 
-// Characteristic variables: the basis at the mean of the two cells sharing the face ...
-__device__ __forceinline__ void char_basis(const RegK& r, double gamma, const double Qa[4][4], double& rho, CharState& cs)
-{
-    double Wref[4];
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) Wref[kk] = r.mul(0.5, r.add(Qa[kk][1], Qa[kk][2]));
-    char_state(r, Wref, gamma, cs);
-    rho = Wref[0];
-}
+// Characteristic variables: the basis is taken at the mean of the two cells sharing the face (b, c) ...
+__device__ __forceinline__ double char_mean(const RegK& r, double b, double c) { return r.mul(0.5, r.add(b, c)); }
 
-// ... and field m: projected on its left eigenvector, WENO-Z, slopes per unit length.
-// w[0..3]: left and right value, left and right slope.
+// ... and a field's WENO-Z step, from its projections Q and h times its projected gradients S;
+// w[0..3]: left and right value, left and right slope per unit length.
 template <int ORDER>
-__device__ __forceinline__ void char_field(const RegK& r, const CharState& cs, double rho, int m, const double Qa[4][4],
-                                           const double Na[4][4], double h, double ih, double weno_eps, double w[4])
+__device__ __forceinline__ void char_weno(const RegK& r, double rho, const double Q[4], const double S[4], double ih,
+                                          double weno_eps, double w[4])
 {
-    double l[4], Q[4], S[4];
-    char_left_row(r, cs, m, l);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
-        S[c] = r.mul(h, char_project(r, m, l, Na[0][c], Na[1][c], Na[2][c], Na[3][c]));
-    }
 #ifdef CGKS_OPCOUNT_HOST
     weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, w[0], w[2], w[1], w[3]);
 #else
@@ -274,12 +280,20 @@ __device__ __forceinline__ void char_record(const RegK& r, double gamma, const d
     for (int k = 0; k < 4; ++k) linear_fields<ORDER>(r, Qa[k], Na[k], h, ih, k, out);
     if (!inner) return;
     CharState cs;
-    double rho, w[4][4], o4[4];
-    char_basis(r, gamma, Qa, rho, cs);
+    double Wref[4], w[4][4], o4[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Wref[k] = char_mean(r, Qa[k][1], Qa[k][2]);
+    char_state(r, Wref, gamma, cs);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        double v[4];
-        char_field<ORDER>(r, cs, rho, m, Qa, Na, h, ih, weno_eps, v);
+        double l[4], Q[4], S[4], v[4];
+        char_left_row(r, cs, m, l);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
+            S[c] = r.mul(h, char_project(r, m, l, Na[0][c], Na[1][c], Na[2][c], Na[3][c]));
+        }
+        char_weno<ORDER>(r, Wref[0], Q, S, ih, weno_eps, v);
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[q][m] = v[q];
     }
@@ -325,6 +339,7 @@ __device__ __forceinline__ void cons_row(const RegK& r, const GridDev& G, const 
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
 
+#ifdef CGKS_OPCOUNT_HOST
 // the stencil cells of a row, all four variables in the face frame
 __device__ __forceinline__ void char_stencil(const GridDev& G, const double* src, size_t PL, const RowRef& q,
                                              double Qa[4][4], double Na[4][4])
@@ -352,8 +367,7 @@ __device__ __forceinline__ void char_stencil(const GridDev& G, const double* src
     }
 }
 
-// Characteristic variables: all four variables of face row `row` by one thread (the host
-// count) ...
+// Characteristic variables: all four variables of face row `row` by one thread (the host count)
 template <int ORDER>
 __device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const double* src, size_t PL,
                                          int row)
@@ -367,49 +381,77 @@ __device__ __forceinline__ void char_row(const RegK& r, const GridDev& G, const 
     char_record<ORDER>(r, G.gamma, Qa, Na, q.h, q.ih, G.weno_eps, q.inner,
                        [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
 }
+#else
+// a 4x4 matrix over a quad of lanes, lane m holding row m, becomes its transpose
+__device__ __forceinline__ void quad_transpose(unsigned quad, int m, double a[4])
+{
+#pragma unroll
+    for (int s = 1; s < 4; s <<= 1) {
+        const bool up = m & s;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (i & s) continue;                // the pair of columns i, i + s
+            const double got = __shfl_xor_sync(quad, up ? a[i] : a[i | s], s);
+            if (up) a[i] = got;
+            else a[i | s] = got;
+        }
+    }
+}
 
-#ifndef CGKS_OPCOUNT_HOST
-// ... or by four lanes (a quad of a warp), lane m with variable m of the linear fields and
-// field m of the WENO-Z step; the four fields' results are transposed by shuffles, and
-// lane m brings quantity m (left, right value, left, right slope) back to conservative
-// variables.  One thread per row ran the four fields in turn: 600 FP64 instructions in
-// one chain and 254 registers.
+// Characteristic variables: face row `row` by four lanes (a quad of a warp).  Lane m reads cell m of the stencil and projects it on
+// the four left eigenvectors; transposed, it has variable m of the four cells for the linear
+// fields and field m for the WENO-Z step, and, transposed again, quantity m (left, right value, left,
+// right slope) of the four fields, which it brings back to conservative variables.  One thread per row
+// ran the four fields in turn: 600 FP64 instructions in one chain and 254 registers; with every lane
+// of the quad reading the whole stencil the kernel waited for its instructions (200x50: 65 us, 58 here).
 template <int ORDER>
 __device__ __forceinline__ void char_row_quad(const RegK& r, const GridDev& G, const double* src, size_t PL,
                                               int row, int m, unsigned quad)
 {
     const RowRef q = row_ref(G, row);
     if (!CGKS_IN_BOUNDS(q.idx < q.stride, G.ctrl)) return;
-    double Qa[4][4], Na[4][4], Qm[4], Nm[4];
-    char_stencil(G, src, PL, q, Qa, Na);
+    const int p1 = q.xo ? 1 : 2, p2 = q.xo ? 2 : 1;         // planes of the normal and tangential momentum
+    StencilCell c;
+    map_cell(G, q, m, c);
+    const double *v = src + c.at, *n = v + (size_t)q.gn * PL;
+    double Q[4] = {v[0], v[p1 * PL], v[p2 * PL], v[3 * PL]}, N[4] = {n[0], n[p1 * PL], n[p2 * PL], n[3 * PL]};
+    if (c.kn | c.kt) {
+        const int pk[4] = {0, p1, p2, 3};
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        Qm[c] = m == 0 ? Qa[0][c] : m == 1 ? Qa[1][c] : m == 2 ? Qa[2][c] : Qa[3][c];
-        Nm[c] = m == 0 ? Na[0][c] : m == 1 ? Na[1][c] : m == 2 ? Na[2][c] : Na[3][c];
+        for (int k = 0; k < 4; ++k) {
+            Q[k] = c.value(G, q, m, Q[k], pk[k]);
+            N[k] = c.value(G, q, m, N[k], q.gn + pk[k]);
+        }
     }
+    double Qm[4] = {Q[0], Q[1], Q[2], Q[3]}, Nm[4] = {N[0], N[1], N[2], N[3]};
+    quad_transpose(quad, m, Qm);
+    quad_transpose(quad, m, Nm);
     double* o = q.base + q.idx;
     const size_t st = q.stride;
     linear_fields<ORDER>(r, Qm, Nm, q.h, q.ih, m, [&](int f, int kk, double x) { o[(f * 4 + kk) * st] = x; });
     if (!q.inner) return;                     // the same for the quad's lanes (one row)
     CharState cs;
-    double rho, w[4], t[4], o4[4];
-    char_basis(r, G.gamma, Qa, rho, cs);
-    char_field<ORDER>(r, cs, rho, m, Qa, Na, q.h, q.ih, G.weno_eps, w);
-    // t[j] = field j of quantity m: step s sends quantity m ^ s to lane m ^ s
+    const double mean = char_mean(r, Qm[1], Qm[2]);
+    double Wref[4], P[4], S[4], w[4], o4[4];
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int j = m ^ s;
-        const double mine = j == 0 ? w[0] : j == 1 ? w[1] : j == 2 ? w[2] : w[3];
-        const double got = __shfl_xor_sync(quad, mine, s);
+    for (int k = 0; k < 4; ++k) Wref[k] = __shfl_sync(quad, mean, k, 4);
+    char_state(r, Wref, G.gamma, cs);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) t[i] = i == j ? got : t[i];
+    for (int f = 0; f < 4; ++f) {
+        double l[4];
+        char_left_row(r, cs, f, l);
+        P[f] = char_project(r, f, l, Q[0], Q[1], Q[2], Q[3]);
+        S[f] = r.mul(q.h, char_project(r, f, l, N[0], N[1], N[2], N[3]));
     }
-    char_to_cons(r, cs, t, o4);
+    quad_transpose(quad, m, P);
+    quad_transpose(quad, m, S);
+    char_weno<ORDER>(r, Wref[0], P, S, q.ih, G.weno_eps, w);
+    quad_transpose(quad, m, w);
+    char_to_cons(r, cs, w, o4);
     const int f = m == 0 ? RL : m == 1 ? RR : m == 2 ? RLN : RRN;
 #pragma unroll
     for (int k = 0; k < 4; ++k) o[(f * 4 + k) * st] = o4[k];
 }
 #endif
-
 
 }  // namespace cgks
