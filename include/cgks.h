@@ -156,8 +156,8 @@ cgks_status cgks_batch_step(cgks_solver* const* solvers, int n, int nsteps);
  * 0: 16x8, 1: 8x16, 2: 32x4, 3: 64x1, 4: 16x7, 5: 7x16, 6: 14x8, 7: 24x8,
  * 8: 16x14, 9: 20x11, 10: 15x15, 11: 22x10, 12: 18x12, 13: 20x12, 14: 15x16,
  * 15: 17x14, 16: 16x16, 17: 24x16, 18: 32x12; -1
- * restores the default (64x1 in 1D; in 2D 8x16, or 14x8 where it needs no more
- * passes of the persistent grid, as on small grids).  The shape changes only the
+ * restores the default (64x1 in 1D, 8x16 in 2D, which is worked on as 8x4 strips).
+ * The shape changes only the
  * decomposition of the work, never the results.  Errors: CGKS_E_INVAL (1D
  * solvers take only 64x1; 2D solvers any other shape). */
 cgks_status cgks_set_tile_shape(cgks_solver* s, int shape);
@@ -169,10 +169,9 @@ int cgks_tile_shape(const cgks_solver* s);
 /* Tile shape (numbered as for cgks_set_tile_shape) that the autotuner of
  * cgks_batch_step chose for this exact batch, or -1 while it is still timing
  * the candidates.  The tuner times, on the first steps of a new batch
- * composition, the flux kernel's tile shapes 8x16, 14x8, 16x8 and 16x16 (with
- * 2, 1.75, 2 and 4 face segments per thread), then the update kernel at 2
- * and 4 cells per thread with the best shape (12 steps in all); neither choice
- * changes a result. */
+ * composition, the flux kernel's tile shapes 8x16 and 14x8, then the update
+ * kernel at 2 and 4 cells per thread with the best shape (8 steps in all);
+ * neither choice changes a result. */
 int cgks_batch_tile_shape(cgks_solver* const* solvers, int n);
 
 /* Cells per thread of the update kernel (1, 2 or 4) that the autotuner chose
@@ -183,7 +182,8 @@ int cgks_batch_update_cpt(cgks_solver* const* solvers, int n);
  * solver's stream around every kernel of every step; stage_ms[0..7] receive
  * the average duration in milliseconds of the step-begin, stage-1 record,
  * stage-1 flux, stage-1 update, stage-2 record, stage-2 flux, stage-2 update
- * and step-end kernels.  For measurement only (the events serialise nothing
+ * and step-end kernels (the first and the last are empty: the stage-2 update
+ * kernel ends a step and starts the next).  For measurement only (the events serialise nothing
  * but add host work per launch). */
 cgks_status cgks_step_profiled(cgks_solver* s, int nsteps, double stage_ms[8]);
 

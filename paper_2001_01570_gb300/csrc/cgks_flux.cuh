@@ -20,8 +20,8 @@ namespace cgks {
 #define CGKS_BRANCH(cond) _Pragma("unroll 1") for (bool go_ = (cond); go_; go_ = false)
 
 // Layout of the flux kernel's shared-memory table.  Fixed constants first
-// (copied from kFluxFixed), then the values of the tile's grid and time step
-// (written by the CTA's first thread at the start of each tile).
+// (copied from global memory), then the values of the tile's grid and time step
+// (written by the CTA's four warps when a tile's grid is not the tile's before).
 enum FluxK {
     FK_ONE = 0, FK_NZERO, FK_HALF, FK_MHALF, FK_2, FK_M2, FK_3, FK_4, FK_M4,
     FK_T13_3, FK_DLO, FK_DHI,              // tangential WENO-Z: 4 x beta weight, linear weights at the Gauss points

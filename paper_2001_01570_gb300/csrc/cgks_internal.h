@@ -139,8 +139,8 @@ enum TileShape { CGKS_FOR_EACH_TILE(CGKS_TILE_ENUM) TILE_COUNT };
 // The tiles of a shape's queue: the shape itself, except that 8x16, the 2D default, is
 // worked on (queued and staged) as 8x4 strips of 64 segments, one pass of a CTA.  The
 // strips' records and slices take 49 KB, so three CTAs fit an SM; a small grid spreads
-// over twice the CTAs of 8x8 strips (64^2: stage-1 flux 75.8 -> 42.9 us; 2048^2: 18.4 ->
-// 17.8 ms).
+// over twice the CTAs of 8x8 strips (when it was chosen, stage 1: 64^2 75.8 -> 42.9 us,
+// 2048^2 18.4 -> 17.8 ms).
 constexpr int work_w(int w, int) { return w; }
 constexpr int work_h(int w, int h) { return w == 8 && h == 16 ? 4 : h; }
 #define CGKS_TILE_W(w, h) work_w(w, h),
@@ -175,12 +175,14 @@ inline int update_blocks(int nchunks, int nsm, int cpt = 1)
 }
 // cells per thread for one grid run by itself: one while the cells are at most four warps
 // per FP64 unit (four units per SM), where the chain of one thread's instructions counts;
-// two above, where the loads in flight do
+// two above, where half the CTAs end a chunk (2048^2, stage 1 / 2: one 540 / 585 us, two
+// 543 / 561, four 593 / 628)
 inline int update_cpt(long long cells, int nsm) { return cells <= 4LL * 32 * 4 * nsm ? 1 : 2; }
 // flux kernel: resident CTAs of 128 threads per SM.  The 8x4 strips run three at 168
-// registers (250 B of spills in stage 1): with two CTAs the FP64 unit was 57 % busy, its
+// registers (180 B of spills in stage 2): with two CTAs the FP64 unit was 57 % busy, its
 // warps waiting for one another's FP64 and FP32 chains; four at 128 registers spill more
-// and are no faster (2048^2, stage 1: 21.4, 17.8, 18.3 ms with two, three, four).
+// and are no faster (2048^2, stage 1: 21.4, 17.8, 18.3 ms with two, three, four; later
+// 16.05 and 16.42 ms with three and four).
 constexpr int stage_ctas(int tx, int ty) { return tx == 8 && ty == 4 ? 3 : 2; }
 inline int stage_blocks(int ntiles, int nsm, int shape)
 {

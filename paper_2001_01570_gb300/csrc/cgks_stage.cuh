@@ -21,12 +21,13 @@
 //            W* and R flux combinations and the interface states W(dt/2), W(dt);
 //            stage 2: dt^2/3 F_t and dt^2/3 W_tt)
 // What bounds it: the FP64 unit (68 cycles per warp instruction) with FP32 issue beside
-// it; about 1,000 FP64 instructions and 18,000 others per warp and 32 segments.  One
+// it: 792 (stage 1) and 690 FP64 instructions and some 20,000 others per 32 segments.  One
 // thread per segment ran both points in turn with the first one's sums and the shared
 // parts in registers (255 of them, 1.8 KB of spills once the FP32 pairs came in); one
 // thread per point needs 168 and halves the chain of dependent instructions that a small
 // grid waits for.  Measured per launch, stage 1 / 2: 2048^2 27.66 / 25.41 -> 17.8 / 14.4
-// ms, 512^2 1.93 / 1.77 -> 1.14 / 0.94 ms, 64^2 155 / 138 -> 43 / 38 us.
+// ms with this split, 13.9 / 12.1 now; 512^2 1.93 / 1.77 -> 1.14 / 0.94, 0.90 / 0.79 ms now;
+// 64^2 155 / 138 -> 43 / 38, 37 / 34 us now.
 // Coefficients (fixed, and the tile's grid and dt) come from the shared-memory
 // table of cgks_flux.cuh; all arithmetic is in the register-only DFMA forms.
 // The kernel is persistent: CTAs stride over a flattened tile queue that may

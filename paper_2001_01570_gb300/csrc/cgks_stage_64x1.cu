@@ -10,7 +10,7 @@
 // shuffles.  What bounds it on the grids 1D is used for (12 to a few hundred cells) is the
 // chain of dependent FP64 instructions of one warp, 68 cycles each: about 220 here
 // against some 550 per lane of the 2D kernel (100 cells, stage 1: 81.9 us with one thread
-// per face, 43.7 with one per Gauss point, 18.5 here).
+// per face, 43.7 with one per Gauss point, 18.3 here).
 #include "cgks_flux.cuh"
 #include "cgks_segment.cuh"
 

@@ -20,8 +20,8 @@ namespace cgks {
 // What bounds it: HBM on large grids; on small ones the chain of one thread's 80 (stage 1)
 // to 150 FP64 instructions per cell, so those run one cell per thread.  Measured, stage 1 / 2,
 // before (four cells per thread, chunks of 256, two quotients per cell, the step's end and
-// start in launches of their own) and now: 64^2 27 / 29 -> 14 / 17 us (5 of them the event
-// pair's), 2048^2 537 / 693 -> 575 / 607 us (one cell per thread 573 / 673, four 844 / 590).
+// start in launches of their own) and now: 64^2 27 / 29 -> 10.3 / 14.5 us (5 of them the event
+// pair's), 2048^2 537 / 693 -> 543 / 561 us.
 template <int STAGE, int CPT>
 __global__ void __launch_bounds__(kCellChunk / CPT) update_kernel(const GridDev* __restrict__ grids,
                                                                   const TileRef* __restrict__ chunks, int nchunks,
