@@ -54,8 +54,8 @@ UNIT = "cell-updates/s"
 # each: linear P7 + WENO-Z pair of 4 variables), two face segments (3,076.44 in stage 1, 2,878.44 in
 # stage 2: two Gauss points each) and the update (80 / 121).  The kernels issue their adds and
 # multiplies as DFMAs, so the operations are counted by ncu on a build with plain adds and
-# multiplies; each per-unit figure is the smallest count of the formulations measured (the current
-# code spends 1,916 per record and 3,076.44 / 2,878.44 per segment).
+# multiplies; each per-unit figure is the smallest count of the FP64 formulations measured (the current code
+# computes the corrections among them in pairs of FP32, whose instructions are not counted).
 # The compact 6th-order variant (--order 6) changes only the record kernel's linear reconstruction:
 # 1,840 per face row with WENO-Z.
 RECORD_FLOP_PER_CELL = {8: 3776.0, 6: 3680.0}
@@ -68,11 +68,14 @@ FLOP_PER_CELL = {s: RECORD_FLOP_PER_CELL[8] + FLUX_FLOP_PER_CELL[s] + UPDATE_FLO
 # every divide, square root, reciprocal, exponential and erfc as 1 however the GPU expands it.
 OPCOUNT_FLOP_PER_CELL = {"records": 3854.022, "flux": {1: 4746.316, 2: 4466.180}, "update": {1: 80.0, 2: 71.0}}
 TRAFFIC_TILE = "8x16"     # the tile shape the DRAM bytes below were captured on
-# DRAM bytes (read + write) per cell of one stage-1 flux-kernel launch with 8x16 tiles: ncu
+# DRAM bytes (read + write) per cell of one stage-1 flux-kernel launch with 8x16 tiles (8x4 strips): ncu
 # dram__bytes_{read,write}.sum of the current kernel on the 1024^2 vortex (records and state larger
-# than L2), 478.90 + 244.60 MB, divided by the cells; the 2048^2 bench grid moves the same bytes per
+# than L2), 480.56 + 246.52 MB, divided by the cells; the 2048^2 bench grid moves the same bytes per
 # cell (its launch is too large to capture under the profiling size rule).
-FLUX_DRAM_BYTES_PER_CELL = {1: (478.897664e6 + 244.597504e6) / 1048576}
+FLUX_DRAM_BYTES_PER_CELL = {1: (480.558336e6 + 246.522112e6) / 1048576}
+# FP64 thread instructions per cell of a stage-1 flux launch (ncu sm__inst_executed_pipe_fp64.sum x 32 on the
+# 1024^2 vortex): what the kernel issues to the FP64 pipe itself; the rest of its formulas runs in pairs of FP32
+FLUX_FP64_INST_PER_CELL = {1: 51522648 * 32 / 1048576}
 # algorithmic bytes per cell of the flux kernel: the two face rows' records (2 x 28 doubles) read and
 # the two faces' results written (stage 1: 16 doubles each, stage 2: 8)
 FLUX_ALGO_BYTES_PER_CELL = {1: 448 + 256, 2: 448 + 128}
@@ -279,6 +282,12 @@ def run_cgks(args, world, rank, local):
                 "peak_source": "measured FP64 DFMA rate (register operands, FMA = 2): %.2f per SM and cycle x %d SMs "
                                "x %.0f MHz (median SM clock in the timed region), of measured"
                                % (FP64_DFMA_PER_SM_CYCLE, nsm, peak_mhz)}
+    roofline["fp64_pipe"] = {
+        "instructions_per_cell": FLUX_FP64_INST_PER_CELL[1],
+        "busy": FLUX_FP64_INST_PER_CELL[1] * cells / (flux_ms * 1e-3)
+                / (FP64_DFMA_PER_SM_CYCLE * nsm * peak_mhz * 1e6),
+        "note": "frac counts the method's operations in FP64 equivalents; corrections are computed in pairs of FP32, "
+                "so it is not bounded by 1, busy is"} if tile == TRAFFIC_TILE and args.order == 8 else None
     # the same kernels against the operation count of their formulas (exp, erfc, reciprocal,
     # divide, square root one operation each): the convention of the algorithmic FP64 count
     oc_flux = OPCOUNT_FLOP_PER_CELL["flux"][1]
