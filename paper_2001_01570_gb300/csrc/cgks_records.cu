@@ -29,11 +29,12 @@ static __device__ const ReconTab kReconTab = make_recon_tab();
 // 512^2: 1.010 -> 0.257 ms; 64^2 (two warps per FP64 unit): 24 -> 14.3 us.
 // Characteristic mode with a thread per row ran 600 FP64 instructions and four WENO-Z pairs
 // in one chain (401 cells in 1D: 78 us; a lane per field, and only the grid's own row of the
-// five a 1D stencil would take: 41 us, with the stencil mapped once 26, a cell per lane 24.7; 200x50: 99 -> 58 us).
-// Two lanes per row, one for each
-// side of the face, changed nothing on small grids (100 cells in 1D: 69.1 and 69.4 us per step).
+// five a 1D stencil would take: 41 us; the stencil mapped once: 26; a cell per lane: 24.7;
+// 200x50: 99 -> 58 us).  Two lanes per row, one for each side of the face, changed nothing
+// on small grids (100 cells in 1D: 69.1 and 69.4 us per step).
 // CTAs of 128 threads, four per SM: one of 256 left a small grid's items on half
 // of the SMs (100 cells in 1D: 24.7 us; spread over twice the CTAs: 20.9, 12.6 now).
+// Three, four, five per SM: 2048^2 3.98, 3.73, 3.78 ms; 512^2 272, 258, 256 us.
 template <int STAGE, int CHAR>
 __global__ void __launch_bounds__(kRecordChunk, 4) records_kernel(const GridDev* __restrict__ grids,
                                                                     const TileRef* __restrict__ chunks, int nchunks,
