@@ -22,7 +22,10 @@
 #include <stdint.h>
 
 #include "cgks_erfcx_table.h"
-#ifndef CGKS_OPCOUNT_HOST
+// CGKS_PAIRS: the forms in pairs of FP32 and the choices between them and FP64 are compiled (everywhere
+// but in the host operation count, which counts the FP64 formulas)
+#if !defined(CGKS_OPCOUNT_HOST) || defined(CGKS_SPLIT_CHECK)
+#define CGKS_PAIRS 1
 #include "cgks_split.cuh"
 #endif
 #include "../../include/cgks.h"
@@ -304,7 +307,7 @@ __device__ __forceinline__ void weno_pair_rk(const RegK& r, double a, double b, 
     sr = -s;
 }
 
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
 // The pair of one row: the split form of cgks_split.cuh where it loses nothing
 // (split_ok), else the FP64 form above.  Same outputs as weno_pair_rk.
 template <int ORDER>

@@ -118,7 +118,7 @@ __device__ __forceinline__ void flux_table_part(double* t, const GridDev& G, dou
         t[FK_WEPS] = G.weno_eps;
         t[FK_WEPS4] = 4.0 * G.weno_eps;
     } else {
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
         t[FK_PGAMMA] = ff_pack(ff_from(G.gamma));
         t[FK_PGM1] = ff_pack(ff_from(G.gamma - 1.0));
         t[FK_PK1] = ff_pack(ff_from(G.K + 1.0));
@@ -229,7 +229,7 @@ __device__ __forceinline__ void tang_weno3_parts(const RegK& r, double vm, doubl
 
 // Twice one row's slope in the split form: false where the correction it carries is not
 // below 2^-11 of the scale (its relative error is about 2^-44).
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
 __device__ __forceinline__ bool tang_weno3_small(const RegK& r, double vm, double v0, double vp, double eps,
                                                  int scale_hi, double& slope2)
 {
@@ -247,7 +247,7 @@ __device__ __forceinline__ void tang_weno3_slopes(const RegK& r, double lm, doub
                                                   double r0, double rp, double eps, int scale_hi, double& sl,
                                                   double& sr)
 {
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
     if (tang_weno3_small(r, lm, l0, lp, eps, scale_hi, sl) && tang_weno3_small(r, rm, r0, rp, eps, scale_hi, sr)) return;
 #endif
     double nl, dl, nr, dr;
@@ -440,7 +440,7 @@ struct Ar64 {
     __device__ __forceinline__ double K3() const { return r.k(FK_K3); }
 };
 
-#if !defined(CGKS_OPCOUNT_HOST) || defined(CGKS_SPLIT_CHECK)
+#ifdef CGKS_PAIRS
 // the same in pairs of FP32 (cgks_split.cuh), not renormalised: the results' weights leave room
 struct ArSplit {
     using T = ff;
@@ -523,17 +523,20 @@ __device__ __forceinline__ void euler_second(const Ar& q, const EulerFirst<T>& f
                    q.mad(rt2, f.uut, q.mad(rtt, f.hq2, ett)));
 }
 
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
 // W_tt in pairs of FP32: it enters the interface state as dt^2/8 W_tt and dt^2/6 W_tt,
 // second order in the changes over a time step.  False (nothing written) unless
 //   (a dt)^2 (sum of second derivatives + squared sum of first ones) < 2^-6
 // of the variables' scales rho, rho a, rho a^2 (a = |U| + |V| + 2 sqrt(theta)), so that
 // the pairs' rounding of W_tt (about 2^-45 of its largest term) stays below the last bit
-// of the state.
+// of the state, and unless the units let the pairs hold all terms (wtt_range_ok).  A derivative
+// that is out of a float's range itself, infinite or NaN is so in the sum, which then is not
+// below the bound.
 template <class Src>
 __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src, const EulerFirst<double>& f,
-                                                   double Wtt[4])
+                                                   double E, double Wtt[4])
 {
+    if (!wtt_range_ok(hi_log(f.rho), hi_log(E), hi_log(r.k(FK_DT)))) return false;
     EulerFirst<ff> g;
     g.rho = ff_from(f.rho); g.U = ff_from(f.U); g.V = ff_from(f.V); g.ir = ff_from(f.ir); g.gir = ff_from(f.gir);
     g.hq2 = ff_from(f.hq2); g.e = ff_from(f.e);
@@ -546,7 +549,7 @@ __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src
         // theta = (gamma - 1) e / rho; e * gir
         const float th = f_mul(g.e.h, g.gir.h), a = f_add(f_add(fabsf(g.U.h), fabsf(g.V.h)), f_mul(2.0f, f_mul(th, f_rsqrt(th))));
         const float ia = f_rcp(a), ad = f_mul(a, f_lead(r.k(FK_DT))), ir = g.ir.h, ir1 = f_mul(ir, ia), ir2 = f_mul(ir1, ia);
-        // sums, not maxima: a NaN has to fail the comparison
+        // sums, not maxima: a NaN has to fail the comparison (a maximum drops it)
         auto m3 = [](ff a, ff b, ff c) { return f_add(f_add(fabsf(a.h), fabsf(b.h)), fabsf(c.h)); };
         const float s2 = f_fma(m3(xx[3], xy[3], yy[3]), ir2,
                                f_fma(f_add(m3(xx[1], xy[1], yy[1]), m3(xx[2], xy[2], yy[2])), ir1, f_mul(m3(xx[0], xy[0], yy[0]), ir)));
@@ -612,27 +615,29 @@ __device__ __forceinline__ void euler_time_derivs(const RegK& r, const Src& src,
     o.TNS[1] = sxx;
     o.TNS[2] = sxy;
     o.TNS[3] = fma(r.mul(r.k(FK_KHEAT), p), thx, fma(V, sxy, r.mul(U, sxx)));
-#ifndef CGKS_OPCOUNT_HOST
-    if (euler_second_split(r, src, f, o.Wtt)) return;
+#ifdef CGKS_PAIRS
+    if (euler_second_split(r, src, f, E, o.Wtt)) return;
 #endif
     double Wxx[4], Wxy[4], Wyy[4];
     src.eq_second(Wxx, Wxy, Wyy);
     euler_second(Ar64{r}, f, gamma, Wxx, Wxy, Wyy, o.Wtt);
 }
 
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
 // The slope moments in pairs of FP32.  They enter a face's flux through the weights
 // of order tau^2/dt and its state through h dt, a small correction where the
-// collision time is: false (nothing written) unless every weighted term is below
+// collision time is: false (nothing to be used) unless every weighted term is below
 // 2^-7 of the side's half-line flux of the same kind (a momentum's scale is the
 // normal momentum flux), so that the pairs' rounding stays below that flux's last
-// bit.  wth, wsl: the weights' magnitudes.
-
+// bit, and unless the units let the pairs hold the terms (slopes_range_ok).  wth, wsl:
+// the weights' magnitudes.
 template <class Src>
 __device__ __forceinline__ bool slope_moments_split(const RegK& r, const Src& src, int side, bool ne, double rho,
                                                     double U, double V, double th, double sq, const HalfMoments& h,
                                                     float wth, float wsl, ff Th[4], ff Wsl[4])
 {
+    if (!slopes_range_ok(hi_log(rho), hi_log(th), i_max(hi_log(U), hi_log(V)), hi_log(src.iht), f_log(wth > wsl ? wth : wsl)))
+        return false;
     const ff K1 = ff_unpack(r.k(FK_PK1));
     const ArSplit q{ff_unpack(r.k(FK_PGM1)), K1, ff_unpack(r.k(FK_PK3))};
     ff m[4], n[4], s[4], T[4], S[4];
@@ -645,7 +650,7 @@ __device__ __forceinline__ bool slope_moments_split(const RegK& r, const Src& sr
     const float fr = f_lead(rho), qt = f_fma(fV.h, fV.h, f_mul(K1.h, fth.h)), f0 = f_mul(fr, fabsf(m[1].h)),
                 f1 = f_mul(fr, m[2].h), f3 = f_mul(f_mul(0.5f, fr), f_fma(fabsf(m[1].h), qt, fabsf(m[3].h)));
     const float w = f_mul(128.0f, wth), v = f_mul(128.0f, wsl);
-    // sums, not maxima: a NaN has to fail the comparisons
+    // sums, not maxima: a NaN has to fail the comparisons (a maximum drops it)
     bool ok = f0 > 1e-15f && f1 > 1e-15f && f3 > 1e-15f && f_mul(w, fabsf(T[0].h)) < f0 &&
               f_mul(w, f_add(fabsf(T[1].h), fabsf(T[2].h))) < f1 && f_mul(w, fabsf(T[3].h)) < f3;
     if (ne)
@@ -672,7 +677,7 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
                                           double Ul, double Vl, double thl, double Ur, double Vr, double thr,
                                           bool need_ne, float wth, float wsl, HalfSums& o)
 {
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
     bool split = false;
 #else
     bool split = true;
@@ -682,7 +687,7 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
         bool ok = true;
 #pragma unroll
         for (int k = 0; k < 4; ++k) { o.Fh[k] = 0.0; o.Th[k] = 0.0; o.Wh[k] = 0.0; o.Wsl[k] = 0.0; }
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
 #pragma unroll
         for (int k = 0; k < 4; ++k) { Ts[k] = ff{0.0f, 0.0f}; Ss[k] = ff{0.0f, 0.0f}; }
 #endif
@@ -705,7 +710,7 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
                 o.Wh[2] = fma(rho, r.mul(V, h.m[0]), o.Wh[2]);
                 o.Wh[3] = fma(rho, r.kmul(FK_HALF, fma(h.m[0], qt, h.m[2])), o.Wh[3]);
             }
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
             if (split) {
                 ok &= slope_moments_split(r, src, side, need_ne, rho, U, V, th, sq, h, wth, wsl, Ts, Ss);
                 continue;
@@ -722,7 +727,7 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
             for (int k = 0; k < 4; ++k) o.Wsl[k] = r.add(o.Wsl[k], ws[k]);
         }
         if (!split) return;
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
         if (ok) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) o.Th[k] = r.add(d_from(Ts[k].h), d_from(Ts[k].l));
@@ -787,15 +792,17 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
 #ifdef CGKS_OPCOUNT_HOST
     if (tau > 0.0 && dt < 80.0 * tau) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
     const bool need_ne = (STAGE == 1) && (h >= 1e-20);
-    const float wth = 0.0f, wsl = 0.0f;
 #else
-    const float ft = f_lead(tau), fdt = f_lead(dt);
-    CGKS_BRANCH(ft > 0.0f && fdt < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
+    CGKS_BRANCH(f_lead(tau) > 0.0f && f_lead(dt) < f_mul(80.0f, f_lead(tau))) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
     const bool need_ne = (STAGE == 1) && d_hi(h) >= 0x3bc79ca1;       // high word of 1e-20
+#endif
+#ifdef CGKS_PAIRS
     // bounds of the slope terms' weights (FP32, for the choice of their arithmetic): beside F
     // |b4| and |f4| dt/4 below are at most 4 tau (tau + h dt) / dt, beside W it is h dt
-    const float wsl = f_mul(fdt, f_lead(h));
-    const float wth = f_mul(f_mul(4.0f, f_mul(ft, f_add(ft, wsl))), f_lead(r.k(FK_IDT)));
+    const float ft = f_lead(tau), wsl = f_mul(f_lead(dt), f_lead(h));
+    const float wth = f_mul(f_mul(4.0f, ft), f_mul(f_add(ft, wsl), f_lead(r.k(FK_IDT))));
+#else
+    const float wth = 0.0f, wsl = 0.0f;
 #endif
 
     HalfSums o;

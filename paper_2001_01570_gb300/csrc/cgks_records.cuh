@@ -202,7 +202,7 @@ __device__ __forceinline__ void cons_record(const RegK& r, const double Q[4], co
     out(RNN, k, r.mul(r.mul(h2vxx, ih), ih));
     if (inner) {
         double vl, sl, vr, sr;
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
         weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, vl, sl, vr, sr);
 #else
         weno_pair_row<ORDER>(r, Q, S, x, hd2, weno_eps, scale_hi, vl, sl, vr, sr);
@@ -214,7 +214,7 @@ __device__ __forceinline__ void cons_record(const RegK& r, const double Q[4], co
     }
 }
 
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
 inline int scale_of(int, double, double, double, double) { return 0; }
 #else
 // High word of the scale a variable's rounding is measured against: density and
@@ -256,7 +256,7 @@ template <int ORDER>
 __device__ __forceinline__ void char_weno(const RegK& r, double rho, const double Q[4], const double S[4], double ih,
                                           double weno_eps, double w[4])
 {
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
     weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, w[0], w[2], w[1], w[3]);
 #else
     // every characteristic field is measured against the density, whose dimension it has

@@ -110,7 +110,7 @@ struct SegmentPoint {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             W0nn[k] = at(RNN, k, 0);
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
             W0tt[k] = r.mul(fma(eta, P(k, PTT1), P(k, PTT0)), iht2);
             W0nt[k] = r.mul(fma(eta, P(k, PNT1), P(k, PNT0)), iht);
 #else
@@ -123,7 +123,7 @@ struct SegmentPoint {
         }
     }
 
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
     __device__ __forceinline__ void eq_second_split(ff W0nn[4], ff W0nt[4], ff W0tt[4]) const
     {
         const ff ih = ff_unpack(r.k(ihp)), ih2 = ff_mul(ih, ih), et = gp ? CGKS_FF(kGauss) : CGKS_FF(-kGauss);
@@ -155,7 +155,7 @@ struct SegmentPoint {
         }
     }
 
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
     __device__ __forceinline__ void ne_slopes_split(int side, ff Wn[4], ff Wt[4]) const
     {
         const int f = side ? RRN : RLN;
@@ -178,7 +178,7 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
 {
     const double weps = r.k(FK_WEPS), weps4 = r.k(FK_WEPS4);
     auto R = [&](int f, int k, int off) { return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off); };
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
     // scales (high words): the smallest of the three states' densities and energies; a
     // momentum also against sqrt(rho E)
     const int sc0 = i_min(i_min(hi_abs(R(RV, 0, 0)), hi_abs(R(RL, 0, 0))), hi_abs(R(RR, 0, 0)));
@@ -190,7 +190,7 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
         int sc = 0;
         bool split = false;
         const double m0 = R(RV, k, 0), n0 = R(RN, k, 0);
-#ifndef CGKS_OPCOUNT_HOST
+#ifdef CGKS_PAIRS
         sc = k == 0 ? sc0 : k == 3 ? sc3 : i_max(hi_abs(m0), (sc0 >> 1) + (sc3 >> 1));
         {
             const double vm = R(RV, k, -1), vp = R(RV, k, 1), nm = R(RN, k, -1), np = R(RN, k, 1);
@@ -200,7 +200,7 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
             const int m1 = i_max(i_max(hi_abs(va), hi_abs(vb)), i_max(hi_abs(vc), hi_abs(vd)));
             const int mn = i_max(i_max(hi_abs(na), hi_abs(nb)), i_max(hi_abs(nc), hi_abs(nd)));
             const int lim = sc + kTangFirst * (1 << 20);
-            split = split_scale_ok(sc, weps4) && m1 < lim && mn < lim + i_min(hi_abs(ihn), kHiOne + (60 << 20)) - kHiOne &&
+            split = split_scale_ok(sc, weps4) && deriv_rows_range_ok(sc - kHiOne, hi_log(ihn)) && m1 < lim && mn < lim + i_min(hi_abs(ihn), kHiOne + (60 << 20)) - kHiOne &&
                     i_max(f_abs_word(v.t0.h), f_abs_word(v.t1.h)) < f_scale_word(sc) + kTangThird * (1 << 23);
             if (split) {
                 const ff g = CGKS_FF(kGauss), m12 = CGKS_FF(-1.0 / 12.0), c9 = CGKS_FF(1.0 / 9.0);
@@ -234,7 +234,7 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
             const double t0 = quartic_t0(r, x), t2 = r.add(t0, t0), gt = r.mul(2.0 * kGauss, quartic_t1(r, x));
             p[(PT + 0) * stride] = r.sub(t2, gt);
             p[(PT + 1) * stride] = r.add(t2, gt);
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
             p[PTT0 * stride] = quartic_tt0(r, x);
             p[PTT1 * stride] = quartic_tt1(r, x);
 #else
@@ -245,7 +245,7 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
             const double v0 = quartic_v0(r, n0, x), gv = r.mul(kGauss, quartic_v1(r, x));
             p[(PN + 0) * stride] = r.sub(v0, gv);
             p[(PN + 1) * stride] = r.add(v0, gv);
-#ifdef CGKS_OPCOUNT_HOST
+#ifndef CGKS_PAIRS
             p[PNT0 * stride] = quartic_t0(r, x);
             p[PNT1 * stride] = quartic_t1(r, x);
 #else

@@ -74,15 +74,28 @@ inline int i_min(int a, int b) { return a < b ? a : b; }
 
 struct ff { float h, l; };
 
+// The exponent field and the leading mantissa bits of |x|, from its high word, as a float's:
+// the float's bits shifted right by 3.  A float below 2^-126 for |x| below that; infinity's bits from
+// 2^128 on (NaN included).
+CGKS_SPLIT_FN uint32_t f_upper(uint32_t hi)
+{
+#ifdef __CUDACC__
+    return (uint32_t)__viaddmin_s32_relu((int)(hi & 0x7fffffffu), -(896 << 20), 0x0ff00000);
+#else
+    return (uint32_t)i_max(i_min((int)(hi & 0x7fffffffu) - (896 << 20), 0x0ff00000), 0);
+#endif
+}
+
 // the pair nearest below |x| in its leading 24 bits, the remaining 29 bits rounded
 // to 24; integer operations, since a conversion instruction occupies the FP64
-// unit like an addition.  For |x| in [2^-70, 2^127); smaller values lose low bits
-// (absolute error below 2^-126).
+// unit like an addition.  For |x| in [2^-74, 2^128) the pair has 47 bits; below 2^-74 it
+// has the leading 24 alone (error below 2^-97) and below 2^-126 next to nothing.  From 2^128
+// on, infinite and NaN, h is infinite or NaN.
 CGKS_SPLIT_FN ff ff_from(double x)
 {
     const uint32_t hi = (uint32_t)d_hi(x), lo = (uint32_t)d_lo(x);
     const uint32_t sgn = hi & 0x80000000u;
-    const uint32_t t = (uint32_t)i_max((int)(hi & 0x7fffffffu) - (896 << 20), 0);
+    const uint32_t t = f_upper(hi);
 #ifdef __CUDACC__
     const uint32_t hb = __funnelshift_l(lo, t, 3);
 #else
@@ -95,15 +108,16 @@ CGKS_SPLIT_FN ff ff_from(double x)
     return r;
 }
 
-// the leading 24 bits of x as a float (truncated; zero below 2^-126)
+// the leading 21 bits of x as a float (truncated; something below 2^-126 for |x| below that, infinite from
+// 2^128 on and for NaN)
 CGKS_SPLIT_FN float f_lead(double x)
 {
     const uint32_t hi = (uint32_t)d_hi(x);
-    const uint32_t t = (uint32_t)i_max((int)(hi & 0x7fffffffu) - (896 << 20), 0);
-    return f_bits((hi & 0x80000000u) | (t << 3));
+    return f_bits((hi & 0x80000000u) | (f_upper(hi) << 3));
 }
 
-// a float as a double (zero and denormals give zero), integer operations
+// a finite float as a double (zero and denormals give zero; infinity and NaN give 2^128 and more,
+// which no bound on a correction admits), integer operations
 CGKS_SPLIT_FN double d_from(float a)
 {
     const uint32_t b = f_word(a), m = b & 0x7fffffffu;
@@ -324,5 +338,45 @@ CGKS_SPLIT_FN ff tang_weno3_split(ff A, ff s, ff eps)
     const ff den = ff_addp(ff_scale(2.0f, ff_mul(e0, e1)), ff_mul(Z, ff_addp(e0, e1)));
     return ff_mul(ff_mul(ff_mul(Z, sA), s), ff_rcp(den));
 }
+
+// ------------------------------------------------------------------------
+// Ranges.  The pairs' floats hold a number's 47 bits from 2^-74 to 2^128, and its leading 24 with an
+// error below 2^-97 beneath that; the quantities of a face's time derivatives and slope moments carry
+// units (density rho, a speed a, a rate or length), so their pairs are used only where the units keep
+// the operands that matter and all results inside.  Logarithms here are base 2, in units of 2^-20, read
+// off the high words (exact at powers of two, less than 0.09 too large between them); zero gives -1023,
+// infinity and NaN 1024.
+constexpr int kOct = 1 << 20;
+CGKS_SPLIT_FN int hi_log(double x) { return hi_abs(x) - kHiOne; }
+CGKS_SPLIT_FN int clamp_log(int x) { return i_max(i_min(x, 60 * kOct), -60 * kOct); }
+
+// W_tt.  Density rho, energy E (so a = sqrt(E / rho)) and the time step: with the rate k = 1/(a dt) and
+// derivatives up to k and k^2 times their variables (the caller's bound), the operands are of size rho^i
+// a^j k^m with |i| <= 1, j <= 3, m <= 2 and no result exceeds rho^i a^j k^m with i <= 2, j <= 4, m <= 2.  Operands
+// of 2^-50 and more lose at most 2^-47 of themselves, results stay below 2^110 (16 orders left for the
+// sums).
+CGKS_SPLIT_FN bool wtt_range_ok(int lrho, int lE, int ldt)
+{
+    const int r = clamp_log(lrho), a = clamp_log((lE - lrho) >> 1), k = clamp_log(-ldt - a);
+    return i_max(2 * r, -r) + i_max(4 * a, 0) + i_max(2 * k, 0) <= 110 * kOct &&
+           -i_max(r, -r) + i_min(3 * a, 0) + i_min(2 * k, 0) >= -50 * kOct;
+}
+
+// Slope moments.  Density rho, theta, the larger of |U| and |V|, the inverse spacing along the face and the
+// weight's word (a float >= 0): moments to the third power of the speeds a (2^-16 to 2^16) are operands,
+// and a slope's absolute error of 2^-97 (times the inverse spacing where that is above 1) reaches the
+// fluxes of size rho a, rho a^2, rho a^3 as weight a, weight and weight / a times itself over rho, which has to
+// stay below 2^-56.  Slopes too large for a float give results that no bound admits.
+CGKS_SPLIT_FN int f_log(float w) { return (int)(f_word(w) >> 3) - (127 << 20); }
+CGKS_SPLIT_FN bool slopes_range_ok(int lrho, int ltheta, int lspeed, int linv, int lweight)
+{
+    const int lc = ltheta >> 1, la = i_max(lc, lspeed);
+    return i_max(lrho, -lrho) <= 40 * kOct && lc >= -16 * kOct && la <= 16 * kOct && linv <= 60 * kOct &&
+           lweight - lrho + i_max(la, -lc) + i_max(linv, 0) <= 40 * kOct;
+}
+
+// The rows of normal derivatives along a face, of size scale x inverse spacing: operands of 2^-45 and more
+// keep the absolute error of 2^-97 below 2^-52 of the row.
+CGKS_SPLIT_FN bool deriv_rows_range_ok(int lscale, int linv) { return i_min(linv, 60 * kOct) + lscale >= -45 * kOct; }
 
 }  // namespace cgks
