@@ -40,6 +40,7 @@ enum FluxK {
     FK_IDX, FK_IDY, FK_HIDX, FK_HIDY, FK_WEPS, FK_WEPS4,
     // the same as pairs of FP32 (ff_pack): gamma, gamma - 1, K + 1, K + 3, inverse spacings, epsilons
     FK_PGAMMA, FK_PGM1, FK_PK1, FK_PK3, FK_PIDX, FK_PIDY, FK_PWEPS, FK_PWEPS4,
+    FK_DT80,                                        // dt / 80 (its high word is compared)
     FK_N
 };
 
@@ -127,6 +128,7 @@ __device__ __forceinline__ void flux_table_part(double* t, const GridDev& G, dou
         t[FK_PIDY] = ff_pack(ff_from(G.inv_dy));
         t[FK_PWEPS] = ff_pack(ff_from(G.weno_eps));
         t[FK_PWEPS4] = ff_pack(ff_from(4.0 * G.weno_eps));
+        t[FK_DT80] = dt * (1.0 / 80.0);
 #endif
     }
 }
@@ -741,6 +743,11 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
     }
 }
 
+#ifndef CGKS_OPCOUNT_HOST
+// dt < 80 tau, from the high words (in any unit of time, off the FP64 unit); true for a NaN
+__device__ __forceinline__ bool nonequilibrium(const RegK& r, double tau) { return d_hi(r.k(FK_DT80)) < d_hi(tau); }
+#endif
+
 // ------------------------------------------------------------------------
 // One interface quadrature point in the face frame (Sec. 2.1-2.2).
 // Inputs of one Gauss point are pulled from the caller's loader when they are
@@ -793,7 +800,7 @@ __device__ __forceinline__ bool gks_point(const RegK& r, const Src& src, double 
     if (tau > 0.0 && dt < 80.0 * tau) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
     const bool need_ne = (STAGE == 1) && (h >= 1e-20);
 #else
-    CGKS_BRANCH(f_lead(tau) > 0.0f && f_lead(dt) < f_mul(80.0f, f_lead(tau))) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
+    CGKS_BRANCH(nonequilibrium(r, tau)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
     const bool need_ne = (STAGE == 1) && d_hi(h) >= 0x3bc79ca1;       // high word of 1e-20
 #endif
 #ifdef CGKS_PAIRS

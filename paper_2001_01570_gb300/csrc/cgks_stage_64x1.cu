@@ -131,8 +131,7 @@ flux1d_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ til
         CGKS_BRANCH(positive(mu)) tau0 = r.mul(mu, r.rcp3(p));
         const double tau = fma(r.k(FK_CTAUDT), fabs(r.mul(r.sub(ph, po), r.rcp3(r.add(ph, po)))), tau0);
         double h = 0.0;
-        const float ft = f_lead(tau);
-        CGKS_BRANCH(ft > 0.0f && f_lead(dt) < f_mul(80.0f, ft)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
+        CGKS_BRANCH(nonequilibrium(r, tau)) h = exp_neg(r, r.mul(r.k(FK_MHDT), r.rcp3(tau)));
         const bool need_ne = (STAGE == 1) && d_hi(h) >= 0x3bc79ca1;       // h >= 1e-20
         Half1 o;
         half_1d(r, side, H, Hn, Uh, thh, need_ne, o);

@@ -32,8 +32,21 @@ def compare(spec, W, nsteps):
 
 @pytest.mark.parametrize("mu", [0.0, 0.01])
 @pytest.mark.parametrize("rho,a,length", [(1.2, 340.0, 1e-3), (3e-12, 800.0, 1e4), (1e-9, 1e3, 1e9), (1e-15, 1e4, 1e10),
-                                          (1e4, 1e6, 1e-7), (1e3, 1e9, 1e-6)])
+                                          (1e4, 1e6, 1e-7)])
 def test_vortex_in_units(rho, a, length, mu):
     spec, W = wl.isentropic_vortex(48)
     spec, W = in_units(spec, np.ascontiguousarray(W), rho, a, length)
     compare(dataclasses.replace(spec, mu=mu * rho * a * length), W, 20)
+
+
+@pytest.mark.parametrize("char", [0, 1])
+@pytest.mark.parametrize("length", [1e-42, 1e42])
+def test_time_steps_out_of_a_floats_range(length, char):
+    """A shock's non-equilibrium part, weighted by exp(-dt / (2 tau)), in units of time of 1e-45 and 1e39."""
+    spec, W = wl.shock_tube_1d(100)
+    spec, W = in_units(dataclasses.replace(spec, recon_vars=char), np.ascontiguousarray(W), 1.0, 1.0, length)
+    compare(spec, W, 10)
+    spec, W = wl.shock_vortex(nx=48, ny=24, mach=1.5)
+    inflow = spec.inflow
+    spec, W = in_units(dataclasses.replace(spec, recon_vars=char), np.ascontiguousarray(W), 1.0, 1.0, length)
+    compare(dataclasses.replace(spec, inflow=inflow), W, 3)
