@@ -120,14 +120,14 @@ __device__ __forceinline__ void flux_table_part(double* t, const GridDev& G, dou
         t[FK_WEPS4] = 4.0 * G.weno_eps;
     } else {
 #ifdef CGKS_PAIRS
-        t[FK_PGAMMA] = ff_pack(ff_from(G.gamma));
-        t[FK_PGM1] = ff_pack(ff_from(G.gamma - 1.0));
-        t[FK_PK1] = ff_pack(ff_from(G.K + 1.0));
-        t[FK_PK3] = ff_pack(ff_from(G.K + 3.0));
-        t[FK_PIDX] = ff_pack(ff_from(G.inv_dx));
-        t[FK_PIDY] = ff_pack(ff_from(G.inv_dy));
-        t[FK_PWEPS] = ff_pack(ff_from(G.weno_eps));
-        t[FK_PWEPS4] = ff_pack(ff_from(4.0 * G.weno_eps));
+        t[FK_PGAMMA] = ff_pack(ff_from_any(G.gamma));
+        t[FK_PGM1] = ff_pack(ff_from_any(G.gamma - 1.0));
+        t[FK_PK1] = ff_pack(ff_from_any(G.K + 1.0));
+        t[FK_PK3] = ff_pack(ff_from_any(G.K + 3.0));
+        t[FK_PIDX] = ff_pack(ff_from_any(G.inv_dx));
+        t[FK_PIDY] = ff_pack(ff_from_any(G.inv_dy));
+        t[FK_PWEPS] = ff_pack(ff_from_any(G.weno_eps));
+        t[FK_PWEPS4] = ff_pack(ff_from_any(4.0 * G.weno_eps));
         t[FK_DT80] = dt * (1.0 / 80.0);
 #endif
     }
@@ -538,12 +538,13 @@ template <class Src>
 __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src, const EulerFirst<double>& f,
                                                    double E, double Wtt[4])
 {
-    if (!wtt_range_ok(hi_log(f.rho), hi_log(E), hi_log(r.k(FK_DT)))) return false;
+    // (with the size below, not as a branch of its own: the conversions wait for no FP64 result so)
+    const bool in = wtt_range_ok(hi_log(f.rho), hi_log(E), hi_log(r.k(FK_DT)));
     EulerFirst<ff> g;
     g.rho = ff_from(f.rho); g.U = ff_from(f.U); g.V = ff_from(f.V); g.ir = ff_from(f.ir); g.gir = ff_from(f.gir);
     g.hq2 = ff_from(f.hq2); g.e = ff_from(f.e);
-    g.rx = ff_from(f.rx); g.ry = ff_from(f.ry); g.Ux = ff_from(f.Ux); g.Uy = ff_from(f.Uy);
-    g.Vx = ff_from(f.Vx); g.Vy = ff_from(f.Vy); g.ex = ff_from(f.ex); g.ey = ff_from(f.ey); g.Dv = ff_from(f.Dv);
+    g.rx = ff_from_any(f.rx); g.ry = ff_from_any(f.ry); g.Ux = ff_from_any(f.Ux); g.Uy = ff_from_any(f.Uy);
+    g.Vx = ff_from_any(f.Vx); g.Vy = ff_from_any(f.Vy); g.ex = ff_from_any(f.ex); g.ey = ff_from_any(f.ey); g.Dv = ff_from(f.Dv);
     g.rt = ff_from(f.rt); g.Ut = ff_from(f.Ut); g.Vt = ff_from(f.Vt); g.et = ff_from(f.et); g.uut = ff_from(f.uut);
     ff xx[4], xy[4], yy[4], o[4];
     src.eq_second_split(xx, xy, yy);
@@ -557,7 +558,7 @@ __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src
                                f_fma(f_add(m3(xx[1], xy[1], yy[1]), m3(xx[2], xy[2], yy[2])), ir1, f_mul(m3(xx[0], xy[0], yy[0]), ir)));
         const float s1 = f_fma(f_add(fabsf(g.ex.h), fabsf(g.ey.h)), ir2,
                                f_fma(f_add(m3(g.Ux, g.Uy, g.Vx), fabsf(g.Vy.h)), ia, f_mul(f_add(fabsf(g.rx.h), fabsf(g.ry.h)), ir)));
-        if (!(f_mul(f_mul(ad, ad), f_fma(s1, s1, s2)) < 1.0f / 64.0f)) return false;
+        if (!(in & (f_mul(f_mul(ad, ad), f_fma(s1, s1, s2)) < 1.0f / 64.0f))) return false;
     }
     euler_second(ArSplit{}, g, ff_unpack(r.k(FK_PGAMMA)), xx, xy, yy, o);
 #pragma unroll
@@ -631,15 +632,13 @@ __device__ __forceinline__ void euler_time_derivs(const RegK& r, const Src& src,
 // collision time is: false (nothing to be used) unless every weighted term is below
 // 2^-7 of the side's half-line flux of the same kind (a momentum's scale is the
 // normal momentum flux), so that the pairs' rounding stays below that flux's last
-// bit, and unless the units let the pairs hold the terms (slopes_range_ok).  wth, wsl:
+// bit.  Only where the units let the pairs hold the terms (slopes_range_ok).  wth, wsl:
 // the weights' magnitudes.
 template <class Src>
 __device__ __forceinline__ bool slope_moments_split(const RegK& r, const Src& src, int side, bool ne, double rho,
                                                     double U, double V, double th, double sq, const HalfMoments& h,
                                                     float wth, float wsl, ff Th[4], ff Wsl[4])
 {
-    if (!slopes_range_ok(hi_log(rho), hi_log(th), i_max(hi_log(U), hi_log(V)), hi_log(src.iht), f_log(wth > wsl ? wth : wsl)))
-        return false;
     const ff K1 = ff_unpack(r.k(FK_PK1));
     const ArSplit q{ff_unpack(r.k(FK_PGM1)), K1, ff_unpack(r.k(FK_PK3))};
     ff m[4], n[4], s[4], T[4], S[4];
@@ -682,7 +681,10 @@ __device__ __forceinline__ void half_sums(const RegK& r, const Src& src, const d
 #ifndef CGKS_PAIRS
     bool split = false;
 #else
-    bool split = true;
+    const int rl = hi_log(Wl[0]), rr = hi_log(Wr[0]), tl = hi_log(thl), tr = hi_log(thr);
+    const int speed = i_max(i_max(hi_log(Ul), hi_log(Vl)), i_max(hi_log(Ur), hi_log(Vr)));
+    bool split = slopes_range_ok(i_min(rl, rr), i_max(rl, rr), i_min(tl, tr), i_max(tl, tr), speed, hi_log(src.iht),
+                                 f_log(wth > wsl ? wth : wsl));
     ff Ts[4], Ss[4];
 #endif
     for (;;) {

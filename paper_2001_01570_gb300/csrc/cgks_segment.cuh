@@ -131,7 +131,7 @@ struct SegmentPoint {
         for (int k = 0; k < 4; ++k) {
             W0tt[k] = ff_mul(ff_addp(ff_unpack(P(k, PTT0)), ff_mul(et, ff_unpack(P(k, PTT1)))), ih2);
             W0nt[k] = ff_mul(ff_addp(ff_unpack(P(k, PNT0)), ff_mul(et, ff_unpack(P(k, PNT1)))), ih);
-            W0nn[k] = ff_from(at(RNN, k, 0));
+            W0nn[k] = ff_from_any(at(RNN, k, 0));
         }
     }
 #endif
@@ -162,8 +162,8 @@ struct SegmentPoint {
         const ff he = gp ? CGKS_FF(0.5 * kGauss) : CGKS_FF(-0.5 * kGauss), ih = ff_scale(0.5f, ff_unpack(r.k(ihp)));
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            Wn[k] = ff_addp(ff_mul(he, ff_addp(ff_from(at(f, k, 1)), ff_neg(ff_from(at(f, k, -1))))), ff_from(at(f, k, 0)));
-            Wt[k] = ff_mul(ff_from(P(k, PS + side)), ih);
+            Wn[k] = ff_addp(ff_mul(he, ff_addp(ff_from_any(at(f, k, 1)), ff_neg(ff_from_any(at(f, k, -1))))), ff_from_any(at(f, k, 0)));
+            Wt[k] = ff_mul(ff_from_any(P(k, PS + side)), ih);
         }
     }
 #endif
@@ -238,8 +238,8 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
             p[PTT0 * stride] = quartic_tt0(r, x);
             p[PTT1 * stride] = quartic_tt1(r, x);
 #else
-            p[PTT0 * stride] = ff_pack(ff_from(quartic_tt0(r, x)));
-            p[PTT1 * stride] = ff_pack(ff_from(quartic_tt1(r, x)));
+            p[PTT0 * stride] = ff_pack(ff_from_any(quartic_tt0(r, x)));
+            p[PTT1 * stride] = ff_pack(ff_from_any(quartic_tt1(r, x)));
 #endif
             tang_diffs(r, R(RN, k, -2), R(RN, k, -1), n0, R(RN, k, 1), R(RN, k, 2), x);
             const double v0 = quartic_v0(r, n0, x), gv = r.mul(kGauss, quartic_v1(r, x));
@@ -249,8 +249,8 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
             p[PNT0 * stride] = quartic_t0(r, x);
             p[PNT1 * stride] = quartic_t1(r, x);
 #else
-            p[PNT0 * stride] = ff_pack(ff_from(quartic_t0(r, x)));
-            p[PNT1 * stride] = ff_pack(ff_from(quartic_t1(r, x)));
+            p[PNT0 * stride] = ff_pack(ff_from_any(quartic_t0(r, x)));
+            p[PNT1 * stride] = ff_pack(ff_from_any(quartic_t1(r, x)));
 #endif
         }
         tang_weno3_slopes(r, R(RL, k, -1), R(RL, k, 0), R(RL, k, 1), R(RR, k, -1), R(RR, k, 0), R(RR, k, 1), weps, sc,

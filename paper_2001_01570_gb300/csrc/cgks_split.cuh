@@ -89,13 +89,13 @@ CGKS_SPLIT_FN uint32_t f_upper(uint32_t hi)
 // the pair nearest below |x| in its leading 24 bits, the remaining 29 bits rounded
 // to 24; integer operations, since a conversion instruction occupies the FP64
 // unit like an addition.  For |x| in [2^-74, 2^128) the pair has 47 bits; below 2^-74 it
-// has the leading 24 alone (error below 2^-97) and below 2^-126 next to nothing.  From 2^128
-// on, infinite and NaN, h is infinite or NaN.
-CGKS_SPLIT_FN ff ff_from(double x)
+// has the leading 24 alone (error below 2^-97) and below 2^-126 next to nothing.  ff_from is for
+// numbers that a bound on the FP64 values keeps below 2^128 (from there on its exponent wraps
+// around); with ff_from_any, h is infinite or NaN from 2^128 on and for infinity and NaN.  (One
+// instruction more at every conversion of the flux kernel: 512^2, stage 1 907 us, so 902.)
+CGKS_SPLIT_FN ff ff_of(uint32_t hi, uint32_t lo, uint32_t t)
 {
-    const uint32_t hi = (uint32_t)d_hi(x), lo = (uint32_t)d_lo(x);
     const uint32_t sgn = hi & 0x80000000u;
-    const uint32_t t = f_upper(hi);
 #ifdef __CUDACC__
     const uint32_t hb = __funnelshift_l(lo, t, 3);
 #else
@@ -106,6 +106,16 @@ CGKS_SPLIT_FN ff ff_from(double x)
     r.h = f_bits(hb | sgn);
     r.l = f_mul(f_int((int)(lo & 0x1fffffffu)), f_bits(sc | sgn));
     return r;
+}
+CGKS_SPLIT_FN ff ff_from(double x)
+{
+    const uint32_t hi = (uint32_t)d_hi(x);
+    return ff_of(hi, (uint32_t)d_lo(x), (uint32_t)i_max((int)(hi & 0x7fffffffu) - (896 << 20), 0));
+}
+CGKS_SPLIT_FN ff ff_from_any(double x)
+{
+    const uint32_t hi = (uint32_t)d_hi(x);
+    return ff_of(hi, (uint32_t)d_lo(x), f_upper(hi));
 }
 
 // the leading 21 bits of x as a float (truncated; something below 2^-126 for |x| below that, infinite from
@@ -358,21 +368,22 @@ CGKS_SPLIT_FN int clamp_log(int x) { return i_max(i_min(x, 60 * kOct), -60 * kOc
 CGKS_SPLIT_FN bool wtt_range_ok(int lrho, int lE, int ldt)
 {
     const int r = clamp_log(lrho), a = clamp_log((lE - lrho) >> 1), k = clamp_log(-ldt - a);
-    return i_max(2 * r, -r) + i_max(4 * a, 0) + i_max(2 * k, 0) <= 110 * kOct &&
-           -i_max(r, -r) + i_min(3 * a, 0) + i_min(2 * k, 0) >= -50 * kOct;
+    return (i_max(2 * r, -r) + i_max(4 * a, 0) + i_max(2 * k, 0) <= 110 * kOct) &
+           (-i_max(r, -r) + i_min(3 * a, 0) + i_min(2 * k, 0) >= -50 * kOct);
 }
 
-// Slope moments.  Density rho, theta, the larger of |U| and |V|, the inverse spacing along the face and the
-// weight's word (a float >= 0): moments to the third power of the speeds a (2^-16 to 2^16) are operands,
-// and a slope's absolute error of 2^-97 (times the inverse spacing where that is above 1) reaches the
-// fluxes of size rho a, rho a^2, rho a^3 as weight a, weight and weight / a times itself over rho, which has to
-// stay below 2^-56.  Slopes too large for a float give results that no bound admits.
+// Slope moments of both sides.  Their densities and thetas lie between rlo, rhi and tlo, thi, |U| and |V|
+// below speed; inv is the inverse spacing along the face, weight the larger weight's word (a float >= 0).
+// Moments to the third power of the speeds a (2^-16 to 2^16) are operands, and a slope's absolute error
+// of 2^-97 (times the inverse spacing where that is above 1) reaches the fluxes of size rho a, rho a^2,
+// rho a^3 as weight a, weight and weight / a times itself over rho, which has to stay below 2^-56.  Slopes too
+// large for a float give results that no bound admits.
 CGKS_SPLIT_FN int f_log(float w) { return (int)(f_word(w) >> 3) - (127 << 20); }
-CGKS_SPLIT_FN bool slopes_range_ok(int lrho, int ltheta, int lspeed, int linv, int lweight)
+CGKS_SPLIT_FN bool slopes_range_ok(int rlo, int rhi, int tlo, int thi, int speed, int inv, int weight)
 {
-    const int lc = ltheta >> 1, la = i_max(lc, lspeed);
-    return i_max(lrho, -lrho) <= 40 * kOct && lc >= -16 * kOct && la <= 16 * kOct && linv <= 60 * kOct &&
-           lweight - lrho + i_max(la, -lc) + i_max(linv, 0) <= 40 * kOct;
+    const int lc = tlo >> 1, la = i_max(thi >> 1, speed);
+    return (i_max(rhi, -rlo) <= 40 * kOct) & (lc >= -16 * kOct) & (la <= 16 * kOct) & (inv <= 60 * kOct) &
+           (weight - rlo + i_max(la, -lc) + i_max(inv, 0) <= 40 * kOct);
 }
 
 // The rows of normal derivatives along a face, of size scale x inverse spacing: operands of 2^-45 and more

@@ -48,7 +48,7 @@ def test_pairs_are_used_in_units_of_order_one(points, k):
 
 
 def test_numbers_out_of_a_floats_range(tmp_path):
-    """ff_from keeps 47 bits from 2^-74 to 2^128 and errors below 2^-97 beneath; from 2^128 on, and for NaN,
+    """ff_from_any keeps 47 bits from 2^-74 to 2^128 and errors below 2^-97 beneath; from 2^128 on, and for NaN,
     it and f_lead give no finite number, so that no bound on a result admits it."""
     src = tmp_path / "c.cpp"
     src.write_text('''
@@ -65,7 +65,7 @@ int main()
         for (int m = 0; m < 64; ++m)
             for (int sgn = -1; sgn <= 1; sgn += 2) {
                 const double x = sgn * std::ldexp(1.0 + (m * 2654435761u % 1000003) / 1000003.0, e);
-                const ff p = ff_from(x);
+                const ff p = ff_from_any(x);
                 const float f = f_lead(x);
                 if (e >= 128) { bad += std::isfinite(p.h) + std::isfinite(f); continue; }
                 const double err = std::fabs((double)p.h + (double)p.l - x), el = std::fabs((double)f - x);
@@ -75,7 +75,7 @@ int main()
                 else bad += !(std::fabs((double)f) < std::ldexp(1.0, -126));
             }
     for (double x : {std::numeric_limits<double>::infinity(), -std::numeric_limits<double>::infinity(), (double)NAN})
-        bad += std::isfinite(ff_from(x).h) + std::isfinite(f_lead(x));
+        bad += std::isfinite(ff_from_any(x).h) + std::isfinite(f_lead(x));
     printf("%.17g %.17g %d\\n", rel, low, bad);
 }
 ''')
