@@ -533,13 +533,14 @@ __device__ __forceinline__ void euler_second(const Ar& q, const EulerFirst<T>& f
 // the pairs' rounding of W_tt (about 2^-45 of its largest term) stays below the last bit
 // of the state, and unless the units let the pairs hold all terms (wtt_range_ok).  A derivative
 // that is out of a float's range itself, infinite or NaN is so in the sum, which then is not
-// below the bound.
+// below the bound.  Nor on a rough segment (its bound hardly ever holds, and its slice holds the
+// second derivatives' parts in FP64).
 template <class Src>
 __device__ __forceinline__ bool euler_second_split(const RegK& r, const Src& src, const EulerFirst<double>& f,
                                                    double E, double Wtt[4])
 {
     // (with the size below, not as a branch of its own: the conversions wait for no FP64 result so)
-    const bool in = wtt_range_ok(hi_log(f.rho), hi_log(E), hi_log(r.k(FK_DT)));
+    const bool in = wtt_range_ok(hi_log(f.rho), hi_log(E), hi_log(r.k(FK_DT))) & (src.rough() == 0);
     EulerFirst<ff> g;
     g.rho = ff_from(f.rho); g.U = ff_from(f.U); g.V = ff_from(f.V); g.ir = ff_from(f.ir); g.gir = ff_from(f.gir);
     g.hq2 = ff_from(f.hq2); g.e = ff_from(f.e);

@@ -32,6 +32,12 @@ __device__ __forceinline__ double rec_at(const double* rec, int pa, int pb, int 
     return rec[8 * pa + ((f - RL) * 4 + k) * pb + r0 + (off + 1) * F];
 }
 
+// Parts of a variable: W0, twice its tangential slope per unit eta and its normal derivative
+// at eta = -g and +g; twice the slopes of W_l and W_r; what the second derivatives need (d2/deta2 =
+// PTT0 + eta PTT1, d2/dn deta = PNT0 + eta PNT1), as pairs of FP32, or in FP64 where the other
+// parts are (and in the host operation count).  kRough: the slot of a bit per variable with FP64 parts.
+enum { PV = 0, PT = 2, PN = 4, PS = 6, PTT0 = 8, PTT1, PNT0, PNT1, kPartsVar, kRough = 4 * kPartsVar, kParts };
+
 template <int TX, int TY, int STAGE>
 struct StageLayout {
     static constexpr int NF = FaceQ<STAGE>::n;
@@ -39,7 +45,7 @@ struct StageLayout {
     static constexpr int n_ry = RecGroups<TX, TY + 1>::n;
     static constexpr int n_rec = n_rx + n_ry;
     // a slice per pair of threads: what the two Gauss points of its segment share
-    static constexpr int n_parts = 48 * kPairs;
+    static constexpr int n_parts = kParts * kPairs;
     // record buffers: two where the shape's CTAs still fit an SM (static shared memory and
     // the 1 KB the system takes per CTA included)
     static constexpr int buffers =
@@ -65,11 +71,6 @@ __device__ __forceinline__ double quartic_tt1(const RegK& r, const TangDiffs& x)
 // j-2..j+2 of one face) and the reconstruction along the face there.  The
 // segment's slice (segment_parts; part j of variable k at part[(kPartsVar k + j)
 // * stride]) holds what its two Gauss points share.
-// Parts of a variable: W0, twice its tangential slope per unit eta and its normal derivative
-// at eta = -g and +g; twice the slopes of W_l and W_r; as pairs of FP32 what the second derivatives
-// need (d2/deta2 = PTT0 + eta PTT1, d2/dn deta = PNT0 + eta PNT1; the host operation
-// count keeps them in FP64).
-enum { PV = 0, PT = 2, PN = 4, PS = 6, PTT0 = 8, PTT1, PNT0, PNT1, kPartsVar, kParts = 4 * kPartsVar };
 constexpr double kGauss = 0.28867513459481287;   // 1/(2 sqrt 3): Gauss points at +-kGauss
 
 struct SegmentPoint {
@@ -87,6 +88,17 @@ struct SegmentPoint {
         return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off);
     }
     __device__ __forceinline__ double P(int k, int j) const { return part[(kPartsVar * k + j) * stride]; }
+#ifdef CGKS_PAIRS
+    // the same where a slot may hold a pair instead: read again where it is used (a value kept from the
+    // pair's read to there costs two registers for each of 16 slots, 100 B of spills in all)
+    __device__ __forceinline__ double P64(int k, int j) const { return ((volatile const double*)part)[(kPartsVar * k + j) * stride]; }
+    // the variables with FP64 parts (segment_parts), a bit each
+    __device__ __forceinline__ int rough() const
+    {
+        const volatile int* m = (const volatile int*)(part + kRough * stride);
+        return m[0] | m[1];
+    }
+#endif
 
     __device__ __forceinline__ void eq_value(double W[4]) const
     {
@@ -103,7 +115,8 @@ struct SegmentPoint {
         }
     }
 
-    // the second derivatives in FP64, from the rows
+    // the second derivatives in FP64: from the slice where it holds their parts so, else from the rows (always
+    // from the rows took 124 of a rough point's FP64 instructions)
     __device__ __forceinline__ void eq_second(double W0nn[4], double W0nt[4], double W0tt[4]) const
     {
         const double iht2 = r.mul(iht, iht);
@@ -114,6 +127,11 @@ struct SegmentPoint {
             W0tt[k] = r.mul(fma(eta, P(k, PTT1), P(k, PTT0)), iht2);
             W0nt[k] = r.mul(fma(eta, P(k, PNT1), P(k, PNT0)), iht);
 #else
+            if (rough() >> k & 1) {
+                W0tt[k] = r.mul(fma(eta, P64(k, PTT1), P64(k, PTT0)), iht2);
+                W0nt[k] = r.mul(fma(eta, P64(k, PNT1), P64(k, PNT0)), iht);
+                continue;
+            }
             TangDiffs x;
             tang_diffs(r, at(RV, k, -2), at(RV, k, -1), at(RV, k, 0), at(RV, k, 1), at(RV, k, 2), x);
             W0tt[k] = r.mul(fma(eta, quartic_tt1(r, x), quartic_tt0(r, x)), iht2);
@@ -172,11 +190,16 @@ struct SegmentPoint {
 // What the Gauss points of a segment share, for variables k0..k1-1.  Corrections in
 // pairs of FP32 where the rows' differences are small beside the variable's scale (ihn:
 // inverse spacing along the normal, for the derivative rows' differences), else in FP64.
+// A variable whose rows are too rough for that has its second derivatives' parts in FP64 and its bit in the
+// kRough slot set.  On rough data everywhere (512^2, stage 1 / 2) an all-FP64 kernel took 2170 /
+// 1805 us, this one 2411 / 2050 with pairs tried first for every part of every point, and 2137 / 1800 where a rough
+// variable is left out of what hardly ever qualifies then.
 // A rolled loop: unrolled, its instructions alone outgrow the instruction cache.
 __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, int pa, int pb, int pc, int r0,
                                               int rstride, double ihn, int k0, int k1, double* part, int stride)
 {
     const double weps = r.k(FK_WEPS), weps4 = r.k(FK_WEPS4);
+    int rough = 0;
     auto R = [&](int f, int k, int off) { return rec_at(rec, pa, pb, pc, r0, rstride, f, k, off); };
 #ifdef CGKS_PAIRS
     // scales (high words): the smallest of the three states' densities and energies; a
@@ -228,34 +251,32 @@ __device__ __forceinline__ void segment_parts(const RegK& r, const double* rec, 
         }
 #endif
         if (!split) {
+            rough |= 1 << k;
             TangDiffs x;
             tang_diffs(r, R(RV, k, -2), R(RV, k, -1), m0, R(RV, k, 1), R(RV, k, 2), x);
             tang_weno5_pair(r, m0, x, weps4, p[(PV + 0) * stride], p[(PV + 1) * stride]);
             const double t0 = quartic_t0(r, x), t2 = r.add(t0, t0), gt = r.mul(2.0 * kGauss, quartic_t1(r, x));
             p[(PT + 0) * stride] = r.sub(t2, gt);
             p[(PT + 1) * stride] = r.add(t2, gt);
-#ifndef CGKS_PAIRS
             p[PTT0 * stride] = quartic_tt0(r, x);
             p[PTT1 * stride] = quartic_tt1(r, x);
-#else
-            p[PTT0 * stride] = ff_pack(ff_from_any(quartic_tt0(r, x)));
-            p[PTT1 * stride] = ff_pack(ff_from_any(quartic_tt1(r, x)));
-#endif
             tang_diffs(r, R(RN, k, -2), R(RN, k, -1), n0, R(RN, k, 1), R(RN, k, 2), x);
             const double v0 = quartic_v0(r, n0, x), gv = r.mul(kGauss, quartic_v1(r, x));
             p[(PN + 0) * stride] = r.sub(v0, gv);
             p[(PN + 1) * stride] = r.add(v0, gv);
-#ifndef CGKS_PAIRS
             p[PNT0 * stride] = quartic_t0(r, x);
             p[PNT1 * stride] = quartic_t1(r, x);
-#else
-            p[PNT0 * stride] = ff_pack(ff_from_any(quartic_t0(r, x)));
-            p[PNT1 * stride] = ff_pack(ff_from_any(quartic_t1(r, x)));
-#endif
         }
-        tang_weno3_slopes(r, R(RL, k, -1), R(RL, k, 0), R(RL, k, 1), R(RR, k, -1), R(RR, k, 0), R(RR, k, 1), weps, sc,
-                          p[(PS + 0) * stride], p[(PS + 1) * stride]);
+        // (a scale of 0 admits no pairs)
+        tang_weno3_slopes(r, R(RL, k, -1), R(RL, k, 0), R(RL, k, 1), R(RR, k, -1), R(RR, k, 0), R(RR, k, 1), weps,
+                          split ? sc : 0, p[(PS + 0) * stride], p[(PS + 1) * stride]);
     }
+#ifdef CGKS_PAIRS
+    // each of a pair's lanes has a half of the slot (one thread with all variables has both)
+    int* m = (int*)(part + kRough * stride);
+    m[k0 >> 1] = rough;
+    if (k1 - k0 == 4) m[1] = rough;
+#endif
 }
 
 // The results of one Gauss point (stage 1: Fb, Ft, Wm, Wb; stage 2: Ft, Wtt in a, b).

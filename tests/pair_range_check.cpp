@@ -103,7 +103,7 @@ int main()
     for (int er : {-60, -50, -38, -30, -20, 0, 10, 13, 20})
         for (int ea : {-24, -12, 0, 10, 15, 20, 26, 30})
             for (int el : {-120, -60, -30, -23, -13, -7, 0, 10, 13, 17, 30, 33, 60, 120})
-                for (int lev : {3, 6, 10})
+                for (int lev : {2, 3, 6, 10})
                     for (int n = 0; n < 6; ++n) segment(g, Case{er, ea, el, std::ldexp(1.0, -lev), n % 2 == 1});
     return 0;
 }
