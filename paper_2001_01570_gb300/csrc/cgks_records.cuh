@@ -216,6 +216,7 @@ __device__ __forceinline__ void cons_record(const RegK& r, const double Q[4], co
 
 #ifndef CGKS_PAIRS
 inline int scale_of(int, double, double, double, double) { return 0; }
+inline int char_scale(int, double, double) { return 0; }
 #else
 // High word of the scale a variable's rounding is measured against: density and
 // energy against the values on the face's two sides (b, c); a momentum also
@@ -227,6 +228,14 @@ __device__ __forceinline__ int scale_of(int k, double b, double c, double rho, d
     int s = i_max(hi_abs(b), hi_abs(c));
     if (k == 1 || k == 2) s = i_max(s, (int)(((unsigned)hi_abs(rho) + (unsigned)hi_abs(E)) >> 1));
     return s;
+}
+
+// The same for characteristic field m: the density, whose dimension the acoustic and the entropy fields
+// have; the shear field (2) has a momentum's, so sqrt(rho E).
+__device__ __forceinline__ int char_scale(int m, double rho, double E)
+{
+    const int s = hi_abs(rho);
+    return m == 2 ? (int)(((unsigned)s + (unsigned)hi_abs(E)) >> 1) : s;
 }
 #endif
 
@@ -250,19 +259,18 @@ __device__ __forceinline__ void linear_fields(const RegK& r, const double Q[4], 
 // Characteristic variables: the basis is taken at the mean of the two cells sharing the face (b, c) ...
 __device__ __forceinline__ double char_mean(const RegK& r, double b, double c) { return r.mul(0.5, r.add(b, c)); }
 
-// ... and a field's WENO-Z step, from its projections Q and h times its projected gradients S;
-// w[0..3]: left and right value, left and right slope per unit length.
+// ... and a field's WENO-Z step, from its projections Q and h times its projected gradients S (scale_hi:
+// char_scale); w[0..3]: left and right value, left and right slope per unit length.
 template <int ORDER>
-__device__ __forceinline__ void char_weno(const RegK& r, double rho, const double Q[4], const double S[4], double ih,
+__device__ __forceinline__ void char_weno(const RegK& r, int scale_hi, const double Q[4], const double S[4], double ih,
                                           double weno_eps, double w[4])
 {
 #ifndef CGKS_PAIRS
     weno_pair_rk(r, Q[0], Q[1], Q[2], Q[3], S[0], S[1], S[2], S[3], weno_eps, w[0], w[2], w[1], w[3]);
 #else
-    // every characteristic field is measured against the density, whose dimension it has
     RowDiffs x;
     row_diffs_rk(r, Q, S, x);
-    weno_pair_row<ORDER>(r, Q, S, x, r.kmul(RK_HALF, x.d2), weno_eps, hi_abs(rho), w[0], w[2], w[1], w[3]);
+    weno_pair_row<ORDER>(r, Q, S, x, r.kmul(RK_HALF, x.d2), weno_eps, scale_hi, w[0], w[2], w[1], w[3]);
 #endif
     w[2] = r.mul(w[2], ih);
     w[3] = r.mul(w[3], ih);
@@ -293,7 +301,7 @@ __device__ __forceinline__ void char_record(const RegK& r, double gamma, const d
             Q[c] = char_project(r, m, l, Qa[0][c], Qa[1][c], Qa[2][c], Qa[3][c]);
             S[c] = r.mul(h, char_project(r, m, l, Na[0][c], Na[1][c], Na[2][c], Na[3][c]));
         }
-        char_weno<ORDER>(r, Wref[0], Q, S, ih, weno_eps, v);
+        char_weno<ORDER>(r, char_scale(m, Wref[0], Wref[3]), Q, S, ih, weno_eps, v);
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[q][m] = v[q];
     }
@@ -445,7 +453,7 @@ __device__ __forceinline__ void char_row_quad(const RegK& r, const GridDev& G, c
     }
     quad_transpose(quad, m, P);
     quad_transpose(quad, m, S);
-    char_weno<ORDER>(r, Wref[0], P, S, q.ih, G.weno_eps, w);
+    char_weno<ORDER>(r, char_scale(m, Wref[0], Wref[3]), P, S, q.ih, G.weno_eps, w);
     quad_transpose(quad, m, w);
     char_to_cons(r, cs, w, o4);
     const int f = m == 0 ? RL : m == 1 ? RR : m == 2 ? RLN : RRN;

@@ -83,3 +83,13 @@ int main()
     subprocess.run(["g++", "-O1", "-std=c++17", "-I", CSRC, "-o", exe, str(src)], check=True)
     rel, low, bad = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
     assert float(rel) <= 2.0 ** -47 and float(low) < 2.0 ** -97 and int(bad) == 0
+
+
+def test_shear_is_measured_against_its_own_scale(tmp_path):
+    """Characteristic variables, a shear layer in gases whose speed of sound is 1 to 2^-12 of the unit of
+    velocity: the WENO-Z values' bound of tests/test_split_host.py (2^-51 of the scale, here rho, rho c and rho c^2)
+    once for the field and once for the basis it goes through."""
+    a, b = (np.frombuffer(subprocess.run([build(tmp_path, "char_scale_check.cpp", *d)], check=True, capture_output=True).stdout)
+            .reshape(13, -1, 2, 2, 4) for d in ((), ("-DCGKS_SPLIT_CHECK=1",)))
+    worst = (np.abs(a[:, :, 0] - b[:, :, 0]) / a[:, :, 1]).max(axis=(1, 2))
+    assert (worst[0, 2] > 0) and np.all(worst <= 2.0 ** -50), np.log2(np.maximum(worst, 2.0 ** -60)).round(1)
