@@ -306,7 +306,7 @@ static cgks_status set_state_impl(cgks_solver* s, const double* planes, int on_d
     if (s->prob.dim == 1) {
         const bool direct = on_device && kernel_access(s, planes);
         if (!direct) CK(cudaMemcpyAsync(s->d_stage1d, planes, 6 * PL * sizeof(double), kind, s->stream));
-        CK(launch_set_state_1d(s->d_desc, direct ? planes : s->d_stage1d, t, steps, s->stream));
+        CK(launch_set_state_1d(s->d_desc, s->host_desc, direct ? planes : s->d_stage1d, t, steps, s->stream));
     } else {
         CK(launch_set_ctrl(s->d_ctrl, t, 0.0, -1, 1, s->stream, steps));
         CK(cudaMemcpyAsync(s->host_desc.buf[0], planes, 12 * PL * sizeof(double), kind, s->stream));

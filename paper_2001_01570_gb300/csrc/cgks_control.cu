@@ -101,22 +101,24 @@ __global__ void batch_resume_kernel(const GridDev* grids, int n)
 }
 
 // The state of a 1D grid (6 planes: rho, rhoU, rhoE, their x-gradients) into the internal
-// 2D layout, with the control block of a solve that starts there and the state's speed
-// maxima: one CTA, one launch (a batch of small grids is set one by one).
+// 2D layout, with the state's speed maxima and, run by one CTA (one_cta), the control block of a solve
+// that starts there; before several CTAs a launch of its own has reset the block.
 __global__ void __launch_bounds__(256) set_state_1d_kernel(const GridDev* grids, const double* src, double t,
-                                                           long long steps0)
+                                                           long long steps0, int one_cta)
 {
     const GridDev& G = grids[0];
     Ctrl* C = G.ctrl;
-    if (threadIdx.x == 0) {
-        set_ctrl(C, t, 0.0, -1, 1, steps0);
-        __threadfence_block();
+    if (one_cta) {
+        if (threadIdx.x == 0) {
+            set_ctrl(C, t, 0.0, -1, 1, steps0);
+            __threadfence_block();
+        }
+        __syncthreads();
     }
-    __syncthreads();
     const int nx = G.nx;
     double* dst = G.buf[0];
     SpeedMax s;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nx; i += gridDim.x * blockDim.x) {
         double v[6];
 #pragma unroll
         for (int p = 0; p < 6; ++p) v[p] = src[(size_t)p * nx + i];
@@ -175,9 +177,18 @@ cudaError_t launch_batch_resume(const GridDev* grids, int n, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_set_state_1d(const GridDev* grids, const double* src, double t, long long steps0, cudaStream_t st)
+// A thread per cell; one CTA's worth in one launch (a batch of small grids is set one by one), more after
+// a launch for the control block.  A whole call with one CTA at any size / so: 256 cells 14.7 / 14.9 us,
+// 512 17.9 / 16.5, 2048 33 / 16, 2^20 10766 / 89 (four launches of a kind each: 24, 23, 23, 136).
+cudaError_t launch_set_state_1d(const GridDev* grids, const GridDev& host, const double* src, double t, long long steps0,
+                                cudaStream_t st)
 {
-    set_state_1d_kernel<<<1, 256, 0, st>>>(grids, src, t, steps0);
+    const int blocks = host.nx < 1024 * 256 ? (host.nx + 255) / 256 : 1024;
+    if (blocks > 1) {
+        const cudaError_t e = launch_set_ctrl(host.ctrl, t, 0.0, -1, 1, st, steps0);
+        if (e != cudaSuccess) return e;
+    }
+    set_state_1d_kernel<<<blocks, 256, 0, st>>>(grids, src, t, steps0, blocks == 1);
     return cudaGetLastError();
 }
 

@@ -249,7 +249,8 @@ cudaError_t launch_end_step(const GridDev* grids, int ngrids, cudaStream_t st);
 cudaError_t launch_cfl(const GridDev* grids, int gidx, const GridDev& host, cudaStream_t st);
 // grids[0]'s state from 6 device planes (1D), with its control block reset; its current state
 // to device planes
-cudaError_t launch_set_state_1d(const GridDev* grids, const double* src, double t, long long steps0, cudaStream_t st);
+cudaError_t launch_set_state_1d(const GridDev* grids, const GridDev& host, const double* src, double t, long long steps0,
+                                cudaStream_t st);
 cudaError_t launch_get_state(const GridDev* grids, const GridDev& host, double* dst, cudaStream_t st);
 // reset != 0: the control block starts a solve at time t with `steps0` steps
 // already taken (0 for a new solve, the checkpoint's count on a restore)
