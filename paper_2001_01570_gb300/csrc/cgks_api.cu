@@ -288,13 +288,13 @@ cgks_status cgks_destroy(cgks_solver* s)
     return CGKS_OK;
 }
 
-// whether this solver's kernels may read and write device planes at p directly: memory of its
-// own device, aligned (a copy takes any other)
+// planes_direct for this solver and a pointer from the caller
 static bool kernel_access(const cgks_solver* s, const void* p)
 {
     cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
-    return a.type == cudaMemoryTypeDevice && a.device == s->device && ((uintptr_t)p & 7) == 0;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+    return planes_direct(a.type == cudaMemoryTypeDevice ? a.device : -1, s->device, dev, p);
 }
 
 static cgks_status set_state_impl(cgks_solver* s, const double* planes, int on_device, double t, long long steps)

@@ -228,6 +228,14 @@ cudaError_t launch_chained(void (*kernel)(P...), int blocks, int threads, size_t
 }
 #endif
 
+// Whether a kernel launched now may read and write a caller's planes at p directly: memory of the solver's
+// own device (planes_device: -1 if no device's), which is also the current one (a kernel on the NULL stream
+// runs there), aligned.  A copy takes any other.
+inline bool planes_direct(int planes_device, int solver_device, int current_device, const void* p)
+{
+    return planes_device >= 0 && planes_device == solver_device && current_device == solver_device && ((uintptr_t)p & 7) == 0;
+}
+
 // launchers (defined in the kernel translation units).  The persistent kernels
 // stride over a work queue of `n` entries; a non-NULL `dcount` points to an int
 // in device memory that holds the queue's current length instead (read when the
