@@ -332,8 +332,12 @@ cgks_status cgks_get_state(cgks_solver* s, double* planes, int on_device, double
     Ctrl c;
     const size_t PL = (size_t)s->nx * s->ny;
     // device planes: a kernel picks the buffer, so one synchronisation serves the planes and the
-    // control block
-    const bool direct = planes && on_device && kernel_access(s, planes);
+    // control block.  2D planes above kDirectCells are copied once the control block has told the buffer: the
+    // copy engine is faster than the kernel by more than a synchronisation (kernel / copy, a whole call: 64^2
+    // 21 / 25 us, 256^2 24 / 27, 384^2 31 / 27, 512^2 32 / 31, 2048^2 167 / 143); 1D planes have no copy of
+    // one piece (2^20 cells 44 / 59).
+    constexpr size_t kDirectCells = 65536;
+    const bool direct = planes && on_device && (s->prob.dim == 1 || PL <= kDirectCells) && kernel_access(s, planes);
     if (direct) CK(launch_get_state(s->d_desc, s->host_desc, planes, s->stream));
     cgks_status st = read_ctrl(s, &c);
     if (st != CGKS_OK) return st;
