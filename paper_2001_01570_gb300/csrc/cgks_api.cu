@@ -410,7 +410,7 @@ static cgks_status step_impl(cgks_solver* s, int nsteps, double t_end, double* t
     long launches = 0;
     CK(launch_set_ctrl(s->d_ctrl, 0.0, t_end > 0.0 ? t_end : 0.0, -1, 0, s->stream));
     launches += 1;
-    if (!fused) {
+    if (!fused && nsteps > 0) {
         CK(launch_begin_step(s->d_desc, 1, s->stream));   // the later steps start where the one before ends
         launches += 1;
     }

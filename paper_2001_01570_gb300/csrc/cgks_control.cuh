@@ -7,12 +7,17 @@
 
 namespace cgks {
 
+// whether a step can be taken with dt
+__device__ __forceinline__ bool usable_dt(double dt) { return dt > 0.0 && !isinf(dt); }
+
 // Start of a step: dt = CFL * (min over cells of dx/(|U|+c+2 nu/dx), dy/(|V|+c+2 nu/dy)) of the
 // current state, clipped so that t does not pass t_end; marks a grid that is finished.  A
 // function of the control block alone that it leaves valid: running it again before the
-// step gives the same dt.
+// step gives the same dt.  A state without a usable dt is an error if a step is asked of it: right away
+// (raise), or at the end of the step that was begun with it (turn_step, which cannot know whether
+// another step follows).
 template <class C_>
-__device__ __forceinline__ void begin_step(const GridDev& G, C_* C)
+__device__ __forceinline__ void begin_step(const GridDev& G, C_* C, bool raise = true)
 {
     if (C->done) return;
     if (C->status) { C->done = 1; return; }
@@ -21,7 +26,11 @@ __device__ __forceinline__ void begin_step(const GridDev& G, C_* C)
     double d = G.dx / __longlong_as_double((long long)C->amax_bits[0]);
     if (G.dim != 1) d = fmin(d, G.dy / __longlong_as_double((long long)C->amax_bits[1]));
     double dt = G.cfl * d;
-    if (!(dt > 0.0) || isinf(dt)) { C->status |= CGKS_E_NONPHYSICAL; C->done = 1; return; }
+    if (!usable_dt(dt)) {
+        if (raise) { C->status |= CGKS_E_NONPHYSICAL; C->done = 1; }
+        else C->dt = dt;
+        return;
+    }
     if (C->t_end > 0.0 && C->t + dt > C->t_end) dt = C->t_end - C->t;
     C->dt = dt;
 }
@@ -45,8 +54,9 @@ __device__ __forceinline__ void turn_step(const GridDev& G, volatile Ctrl* C)
     Ctrl c;
     c.dt = C->dt; c.t = C->t; c.t_end = C->t_end; c.amax_bits[0] = C->amax_bits[0]; c.amax_bits[1] = C->amax_bits[1];
     c.status = C->status; c.done = C->done; c.par = C->par; c.steps = C->steps; c.steps_target = C->steps_target;
+    if (!usable_dt(c.dt)) c.status |= CGKS_E_NONPHYSICAL;   // the step just run had none: the state before it stays
     end_step(&c);
-    begin_step(G, &c);
+    begin_step(G, &c, false);
     C->dt = c.dt; C->t = c.t; C->status = c.status; C->done = c.done; C->par = c.par; C->steps = c.steps;
 }
 

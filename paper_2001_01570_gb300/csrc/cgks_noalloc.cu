@@ -198,7 +198,7 @@ cgks_status cgks_step_noalloc(const cgks_problem* prob, double* planes, int nste
     NCK(launch_cfl(sym->desc, 0, G, stream));
     const int rblocks = record_blocks(nrc, nsm);
     const int cpt = update_cpt((long long)cells, nsm), ublocks = update_blocks(ncc, nsm, cpt);
-    NCK(launch_begin_step(sym->desc, 1, stream));
+    if (nsteps > 0) NCK(launch_begin_step(sym->desc, 1, stream));
     for (int k = 0; k < nsteps; ++k) {
         for (int stage = 1; stage <= 2; ++stage) {
             NCK(launch_records(stage, cv, sym->desc, sym->rchunks, nrc, rblocks, stream));
