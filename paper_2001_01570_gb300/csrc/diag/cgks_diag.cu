@@ -8,6 +8,9 @@
 //                              units in the last place over n arguments
 //   cgks_diag_rcp_maxulp       RegK::rcp (cgks_device.cuh: rcp.approx + two
 //                              Newton-Raphson steps) against __drcp_rn
+//   cgks_diag_rcp3_maxrel      RegK::rcp3 (one third-order step) and RegK::rsq (1/sqrt, one
+//                              third-order step): largest relative error, from residuals that
+//                              are exact or have twice the precision
 //   cgks_diag_erfc_maxrel      erfc_scaled (the erfcx table of cgks_erfcx_table.h
 //                              times exp_neg(-t^2)) against CUDA's erfc, largest
 //                              relative difference over t in [0, 26]
@@ -66,6 +69,27 @@ __global__ void rcp_kernel(unsigned long long* maxulp, int n)
     x *= (i & 1) ? 1e150 : 1e-150;
     if (i & 2) x = -x;
     atomicMax(maxulp, ulp_diff(r.rcp(x), __drcp_rn(x)));
+}
+
+// relative errors of rcp3 (out[0]) and rsq (out[1]) on the arguments of rcp_kernel (rsq: their
+// magnitudes times 1 and 2), as the bits of non-negative doubles: 1 - x y is exact in one FMA, and 1 - x y^2
+// takes x y as a sum of two
+__global__ void rcp3_kernel(unsigned long long* out, int n)
+{
+    __shared__ double s_fk[FK_NFIX2];
+    const RegK r = diag_table(s_fk);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const unsigned long long mant = ((unsigned long long)i * 0x0000001000000001ULL) & 0x000FFFFFFFFFFFFFULL;
+    double x = __longlong_as_double((long long)(0x3FF0000000000000ULL | mant));
+    x *= (i & 1) ? 1e150 : 1e-150;
+    const double z = (i & 4) ? 2.0 * x : x;
+    if (i & 2) x = -x;
+    const double a = fabs(fma(-x, r.rcp3(x), 1.0));
+    const double y = r.rsq(z), p = __dmul_rn(z, y), q = fma(z, y, -p);
+    const double b = 0.5 * fabs(__dsub_rn(fma(-p, y, 1.0), __dmul_rn(q, y)));
+    atomicMax(out, (unsigned long long)__double_as_longlong(a));
+    atomicMax(out + 1, (unsigned long long)__double_as_longlong(b));
 }
 
 // relative difference as the bits of a non-negative double (ordered like the value)
@@ -158,16 +182,16 @@ void launch_fp64(int op, int blocks, int threads, double* d, unsigned long long*
 }
 
 template <typename F>
-cudaError_t run_max(F launch, unsigned long long* host_out)
+cudaError_t run_max(F launch, unsigned long long* host_out, int count = 1)
 {
     unsigned long long* d = nullptr;
-    cudaError_t e = cudaMalloc(&d, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(d, 0, sizeof(unsigned long long));
+    cudaError_t e = cudaMalloc(&d, count * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(d, 0, count * sizeof(unsigned long long));
     if (e == cudaSuccess) {
         launch(d);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpy(host_out, d, sizeof(unsigned long long), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(host_out, d, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost);
     cudaFree(d);
     return e;
 }
@@ -186,6 +210,15 @@ int cgks_diag_rcp_maxulp(int n, unsigned long long* maxulp)
 {
     if (n <= 0 || !maxulp) return (int)cudaErrorInvalidValue;
     return (int)run_max([n](unsigned long long* d) { rcp_kernel<<<(n + 255) / 256, 256>>>(d, n); }, maxulp);
+}
+
+int cgks_diag_rcp3_maxrel(int n, double maxrel[2])
+{
+    if (n <= 0 || !maxrel) return (int)cudaErrorInvalidValue;
+    unsigned long long bits[2] = {};
+    cudaError_t e = run_max([n](unsigned long long* d) { rcp3_kernel<<<(n + 255) / 256, 256>>>(d, n); }, bits, 2);
+    for (int k = 0; k < 2; ++k) maxrel[k] = __builtin_bit_cast(double, bits[k]);
+    return (int)e;
 }
 
 int cgks_diag_erfc_maxrel(int n, double* maxrel)

@@ -28,6 +28,7 @@ def load():
         u64p = ctypes.POINTER(ctypes.c_ulonglong)
         L.cgks_diag_exp_neg_maxulp.argtypes = [ctypes.c_int, u64p]
         L.cgks_diag_rcp_maxulp.argtypes = [ctypes.c_int, u64p]
+        L.cgks_diag_rcp3_maxrel.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_double)]
         L.cgks_diag_erfc_maxrel.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_double)]
         L.cgks_diag_fp64_rate.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double)]
         _lib = L
@@ -49,6 +50,13 @@ def rcp_maxulp(n=1 << 22) -> int:
     v = ctypes.c_ulonglong()
     _ok(load().cgks_diag_rcp_maxulp(int(n), ctypes.byref(v)), "rcp check")
     return int(v.value)
+
+
+def rcp3_rsq_maxrel(n=1 << 22):
+    """Largest relative errors of RegK::rcp3 and RegK::rsq."""
+    v = (ctypes.c_double * 2)()
+    _ok(load().cgks_diag_rcp3_maxrel(int(n), v), "rcp3 check")
+    return float(v[0]), float(v[1])
 
 
 def erfc_maxrel(n=1 << 22) -> float:
@@ -73,7 +81,8 @@ def main():
     for r in rows:
         print(f"{r['op']:32s} {r['gops']:10.2f} G/s  {r['per_sm_cycle']:6.3f} per SM and cycle  "
               f"SM clock {r['sm_mhz']:7.1f} MHz")
-    checks = {"exp_neg_vs_exp_max_ulp": exp_neg_maxulp(), "rcp_vs_drcp_rn_max_ulp": rcp_maxulp(),
+    rcp3, rsq = rcp3_rsq_maxrel()
+    checks = {"rcp3_max_rel": rcp3, "rsq_max_rel": rsq, "exp_neg_vs_exp_max_ulp": exp_neg_maxulp(), "rcp_vs_drcp_rn_max_ulp": rcp_maxulp(),
               "erfc_scaled_vs_erfc_max_rel": erfc_maxrel()}
     print(json.dumps(checks))
 
