@@ -214,12 +214,12 @@ const char* cgks_last_error(void);
  * state buffer, the intermediate state, the face-row records, the control
  * block and the work queues live in fixed-size device arrays of the library
  * (file-scope __device__ storage, about 12.6 MB of state, 34 MB of face-row
- * records, 17 MB of face results and 300 KB of queues), which every GPU that
+ * records, 17 MB of face results and 350 KB of queues), which every GPU that
  * loads the library holds until the process exits.
  *
  * prob:        2D problem, nx*ny <= CGKS_NOALLOC_MAX_CELLS, nx and ny <=
  *              CGKS_NOALLOC_MAX_SIDE, at most CGKS_NOALLOC_MAX_TILES tiles of
- *              16x8 cells
+ *              8x4 cells (the other two limits allow 3,074)
  * planes:      device pointer, 12 planes of ny*nx doubles (layout above); read
  *              as the initial state and overwritten with the state after the
  *              steps (or the last valid state on CGKS_E_NONPHYSICAL)

@@ -5,9 +5,10 @@
 // On GB300 the FP64 pipe issues about one warp instruction per 16 SM cycles, and
 // only in the register-only DFMA form (RegK below), so the arithmetic is
 // written in that form and to minimise the FP64 instruction count:
-//   * WENO smoothness indicators as quadratic forms in first differences, with
-//     the 19 pair products shared by the left and the mirrored right stencil;
-//   * WENO-Z weights normalised with one reciprocal (leave-one-out products);
+//   * the reconstruction in differences of the stencil data, its WENO-Z corrections in
+//     pairs of FP32 where that loses nothing; where it would, smoothness indicators as
+//     quadratic forms in first differences (19 pair products shared by the left and the
+//     mirrored right stencil) and weights normalised with one reciprocal (leave-one-out products);
 //   * the Euler flux and its time derivative in closed form; only the terms that
 //     genuinely need velocity-space moments (the tau-terms and the half-line
 //     moments of the non-equilibrium states) use them;

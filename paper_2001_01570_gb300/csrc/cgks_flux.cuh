@@ -23,7 +23,7 @@ namespace cgks {
 // (copied from global memory), then the values of the tile's grid and time step
 // (written by the CTA's four warps when a tile's grid is not the tile's before).
 enum FluxK {
-    FK_ONE = 0, FK_NZERO, FK_HALF, FK_MHALF, FK_2, FK_M2, FK_3, FK_4, FK_M4,
+    FK_ONE = 0, FK_NZERO, FK_HALF, FK_MHALF, FK_2, FK_3,
     FK_T13_3, FK_DLO, FK_DHI,              // tangential WENO-Z: 4 x beta weight, linear weights at the Gauss points
     FK_HG, FK_MHG,                         // +-eta/2 at the Gauss point eta = 1/(2 sqrt 3)
     FK_M12TH, FK_M9TH, FK_M4320TH, FK_M7_72,         // quartic through the five means: coefficients
@@ -54,14 +54,14 @@ constexpr FluxFixed make_flux_fixed()
 {
     FluxFixed t{};
     double* k = t.v;
-    k[FK_ONE] = 1.0; k[FK_NZERO] = -0.0; k[FK_HALF] = 0.5; k[FK_MHALF] = -0.5; k[FK_2] = 2.0; k[FK_M2] = -2.0;
-    k[FK_3] = 3.0; k[FK_4] = 4.0; k[FK_M4] = -4.0;
+    k[FK_ONE] = 1.0; k[FK_NZERO] = -0.0; k[FK_HALF] = 0.5; k[FK_MHALF] = -0.5; k[FK_2] = 2.0;
+    k[FK_3] = 3.0;
     const double gq = 0.28867513459481287;               // 1/(2 sqrt 3)
     k[FK_T13_3] = 13.0 / 3.0;
     k[FK_DLO] = kTangLo;
     k[FK_DHI] = kTangHi;
     k[FK_HG] = 0.5 * gq; k[FK_MHG] = -0.5 * gq;
-    // the quartic p(eta) through the five segment means (see SegmentRows::deriv_parts)
+    // the quartic p(eta) through the five segment means (quartic_v0 and the functions after it, cgks_segment.cuh)
     k[FK_M12TH] = -1.0 / 12.0; k[FK_M9TH] = -1.0 / 9.0; k[FK_M4320TH] = -1.0 / 4320.0; k[FK_M7_72] = -7.0 / 72.0;
     k[FK_C1P] = 0.56418958354775628; k[FK_C1M] = -0.56418958354775628;
     k[FK_X32LN2] = 32.0 / 0.6931471805599453;             // 32 / ln 2

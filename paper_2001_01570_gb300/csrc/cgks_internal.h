@@ -138,7 +138,7 @@ enum TileShape { CGKS_FOR_EACH_TILE(CGKS_TILE_ENUM) TILE_COUNT };
 #undef CGKS_TILE_ENUM
 // The tiles of a shape's queue: the shape itself, except that 8x16, the 2D default, is
 // worked on (queued and staged) as 8x4 strips of 64 segments, one pass of a CTA.  The
-// strips' records and slices take 49 KB, so three CTAs fit an SM; a small grid spreads
+// strips' records (two buffers) and slices take 73 KB, so three CTAs fit an SM; a small grid spreads
 // over twice the CTAs of 8x8 strips (when it was chosen, stage 1: 64^2 75.8 -> 42.9 us,
 // 2048^2 18.4 -> 17.8 ms).
 constexpr int work_w(int w, int) { return w; }

@@ -1,6 +1,6 @@
 // cgks_segment.cuh -- the per-face-segment arithmetic of the flux kernel
 // (cgks_stage.cuh): the layout of a tile's face-row records in shared memory,
-// the reconstruction along a face at a Gauss point (SegmentRows) and one
+// the reconstruction along a face at a Gauss point (SegmentPoint) and one
 // segment's two Gauss points with their Gauss average (segment_results).
 #pragma once
 #include "cgks_device.cuh"
@@ -40,7 +40,6 @@ enum { PV = 0, PT = 2, PN = 4, PS = 6, PTT0 = 8, PTT1, PNT0, PNT1, kPartsVar, kR
 
 template <int TX, int TY, int STAGE>
 struct StageLayout {
-    static constexpr int NF = FaceQ<STAGE>::n;
     static constexpr int n_rx = RecGroups<TY, TX + 1>::n;
     static constexpr int n_ry = RecGroups<TX, TY + 1>::n;
     static constexpr int n_rec = n_rx + n_ry;

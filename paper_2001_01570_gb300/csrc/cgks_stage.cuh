@@ -50,7 +50,6 @@ stage_kernel(const GridDev* __restrict__ grids, const TileRef* __restrict__ tile
              const int* __restrict__ dcount)
 {
     using L = StageLayout<TX, TY, STAGE>;
-    constexpr int NF = L::NF;
     extern __shared__ double smem[];
     double* part = smem + L::buffers * L::n_rec + (threadIdx.x >> 1);   // [kParts][kPairs]: this pair's slice
     __shared__ double s_fk[FK_N];       // coefficient table (fixed part, then the tile's grid and dt)
@@ -233,7 +232,8 @@ cudaError_t launch_stage_t(const GridDev* grids, const TileRef* tiles, int ntile
 // per shape, so the shapes compile in parallel).
 #define CGKS_STAGE_INSTANCE(W, H) CGKS_STAGE_INSTANCE_(W, H, work_w(W, H), work_h(W, H))
 #define CGKS_STAGE_INSTANCE_(W, H, TX, TY)                                                                  \
-    static_assert(StageLayout<TX, TY, 1>::bytes + 64 <= 227 * 1024, "stage-1 tile exceeds shared memory");  \
+    static_assert(StageLayout<TX, TY, 1>::bytes + sizeof(double) * FK_N + 16 <= 227 * 1024,                 \
+                  "stage-1 tile exceeds shared memory");                                                    \
     cudaError_t launch_stage_##W##x##H(int stage, const GridDev* grids, const TileRef* tiles, int ntiles,  \
                                          int nblocks, cudaStream_t st, const int* dcount)                   \
     {                                                                                                       \
