@@ -354,7 +354,7 @@ CGKS_SPLIT_FN ff tang_weno3_split(ff A, ff s, ff eps)
 // error below 2^-97 beneath that; the quantities of a face's time derivatives and slope moments carry
 // units (density rho, a speed a, a rate or length), so their pairs are used only where the units keep
 // the operands that matter and all results inside.  Logarithms here are base 2, in units of 2^-20, read
-// off the high words (exact at powers of two, less than 0.09 too large between them); zero gives -1023,
+// off the high words (exact at powers of two, up to 0.09 too small between them); zero gives -1023,
 // infinity and NaN 1024.
 constexpr int kOct = 1 << 20;
 CGKS_SPLIT_FN int hi_log(double x) { return hi_abs(x) - kHiOne; }

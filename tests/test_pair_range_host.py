@@ -93,3 +93,14 @@ def test_shear_is_measured_against_its_own_scale(tmp_path):
             .reshape(13, -1, 2, 2, 4) for d in ((), ("-DCGKS_SPLIT_CHECK=1",)))
     worst = (np.abs(a[:, :, 0] - b[:, :, 0]) / a[:, :, 1]).max(axis=(1, 2))
     assert (worst[0, 2] > 0) and np.all(worst <= 2.0 ** -50), np.log2(np.maximum(worst, 2.0 ** -60)).round(1)
+
+
+def test_each_choice_is_its_bound(tmp_path):
+    """Every function that chooses between the pairs and FP64, on data on both sides of its bound (1 % around it
+    left out), against the bound worked out in FP64; slopes, second derivatives and rows that are infinite, NaN or
+    out of a float's range are refused (tests/pair_choice_check.cpp)."""
+    out = subprocess.run([build(tmp_path, "pair_choice_check.cpp")], check=True, capture_output=True, text=True).stdout
+    rows = [(a[0], *map(int, a[1:])) for a in (ln.split() for ln in out.splitlines())]
+    assert len(rows) == 9
+    for name, yes, no, bad in rows:
+        assert yes > 1000 and no > 1000 and bad == 0, (name, yes, no, bad)
