@@ -70,12 +70,12 @@ OPCOUNT_FLOP_PER_CELL = {"records": 3854.022, "flux": {1: 4746.316, 2: 4466.180}
 TRAFFIC_TILE = "8x16"     # the tile shape the DRAM bytes below were captured on
 # DRAM bytes (read + write) per cell of one stage-1 flux-kernel launch with 8x16 tiles (8x4 strips): ncu
 # dram__bytes_{read,write}.sum of the current kernel on the 1024^2 vortex (records and state larger
-# than L2), 480.56 + 246.52 MB, divided by the cells; the 2048^2 bench grid moves the same bytes per
+# than L2), 480.99 + 247.14 MB, divided by the cells; the 2048^2 bench grid moves the same bytes per
 # cell (its launch is too large to capture under the profiling size rule).
-FLUX_DRAM_BYTES_PER_CELL = {1: (480.558336e6 + 246.522112e6) / 1048576}
+FLUX_DRAM_BYTES_PER_CELL = {1: (480.992768e6 + 247.13728e6) / 1048576}
 # FP64 thread instructions per cell of a stage-1 flux launch (ncu sm__inst_executed_pipe_fp64.sum x 32 on the
 # 1024^2 vortex): what the kernel issues to the FP64 pipe itself; the rest of its formulas runs in pairs of FP32
-FLUX_FP64_INST_PER_CELL = {1: 51522648 * 32 / 1048576}
+FLUX_FP64_INST_PER_CELL = {1: 51786528 * 32 / 1048576}
 # algorithmic bytes per cell of the flux kernel: the two face rows' records (2 x 28 doubles) read and
 # the two faces' results written (stage 1: 16 doubles each, stage 2: 8)
 FLUX_ALGO_BYTES_PER_CELL = {1: 448 + 256, 2: 448 + 128}

@@ -26,7 +26,7 @@
 // parts in registers (255 of them, 1.8 KB of spills once the FP32 pairs came in); one
 // thread per point needs 168 and halves the chain of dependent instructions that a small
 // grid waits for.  Measured per launch, stage 1 / 2: 2048^2 27.66 / 25.41 -> 17.8 / 14.4
-// ms with this split, 13.9 / 12.1 now; 512^2 1.93 / 1.77 -> 1.14 / 0.94, 0.90 / 0.79 ms now;
+// ms with this split, 14.0 / 12.2 now; 512^2 1.93 / 1.77 -> 1.14 / 0.94, 0.90 / 0.79 ms now;
 // 64^2 155 / 138 -> 43 / 38, 37 / 34 us now.
 // Coefficients (fixed, and the tile's grid and dt) come from the shared-memory
 // table of cgks_flux.cuh; all arithmetic is in the register-only DFMA forms.
